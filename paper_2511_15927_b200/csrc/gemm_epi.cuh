@@ -1,0 +1,184 @@
+// Epilogue shared by the tensor-core GEMM kernels: what happens to 32 consecutive accumulator columns of one output row.
+#pragma once
+
+#include "dm_internal.h"
+#include "tc_ptx.cuh"
+
+namespace dm {
+namespace tc {
+
+struct EpiArgs {
+    void *C; int64_t ldc; int c_is_f32;
+    const float *row_scale; const float *addend; int64_t ld_add;
+    int M, N, K;
+    int silu_cols;   // SiLU on output columns below this one
+    const float *col_bias; int gelu; const float *col_scale; int cs_rows; int64_t ld_cs;   // see GemmArgs
+    const int *m_dev; int m_off;
+    int k_off;       // first element along K of this problem's share (split K: the second half of a product is a problem of its own)
+};
+
+// Up to two products of the same M, N, K in one launch (the two directions' in_proj, or their out_proj on short inputs), each optionally
+// cut in two along K (ksplit: problems 2 i and 2 i + 1 are the halves of product i, each with an output of its own that the caller adds): the tile
+// loop runs over all of them, so that they share one tail round and -- for in_proj, whose A operand is the same x -- the rows of A in L2.
+struct EpiPair {
+    EpiArgs p[4];
+    int nprob, ksplit;
+    int n_fast;      // tile order: consecutive tiles step along N (the A rows are streamed once, B stays in L2) or along M
+};
+
+inline EpiArgs epi_of(const GemmArgs &a) {
+    return EpiArgs{a.C, a.ldc, a.c_dtype == DM_F32 ? 1 : 0, a.row_scale, a.addend, a.ld_add, a.M, a.N, a.K, a.silu_cols,
+                   a.col_bias, a.gelu, a.col_scale, a.cs_rows > 0 ? a.cs_rows : 1, a.ld_cs > 0 ? a.ld_cs : (int64_t)a.N, a.m_dev, a.m_off, 0};
+}
+
+// The launch's problems: one product, two (b), or two that are each cut in two along K (hi: fp32 outputs of the second halves, same pitch).
+inline EpiPair epi_pair_of(const GemmArgs &a, const GemmArgs *b, float *const *hi) {
+    EpiPair epp{};
+    if (hi) {
+        const GemmArgs *prod[2] = {&a, b};
+        for (int i = 0; i < 2; ++i) {
+            EpiArgs lo = epi_of(*prod[i]), up = lo;
+            lo.K = up.K = prod[i]->K / 2;
+            up.k_off = lo.K;
+            up.C = hi[i]; up.addend = nullptr; up.col_bias = nullptr;
+            epp.p[2 * i] = lo; epp.p[2 * i + 1] = up;
+        }
+        epp.nprob = 4; epp.ksplit = 1;
+    } else {
+        epp.p[0] = epi_of(a);
+        epp.p[1] = b ? epi_of(*b) : epp.p[0];
+        epp.nprob = b ? 2 : 1;
+    }
+    epp.n_fast = a.M > a.N ? 1 : 0;
+    return epp;
+}
+
+// What is the same for every column of a thread's row
+struct EpiRow {
+    bool wide_c, wide_add;     // 32-byte stores / loads (one full sector per thread): every row of C / of the addend starts on a 32-byte boundary
+    const float *add_row, *cs_row;
+    __device__ __forceinline__ EpiRow(const EpiArgs &ep, int row) {
+        const int c_es = ep.c_is_f32 ? 4 : 2;
+        wide_c = (reinterpret_cast<uintptr_t>(ep.C) & 31u) == 0 && ((ep.ldc * c_es) & 31) == 0;
+        wide_add = ep.addend && (reinterpret_cast<uintptr_t>(ep.addend) & 31u) == 0 && ((ep.ld_add * 4) & 31) == 0;
+        add_row = ep.addend ? ep.addend + (int64_t)row * ep.ld_add : nullptr;
+        cs_row = ep.col_scale ? ep.col_scale + (int64_t)(row / ep.cs_rows) * ep.ld_cs : nullptr;
+    }
+};
+
+// v[j] = accumulator of column col + j, already times the row scale.  ACT: bias and activations may occur.
+template <bool ACT>
+__device__ __forceinline__ void epi_cols32(const EpiArgs &ep, const EpiRow &er, int row, int col, float (&v)[32]) {
+    const bool full = col + 32 <= ep.N;
+    if constexpr (ACT) {
+        if (ep.col_bias) {
+            if (full) {
+#pragma unroll
+                for (int j = 0; j < 32; j += 4) {
+                    const float4 b4 = *reinterpret_cast<const float4 *>(ep.col_bias + col + j);
+                    v[j] += b4.x; v[j + 1] += b4.y; v[j + 2] += b4.z; v[j + 3] += b4.w;
+                }
+            } else {
+#pragma unroll
+                for (int j = 0; j < 32; ++j) if (col + j < ep.N) v[j] += ep.col_bias[col + j];
+            }
+        }
+        if (col < ep.silu_cols) {                  // gate columns: SiLU here, where the ALUs idle, not in the scan
+#pragma unroll
+            for (int j = 0; j < 32; ++j)
+                if (col + j < ep.silu_cols) { const float hv = 0.5f * v[j]; v[j] = fmaf(hv, tanh_fast(hv), hv); }   // SiLU(v) = v/2 + v/2 tanh(v/2)
+        }
+        if (ep.gelu) {
+#pragma unroll
+            for (int j = 0; j < 32; ++j) {                  // GELU, tanh form
+                const float x = v[j], hx = 0.5f * x;
+                v[j] = fmaf(hx, tanh_fast(0.7978845608028654f * fmaf(0.044715f * x, x * x, x)), hx);
+            }
+        }
+    }
+    if (er.cs_row) {
+        const float *cs = er.cs_row + col;
+        if (full) {
+#pragma unroll
+            for (int j = 0; j < 32; j += 4) {
+                const float4 c4 = *reinterpret_cast<const float4 *>(cs + j);
+                v[j] *= c4.x; v[j + 1] *= c4.y; v[j + 2] *= c4.z; v[j + 3] *= c4.w;
+            }
+        } else {
+#pragma unroll
+            for (int j = 0; j < 32; ++j) if (col + j < ep.N) v[j] *= cs[j];
+        }
+    }
+    if (er.add_row) {
+        if (full && er.wide_add) {
+#pragma unroll
+            for (int j = 0; j < 32; j += 8) {
+                uint32_t a8[8];
+                ld_global_256(er.add_row + col + j, a8);
+#pragma unroll
+                for (int e = 0; e < 8; ++e) v[j + e] += __uint_as_float(a8[e]);
+            }
+        } else if (full && (ep.ld_add & 3) == 0) {
+#pragma unroll
+            for (int j = 0; j < 32; j += 4) {
+                const float4 a4 = *reinterpret_cast<const float4 *>(er.add_row + col + j);
+                v[j] += a4.x; v[j + 1] += a4.y; v[j + 2] += a4.z; v[j + 3] += a4.w;
+            }
+        } else {
+#pragma unroll
+            for (int j = 0; j < 32; ++j) if (col + j < ep.N) v[j] += er.add_row[col + j];
+        }
+    }
+    if (ep.c_is_f32) {
+        float *crow = static_cast<float *>(ep.C) + (int64_t)row * ep.ldc + col;
+        if (full && er.wide_c) {
+#pragma unroll
+            for (int j = 0; j < 32; j += 8) {
+                uint32_t o[8];
+#pragma unroll
+                for (int e = 0; e < 8; ++e) o[e] = __float_as_uint(v[j + e]);
+                st_global_256(crow + j, o);
+            }
+        } else if (full && (ep.ldc & 3) == 0) {
+#pragma unroll
+            for (int j = 0; j < 32; j += 4) *reinterpret_cast<float4 *>(crow + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+        } else {
+#pragma unroll
+            for (int j = 0; j < 32; ++j) if (col + j < ep.N) crow[j] = v[j];
+        }
+    } else {
+        __nv_bfloat16 *crow = static_cast<__nv_bfloat16 *>(ep.C) + (int64_t)row * ep.ldc + col;
+        if (full && er.wide_c) {
+#pragma unroll
+            for (int j = 0; j < 32; j += 16) {
+                uint32_t o[8];
+#pragma unroll
+                for (int e = 0; e < 8; ++e) o[e] = pack_bf16(v[j + 2 * e], v[j + 2 * e + 1]);
+                st_global_256(crow + j, o);
+            }
+        } else if (full && (ep.ldc & 7) == 0) {
+#pragma unroll
+            for (int j = 0; j < 32; j += 8)
+                *reinterpret_cast<uint4 *>(crow + j) = make_uint4(pack_bf16(v[j], v[j + 1]), pack_bf16(v[j + 2], v[j + 3]),
+                                                                 pack_bf16(v[j + 4], v[j + 5]), pack_bf16(v[j + 6], v[j + 7]));
+        } else {
+#pragma unroll
+            for (int j = 0; j < 32; ++j) if (col + j < ep.N) crow[j] = __float2bfloat16_rn(v[j]);
+        }
+    }
+}
+
+// 2-D bf16 tensor [rows, cols] with row pitch ld elements; box = [box_rows, 64 columns], 128-byte swizzle.
+inline bool make_map_2d(CUtensorMap *m, const void *base, int64_t rows, int64_t cols, int64_t ld, int box_rows) {
+    const uint64_t dims[2] = {(uint64_t)cols, (uint64_t)rows};
+    const uint64_t strides[1] = {(uint64_t)ld};
+    const uint32_t box[2] = {64, (uint32_t)box_rows};
+    return make_map_bf16(m, base, 2, dims, strides, box);
+}
+
+}  // namespace tc
+
+// gemm_pair.cu: the two-CTA kernel.  wide: 256 x 256 tiles, else 256 x 128; b, hi: see gemm_tcgen05.cu.
+cudaError_t gemm_pair_launch(bool wide, const GemmArgs &a, const GemmArgs *b, float *const *hi, cudaStream_t s);
+
+}  // namespace dm
