@@ -1,19 +1,24 @@
 // Bidirectional multi-head attention for the hybrid variant (Sec. 3.3: one attention mixer every N mixer blocks):
 //     O_h = softmax(Q_h K_h^T / sqrt(d_h)) V_h        full (non-causal), no position encoding, d_h = 64 or 80.
-// One CTA per (128-query tile, head, sequence) walks the keys in tiles of 128 with the running-maximum form of the
-// softmax, so the L x L score matrix never leaves the SM:
-//     warp 0      TMA loads: the Q tile once, K and V tiles double-buffered
-//     warp 1      one thread issues  S = Q K^T  (both operands K-major in shared memory, fp32 accumulator in TMEM) and
-//                 O += P V  (A = P from TMEM as bf16, B = V [key][d_h] MN-major)
-//     warps 2-5   one query row per thread: S row -> running max m and sum l, P = 2^(s - m) as bf16 into TMEM, O scaled by
-//                 2^(m_old - m_new) in TMEM; at the end O / l -> bf16 -> global
-// A CTA holds 256 TMEM columns (S 128, P 64, O 64) and 82 KB of shared memory, so two CTAs share an SM: while one is in
-// its softmax (latency bound: one warp per scheduler), the other one's products and softmax fill the gaps.
+// One CTA per (256 queries, head, sequence), as two streams of 128 queries that share the key and value tiles; the running-maximum form
+// of the softmax, so the L x L score matrix never leaves the SM:
+//     warp 0       TMA loads: the two Q tiles once, K and V tiles through a ring
+//     warp 1       issues, per key tile and stream, S = Q K^T (both operands K-major in shared memory, fp32 accumulator in TMEM) and
+//                  O += P V (A = P from TMEM as bf16, B = V [key][d_h] MN-major)
+//     warps 4-7, 8-11   softmax of stream 0 and 1, one query row per thread: the row of S into registers, maximum, P = 2^(s - m) as bf16 into TMEM
+//                  and its sum; at the end O / l -> bf16 -> global
+// S(j + 1) of a stream is issued as soon as its softmax warps hold S(j) in registers (P has TMEM columns of its own), so the products run
+// under the softmax, and the two streams fall out of step by themselves: while one waits, the other one has the exponential unit.  What bounds
+// it is that unit: 128 x 128 exponentials take 1024 clocks of an SM, their products 512.  B=4, L=4096, 16 heads of 64: 378 us, 0.73 PFLOP/s (620 us with
+// one stream per CTA, two CTAs per SM, O scaled for every tile); B=8, L=1024, 24 heads of 80: 93 us (230 us).
+// The maximum m that P and O are relative to is only raised when a row's scores exceed it by more than 2^8: P then stays within what bf16 and
+// the fp32 sums hold without loss, and O is read back from TMEM and scaled for a few tiles per row instead of for each one.
 // Heads of 80 channels (the paper's 1.3B hybrid, d = 1920 with 24 heads): every Q, K, V tile is two 64-column sub-tiles, the head's
 // channels 0..63 and the 64 columns from channel 64 on, of which the products use the first 16 (the rest belongs to the next head, or is
-// the zero fill beyond the tensor, and is never read): one more K step of 16 for S, one more product of 16 columns for O.  Twice the
-// shared memory and 512 TMEM columns: one CTA per SM.
+// the zero fill beyond the tensor, and is never read): one more K step of 16 for S, one more product of 16 columns for O.  Key tiles of 96 there:
+// S, P and O of two streams then fit the 512 TMEM columns.
 // Every wait is bounded; on expiry the CTA stores DM_ERR_TIMEOUT in the device status word and leaves.
+// Few queries (block decoding) go to attention_block.cu.
 #include "dm_internal.h"
 #include "tc_ptx.cuh"
 
@@ -21,13 +26,20 @@ namespace dm {
 using namespace tc;
 namespace {
 
-constexpr int BQ = 128, BK = 128, SUB = 64, NTHREADS = 192;       // SUB: columns of a sub-tile (128 bytes: one swizzle atom)
-constexpr uint32_t TILE = BQ * SUB * 2;                     // 16 KB: 128 rows of 128 bytes
-constexpr uint32_t TM_S = 0, TM_P = 128, TM_O = 192;      // S fp32 128 columns, P bf16 64, O fp32 64 or 80
-constexpr uint32_t smem_bytes(int nt) { return 5 * nt * TILE + 1024 + 1024; }
+constexpr int BQ = 128, SUB = 64, NTHREADS = 384;           // SUB: columns of a sub-tile (128 bytes: one swizzle atom)
+constexpr float RESCALE_LOG2 = 8.f;
+
+// NT: sub-tiles per operand tile; 1 = heads of 64 channels, 2 = heads of 80
+template <int NT> struct Cfg {
+    static constexpr int DH = NT == 1 ? 64 : 80, BK = NT == 1 ? 128 : 96, STAGES = NT == 1 ? 4 : 3;
+    static constexpr uint32_t QTILE = BQ * 128, KTILE = BK * 128, Q_BYTES = NT * QTILE, KV_BYTES = NT * KTILE;
+    static constexpr uint32_t OFF_K = 2 * Q_BYTES, OFF_V = OFF_K + STAGES * KV_BYTES, OFF_BAR = OFF_V + STAGES * KV_BYTES, SMEM = OFF_BAR + 1024 + 1024;
+    static constexpr uint32_t TM_P = 2 * BK, TM_O = TM_P + BK;               // S of stream s at s BK, its P at TM_P + s BK / 2, its O at TM_O + s DH
+    static_assert(TM_O + 2 * DH <= 512 && SMEM <= 232448, "TMEM and shared memory budget");
+};
 
 struct Bars {
-    uint64_t q_full, k_full[2], k_empty[2], v_full[2], v_empty[2], s_full, s_empty, p_full, o_done;
+    uint64_t q_full, k_full[4], k_empty[4], v_full[4], v_empty[4], s_full[2], s_empty[2], p_full[2], o_done[2];
     uint32_t tmem_base;
     int abort;
 };
@@ -39,36 +51,34 @@ struct AttnArgs {
     float scale_log2;            // log2(e) / sqrt(d_h)
 };
 
-// NT: sub-tiles per operand tile; 1 = heads of 64 channels, 2 = heads of 80
 template <int NT>
-__global__ void __launch_bounds__(NTHREADS, 3 - NT)
+__global__ void __launch_bounds__(NTHREADS, 1)
 attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                  const __grid_constant__ CUtensorMap map_v, const AttnArgs a, int *status) {
+    using C = Cfg<NT>;
+    constexpr int DH = C::DH, BK = C::BK, STAGES = C::STAGES;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
-    constexpr int DH = NT == 1 ? 64 : 80;
-    constexpr uint32_t OPND = NT * TILE;                        // bytes of one operand tile
-    constexpr uint32_t OFF_Q = 0, OFF_K = OPND, OFF_V = 3 * OPND, OFF_BAR = 5 * OPND;
-    constexpr uint32_t TM_COLS = NT == 1 ? 256 : 512;
-    Bars *bars = reinterpret_cast<Bars *>(smem + OFF_BAR);
+    Bars *bars = reinterpret_cast<Bars *>(smem + C::OFF_BAR);
     volatile int *abort_flag = &bars->abort;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int q0 = blockIdx.x * BQ, h = blockIdx.y, b = blockIdx.z;
+    const int q0 = blockIdx.x * 2 * BQ, h = blockIdx.y, b = blockIdx.z;
     const int n_kv = (a.Lk + BK - 1) / BK;
 
     if (tid == 0) {
         mbar_init(&bars->q_full, 1);
-        for (int i = 0; i < 2; ++i) {
+        for (int i = 0; i < STAGES; ++i) {
             mbar_init(&bars->k_full[i], 1); mbar_init(&bars->k_empty[i], 1);
             mbar_init(&bars->v_full[i], 1); mbar_init(&bars->v_empty[i], 1);
         }
-        mbar_init(&bars->s_full, 1); mbar_init(&bars->s_empty, 128);
-        mbar_init(&bars->p_full, 128);
-        mbar_init(&bars->o_done, 1);
+        for (int i = 0; i < 2; ++i) {              // one arrival per softmax warp of the stream
+            mbar_init(&bars->s_full[i], 1); mbar_init(&bars->s_empty[i], 4);
+            mbar_init(&bars->p_full[i], 4); mbar_init(&bars->o_done[i], 1);
+        }
         bars->abort = 0;
         mbar_fence_init();
     }
-    if (warp == 1) tmem_alloc(&bars->tmem_base, TM_COLS);
+    if (warp == 1) tmem_alloc(&bars->tmem_base, 512);
     fence_before();
     __syncthreads();
     fence_after();
@@ -78,186 +88,178 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     if (warp == 0) {
         // ------------------------------------------------------------ TMA producer
         if (lane == 0) {
-            mbar_expect_tx(&bars->q_full, OPND);
+            mbar_expect_tx(&bars->q_full, 2 * C::Q_BYTES);
 #pragma unroll
-            for (int u = 0; u < NT; ++u) tma_load_3d(smem + OFF_Q + u * TILE, &map_q, h * DH + u * SUB, q0, b, &bars->q_full);
+            for (int i = 0; i < 2; ++i)
+#pragma unroll
+                for (int u = 0; u < NT; ++u) tma_load_3d(smem + i * C::Q_BYTES + u * C::QTILE, &map_q, h * DH + u * SUB, q0 + i * BQ, b, &bars->q_full);
             int issued_k = 0, issued_v = 0;
             for (int j = 0; j < n_kv; ++j) {
-                const int st = j & 1;
-                const uint32_t ph = (j >> 1) & 1;
+                const int st = j % STAGES;
+                const uint32_t ph = (j / STAGES) & 1;
                 if (!WAIT(&bars->k_empty[st], ph ^ 1)) break;
-                mbar_expect_tx(&bars->k_full[st], OPND);
+                mbar_expect_tx(&bars->k_full[st], C::KV_BYTES);
 #pragma unroll
-                for (int u = 0; u < NT; ++u) tma_load_3d(smem + OFF_K + st * OPND + u * TILE, &map_k, a.kx0 + h * DH + u * SUB, j * BK, b, &bars->k_full[st]);
+                for (int u = 0; u < NT; ++u) tma_load_3d(smem + C::OFF_K + st * C::KV_BYTES + u * C::KTILE, &map_k, a.kx0 + h * DH + u * SUB, j * BK, b, &bars->k_full[st]);
                 issued_k = j + 1;
                 if (!WAIT(&bars->v_empty[st], ph ^ 1)) break;
-                mbar_expect_tx(&bars->v_full[st], OPND);
+                mbar_expect_tx(&bars->v_full[st], C::KV_BYTES);
 #pragma unroll
-                for (int u = 0; u < NT; ++u) tma_load_3d(smem + OFF_V + st * OPND + u * TILE, &map_v, a.vx0 + h * DH + u * SUB, j * BK, b, &bars->v_full[st]);
+                for (int u = 0; u < NT; ++u) tma_load_3d(smem + C::OFF_V + st * C::KV_BYTES + u * C::KTILE, &map_v, a.vx0 + h * DH + u * SUB, j * BK, b, &bars->v_full[st]);
                 issued_v = j + 1;
             }
             if (*abort_flag) {             // aborting: bounded wait for the loads still in flight
                 mbar_wait_quiet(&bars->q_full, 0, 100000000ull);
-                for (int j = max(0, issued_k - 2); j < issued_k; ++j) mbar_wait_quiet(&bars->k_full[j & 1], (j >> 1) & 1, 100000000ull);
-                for (int j = max(0, issued_v - 2); j < issued_v; ++j) mbar_wait_quiet(&bars->v_full[j & 1], (j >> 1) & 1, 100000000ull);
+                for (int j = max(0, issued_k - STAGES); j < issued_k; ++j) mbar_wait_quiet(&bars->k_full[j % STAGES], (j / STAGES) & 1, 100000000ull);
+                for (int j = max(0, issued_v - STAGES); j < issued_v; ++j) mbar_wait_quiet(&bars->v_full[j % STAGES], (j / STAGES) & 1, 100000000ull);
             }
         }
     } else if (warp == 1) {
-        // ------------------------------------------------------------ MMA issuer
-        if (lane == 0) {
-            const uint32_t dQ = desc_lo_k(smem_u32(smem + OFF_Q));
-            constexpr uint32_t I_S = idesc_bf16(128, 128, 0, 0), I_O = idesc_bf16(128, 64, 0, 1), I_O16 = idesc_bf16(128, 16, 0, 1);
-            auto issue_pv = [&](int j) -> bool {          // O (+)= P(j) V(j)
-                const int st = j & 1;
-                const uint32_t ph = (j >> 1) & 1;
-                if (!WAIT(&bars->p_full, (uint32_t)(j & 1)) || !WAIT(&bars->v_full[st], ph)) return false;
-                fence_after();
-                const uint32_t dV = desc_lo_mn(smem_u32(smem + OFF_V + st * OPND), TILE), tp = tmem + TM_P;
-                if (j == 0) umma_ts<0>(tmem + TM_O, tp, dV, I_O); else umma_ts<1>(tmem + TM_O, tp, dV, I_O);
-#pragma unroll
-                for (int kk = 1; kk < 8; ++kk) umma_ts<1>(tmem + TM_O, tp + 8 * kk, dV + kk * 128, I_O);
-                if constexpr (NT == 2) {                  // channels 64..79: the first 16 columns of the second sub-tile
-                    const uint32_t dV2 = desc_lo_mn(smem_u32(smem + OFF_V + st * OPND + TILE), TILE);
-                    if (j == 0) umma_ts<0>(tmem + TM_O + 64, tp, dV2, I_O16); else umma_ts<1>(tmem + TM_O + 64, tp, dV2, I_O16);
-#pragma unroll
-                    for (int kk = 1; kk < 8; ++kk) umma_ts<1>(tmem + TM_O + 64, tp + 8 * kk, dV2 + kk * 128, I_O16);
-                }
-                umma_commit(&bars->o_done);               // phase j: O holds tiles 0..j; P(j) and the V stage are free
-                umma_commit(&bars->v_empty[st]);
-                return true;
-            };
-            bool ok = WAIT(&bars->q_full, 0);
-            for (int j = 0; j < n_kv && ok; ++j) {
-                const int st = j & 1;
-                const uint32_t ph = (j >> 1) & 1;
-                if (!WAIT(&bars->k_full[st], ph) || !WAIT(&bars->s_empty, (uint32_t)((j & 1) ^ 1))) { ok = false; break; }
-                fence_after();
-                const uint32_t dK = desc_lo_k(smem_u32(smem + OFF_K + st * OPND)), ts = tmem + TM_S;
+        // ------------------------------------------------------------ MMA issuer: the warp walks the loop, one elected lane issues
+        const bool leader = elect_one();
+        const uint32_t dQ0 = desc_lo_k(smem_u32(smem)), dK0 = desc_lo_k(smem_u32(smem + C::OFF_K)), dV0 = desc_lo_mn(smem_u32(smem + C::OFF_V), C::KTILE);
+        constexpr uint32_t I_S = idesc_bf16(128, BK, 0, 0), I_O = idesc_bf16(128, 64, 0, 1), I_O16 = idesc_bf16(128, 16, 0, 1);
+        auto issue_s = [&](int j, int s) -> bool {        // S of stream s <- Q K(j)^T, once the softmax has taken S(j - 1) out of TMEM
+            if (j > 0 && !WAIT(&bars->s_empty[s], (uint32_t)((j - 1) & 1))) return false;
+            fence_after();
+            const uint32_t dQ = dQ0 + s * (C::Q_BYTES >> 4), dK = dK0 + (j % STAGES) * (C::KV_BYTES >> 4), ts = tmem + s * BK;
+            if (leader) {
                 umma_ss<0>(ts, dQ, dK, I_S);
 #pragma unroll
                 for (int kk = 1; kk < 4; ++kk) umma_ss<1>(ts, dQ + 2 * kk, dK + 2 * kk, I_S);
-                if constexpr (NT == 2) umma_ss<1>(ts, dQ + (TILE >> 4), dK + (TILE >> 4), I_S);      // channels 64..79: one K step of the second sub-tiles
-                umma_commit(&bars->s_full);
-                umma_commit(&bars->k_empty[st]);
-                if (j > 0) ok = issue_pv(j - 1);
+                if constexpr (NT == 2) umma_ss<1>(ts, dQ + (C::QTILE >> 4), dK + (C::KTILE >> 4), I_S);      // channels 64..79: one K step of the second sub-tiles
+                umma_commit(&bars->s_full[s]);
+                if (s == 1) umma_commit(&bars->k_empty[j % STAGES]);
             }
-            if (ok) issue_pv(n_kv - 1);
+            __syncwarp();
+            return true;
+        };
+        auto issue_pv = [&](int j, int s) -> bool {       // O of stream s (+)= P(j) V(j)
+            if (!WAIT(&bars->p_full[s], (uint32_t)(j & 1))) return false;
+            fence_after();
+            const uint32_t dV = dV0 + (j % STAGES) * (C::KV_BYTES >> 4), tp = tmem + C::TM_P + s * (BK / 2), to = tmem + C::TM_O + s * DH;
+            if (leader) {
+                if (j == 0) umma_ts<0>(to, tp, dV, I_O); else umma_ts<1>(to, tp, dV, I_O);
+#pragma unroll
+                for (int kk = 1; kk < BK / 16; ++kk) umma_ts<1>(to, tp + 8 * kk, dV + kk * 128, I_O);
+                if constexpr (NT == 2) {                  // channels 64..79: the first 16 columns of the second sub-tile
+                    const uint32_t dV2 = dV + (C::KTILE >> 4);
+                    if (j == 0) umma_ts<0>(to + 64, tp, dV2, I_O16); else umma_ts<1>(to + 64, tp, dV2, I_O16);
+#pragma unroll
+                    for (int kk = 1; kk < BK / 16; ++kk) umma_ts<1>(to + 64, tp + 8 * kk, dV2 + kk * 128, I_O16);
+                }
+                umma_commit(&bars->o_done[s]);            // phase j: O holds tiles 0..j and P(j) has been read
+                if (s == 1) umma_commit(&bars->v_empty[j % STAGES]);
+            }
+            __syncwarp();
+            return true;
+        };
+        bool ok = WAIT(&bars->q_full, 0) && WAIT(&bars->k_full[0], 0) && issue_s(0, 0) && issue_s(0, 1);
+        for (int j = 0; j < n_kv && ok; ++j) {
+            const bool more = j + 1 < n_kv;
+            if (more) ok = WAIT(&bars->k_full[(j + 1) % STAGES], ((j + 1) / STAGES) & 1);
+            ok = ok && WAIT(&bars->v_full[j % STAGES], (j / STAGES) & 1);
+            for (int s = 0; s < 2 && ok; ++s) ok = (!more || issue_s(j + 1, s)) && issue_pv(j, s);
         }
-    } else {
+    } else if (warp >= 4) {
         // ------------------------------------------------------------ softmax, O scaling, output
+        const int s = (warp - 4) >> 2;                            // stream
         const int q = warp & 3;                                   // TMEM lane quarter of this warp
-        const int row = q * 32 + lane;                            // query row of the tile
-        const uint32_t tlane = tmem + ((uint32_t)(q * 32) << 16);
-        float m = -INFINITY, l = 0.f;
+        const uint32_t tlane = tmem + ((uint32_t)(q * 32) << 16), ts = tlane + s * BK, tp = tlane + C::TM_P + s * (BK / 2), to = tlane + C::TM_O + s * DH;
+        float m = 0.f;
+        f32x2 l2 = pk2(0.f, 0.f);
         bool ok = true;
         for (int j = 0; j < n_kv; ++j) {
-            ok = ok && WAIT(&bars->s_full, (uint32_t)(j & 1));
+            ok = WAIT(&bars->s_full[s], (uint32_t)(j & 1));
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
             fence_after();
-            const uint32_t ts = tlane + TM_S, tp = tlane + TM_P;
-            const int valid = min(BK, a.Lk - j * BK);             // keys of this tile inside the sequence
-            // pass 1: the row maximum of the scaled scores
-            float mx = -INFINITY;
-#pragma unroll 1
-            for (int c0 = 0; c0 < BK; c0 += 32) {
-                uint32_t r[32];
-                tmem_ld_x32(ts + c0, r);
-                tmem_wait_ld();
+            uint32_t r[BK];
 #pragma unroll
-                for (int i = 0; i < 32; ++i) if (c0 + i < valid) mx = fmaxf(mx, __uint_as_float(r[i]));
+            for (int c0 = 0; c0 < BK; c0 += 32) tmem_ld_x32(ts + c0, r + c0);
+            tmem_wait_ld();
+            fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&bars->s_empty[s]);
+            const int valid = a.Lk - j * BK;                      // keys of this tile inside the sequence
+            if (valid < BK) {
+#pragma unroll
+                for (int i = 0; i < BK; ++i) if (i >= valid) r[i] = __float_as_uint(-INFINITY);
             }
-            const float m_new = fmaxf(m, mx * a.scale_log2);
-            const float alpha = ex2f(m - m_new);                  // 0 on the first tile (m = -inf)
-            // P is single-buffered: P V of the previous tile must have read it (that product also completes O for the scaling below)
+            float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+            for (int i = 0; i < BK; ++i) mx[i & 3] = fmaxf(mx[i & 3], __uint_as_float(r[i]));
+            const float mj = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * a.scale_log2;
+            float alpha = 1.f;
+            if (j == 0) m = mj;
+            else if (mj > m + RESCALE_LOG2) { alpha = ex2f(m - mj); m = mj; }
+            // P V of the previous tile has read P (and completed O for a scaling)
             if (j > 0) {
-                ok = WAIT(&bars->o_done, (uint32_t)((j - 1) & 1));
+                ok = WAIT(&bars->o_done[s], (uint32_t)((j - 1) & 1));
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
                 fence_after();
             }
-            // pass 2: P = 2^(s - m_new) as bf16 into TMEM, and its row sum
-            float sum = 0.f;
-#pragma unroll 1
+            const f32x2 sc2 = pk2(a.scale_log2, a.scale_log2), nm2 = pk2(-m, -m);
+            l2 = mul2(l2, pk2(alpha, alpha));
+#pragma unroll
             for (int c0 = 0; c0 < BK; c0 += 32) {
-                uint32_t r[32], pk[16];
-                tmem_ld_x32(ts + c0, r);
-                tmem_wait_ld();
+                uint32_t pk[16];
 #pragma unroll
                 for (int i = 0; i < 32; i += 2) {
-                    const float p0 = c0 + i < valid ? ex2f(fmaf(__uint_as_float(r[i]), a.scale_log2, -m_new)) : 0.f;
-                    const float p1 = c0 + i + 1 < valid ? ex2f(fmaf(__uint_as_float(r[i + 1]), a.scale_log2, -m_new)) : 0.f;
+                    float x, y;
+                    upk2(fma2(pk2(__uint_as_float(r[c0 + i]), __uint_as_float(r[c0 + i + 1])), sc2, nm2), x, y);
+                    const float p0 = ex2f(x), p1 = ex2f(y);
+                    l2 = add2(l2, pk2(p0, p1));
                     pk[i >> 1] = pack_bf16(p0, p1);
-                    sum += p0 + p1;
                 }
                 tmem_st_x16(tp + (c0 >> 1), pk);
             }
-            l = fmaf(l, alpha, sum);
-            m = m_new;
-            fence_before();
-            mbar_arrive(&bars->s_empty);                          // every read of S(j) has completed
-            // O holds tiles 0..j-1 once PV(j-1) has completed: scale it to the new maximum
-            if (j > 0) {
+            if (__any_sync(0xffffffffu, alpha != 1.f)) {          // rare: O moves to the new maximum
 #pragma unroll 1
-                for (int c0 = 0; c0 < 64; c0 += 32) {
-                    uint32_t r[32];
-                    tmem_ld_x32(tlane + TM_O + c0, r);
+                for (int c0 = 0; c0 < DH; c0 += 16) {
+                    uint32_t t[16];
+                    tmem_ld_x16(to + c0, t);
                     tmem_wait_ld();
 #pragma unroll
-                    for (int i = 0; i < 32; ++i) r[i] = __float_as_uint(__uint_as_float(r[i]) * alpha);
-                    tmem_st_x32(tlane + TM_O + c0, r);
-                }
-                if constexpr (NT == 2) {
-                    uint32_t r[16];
-                    tmem_ld_x16(tlane + TM_O + 64, r);
-                    tmem_wait_ld();
-#pragma unroll
-                    for (int i = 0; i < 16; ++i) r[i] = __float_as_uint(__uint_as_float(r[i]) * alpha);
-                    tmem_st_x16(tlane + TM_O + 64, r);
+                    for (int i = 0; i < 16; ++i) t[i] = __float_as_uint(__uint_as_float(t[i]) * alpha);
+                    tmem_st_x16(to + c0, t);
                 }
             }
             tmem_wait_st();
             fence_before();
-            mbar_arrive(&bars->p_full);
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&bars->p_full[s]);
         }
         if (ok) {
-            ok = WAIT(&bars->o_done, (uint32_t)((n_kv - 1) & 1));
+            ok = WAIT(&bars->o_done[s], (uint32_t)((n_kv - 1) & 1));
             ok = __all_sync(0xffffffffu, ok);
         }
         if (ok) {
             fence_after();
-            const float inv = 1.f / l;
-            const int t = q0 + row;
-            auto store8 = [&](__nv_bfloat16 *dst, const uint32_t *r) {
-                *reinterpret_cast<uint4 *>(dst) =
-                    make_uint4(pack_bf16(__uint_as_float(r[0]) * inv, __uint_as_float(r[1]) * inv), pack_bf16(__uint_as_float(r[2]) * inv, __uint_as_float(r[3]) * inv),
-                               pack_bf16(__uint_as_float(r[4]) * inv, __uint_as_float(r[5]) * inv), pack_bf16(__uint_as_float(r[6]) * inv, __uint_as_float(r[7]) * inv));
-            };
+            float l, lh;
+            upk2(l2, l, lh);
+            const float inv = 1.f / (l + lh);
+            const int t = q0 + s * BQ + q * 32 + lane;
             __nv_bfloat16 *orow = a.out + ((int64_t)b * a.Lq + t) * a.d + h * DH;
-#pragma unroll 1
-            for (int c0 = 0; c0 < 64; c0 += 32) {
-                uint32_t r[32];
-                tmem_ld_x32(tlane + TM_O + c0, r);
-                tmem_wait_ld();
-                if (t < a.Lq) {
 #pragma unroll
-                    for (int i = 0; i < 32; i += 8) store8(orow + c0 + i, r + i);
-                }
-            }
-            if constexpr (NT == 2) {
-                uint32_t r[16];
-                tmem_ld_x16(tlane + TM_O + 64, r);
+            for (int c0 = 0; c0 < DH; c0 += 16) {
+                uint32_t r[16], w[8];
+                tmem_ld_x16(to + c0, r);
                 tmem_wait_ld();
-                if (t < a.Lq) { store8(orow + 64, r); store8(orow + 72, r + 8); }
+#pragma unroll
+                for (int i = 0; i < 8; ++i) w[i] = pack_bf16(__uint_as_float(r[2 * i]) * inv, __uint_as_float(r[2 * i + 1]) * inv);
+                if (t < a.Lq) st_global_256(orow + c0, w);        // heads start on 32-byte boundaries: 16 channels are one sector
             }
         }
     }
     // ---------------------------------------------------------------- teardown
+    __syncwarp();
     fence_before();
     __syncthreads();
     if (warp == 1) {
         fence_after();
-        tmem_dealloc(tmem, TM_COLS);
+        tmem_dealloc(tmem, 512);
     }
 }
 
@@ -286,39 +288,39 @@ cudaError_t attention_forward(const void *qkv, void *out, int B, int Lq, int d, 
     if (!attention_supports(DM_BF16, d, n_heads) || B <= 0 || Lq <= 0 || B > 65535 || n_heads > 65535) return cudaErrorNotSupported;
     const bool cached = k_cache != nullptr;
     if (cached && (!v_cache || cache_len < 0 || cache_len + Lq > cache_cap)) return cudaErrorInvalidValue;
+    if (Lq <= ATTN_BLOCK_MAX_Q) return attention_block(qkv, out, B, Lq, d, n_heads, k_cache, v_cache, cache_len, cache_cap, s);
     const int Lk = cached ? cache_len + Lq : Lq;
     CUtensorMap mq, mk, mv;
-    const uint32_t box[3] = {(uint32_t)SUB, (uint32_t)BQ, 1};
     const int dh = d / n_heads;
+    const uint32_t box[3] = {(uint32_t)SUB, (uint32_t)BQ, 1}, box_kv[3] = {(uint32_t)SUB, (uint32_t)(dh == 64 ? Cfg<1>::BK : Cfg<2>::BK), 1};
     {
         const uint64_t dims[3] = {(uint64_t)3 * d, (uint64_t)Lq, (uint64_t)B};
         const uint64_t str[2] = {(uint64_t)3 * d, (uint64_t)Lq * 3 * d};
-        if (!make_map_bf16(&mq, qkv, 3, dims, str, box)) return cudaErrorInvalidValue;
+        if (!make_map_bf16(&mq, qkv, 3, dims, str, box) || !make_map_bf16(&mk, qkv, 3, dims, str, box_kv)) return cudaErrorInvalidValue;
+        mv = mk;
     }
     if (cached) {
         // the maps end at the last valid key: the rest of a tile is filled with zeros, whatever the cache holds there
         const uint64_t dims[3] = {(uint64_t)d, (uint64_t)Lk, (uint64_t)B};
         const uint64_t str[2] = {(uint64_t)d, (uint64_t)cache_cap * d};
-        if (!make_map_bf16(&mk, k_cache, 3, dims, str, box) || !make_map_bf16(&mv, v_cache, 3, dims, str, box)) return cudaErrorInvalidValue;
+        if (!make_map_bf16(&mk, k_cache, 3, dims, str, box_kv) || !make_map_bf16(&mv, v_cache, 3, dims, str, box_kv)) return cudaErrorInvalidValue;
         kv_append_kernel<<<dim3(Lq, B), 128, 0, s>>>(static_cast<const __nv_bfloat16 *>(qkv), static_cast<__nv_bfloat16 *>(k_cache),
                                                       static_cast<__nv_bfloat16 *>(v_cache), Lq, d, cache_len, cache_cap);
         count_launch();
         cudaError_t e0 = cudaGetLastError();
         if (e0 != cudaSuccess) return e0;
-    } else {
-        mk = mq; mv = mq;
     }
     int *status = device_status_ptr();
     if (!status) return cudaErrorUnknown;
     AttnArgs a{B, Lq, Lk, d, n_heads, cached ? 0 : d, cached ? 0 : 2 * d, static_cast<__nv_bfloat16 *>(out), 1.4426950408889634f / sqrtf((float)dh)};
-    const dim3 grid((Lq + BQ - 1) / BQ, n_heads, B);
+    const dim3 grid((Lq + 2 * BQ - 1) / (2 * BQ), n_heads, B);
     cudaError_t e;
     if (dh == 64) {
-        if ((e = cudaFuncSetAttribute(attention_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes(1))) != cudaSuccess) return e;
-        attention_kernel<1><<<grid, NTHREADS, smem_bytes(1), s>>>(mq, mk, mv, a, status);
+        if ((e = cudaFuncSetAttribute(attention_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg<1>::SMEM)) != cudaSuccess) return e;
+        attention_kernel<1><<<grid, NTHREADS, Cfg<1>::SMEM, s>>>(mq, mk, mv, a, status);
     } else {
-        if ((e = cudaFuncSetAttribute(attention_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes(2))) != cudaSuccess) return e;
-        attention_kernel<2><<<grid, NTHREADS, smem_bytes(2), s>>>(mq, mk, mv, a, status);
+        if ((e = cudaFuncSetAttribute(attention_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg<2>::SMEM)) != cudaSuccess) return e;
+        attention_kernel<2><<<grid, NTHREADS, Cfg<2>::SMEM, s>>>(mq, mk, mv, a, status);
     }
     count_launch();
     return cudaGetLastError();

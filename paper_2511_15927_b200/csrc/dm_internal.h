@@ -94,6 +94,11 @@ bool attention_supports(int dtype, int d, int n_heads);
 cudaError_t attention_forward(const void *qkv, void *out, int B, int L, int d, int n_heads, void *k_cache, void *v_cache,
                               int cache_len, int cache_cap, cudaStream_t s);
 
+// The same for few queries (up to ATTN_BLOCK_MAX_Q): see attention_block.cu.
+constexpr int ATTN_BLOCK_MAX_Q = 64;
+cudaError_t attention_block(const void *qkv, void *out, int B, int L, int d, int n_heads, void *k_cache, void *v_cache, int cache_len,
+                            int cache_cap, cudaStream_t s);
+
 // ---------------------------------------------------------------------------------------------
 // Small row-wise kernels
 // ---------------------------------------------------------------------------------------------

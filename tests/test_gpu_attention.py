@@ -190,6 +190,36 @@ def test_attention_block_step_with_cache(G, dh):
     assert dm.dm_kernel_launch_count() == before
 
 
+@pytest.mark.parametrize("dh", [64, 80])
+@pytest.mark.parametrize("H,G_len,prefix", [(3, 1, 0), (2, 32, 63), (2, 33, 64), (1, 64, 1), (1, 65, 300), (2, 31, 2100), (40, 17, 600)])
+def test_attention_block_splits(G, dh, H, G_len, prefix):
+    """The few-query kernel around its tiles (32 queries, 64 keys) and its splits of the keys (1 to 8 CTAs; the last case has too many heads for
+    one), and 65 queries, which take the other kernel; the cache beyond the valid keys holds NaN."""
+    from paper_2511_15927_b200 import binding as dm
+    B, cap = 2, prefix + G_len + 5
+    d = dh * H
+    x, wq, wo = _case(B, G_len, H, 100 + prefix, 1.0, dh=dh)
+    r = np.random.default_rng(prefix)
+    k0 = I.round_to_bf16(r.standard_normal((B, prefix, d), dtype=np.float32))
+    v0 = I.round_to_bf16(r.standard_normal((B, prefix, d), dtype=np.float32))
+    pad = np.full((B, cap - prefix, d), np.nan, np.float32)
+    kc, vc = G.dev(np.concatenate([k0, pad], 1), I.BF16), G.dev(np.concatenate([v0, pad], 1), I.BF16)
+    xd, wqd, wod = G.dev(x, I.BF16), G.dev(wq, I.BF16), G.dev(wo, I.BF16)
+    yd = torch.empty_like(xd)
+    nb = dm.dm_attention_workspace_bytes(B, G_len, d, dm.DM_BF16)
+    ws = G.workspace(nb)
+    st = torch.cuda.current_stream().cuda_stream
+    dm.dm_attention_block_step(B, G_len, d, H, dm.DM_BF16, wqd.data_ptr(), wod.data_ptr(), xd.data_ptr(), kc.data_ptr(), vc.data_ptr(), prefix, cap,
+                               yd.data_ptr(), ws.data_ptr(), nb, st)
+    dm.dm_check(st)
+    want, k1, v1 = O.attention_block_step(x, wq, wo, H, k0.astype(np.float64), v0.astype(np.float64))
+    got = yd.float().cpu().numpy().astype(np.float64)
+    assert np.all(np.isfinite(got)) and G.rel_l2(got, want) <= BF16_REL and G.max_abs(got, want) <= BF16_ABS
+    n = prefix + G_len
+    assert G.rel_l2(kc[:, :n].float().cpu().numpy().astype(np.float64), k1) <= 5e-3 and G.rel_l2(vc[:, :n].float().cpu().numpy().astype(np.float64), v1) <= 5e-3
+    assert torch.isnan(kc[:, n:]).all() and torch.isnan(vc[:, n:]).all()
+
+
 def test_hybrid_stack_block_mode(G):
     """Prefix pass commits Mamba states and key/value caches, the next block starts from them (Sec. 4.3)."""
     from paper_2511_15927_b200 import binding as dm
