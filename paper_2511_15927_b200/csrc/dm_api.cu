@@ -156,15 +156,36 @@ static cudaError_t gemm(const GemmArgs &a, cudaStream_t s) {
     return gemm_simple(a, s);
 }
 
+// Rows whose RMSNorm scale is still to be applied by the product that reads them: rsqrt(sum(ssq[r, 0..n)) * inv + eps); ssq == NULL: none.
+struct PendingNorm {
+    const float *ssq = nullptr; int n = 0; float inv = 0.f, eps = 0.f;
+    void apply(GemmArgs &a, int64_t row0 = 0) const {
+        if (!ssq) return;
+        a.rs_ssq = ssq + row0 * n; a.rs_n = n; a.rs_inv = inv; a.rs_eps = eps;
+    }
+};
+
 struct MixerOut {
     void *y; int y_dtype; const float *addend; int64_t ld_add;
     const float *col_scale = nullptr; int cs_rows = 0; int64_t ld_cs = 0;   // per-sequence gate on the mixer's output (App. A.1), or NULL
-    // The caller's next step is u = RMSNorm(y; next_norm_w): a mixer that sums its directions in a pass of its own applies it there and sets *next_done
+    // The caller's next step is u = RMSNorm(y; next_norm_w).  A mixer that sums its directions in a pass of its own applies it there; one that sums them inside
+    // the out_proj launch leaves y * next_norm_w in u and the rows' sums of squares in next_ssq ([T][ceil(d / 64)]), the scale pending.  *next_done: u is there.
     const void *next_norm_w = nullptr; void *next_u = nullptr; float next_eps = 0.f; bool *next_done = nullptr;
+    float *next_ssq = nullptr; PendingNorm *pending = nullptr;
+    bool fuse_norm(GemmArgs &a, int d) const {         // asks the product that completes y for u
+        if (!next_norm_w || !next_u || !next_ssq || y_dtype != DM_F32 || a.in_dtype != DM_BF16) return false;
+        GemmArgs f = a;
+        f.u = next_u; f.u_w = next_norm_w; f.u_ssq = next_ssq;
+        if (!gemm_tcgen05_supports(f)) return false;
+        a = f;
+        *next_done = true;
+        *pending = PendingNorm{next_ssq, (d + 63) / 64, 1.f / (float)d, next_eps};
+        return true;
+    }
 };
 
 // in_proj -> fused conv/scan/gate -> out_proj of both directions, summed (Sec. 3.2).
-static int run_mixer(const dm_mixer_cfg *c, const Dims &m, const dm_dir_weights w[2], const void *x, const MixerOut &out,
+static int run_mixer(const dm_mixer_cfg *c, const Dims &m, const dm_dir_weights w[2], const void *x, const PendingNorm &x_norm, const MixerOut &out,
                      const float *ssm_in, const void *conv_in, float *ssm_out, void *conv_out,
                      char *ws, cudaStream_t s) {
     const MixerWs l = mixer_ws(c, m);
@@ -203,6 +224,7 @@ static int run_mixer(const dm_mixer_cfg *c, const Dims &m, const dm_dir_weights 
             a.C = zx + (size_t)(tied ? 0 : dir) * m.T * m.ldz * m.es; a.ldc = m.ldz;
             a.in_dtype = c->dtype; a.c_dtype = c->dtype; a.M = (int)m.T; a.N = m.d_in_proj; a.K = m.d;
             a.silu_cols = ssd ? m.d_inner : 0;
+            x_norm.apply(a);
             ga[n++] = a;
         }
         StageTimer tm(DM_STAGE_IN_PROJ, s);
@@ -255,6 +277,27 @@ static int run_mixer(const dm_mixer_cfg *c, const Dims &m, const dm_dir_weights 
             return DM_OK;
         }
     }
+    if (!tied && c->dir_mask == DM_DIR_BOTH && m.T > PAIR_OUT_MAX_T) {
+        // long inputs: both out_proj and their sum in one launch, each direction's gated-norm scale taken from the sums of squares in the epilogue
+        GemmArgs ga[2];
+        for (int dir = 0; dir < 2; ++dir) {
+            GemmArgs a{};
+            a.A = g + (size_t)dir * m.T * m.d_inner * m.es; a.lda = m.d_inner;
+            a.B = w[dir].w_out; a.ldb = m.d_inner;
+            a.in_dtype = c->dtype; a.M = (int)m.T; a.N = m.d; a.K = m.d_inner;
+            if (norm_on) { a.rs_ssq = ssq + (size_t)dir * m.T * m.H; a.rs_n = m.H; a.rs_inv = 1.f / (float)m.d_inner; a.rs_eps = c->norm_eps; }
+            a.col_scale = out.col_scale; a.cs_rows = out.cs_rows; a.ld_cs = out.ld_cs;        // the gate distributes over the sum of the directions
+            a.addend = out.addend; a.ld_add = out.ld_add;
+            a.C = out.y; a.ldc = m.d; a.c_dtype = out.y_dtype;
+            ga[dir] = a;
+        }
+        if (gemm_tcgen05_sum_supports(ga[0], ga[1])) {
+            out.fuse_norm(ga[1], m.d);
+            StageTimer tm(DM_STAGE_OUT_PROJ, s);
+            if ((e = gemm_tcgen05_sum(ga[0], ga[1], s)) != cudaSuccess) return cuda_fail(e, "out_proj");
+            return DM_OK;
+        }
+    }
     if (norm_on) {
         e = rstd_from_ssq(ssq, rstd, (int)(2 * m.T), m.H, m.d_inner, c->norm_eps, s);
         if (e != cudaSuccess) return cuda_fail(e, "rstd");
@@ -304,7 +347,7 @@ static int check_ws(const void *ws, size_t have, size_t need) {
 }
 
 struct StackWs {
-    size_t r, u, logits, mixer, mod, hmid, idx, count, ug, qkv, att, total;
+    size_t r, u, ussq, logits, mixer, mod, hmid, idx, count, ug, qkv, att, total;
     int logits_rows;
 };
 
@@ -313,6 +356,7 @@ static StackWs stack_ws(const dm_stack_cfg *c, const Dims &m, const dm_block_cfg
     size_t off = 0;
     w.r = off; off += align_up((size_t)m.T * m.d * sizeof(float));
     w.u = off; off += align_up((size_t)m.T * m.d * m.es);
+    w.ussq = off; off += align_up((size_t)m.T * ((m.d + 63) / 64) * sizeof(float));
     w.logits_rows = (int)(m.T < 2048 ? m.T : 2048);
     w.logits = off; off += align_up((size_t)w.logits_rows * c->vocab * m.es);
     w.mixer = off; off += mixer_ws(&c->mixer, m).total;
@@ -453,7 +497,7 @@ int dm_bimamba_forward(const dm_mixer_cfg *cfg, const dm_dir_weights w[2], const
     if (!aligned16(x) || !aligned16(y)) return fail(DM_ERR_INVALID_ARG, "x and y must be 16-byte aligned");
     if ((st = check_ws(workspace, workspace_bytes, mixer_ws(cfg, m).total)) != DM_OK) return st;
     MixerOut out{y, cfg->dtype, nullptr, 0};
-    return run_mixer(cfg, m, w, x, out, nullptr, nullptr, nullptr, nullptr, static_cast<char *>(workspace),
+    return run_mixer(cfg, m, w, x, PendingNorm{}, out, nullptr, nullptr, nullptr, nullptr, static_cast<char *>(workspace),
                      static_cast<cudaStream_t>(cuda_stream));
 }
 
@@ -472,7 +516,7 @@ int dm_bimamba_forward_static(const dm_mixer_cfg *cfg, const dm_dir_weights w[2]
     char *ws = nullptr;
     if ((st = static_ws_ptr(&ws)) != DM_OK) return st;
     MixerOut out{y, cfg->dtype, nullptr, 0};
-    return run_mixer(cfg, m, w, x, out, nullptr, nullptr, nullptr, nullptr, ws, static_cast<cudaStream_t>(cuda_stream));
+    return run_mixer(cfg, m, w, x, PendingNorm{}, out, nullptr, nullptr, nullptr, nullptr, ws, static_cast<cudaStream_t>(cuda_stream));
 }
 
 int dm_bimamba_block_step(const dm_mixer_cfg *cfg, const dm_dir_weights w[2], const void *x_blk,
@@ -494,7 +538,7 @@ int dm_bimamba_block_step(const dm_mixer_cfg *cfg, const dm_dir_weights w[2], co
         return fail(DM_ERR_INVALID_ARG, "state_out needs the left-to-right direction");
     if ((st = check_ws(workspace, workspace_bytes, mixer_ws(cfg, m).total)) != DM_OK) return st;
     MixerOut out{y_blk, cfg->dtype, nullptr, 0};
-    return run_mixer(cfg, m, w, x_blk, out, ssm_state_in, conv_state_in, ssm_state_out, conv_state_out,
+    return run_mixer(cfg, m, w, x_blk, PendingNorm{}, out, ssm_state_in, conv_state_in, ssm_state_out, conv_state_out,
                      static_cast<char *>(workspace), static_cast<cudaStream_t>(cuda_stream));
 }
 
@@ -593,7 +637,8 @@ static int denoise_impl(const dm_stack_cfg *cfg, const dm_block_cfg *blk, const 
     cudaError_t e;
 
     if ((e = embed_gather(weights->embed, dtype, tokens, r, (int)m.T, m.d, cfg->vocab, s)) != cudaSuccess) return cuda_fail(e, "embed");
-    bool u_ready = false;                         // u already holds the norm of r (applied by the previous layer's last pass)
+    bool u_ready = false;                         // u already holds the norm of r (written by the previous layer's last pass),
+    PendingNorm u_norm;                           // up to this scale of its rows
     for (int i = 0; i < cfg->n_layers; ++i) {
         const dm_layer_weights &lw = weights->layers[i];
         MixerOut out{r, DM_F32, r, m.d};          // r <- r + Mamba(u): the residual add rides in the out_proj epilogue
@@ -607,14 +652,19 @@ static int denoise_impl(const dm_stack_cfg *cfg, const dm_block_cfg *blk, const 
             // what follows this layer's mixer is the next layer's (or the final) RMSNorm of r
             out.next_norm_w = i + 1 < cfg->n_layers ? weights->layers[i + 1].norm_w : weights->final_norm_w;
             out.next_u = u; out.next_eps = cfg->rms_eps; out.next_done = &u_ready;
+            // (the sampler gathers rows of the final norm: they are normalised in a pass of their own)
+            out.next_ssq = smp && i + 1 == cfg->n_layers ? nullptr : reinterpret_cast<float *>(ws + l.ussq);
         }
-        u_ready = false;
+        const PendingNorm in_norm = u_norm;
+        u_ready = false; u_norm = PendingNorm{};
+        out.pending = &u_norm;
         if (period > 0 && i % period == 0) {
             // attention mixer (Sec. 3.3): r <- r + [gate *] Attn(u); gate and residual ride in the output projection's epilogue
             void *qkv = ws + l.qkv, *att = ws + l.att;
             GemmArgs a{};
             a.A = u; a.lda = m.d; a.B = hyb->aw[i].w_qkv; a.ldb = m.d; a.C = qkv; a.ldc = 3 * m.d;
             a.in_dtype = dtype; a.c_dtype = dtype; a.M = (int)m.T; a.N = 3 * m.d; a.K = m.d;
+            in_norm.apply(a);
             if ((e = gemm(a, s)) != cudaSuccess) return cuda_fail(e, "qkv projection");
             if ((e = attention_forward(qkv, att, m.B, m.L, m.d, hyb->cfg->attn_heads, hyb->ast ? hyb->ast[i].k_cache : nullptr,
                                        hyb->ast ? hyb->ast[i].v_cache : nullptr, hyb->ast ? hyb->ast[i].len : 0, hyb->ast ? hyb->ast[i].cap : 0, s)) != cudaSuccess) return cuda_fail(e, "attention");
@@ -622,10 +672,11 @@ static int denoise_impl(const dm_stack_cfg *cfg, const dm_block_cfg *blk, const 
             o.A = att; o.lda = m.d; o.B = hyb->aw[i].w_o; o.ldb = m.d; o.C = r; o.ldc = m.d;
             o.in_dtype = dtype; o.c_dtype = DM_F32; o.M = (int)m.T; o.N = m.d; o.K = m.d;
             o.addend = r; o.ld_add = m.d; o.col_scale = out.col_scale; o.cs_rows = out.cs_rows; o.ld_cs = out.ld_cs;
+            out.fuse_norm(o, m.d);
             if ((e = gemm(o, s)) != cudaSuccess) return cuda_fail(e, "attention output projection");
         } else {
             const dm_layer_state *q = states ? &states[i] : nullptr;
-            st = run_mixer(&cfg->mixer, m, lw.dir, u, out, q ? q->ssm_in : nullptr, q ? q->conv_in : nullptr,
+            st = run_mixer(&cfg->mixer, m, lw.dir, u, in_norm, out, q ? q->ssm_in : nullptr, q ? q->conv_in : nullptr,
                            q ? q->ssm_out : nullptr, q ? q->conv_out : nullptr, ws + l.mixer, s);
             if (st != DM_OK) return st;
         }
@@ -677,6 +728,7 @@ static int denoise_impl(const dm_stack_cfg *cfg, const dm_block_cfg *blk, const 
         a.B = weights->w_vocab; a.ldb = m.d;
         a.C = logits ? static_cast<char *>(logits) + (size_t)t0 * cfg->vocab * m.es : ws + l.logits; a.ldc = cfg->vocab;
         a.in_dtype = dtype; a.c_dtype = dtype; a.M = rows; a.N = cfg->vocab; a.K = m.d;
+        u_norm.apply(a, t0);
         if ((e = gemm(a, s)) != cudaSuccess) return cuda_fail(e, "vocab projection");
         if (argmax_out && (e = argmax_rows(a.C, dtype, argmax_out + t0, rows, cfg->vocab, s)) != cudaSuccess) return cuda_fail(e, "argmax");
     }

@@ -14,6 +14,8 @@ struct EpiArgs {
     int silu_cols;   // SiLU on output columns below this one
     const float *col_bias; int gelu; const float *col_scale; int cs_rows; int64_t ld_cs;   // see GemmArgs
     const int *m_dev; int m_off;
+    const float *rs_ssq; int rs_n; float rs_inv, rs_eps;
+    __nv_bfloat16 *u; const __nv_bfloat16 *u_w; float *u_ssq;
     int k_off;       // first element along K of this problem's share (split K: the second half of a product is a problem of its own)
 };
 
@@ -28,7 +30,8 @@ struct EpiPair {
 
 inline EpiArgs epi_of(const GemmArgs &a) {
     return EpiArgs{a.C, a.ldc, a.c_dtype == DM_F32 ? 1 : 0, a.row_scale, a.addend, a.ld_add, a.M, a.N, a.K, a.silu_cols,
-                   a.col_bias, a.gelu, a.col_scale, a.cs_rows > 0 ? a.cs_rows : 1, a.ld_cs > 0 ? a.ld_cs : (int64_t)a.N, a.m_dev, a.m_off, 0};
+                   a.col_bias, a.gelu, a.col_scale, a.cs_rows > 0 ? a.cs_rows : 1, a.ld_cs > 0 ? a.ld_cs : (int64_t)a.N, a.m_dev, a.m_off,
+                   a.rs_ssq, a.rs_n, a.rs_inv, a.rs_eps, static_cast<__nv_bfloat16 *>(a.u), static_cast<const __nv_bfloat16 *>(a.u_w), a.u_ssq, 0};
 }
 
 // The launch's problems: one product, two (b), or two that are each cut in two along K (hi: fp32 outputs of the second halves, same pitch).
@@ -66,9 +69,28 @@ struct EpiRow {
     }
 };
 
-// v[j] = accumulator of column col + j, already times the row scale.  ACT: bias and activations may occur.
+// The row's scale: given, or from sums of squares (of the gated output per head, or of the residual stream per 64 channels), added in their order.
+__device__ __forceinline__ float epi_row_scale(const EpiArgs &ep, int row) {
+    if (ep.row_scale) return ep.row_scale[row];
+    if (!ep.rs_ssq) return 1.f;
+    const float *q = ep.rs_ssq + (int64_t)row * ep.rs_n;
+    float s = 0.f;
+    if ((ep.rs_n & 3) == 0) {
+#pragma unroll 8
+        for (int i = 0; i < ep.rs_n; i += 4) {
+            const float4 v = __ldg(reinterpret_cast<const float4 *>(q + i));
+            s += (v.x + v.y) + (v.z + v.w);
+        }
+    } else {
+#pragma unroll 8
+        for (int i = 0; i < ep.rs_n; ++i) s += __ldg(q + i);
+    }
+    return rsqrtf(s * ep.rs_inv + ep.rs_eps);
+}
+
+// v[j] = accumulator of column col + j, already times the row scale: bias, activation (ACT: they may occur), column scale.
 template <bool ACT>
-__device__ __forceinline__ void epi_cols32(const EpiArgs &ep, const EpiRow &er, int row, int col, float (&v)[32]) {
+__device__ __forceinline__ void epi_pre(const EpiArgs &ep, const EpiRow &er, int col, float (&v)[32]) {
     const bool full = col + 32 <= ep.N;
     if constexpr (ACT) {
         if (ep.col_bias) {
@@ -109,6 +131,11 @@ __device__ __forceinline__ void epi_cols32(const EpiArgs &ep, const EpiRow &er, 
             for (int j = 0; j < 32; ++j) if (col + j < ep.N) v[j] *= cs[j];
         }
     }
+}
+
+// Addend and output by the thread itself, one row per lane.
+__device__ __forceinline__ void epi_add_store(const EpiArgs &ep, const EpiRow &er, int row, int col, float (&v)[32]) {
+    const bool full = col + 32 <= ep.N;
     if (er.add_row) {
         if (full && er.wide_add) {
 #pragma unroll
@@ -176,9 +203,24 @@ inline bool make_map_2d(CUtensorMap *m, const void *base, int64_t rows, int64_t 
     return make_map_bf16(m, base, 2, dims, strides, box);
 }
 
+// The next norm's input: box = 32 rows x 32 columns, 64-byte swizzle.
+inline bool make_map_u(CUtensorMap *m, const void *base, int64_t rows, int64_t cols) {
+    EncodeTiledFn fn = encode_fn();
+    if (!fn) return false;
+    const cuuint64_t d[2] = {(cuuint64_t)cols, (cuuint64_t)rows}, st[1] = {(cuuint64_t)cols * 2};
+    const cuuint32_t b[2] = {32, 32}, e[2] = {1, 1};
+    return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(base), d, st, b, e, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B,
+              CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 }  // namespace tc
 
-// gemm_pair.cu: the two-CTA kernel.  wide: 256 x 256 tiles, else 256 x 128; b, hi: see gemm_tcgen05.cu.
+// gemm_pair.cu: the two-CTA kernel.  wide: 256 x 256 tiles, else 256 x 128; b, hi: see gemm_tcgen05.cu.  gemm_pair_sum_launch: both products into one output.
 cudaError_t gemm_pair_launch(bool wide, const GemmArgs &a, const GemmArgs *b, float *const *hi, cudaStream_t s);
+cudaError_t gemm_pair_sum_launch(const GemmArgs &a, const GemmArgs &b, cudaStream_t s);
+// Output and addend can go through TMA: 16-byte aligned rows.
+inline bool gemm_pair_tma_io(const GemmArgs &a) {
+    return (a.ldc * (int64_t)dtype_size(a.c_dtype)) % 16 == 0 && (!a.addend || a.ld_add % 4 == 0);
+}
 
 }  // namespace dm

@@ -2,7 +2,7 @@
 // tile, each holding half of its rows of A and of its accumulators, and each loading half of B -- the tensor cores read the other half
 // out of the partner's shared memory.  Per product that is two thirds of the operand traffic (L2 to shared memory) of a single CTA's 128 x 256
 // tile.  Bound by the tensor cores under the power limit on large products (about 1.3 GHz in a long run): 16384 x 8512 x 2048 in 438 us =
-// 1.30 PFLOP/s, 367 us = 1.56 PFLOP/s after a pause (single-CTA 128 x 256 tiles: 500 and 410 us); by the operand stream from L2, 14 to 15 TB/s over
+// 1.30 PFLOP/s, 364 us = 1.57 PFLOP/s after a pause (single-CTA 128 x 256 tiles: 500 and 410 us); by the operand stream from L2, 14 to 15 TB/s over
 // all SMs, on small ones (512 x 17024 x 2048: 31 us).
 //
 // Persistent, one CTA per SM, warp roles per CTA: warp 0 issues this CTA's TMA loads (A: its 128 rows, B: its half of the columns), which
@@ -10,6 +10,8 @@
 // Tile order: the larger operand is streamed from HBM once, the other one stays in L2 (n_fast: consecutive tiles step along N).
 //
 // Waits and abort as in gemm_tcgen05.cu: every mbarrier wait is bounded, in both CTAs; the CTAs of a pair leave together.
+#include <cstring>
+
 #include "gemm_epi.cuh"
 
 namespace dm {
@@ -20,6 +22,7 @@ using namespace tc;
 constexpr int BM = 128, BK = 64;             // rows of A per CTA and row block, K step
 constexpr int NTHREADS = 64 + 8 * 32;
 constexpr int MAX_STAGES = 8;
+constexpr uint32_t STG_BYTES = 32 * 128;     // staging of one epilogue warp
 
 // 256 rows x BN columns per pair.  Stage of one CTA: 128 rows of A and BN / 2 rows of B.
 template <int BN> struct Tile {
@@ -29,22 +32,34 @@ template <int BN> struct Tile {
 };
 
 struct __align__(8) Bars {
-    uint64_t full[MAX_STAGES], empty[MAX_STAGES], tmem_full[2], tmem_empty[2];
+    uint64_t full[MAX_STAGES], empty[MAX_STAGES], tmem_full[2], tmem_empty[2], add_full[8];
     uint32_t tmem_base;
     int abort;
 };
 
-template <int BN>
+// Tensor maps of the outputs (boxes of 32 rows x 128 bytes), the addend and the next norm's input.
+struct IoMaps { CUtensorMap c[4], add, u; };
+
+// How a tile leaves the kernel:
+//   DIRECT  every lane reads and writes its own row: for outputs whose rows do not start on 16-byte boundaries
+//   TMA     32 rows x 128 bytes at a time through 4 KB of shared memory per warp: the addend arrives and the results leave as whole 128-byte lines (a lane
+//           storing 32 bytes of its own row makes a transaction of its own of each: 16384 x 4160 x 1024 spent 8.6 k clocks per tile on that
+//           where its products take 8.2 k)
+//   SUM     TMA, and the two problems are summed (s_0 A_0 B_0^T + s_1 A_1 B_1^T into problem 1's output): a pair runs both on a tile, one after the other in the
+//           two accumulator buffers; the epilogue warps take the first product out of TMEM into registers (128 per thread, scaled by its
+//           rows' factor, the addend added) while the second one runs, so the sum costs no pass over memory and the buffers still alternate
+enum { DIRECT = 0, TMA = 1, SUM = 2 };
+template <int BN, int MODE>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
 gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant__ CUtensorMap map_b0,
                  const __grid_constant__ CUtensorMap map_a1, const __grid_constant__ CUtensorMap map_b1,
-                 const __grid_constant__ EpiPair epp, int *status) {
+                 const __grid_constant__ IoMaps io, const __grid_constant__ EpiPair epp, int *status) {
     using T = Tile<BN>;
     constexpr int STAGES = T::STAGES;
     const EpiArgs &ep = epp.p[0];              // sizes are common to all problems
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
-    Bars *bars = reinterpret_cast<Bars *>(smem + STAGES * T::STAGE);
+    Bars *bars = reinterpret_cast<Bars *>(smem + STAGES * T::STAGE + (MODE == DIRECT ? 0 : 8 * STG_BYTES));
     volatile int *abort_flag = &bars->abort;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -52,8 +67,9 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_consta
     const int pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
     const int M_eff = ep.m_dev ? min(ep.M, max(0, *ep.m_dev - ep.m_off)) : ep.M;
     const int tiles_m = (M_eff + 2 * BM - 1) / (2 * BM), tiles_n = (ep.N + BN - 1) / BN;
-    const int tiles_np = tiles_n * epp.nprob;                  // the problems sit side by side along N
+    const int tiles_np = tiles_n * (MODE == SUM ? 1 : epp.nprob);      // separate problems sit side by side along N
     const int num_tiles = tiles_m * tiles_np;
+    constexpr int NSUB = MODE == SUM ? 2 : 1;                  // products per tile
     auto tile_at = [&](int tile, int &mb, int &cb) {
         mb = epp.n_fast ? tile / tiles_np : tile % tiles_m;
         cb = epp.n_fast ? tile % tiles_np : tile / tiles_m;
@@ -63,8 +79,13 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_consta
     if (threadIdx.x == 0) {
         for (int i = 0; i < STAGES; ++i) { mbar_init(&bars->full[i], 1); mbar_init(&bars->empty[i], 1); }
         for (int i = 0; i < 2; ++i) { mbar_init(&bars->tmem_full[i], 1); mbar_init(&bars->tmem_empty[i], 16); }     // 8 epilogue warps of both CTAs
+        for (int i = 0; i < 8; ++i) mbar_init(&bars->add_full[i], 1);
         bars->abort = 0;
         mbar_fence_init();
+    }
+    if (threadIdx.x == 64) {                   // the maps are on their way while the barriers and TMEM are set up
+        prefetch_map(&map_a0); prefetch_map(&map_b0);
+        if (epp.nprob > 1) { prefetch_map(&map_a1); prefetch_map(&map_b1); }
     }
     if (warp == 1) tmem_alloc_2cta(&bars->tmem_base, T::TMEM_COLS);
     fence_before();
@@ -81,21 +102,22 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_consta
             for (int tile = pair; tile < num_tiles && ok; tile += npairs) {
                 int tm, cb;
                 tile_at(tile, tm, cb);
-                const int prob = cb / tiles_n;
-                const int m0 = tm * 2 * BM + (int)rank * BM, n0 = (cb - prob * tiles_n) * BN + (int)rank * (BN / 2);
-                const int prod = epp.ksplit ? prob >> 1 : prob, k_off = epp.p[prob].k_off;
-                const CUtensorMap *ma = prod ? &map_a1 : &map_a0, *mb = prod ? &map_b1 : &map_b0;
-                for (int kb = 0; kb < kblocks; ++kb, ++it) {
-                    const uint32_t s = it % STAGES, ph = (it / STAGES) & 1u;
-                    if (!(ok = mbar_wait(&bars->empty[s], ph ^ 1u, abort_flag, status))) break;
-                    uint8_t *sa = smem + s * T::STAGE, *sb = sa + T::A_BYTES;
-                    const uint32_t full = cluster_addr(&bars->full[s], 0);
-                    if (leader) {
-                        if (rank == 0) mbar_expect_tx(&bars->full[s], 2 * T::STAGE);        // both CTAs' loads
-                        tma_load_2d_pair(sa, ma, k_off + kb * BK, m0, full);
-                        tma_load_2d_pair(sb, mb, k_off + kb * BK, n0, full);
+                const int prob0 = cb / tiles_n, m0 = tm * 2 * BM + (int)rank * BM, n0 = (cb - prob0 * tiles_n) * BN + (int)rank * (BN / 2);
+                for (int sub = 0; sub < NSUB && ok; ++sub) {
+                    const int prob = prob0 + sub, prod = epp.ksplit ? prob >> 1 : prob, k_off = epp.p[prob].k_off;
+                    const CUtensorMap *ma = prod ? &map_a1 : &map_a0, *mb = prod ? &map_b1 : &map_b0;
+                    for (int kb = 0; kb < kblocks; ++kb, ++it) {
+                        const uint32_t s = it % STAGES, ph = (it / STAGES) & 1u;
+                        if (!(ok = mbar_wait(&bars->empty[s], ph ^ 1u, abort_flag, status))) break;
+                        uint8_t *sa = smem + s * T::STAGE, *sb = sa + T::A_BYTES;
+                        const uint32_t full = cluster_addr(&bars->full[s], 0);
+                        if (leader) {
+                            if (rank == 0) mbar_expect_tx(&bars->full[s], 2 * T::STAGE);        // both CTAs' loads
+                            tma_load_2d_pair(sa, ma, k_off + kb * BK, m0, full);
+                            tma_load_2d_pair(sb, mb, k_off + kb * BK, n0, full);
+                        }
+                        __syncwarp();
                     }
-                    __syncwarp();
                 }
             }
             if (!ok) sleep_ns(100000000ull);       // aborting: the loads already issued get time to land before the pair goes away
@@ -110,7 +132,8 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_consta
             const uint32_t desc_a0 = desc_lo_k(smem_u32(smem));
             uint32_t it = 0, tcount = 0;
             bool ok = true;
-            for (int tile = pair; tile < num_tiles && ok; tile += npairs, ++tcount) {
+            const uint32_t products = (uint32_t)(pair < num_tiles ? (num_tiles - 1 - pair) / npairs + 1 : 0) * NSUB;
+            for (; tcount < products && ok; ++tcount) {
                 const uint32_t buf = tcount & 1u, bph = (tcount >> 1) & 1u;
                 if (!(ok = mbar_wait(&bars->tmem_empty[buf], bph ^ 1u, abort_flag, status))) break;
                 fence_after();
@@ -136,37 +159,174 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_consta
         // ------------------------------------------------------------ epilogue: 8 warps over this CTA's 128 rows
         constexpr int COLS = BN / 2;                           // columns per warp
         const int q = warp & 3, cfirst = ((warp - 2) >> 2) * COLS;       // TMEM lane quarter, first column
+        const uint32_t tlane = tmem_base + ((uint32_t)(q * 32) << 16) + cfirst;
         uint32_t tcount = 0;
         bool ok = true;
-        for (int tile = pair; tile < num_tiles && ok; tile += npairs, ++tcount) {
-            const uint32_t buf = tcount & 1u, bph = (tcount >> 1) & 1u;
-            int tm, cb;
-            tile_at(tile, tm, cb);
-            const int prob = cb / tiles_n;
-            const EpiArgs &pe = epp.p[prob];                   // this tile's problem: its output, scales and addend
-            const int row = tm * 2 * BM + (int)rank * BM + q * 32 + lane, n0 = (cb - prob * tiles_n) * BN + cfirst;
-            const bool row_ok = row < M_eff;
-            const float sc = (pe.row_scale && row_ok) ? pe.row_scale[row] : 1.f;
-            const EpiRow er(pe, row);
-            ok = mbar_wait(&bars->tmem_full[buf], bph, abort_flag, status);
-            ok = __all_sync(0xffffffffu, ok);
-            if (!ok) break;
-            fence_after();
-#pragma unroll 1
-            for (int c0 = 0; c0 < COLS; c0 += 32) {
-                uint32_t r[32];
-                tmem_ld_x32(tmem_base + ((uint32_t)(q * 32) << 16) + buf * BN + cfirst + c0, r);
-                tmem_wait_ld();
-                const int col = n0 + c0;
-                if (!row_ok || col >= pe.N) continue;
-                float v[32];
-#pragma unroll
-                for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]) * sc;
-                epi_cols32<true>(pe, er, row, col, v);
-            }
+        auto drained = [&](uint32_t buf) {                     // this warp has taken the buffer out of TMEM
             fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive_cluster(cluster_addr(&bars->tmem_empty[buf], 0));
+        };
+        auto ready = [&](uint32_t count) -> bool {
+            const bool r = __all_sync(0xffffffffu, mbar_wait(&bars->tmem_full[count & 1u], (count >> 1) & 1u, abort_flag, status));
+            fence_after();
+            return r;
+        };
+        // staging: 16-byte piece j of row `lane` sits at lane * 128 + ((j ^ (lane & 7)) << 4), the 128-byte swizzle of the maps
+        uint8_t *stg = smem + STAGES * T::STAGE + (warp - 2) * STG_BYTES;
+        uint32_t add_count = 0;
+        auto piece = [&](int j) { return reinterpret_cast<uint4 *>(stg + lane * 128 + ((j ^ (lane & 7)) << 4)); };
+        auto stg_free = [&] {                                  // the previous store has read the staging bytes
+            if (lane == 0) bulk_wait_read0();
+            __syncwarp();
+        };
+        auto stg_store = [&](const CUtensorMap *map, int x, int y) {
+            fence_proxy_async();
+            __syncwarp();
+            if (lane == 0) { tma_store_2d(map, stg, x, y); bulk_commit(); }
+        };
+        auto add_fetch = [&](int x, int y) {                   // 32 rows x 32 columns of the addend on their way into the staging bytes
+            stg_free();
+            if (lane == 0) { mbar_expect_tx(&bars->add_full[warp - 2], STG_BYTES); tma_load_2d(stg, &io.add, x, y, &bars->add_full[warp - 2]); }
+        };
+        auto add_take = [&](float *v) -> bool {                // v[0..32) += this lane's row
+            const bool r = __all_sync(0xffffffffu, mbar_wait(&bars->add_full[warp - 2], add_count++ & 1u, abort_flag, status));
+            if (r) {
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const uint4 a4 = *piece(j);
+                    v[4 * j] += __uint_as_float(a4.x); v[4 * j + 1] += __uint_as_float(a4.y); v[4 * j + 2] += __uint_as_float(a4.z); v[4 * j + 3] += __uint_as_float(a4.w);
+                }
+            }
+            __syncwarp();
+            return r;
+        };
+        for (int tile = pair; tile < num_tiles && ok; tile += npairs, tcount += NSUB) {
+            int tm, cb;
+            tile_at(tile, tm, cb);
+            const int prob = MODE == SUM ? 1 : cb / tiles_n;
+            const EpiArgs &pe = epp.p[prob];                   // this tile's problem: its output, scales and addend
+            const int row0 = tm * 2 * BM + (int)rank * BM + q * 32, row = row0 + lane, n0 = (MODE == SUM ? cb : cb - prob * tiles_n) * BN + cfirst;
+            const bool row_ok = row < M_eff;
+            const bool live = row0 < M_eff && n0 < pe.N;       // some of this warp's part of the tile exists
+            const float sc = row_ok ? epi_row_scale(pe, row) : 1.f;
+            const EpiRow er(pe, row_ok ? row : 0);
+            const bool add = MODE != DIRECT && pe.addend && live;
+            if (MODE == TMA && add) add_fetch(n0, row0);       // the first columns' addend arrives while the products run
+            // one 32-column group of results: to the output, and to the next norm's input where that is asked for
+            float ss = 0.f;
+            auto emit = [&](int c0, const float *v) {
+                const int col = n0 + c0;
+                if (pe.c_is_f32) {
+                    stg_free();
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) *piece(j) = make_uint4(__float_as_uint(v[4 * j]), __float_as_uint(v[4 * j + 1]), __float_as_uint(v[4 * j + 2]), __float_as_uint(v[4 * j + 3]));
+                    stg_store(&io.c[prob], col, row0);
+                } else {
+                    if (!(c0 & 32)) stg_free();
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        *piece((c0 & 32) / 8 + j) = make_uint4(pack_bf16(v[8 * j], v[8 * j + 1]), pack_bf16(v[8 * j + 2], v[8 * j + 3]),
+                                                              pack_bf16(v[8 * j + 4], v[8 * j + 5]), pack_bf16(v[8 * j + 6], v[8 * j + 7]));
+                    if ((c0 & 32) || col + 32 >= pe.N) stg_store(&io.c[prob], n0 + (c0 & ~63), row0);
+                }
+                if (pe.u) {                                    // 32 rows x 64 bytes, the 64-byte swizzle of its map
+                    stg_free();
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const bool in = col + 8 * j < pe.N;    // N is a multiple of 8
+                        const uint4 w4 = in ? __ldg(reinterpret_cast<const uint4 *>(pe.u_w + col + 8 * j)) : make_uint4(0u, 0u, 0u, 0u);
+                        const float *x = v + 8 * j;
+                        *reinterpret_cast<uint4 *>(stg + lane * 64 + ((j ^ ((lane >> 1) & 3)) << 4)) =
+                            make_uint4(pack_bf16(x[0] * bf16_lo(w4.x), x[1] * bf16_hi(w4.x)), pack_bf16(x[2] * bf16_lo(w4.y), x[3] * bf16_hi(w4.y)),
+                                       pack_bf16(x[4] * bf16_lo(w4.z), x[5] * bf16_hi(w4.z)), pack_bf16(x[6] * bf16_lo(w4.w), x[7] * bf16_hi(w4.w)));
+                        if (in) {
+#pragma unroll
+                            for (int e = 0; e < 8; ++e) ss = fmaf(x[e], x[e], ss);
+                        }
+                    }
+                    stg_store(&io.u, col, row0);
+                    if ((c0 & 32) || col + 32 >= pe.N) {
+                        if (row_ok) pe.u_ssq[(int64_t)row * ((pe.N + 63) / 64) + col / 64] = ss;
+                        ss = 0.f;
+                    }
+                }
+            };
+            if constexpr (MODE == SUM) {
+                const EpiArgs &p0 = epp.p[0];
+                const float sc0 = row_ok ? epi_row_scale(p0, row) : 1.f;
+                float held[COLS];
+                if (!(ok = ready(tcount))) break;
+#pragma unroll
+                for (int c0 = 0; c0 < COLS; c0 += 32) {
+                    const bool some = n0 + c0 < pe.N;
+                    if (add && some) add_fetch(n0 + c0, row0);
+                    uint32_t r[32];
+                    tmem_ld_x32(tlane + (tcount & 1u) * BN + c0, r);
+                    tmem_wait_ld();
+                    float v[32];
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]) * sc0;
+                    if (some) epi_pre<false>(p0, er, n0 + c0, v);
+                    if (add && some && ok) ok = add_take(v);
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) held[c0 + j] = v[j];
+                }
+                drained(tcount & 1u);
+                if (!ok || !(ok = ready(tcount + 1))) break;
+#pragma unroll
+                for (int c0 = 0; c0 < COLS; c0 += 32) {
+#pragma unroll
+                    for (int c1 = c0; c1 < c0 + 32; c1 += 16) {
+                        uint32_t r[16];
+                        tmem_ld_x16(tlane + ((tcount + 1) & 1u) * BN + c1, r);
+                        tmem_wait_ld();
+                        if (er.cs_row) {
+#pragma unroll
+                            for (int j = 0; j < 16; j += 4) {
+                                const float4 cs = n0 + c1 + j < pe.N ? __ldg(reinterpret_cast<const float4 *>(er.cs_row + n0 + c1 + j)) : make_float4(0.f, 0.f, 0.f, 0.f);      // N is a multiple of 4
+                                held[c1 + j] = fmaf(__uint_as_float(r[j]) * sc, cs.x, held[c1 + j]);
+                                held[c1 + j + 1] = fmaf(__uint_as_float(r[j + 1]) * sc, cs.y, held[c1 + j + 1]);
+                                held[c1 + j + 2] = fmaf(__uint_as_float(r[j + 2]) * sc, cs.z, held[c1 + j + 2]);
+                                held[c1 + j + 3] = fmaf(__uint_as_float(r[j + 3]) * sc, cs.w, held[c1 + j + 3]);
+                            }
+                        } else {
+#pragma unroll
+                            for (int j = 0; j < 16; ++j) held[c1 + j] = fmaf(__uint_as_float(r[j]), sc, held[c1 + j]);
+                        }
+                    }
+                    if (c0 == COLS - 32) drained((tcount + 1) & 1u);
+                    if (live && n0 + c0 < pe.N) emit(c0, held + c0);
+                }
+            } else {
+                if (!(ok = ready(tcount))) break;
+#pragma unroll 1
+                for (int c0 = 0; c0 < COLS; c0 += 32) {
+                    uint32_t r[32];
+                    tmem_ld_x32(tlane + (tcount & 1u) * BN + c0, r);
+                    tmem_wait_ld();
+                    if (c0 == COLS - 32) drained(tcount & 1u);
+                    const int col = n0 + c0;
+                    if (!live || col >= pe.N || (MODE == DIRECT && !row_ok)) continue;
+                    float v[32];
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]) * sc;
+                    epi_pre<true>(pe, er, col, v);
+                    if constexpr (MODE == DIRECT) {
+                        epi_add_store(pe, er, row, col, v);
+                    } else {
+                        if (add) {
+                            if (c0 > 0) add_fetch(col, row0);
+                            if (!(ok = add_take(v))) break;
+                        }
+                        emit(c0, v);
+                    }
+                }
+            }
+        }
+        if (MODE != DIRECT && lane == 0) {
+            bulk_wait_read0();                                 // (what the stores wrote is complete when the launch is)
+            if (!ok) sleep_ns(100000000ull);                   // aborting: an addend load in flight gets time to land
         }
     }
     // ---------------------------------------------------------------- teardown: neither CTA leaves while the other may still signal it
@@ -179,31 +339,47 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_consta
     }
 }
 
-template <int BN>
+template <int BN, int MODE>
 cudaError_t launch(const GemmArgs &a, const GemmArgs *b, float *const *hi, cudaStream_t s) {
     using T = Tile<BN>;
     CUtensorMap ma[2], mb[2];
     if (!make_map_2d(&ma[0], a.A, a.M, a.K, a.lda, BM) || !make_map_2d(&mb[0], a.B, a.N, a.K, a.ldb, BN / 2)) return cudaErrorInvalidValue;
     ma[1] = ma[0]; mb[1] = mb[0];
     if (b && (!make_map_2d(&ma[1], b->A, b->M, b->K, b->lda, BM) || !make_map_2d(&mb[1], b->B, b->N, b->K, b->ldb, BN / 2))) return cudaErrorInvalidValue;
-    constexpr size_t smem = T::STAGES * (size_t)T::STAGE + sizeof(Bars) + 1024;
+    constexpr size_t smem = T::STAGES * (size_t)T::STAGE + (MODE == DIRECT ? 0 : 8 * STG_BYTES) + sizeof(Bars) + 1024;
     static_assert(smem <= 232448, "shared memory budget");
-    cudaError_t e = cudaFuncSetAttribute(gemm_pair_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(gemm_pair_kernel<BN, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     int *status = device_status_ptr();
     if (!status) return cudaErrorUnknown;
     const EpiPair epp = epi_pair_of(a, b, hi);
-    const int64_t tiles = (int64_t)((a.M + 2 * BM - 1) / (2 * BM)) * ((a.N + BN - 1) / BN) * epp.nprob;
+    IoMaps io;
+    memset(&io, 0, sizeof(io));
+    if (MODE != DIRECT) {
+        for (int i = MODE == SUM ? 1 : 0; i < epp.nprob; ++i) {
+            const EpiArgs &p = epp.p[i];
+            if (!(p.c_is_f32 ? make_map_f32_2d(&io.c[i], p.C, p.M, p.N, p.ldc, 32) : make_map_2d(&io.c[i], p.C, p.M, p.N, p.ldc, 32))) return cudaErrorInvalidValue;
+        }
+        const EpiArgs &p = epp.p[MODE == SUM ? 1 : 0];         // (separate problems in one launch have no addend here: see tma_io)
+        if (p.addend && !make_map_f32_2d(&io.add, p.addend, p.M, p.N, p.ld_add, 32)) return cudaErrorInvalidValue;
+        if (p.u && !make_map_u(&io.u, p.u, p.M, p.N)) return cudaErrorInvalidValue;
+    }
+    const int64_t tiles = (int64_t)((a.M + 2 * BM - 1) / (2 * BM)) * ((a.N + BN - 1) / BN) * (MODE == SUM ? 1 : epp.nprob);
     const int pairs = sm_count() / 2, grid = 2 * (int)(tiles < pairs ? tiles : pairs);
-    gemm_pair_kernel<BN><<<grid, NTHREADS, smem, s>>>(ma[0], mb[0], ma[1], mb[1], epp, status);
+    gemm_pair_kernel<BN, MODE><<<grid, NTHREADS, smem, s>>>(ma[0], mb[0], ma[1], mb[1], io, epp, status);
     count_launch();
     return cudaGetLastError();
 }
 
+bool tma_io(const GemmArgs &a, const GemmArgs *b) { return gemm_pair_tma_io(a) && (!b || (gemm_pair_tma_io(*b) && !a.addend && !b->addend && !a.u && !b->u)); }
+
 }  // namespace
 
 cudaError_t gemm_pair_launch(bool wide, const GemmArgs &a, const GemmArgs *b, float *const *hi, cudaStream_t s) {
-    return wide ? launch<256>(a, b, hi, s) : launch<128>(a, b, hi, s);
+    if (tma_io(a, b)) return wide ? launch<256, TMA>(a, b, hi, s) : launch<128, TMA>(a, b, hi, s);
+    return wide ? launch<256, DIRECT>(a, b, hi, s) : launch<128, DIRECT>(a, b, hi, s);
 }
+
+cudaError_t gemm_pair_sum_launch(const GemmArgs &a, const GemmArgs &b, cudaStream_t s) { return launch<256, SUM>(a, &b, nullptr, s); }
 
 }  // namespace dm

@@ -16,7 +16,8 @@ __global__ void __launch_bounds__(256)
 gemm_simple_kernel(const TIn *__restrict__ A, int64_t lda, const TIn *__restrict__ B, int64_t ldb,
                    TOut *C, int64_t ldc, int M, int N, int K,
                    const float *__restrict__ row_scale, const float *addend, int64_t ld_add, int silu_cols,
-                   const float *__restrict__ col_bias, int gelu, const float *__restrict__ col_scale, int cs_rows, int64_t ld_cs, const int *__restrict__ m_dev, int m_off) {
+                   const float *__restrict__ col_bias, int gelu, const float *__restrict__ col_scale, int cs_rows, int64_t ld_cs, const int *__restrict__ m_dev, int m_off,
+                   const float *__restrict__ rs_ssq, int rs_n, float rs_inv, float rs_eps) {
     if (m_dev) M = min(M, max(0, *m_dev - m_off));
     __shared__ float As[BK][BM + 4];
     __shared__ float Bs[BK][BN + 4];
@@ -52,7 +53,12 @@ gemm_simple_kernel(const TIn *__restrict__ A, int64_t lda, const TIn *__restrict
     for (int i = 0; i < TM; ++i) {
         const int gm = m0 + ty * TM + i;
         if (gm >= M) continue;
-        const float sc = row_scale ? row_scale[gm] : 1.f;
+        float sc = row_scale ? row_scale[gm] : 1.f;
+        if (rs_ssq) {
+            float q = 0.f;
+            for (int j = 0; j < rs_n; ++j) q += rs_ssq[(int64_t)gm * rs_n + j];
+            sc = rsqrtf(q * rs_inv + rs_eps);
+        }
 #pragma unroll
         for (int j = 0; j < TN; ++j) {
             const int gn = n0 + tx * TN + j;
@@ -75,7 +81,8 @@ cudaError_t launch(const GemmArgs &a, cudaStream_t s) {
     gemm_simple_kernel<TIn, TOut><<<grid, 256, 0, s>>>(
         static_cast<const TIn *>(a.A), a.lda, static_cast<const TIn *>(a.B), a.ldb,
         static_cast<TOut *>(a.C), a.ldc, a.M, a.N, a.K, a.row_scale, a.addend, a.ld_add, a.silu_cols,
-        a.col_bias, a.gelu, a.col_scale, a.cs_rows > 0 ? a.cs_rows : 1, a.ld_cs > 0 ? a.ld_cs : a.N, a.m_dev, a.m_off);
+        a.col_bias, a.gelu, a.col_scale, a.cs_rows > 0 ? a.cs_rows : 1, a.ld_cs > 0 ? a.ld_cs : a.N, a.m_dev, a.m_off,
+        a.rs_ssq, a.rs_n, a.rs_inv, a.rs_eps);
     count_launch();
     return cudaGetLastError();
 }
@@ -83,7 +90,7 @@ cudaError_t launch(const GemmArgs &a, cudaStream_t s) {
 }  // namespace
 
 cudaError_t gemm_simple(const GemmArgs &a, cudaStream_t s) {
-    if (a.M <= 0 || a.N <= 0 || a.K <= 0) return cudaErrorInvalidValue;
+    if (a.M <= 0 || a.N <= 0 || a.K <= 0 || a.u) return cudaErrorInvalidValue;
     if ((a.M + BM - 1) / BM > 65535) return cudaErrorInvalidValue;
     if (a.in_dtype == DM_F32) {
         return a.c_dtype == DM_F32 ? launch<float, float>(a, s) : launch<float, __nv_bfloat16>(a, s);

@@ -126,7 +126,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
             const uint32_t buf = tcount & 1u, bph = (tcount >> 1) & 1u;
             const int prob = tile / tiles_n, n0 = (tile - prob * tiles_n) * BN;
             const EpiArgs &pe = epp.p[prob];               // this tile's problem: its output, scales and addend
-            const float sc = (pe.row_scale && row_ok) ? pe.row_scale[row] : 1.f;
+            const float sc = row_ok ? epi_row_scale(pe, row) : 1.f;
             const EpiRow er(pe, row);
             ok = mbar_wait(&bars->tmem_full[buf], bph, abort_flag, status);
             ok = __all_sync(0xffffffffu, ok);
@@ -142,7 +142,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant
                 float v[32];
 #pragma unroll
                 for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]) * sc;
-                epi_cols32<true>(pe, er, row, col, v);
+                epi_pre<true>(pe, er, col, v);
+                epi_add_store(pe, er, row, col, v);
             }
             fence_before();
             __syncwarp();
@@ -213,6 +214,8 @@ bool gemm_tcgen05_supports(const GemmArgs &a) {
     if (a.addend && (reinterpret_cast<uintptr_t>(a.addend) & 15u)) return false;
     if (a.col_bias && (reinterpret_cast<uintptr_t>(a.col_bias) & 15u)) return false;
     if (a.col_scale && ((reinterpret_cast<uintptr_t>(a.col_scale) & 15u) || ((a.ld_cs > 0 ? a.ld_cs : (int64_t)a.N) & 3))) return false;
+    if (a.rs_ssq && (reinterpret_cast<uintptr_t>(a.rs_ssq) & 15u)) return false;
+    if (a.u && (a.M <= BM || a.c_dtype != DM_F32 || !gemm_pair_tma_io(a) || ((reinterpret_cast<uintptr_t>(a.u) | reinterpret_cast<uintptr_t>(a.u_w)) & 15u) || (a.N % 8))) return false;
     return encode_fn() != nullptr;
 }
 
@@ -229,6 +232,15 @@ bool gemm_tcgen05_pair_supports(const GemmArgs &a, const GemmArgs &b) {
 cudaError_t gemm_tcgen05_pair(const GemmArgs &a, const GemmArgs &b, cudaStream_t s) {
     if (!gemm_tcgen05_pair_supports(a, b)) return cudaErrorNotSupported;
     return dispatch(a, &b, nullptr, s);
+}
+
+bool gemm_tcgen05_sum_supports(const GemmArgs &a, const GemmArgs &b) {
+    return gemm_tcgen05_supports(b) && gemm_tcgen05_supports(a) && a.M == b.M && a.N == b.N && a.K == b.K && a.M > BM && !a.m_dev && !b.m_dev && gemm_pair_tma_io(b);
+}
+
+cudaError_t gemm_tcgen05_sum(const GemmArgs &a, const GemmArgs &b, cudaStream_t s) {
+    if (!gemm_tcgen05_sum_supports(a, b)) return cudaErrorNotSupported;
+    return gemm_pair_sum_launch(a, b, s);
 }
 
 // Few rows and a long K (the out_proj pair of block decoding): whole products fill less than half of the SMs.  Halving K instead doubles

@@ -45,6 +45,23 @@ def test_denoise_step_full_sequence(G, dtype, N, d, H, layers, V):
     np.testing.assert_array_equal(amax, amax2)
 
 
+@pytest.mark.parametrize("d,H,B,L,d_ff", [(160, 5, 3, 683, 0), (64, 2, 1, 2049, 0), (320, 10, 2, 1100, 640)])
+def test_denoise_step_summed_out_proj(G, d, H, B, L, d_ff):
+    """Above 2048 tokens both directions' out_proj run as one launch that also writes the next norm's input: ragged rows, widths
+    that end inside the 64-column parts of its sums of squares (and inside a 256-column tile); with a gate on the sum."""
+    shape = I.MixerShape(B, L, d, 2, 32, 4, H)
+    sw = I.make_stack_weights(shape, 3, 96, seed=7, dtype=I.BF16, perturb=True)
+    tau = None
+    if d_ff:
+        I.add_block_weights(sw, shape, d_ff, 32, seed=7, dtype=I.BF16)
+        tau = I.make_timestep_embedding(B, 32, seed=7)
+    tok = I.make_tokens(B, L, 95, 95, seed=7)
+    kw = G.oracle_kwargs(shape)
+    want = O.denoise_step_cond(tok, tau, sw, **kw) if d_ff else O.denoise_step(tok, sw, **kw)
+    got, _, _ = G.run_denoise(shape, I.BF16, sw, tok, 96, want_argmax=False, tau=tau, d_ff=d_ff)
+    assert G.rel_l2(got, want) <= 1e-2, G.rel_l2(got, want)
+
+
 @pytest.mark.parametrize("dtype", [I.F32, I.BF16])
 def test_denoise_step_block_mode(G, dtype):
     d, N, H, V, layers = 64, 16, 4, 120, 2
