@@ -231,6 +231,8 @@ static int run_mixer(const dm_mixer_cfg *c, const Dims &m, const dm_dir_weights 
         if (n == 2 && m.T <= PAIR_IN_MAX_T && gemm_tcgen05_pair_supports(ga[0], ga[1])) {
             // both directions in one launch: x is fetched once for the two, and there is one tail round instead of two
             if ((e = gemm_tcgen05_pair(ga[0], ga[1], s)) != cudaSuccess) return cuda_fail(e, "in_proj");
+        } else if (n == 2 && gemm_f32_supports(ga[0], 2) && gemm_f32_supports(ga[1], 2)) {
+            if ((e = gemm_f32(ga[0], &ga[1], false, s)) != cudaSuccess) return cuda_fail(e, "in_proj");
         } else {
             for (int i = 0; i < n; ++i)
                 if ((e = gemm(ga[i], s)) != cudaSuccess) return cuda_fail(e, "in_proj");
@@ -277,8 +279,8 @@ static int run_mixer(const dm_mixer_cfg *c, const Dims &m, const dm_dir_weights 
             return DM_OK;
         }
     }
-    if (!tied && c->dir_mask == DM_DIR_BOTH && m.T > PAIR_OUT_MAX_T) {
-        // long inputs: both out_proj and their sum in one launch, each direction's gated-norm scale taken from the sums of squares in the epilogue
+    if (!tied && c->dir_mask == DM_DIR_BOTH && (m.T > PAIR_OUT_MAX_T || c->dtype == DM_F32)) {
+        // long inputs, and fp32 ones that do not fill the GPU: both out_proj and their sum in one launch, each direction's gated-norm scale taken from the sums of squares in the epilogue
         GemmArgs ga[2];
         for (int dir = 0; dir < 2; ++dir) {
             GemmArgs a{};
@@ -295,6 +297,11 @@ static int run_mixer(const dm_mixer_cfg *c, const Dims &m, const dm_dir_weights 
             out.fuse_norm(ga[1], m.d);
             StageTimer tm(DM_STAGE_OUT_PROJ, s);
             if ((e = gemm_tcgen05_sum(ga[0], ga[1], s)) != cudaSuccess) return cuda_fail(e, "out_proj");
+            return DM_OK;
+        }
+        if (gemm_f32_supports(ga[0], 2) && gemm_f32_supports(ga[1], 2)) {
+            StageTimer tm(DM_STAGE_OUT_PROJ, s);
+            if ((e = gemm_f32(ga[0], &ga[1], true, s)) != cudaSuccess) return cuda_fail(e, "out_proj");
             return DM_OK;
         }
     }

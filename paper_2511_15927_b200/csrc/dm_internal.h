@@ -48,6 +48,9 @@ struct GemmArgs {
     int m_off;
 };
 cudaError_t gemm_simple(const GemmArgs &a, cudaStream_t s);
+// fp32 products that do not fill the GPU: n of them (same sizes) in one launch, or both into b's output (sum).
+bool gemm_f32_supports(const GemmArgs &a, int n);
+cudaError_t gemm_f32(const GemmArgs &a, const GemmArgs *b, bool sum, cudaStream_t s);
 // Tensor-core path (tcgen05 + TMEM + TMA).  Returns cudaErrorNotSupported for shapes it does not take.
 cudaError_t gemm_tcgen05(const GemmArgs &a, cudaStream_t s);
 bool gemm_tcgen05_supports(const GemmArgs &a);

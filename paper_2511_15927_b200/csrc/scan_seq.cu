@@ -7,22 +7,24 @@
 //   scan threads (the first P * LPC):  the state h[p][n] of the head lives in their registers: channel p is served
 //       by LPC adjacent lanes, each holding N / LPC states; the C-contraction is finished with warp shuffles.  They
 //       run the token loop of chunk i from shared memory and leave y_t = h_t C_t + D x_t there.
-//   loader threads (the last 128):  meanwhile they write chunk i-1's gated output (g = y SiLU(z) [* norm_w], per-head
-//       sum of squares) and prepare chunk i+1: conv + SiLU of this head's x channels with one global load per output
-//       (a sliding window along time per channel), B' and C' copied from scratch, z, Delta and the decay.
-// One __syncthreads per chunk hands the buffers over.  The first chunk is prepared, and the last one finished, by all
-// threads.  B' and C' (conv + SiLU of the B and C columns, shared by all heads) come from a small launch of their own.
+//   loader threads (the last 128 or 256):  meanwhile one half of them start the copies of chunk i+2 (x, z, B', C': TMA, straight to shared memory)
+//       and prepare chunk i+1 (conv + SiLU of this head's x channels, Delta and the decay), the other half write chunk i-1's gated output
+//       (g = y SiLU(z) [* norm_w], per-head sum of squares).
+// One __syncthreads per chunk hands the buffers over.  B' and C' (conv + SiLU of the B and C columns, shared by all heads) come from a small launch
+// of their own.  What bounds it is the chain of L tokens in each of the 2 B H CTAs: at 8 heads of 32, d_state 16, L = 256 a chunk of 32 tokens takes 2.9 k clocks, in
+// the scan threads and in the preparing ones alike, and both launches 25 us; with one synchronous loader group, which waited for memory three
+// times a chunk, it was 74 us.
 //
 // This is the exact (fp32) form of the recurrence: the kernel for fp32 I/O (whose 1e-4 tolerance rules out bf16
 // products) and for d_state above 128; bf16 I/O with d_state <= 128 runs the chunked kernels of scan_ssd.cu, block
 // decoding with carried state included.
 #include "dm_internal.h"
+#include "tc_ptx.cuh"
 
 namespace dm {
 namespace {
 
-constexpr int NL = 128;            // loader threads
-constexpr int NSEG = 4;            // time segments per conv channel (parallelism of the sliding windows)
+using namespace tc;
 
 template <typename T> __device__ __forceinline__ float ldf(const T *p);
 template <> __device__ __forceinline__ float ldf<float>(const float *p) { return __ldg(p); }
@@ -33,33 +35,20 @@ template <typename T> __device__ __forceinline__ void stf(T *p, float v);
 template <> __device__ __forceinline__ void stf<float>(float *p, float v) { *p = v; }
 template <> __device__ __forceinline__ void stf<__nv_bfloat16>(__nv_bfloat16 *p, float v) { *p = __float2bfloat16_rn(v); }
 
-// 16 bytes of T -> floats (VEC = 16 / sizeof(T) elements)
-template <typename T> struct Vec16;
-template <> struct Vec16<float> {
-    static constexpr int VEC = 4;
-    static __device__ __forceinline__ void load(const float *p, float *o) {
-        const float4 v = __ldg(reinterpret_cast<const float4 *>(p));
-        o[0] = v.x; o[1] = v.y; o[2] = v.z; o[3] = v.w;
-    }
-};
-template <> struct Vec16<__nv_bfloat16> {
-    static constexpr int VEC = 8;
-    static __device__ __forceinline__ void load(const __nv_bfloat16 *p, float *o) {
-        const uint4 v = __ldg(reinterpret_cast<const uint4 *>(p));
-        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-        for (int i = 0; i < 4; ++i) { o[2 * i] = __uint_as_float(w[i] << 16); o[2 * i + 1] = __uint_as_float(w[i] & 0xFFFF0000u); }
-    }
-};
+__device__ __forceinline__ float to_f(float v) { return v; }
+__device__ __forceinline__ float to_f(__nv_bfloat16 v) { return __bfloat162float(v); }
+inline size_t es_of(const ScanArgs &a) { return dtype_size(a.dtype); }
 
 __device__ __forceinline__ float silu_f(float v) { return __fdividef(v, 1.f + __expf(-v)); }     // ~1e-6 relative: inside the fp32 tolerance
 __device__ __forceinline__ float softplus_f(float v) { return fmaxf(v, 0.f) + log1pf(expf(-fabsf(v))); }
 
 // B' and C' of every token: conv + SiLU of the 2N shared columns, in logical time order semantics (the reverse layer
-// looks at later rows), fp32, layout [dir][B*L][2N].  Thread = one column of one run of `rows` consecutive tokens.
+// looks at later rows), fp32, layout [dir][B*L][2N].  Thread = one column of one run of BC_ROWS consecutive tokens, all its loads in flight at
+// once: the launch is a handful of CTAs and one round trip to memory (runs of 32 tokens took 19 us at L = 256).
+constexpr int BC_ROWS = 8;
 template <typename T>
 __global__ void __launch_bounds__(256)
-bc_prep_kernel(const ScanArgs a, const int dir0, float *__restrict__ bc, const int rows) {
+bc_prep_kernel(const ScanArgs a, const int dir0, float *__restrict__ bc) {
     const int N2 = 2 * a.N, L = a.L, k = a.k;
     const int dir = dir0 + blockIdx.z, b = blockIdx.y;
     const bool rev = dir == 1;
@@ -69,54 +58,64 @@ bc_prep_kernel(const ScanArgs a, const int dir0, float *__restrict__ bc, const i
     const T *conv_in = (!rev && a.conv_in) ? static_cast<const T *>(a.conv_in) + (int64_t)b * (k - 1) * a.conv_ch : nullptr;
     float *out = bc + ((int64_t)dir * T_all + (int64_t)b * L) * N2;
     const bool has_bias = (a.flags & DM_FLAG_CONV_BIAS) && w.conv_b != nullptr;
-    const int tau0 = blockIdx.x * rows;
-    for (int col = threadIdx.x; col < N2; col += blockDim.x) {
-        const int cc = a.d_inner + col;
-        auto raw = [&](int tau) -> float {
-            if (tau >= L) return 0.f;
-            if (tau >= 0) return ldf(zx + (int64_t)(rev ? L - 1 - tau : tau) * a.d_in_proj + a.d_inner + cc);
-            return conv_in ? ldf(conv_in + (int64_t)(k - 1 + tau) * a.conv_ch + cc) : 0.f;
-        };
-        float wl[4];
+    const int task = blockIdx.x * blockDim.x + threadIdx.x, col = task % N2, tau0 = task / N2 * BC_ROWS, cc = a.d_inner + col;
+    if (tau0 >= L) return;
+    float v[BC_ROWS + 3];                                  // pre-conv values of tau0 - 3 .. tau0 + BC_ROWS - 1
 #pragma unroll
-        for (int m = 0; m < 4; ++m) wl[m] = m < k ? ldf(static_cast<const T *>(w.conv_w) + (int64_t)cc * k + (k - 1 - m)) : 0.f;
-        const float bias = has_bias ? ldf(static_cast<const T *>(w.conv_b) + cc) : 0.f;
-        float h1 = raw(tau0 - 1), h2 = k > 2 ? raw(tau0 - 2) : 0.f, h3 = k > 3 ? raw(tau0 - 3) : 0.f;
-#pragma unroll 4
-        for (int i = 0; i < rows; ++i) {
-            const int tau = tau0 + i;
-            if (tau >= L) break;
-            const float cur = raw(tau);
-            float v = bias;
-            v = fmaf(wl[3], h3, v); v = fmaf(wl[2], h2, v); v = fmaf(wl[1], h1, v); v = fmaf(wl[0], cur, v);
-            out[(int64_t)(rev ? L - 1 - tau : tau) * N2 + col] = silu_f(v);
-            h3 = h2; h2 = h1; h1 = cur;
-        }
+    for (int i = 0; i < BC_ROWS + 3; ++i) {
+        const int tau = tau0 + i - 3;
+        v[i] = 0.f;
+        if (tau >= 0 && tau < L) v[i] = ldf(zx + (int64_t)(rev ? L - 1 - tau : tau) * a.d_in_proj + a.d_inner + cc);
+        else if (tau < 0 && conv_in && k - 1 + tau >= 0) v[i] = ldf(conv_in + (int64_t)(k - 1 + tau) * a.conv_ch + cc);
+    }
+    float wl[4];
+#pragma unroll
+    for (int m = 0; m < 4; ++m) wl[m] = m < k ? ldf(static_cast<const T *>(w.conv_w) + (int64_t)cc * k + (k - 1 - m)) : 0.f;
+    const float bias = has_bias ? ldf(static_cast<const T *>(w.conv_b) + cc) : 0.f;
+#pragma unroll
+    for (int i = 0; i < BC_ROWS; ++i) {
+        const int tau = tau0 + i;
+        if (tau >= L) break;
+        float r = fmaf(wl[3], v[i], bias);
+        r = fmaf(wl[2], v[i + 1], r); r = fmaf(wl[1], v[i + 2], r); r = fmaf(wl[0], v[i + 3], r);
+        out[(int64_t)(rev ? L - 1 - tau : tau) * N2 + col] = silu_f(r);
     }
 }
 
-// NQ = float4 groups of state per lane (N / LPC / 4): 4 for N <= 128, 8 for N = 256.
-template <typename T, int NQ>
-__global__ void __launch_bounds__(512 + NL)
-scan_seq_kernel(const ScanArgs a, const int dir0, const int TC, const int LPC, const float *__restrict__ bc_all) {
-    extern __shared__ __align__(16) float smem[];
-    const int P = a.P, N = a.N, L = a.L, k = a.k;
-    const int NS = P * LPC;                            // scan threads
+// Shared memory (bytes).  A raw stage holds one chunk as it comes from memory: [B' | C'] fp32 [TC][2N], x [TC + 3][P] (3 rows of history first) and z [TC][P] of
+// type T; RAW of them: chunk i - 1 (its z), i (B', C'), i + 1 (x) and i + 2 (in flight).  Then, for two chunks each: conv'd x and y [TC][P], Delta and the decay [TC].
+constexpr int RAW = 4;
+__host__ __device__ constexpr int lanes_per_channel(int n) { return n / 4 < 8 ? n / 4 : 8; }
+__host__ __device__ constexpr int loaders(int p, int n) { return p * lanes_per_channel(n) > 256 ? 128 : 256; }      // loader threads
+struct SeqSmem {
+    int TC, P, N, es;
+    __host__ __device__ int xoff() const { return TC * 2 * N * 4; }                                              // a multiple of 128, as TMA wants its tiles
+    __host__ __device__ int zoff() const { return xoff() + up128((TC + 3) * P * es); }
+    __host__ __device__ int raw_bytes() const { return zoff() + up128(TC * P * es); }
+    __host__ __device__ static int up128(int v) { return (v + 127) / 128 * 128; }
+    __host__ __device__ int cooked() const { return RAW * raw_bytes(); }
+    __host__ __device__ int cooked_floats() const { return TC * (2 * P + 2); }
+    __host__ __device__ size_t total() const { return (size_t)cooked() + 2 * (size_t)cooked_floats() * 4; }
+};
+
+// P channels and N states of a head; LPC = lanes per channel, NQ = float4 groups of state per lane
+template <typename T, int P, int N>
+__global__ void __launch_bounds__(P * lanes_per_channel(N) + loaders(P, N))
+scan_seq_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_z, const __grid_constant__ ScanArgs a, const int dir0, const int TC, const float *__restrict__ bc_all, int *status) {
+    extern __shared__ __align__(128) uint8_t smem[];
+    __shared__ uint64_t bars[RAW];                     // raw stage has landed
+    __shared__ int abort_word;
+    volatile int *abort_flag = &abort_word;
+    constexpr int LPC = lanes_per_channel(N), NQ = N / (4 * LPC), NS = P * LPC, NL = loaders(P, N), NP = NL / 2;       // NS: scan threads, NL: loader threads, NP of them preparing
+    const int L = a.L, k = a.k;
     const int h = blockIdx.x, b = blockIdx.z;
     const int dir = dir0 + blockIdx.y;                 // 0 = left-to-right, 1 = right-to-left
     const bool rev = dir == 1;
     const int tid = threadIdx.x;
-
-    // two stages of { xs[TC][P] conv(x), zs[TC][P] z, Bs[TC][N], Cs[TC][N], dl[TC] Delta, da[TC] exp(Delta A) }, then ys[2][TC][P],
-    // then xr[(TC+3)][P]: the pre-conv x rows of the chunk being prepared (3 rows of history first)
-    const int stage_floats = TC * (2 * P + 2 * N + 2);
-    float *ys_all = smem + 2 * stage_floats;
-    float *xr = ys_all + 2 * TC * P;
-    constexpr int VEC = Vec16<T>::VEC;
-    // 16-byte loads need every row slice to start on a 16-byte boundary
-    const bool vec_ok = ((a.d_in_proj * (int)sizeof(T)) % 16 == 0) && (((int64_t)a.d_inner * sizeof(T)) % 16 == 0) &&
-                        ((P * (int)sizeof(T)) % 16 == 0) && ((reinterpret_cast<uintptr_t>(a.zx) & 15u) == 0);
-    auto xs_of = [&](int s) { return smem + s * stage_floats; };
+    const SeqSmem lay{TC, P, N, (int)sizeof(T)};
+    const int raw_bytes = lay.raw_bytes(), xoff = lay.xoff(), zoff = lay.zoff(), cooked_floats = lay.cooked_floats();
+    auto raw_of = [&](int ci) { return smem + (ci % RAW) * raw_bytes; };
+    auto xs_of = [&](int ci) { return reinterpret_cast<float *>(smem + RAW * raw_bytes) + (ci & 1) * cooked_floats; };      // x', then y, Delta, decay
 
     const ScanDir &w = a.dir[dir];
     const T *conv_w = static_cast<const T *>(w.conv_w);
@@ -132,125 +131,138 @@ scan_seq_kernel(const ScanArgs a, const int dir0, const int TC, const int LPC, c
     const T *conv_in = (!rev && a.conv_in) ? static_cast<const T *>(a.conv_in) + (int64_t)b * (k - 1) * a.conv_ch : nullptr;
     const float *bc = bc_all + ((int64_t)dir * T_all + (int64_t)b * L) * (2 * N);
     const int nchunks = (L + TC - 1) / TC;
-    const int nall = blockDim.x;
-
-    const float Ah = -expf(w.A_log[h]);
-    const float dtb = w.dt_bias[h];
-    // pre-conv value of conv channel cc at logical time tau (tau < 0: carried rows or zeros)
-    auto raw = [&](int tau, int cc) -> float {
-        if (tau >= 0) {
-            const int t = rev ? L - 1 - tau : tau;
-            return ldf(zx + (int64_t)t * a.d_in_proj + a.d_inner + cc);
-        }
-        return (conv_in && k - 1 + tau >= 0) ? ldf(conv_in + (int64_t)(k - 1 + tau) * a.conv_ch + cc) : 0.f;
-    };
-    // everything the token loop of chunk ci reads, by threads lt = 0..nthr-1
-    auto prepare = [&](int ci, int lt, int nthr) {
-        const int s = ci & 1, tau0 = ci * TC, tc = min(TC, L - tau0);
-        float *xs = xs_of(s), *zs = xs + TC * P, *Bs = zs + TC * P, *Cs = Bs + TC * N, *dl = Cs + TC * N, *da = dl + TC;
-        // ---- phase 1: global -> shared with independent loads: pre-conv x rows (3 rows of history first), z, B', C'
-        const int upr = P / VEC;                           // 16-byte units per row slice
-        if (vec_ok) {
-#pragma unroll 4
-            for (int u = lt; u < (tc + 3) * upr; u += nthr) {
-                const int r = u / upr, c = (u - r * upr) * VEC, tau = tau0 + r - 3;
-                float o[VEC];
-                if (tau >= 0) {
-                    Vec16<T>::load(zx + (int64_t)(rev ? L - 1 - tau : tau) * a.d_in_proj + a.d_inner + h * P + c, o);
-                } else {
-#pragma unroll
-                    for (int e = 0; e < VEC; ++e) o[e] = raw(tau, h * P + c + e);
-                }
-#pragma unroll
-                for (int e = 0; e < VEC; ++e) xr[r * P + c + e] = o[e];
-            }
-#pragma unroll 4
-            for (int u = lt; u < tc * upr; u += nthr) {
-                const int i = u / upr, c = (u - i * upr) * VEC;
-                const int t = rev ? L - 1 - (tau0 + i) : tau0 + i;
-                float o[VEC];
-                Vec16<T>::load(zx + (int64_t)t * a.d_in_proj + h * P + c, o);
-#pragma unroll
-                for (int e = 0; e < VEC; ++e) zs[i * P + c + e] = o[e];
-            }
-        } else {
-            for (int e = lt; e < (tc + 3) * P; e += nthr) {
-                const int r = e / P, c = e - r * P;
-                xr[r * P + c] = raw(tau0 + r - 3, h * P + c);
-            }
-            for (int e = lt; e < tc * P; e += nthr) {
-                const int i = e / P, c = e - i * P;
-                const int t = rev ? L - 1 - (tau0 + i) : tau0 + i;
-                zs[i * P + c] = ldf(zx + (int64_t)t * a.d_in_proj + h * P + c);
-            }
-        }
-        const int n4 = N / 2;                              // float4 per token row of [B' | C']
-#pragma unroll 4
-        for (int e = lt; e < tc * n4; e += nthr) {
-            const int i = e / n4, c4 = e - i * n4;
-            const int t = rev ? L - 1 - (tau0 + i) : tau0 + i;
-            const float4 v = __ldg(reinterpret_cast<const float4 *>(bc + (int64_t)t * 2 * N) + c4);
-            float *dst = c4 * 4 < N ? Bs + i * N + c4 * 4 : Cs + i * N + (c4 * 4 - N);
-            *reinterpret_cast<float4 *>(dst) = v;
-        }
-        if (nthr == nall) __syncthreads();
-        else asm volatile("bar.sync 1, %0;" ::"n"(NL) : "memory");
-        // ---- phase 2: conv + SiLU of this head's x channels from shared memory: task = (time segment, channel)
-        const int seglen = (tc + NSEG - 1) / NSEG;
-        for (int task = lt; task < NSEG * P; task += nthr) {
-            const int seg = task / P, col = task - seg * P;
-            const int i0 = seg * seglen, i1 = min(tc, i0 + seglen);
-            if (i0 >= i1) continue;
-            const int cc = h * P + col;
-            float wl[4];                                   // wl[m] multiplies the row m steps back in time
-#pragma unroll
-            for (int m = 0; m < 4; ++m) wl[m] = m < k ? ldf(conv_w + (int64_t)cc * k + (k - 1 - m)) : 0.f;
-            const float bias = has_bias ? ldf(conv_b + cc) : 0.f;
-            const float *xc = xr + 3 * P + col;              // xc[i * P] = pre-conv value at chunk row i
-            float h1 = xc[(i0 - 1) * P], h2 = xc[(i0 - 2) * P], h3 = xc[(i0 - 3) * P];
-#pragma unroll 4
-            for (int i = i0; i < i1; ++i) {
-                const float cur = xc[i * P];
-                float v = bias;
-                v = fmaf(wl[3], h3, v); v = fmaf(wl[2], h2, v); v = fmaf(wl[1], h1, v); v = fmaf(wl[0], cur, v);
-                xs[i * P + col] = silu_f(v);
-                h3 = h2; h2 = h1; h1 = cur;
-            }
-        }
-        for (int i = lt; i < tc; i += nthr) {
-            const int t = rev ? L - 1 - (tau0 + i) : tau0 + i;
-            const float dlt = softplus_f(ldf(zx + (int64_t)t * a.d_in_proj + a.d_inner + a.conv_ch + h) + dtb);
-            dl[i] = dlt;
-            da[i] = expf(dlt * Ah);
-        }
-    };
-    // gated output of chunk ci: one warp per token, lanes over the channels; by warps lw = 0..nwarp-1
-    auto finish = [&](int ci, int lw, int nwarp, int lane) {
-        const int s = ci & 1, tau0 = ci * TC, tc = min(TC, L - tau0);
-        const float *zs = xs_of(s) + TC * P, *ys = ys_all + s * TC * P;
-        for (int i = lw; i < tc; i += nwarp) {
-            const int t = rev ? L - 1 - (tau0 + i) : tau0 + i;
-            float sacc = 0.f;
-            for (int c = lane; c < P; c += 32) {
-                float gv = ys[i * P + c] * silu_f(zs[i * P + c]);
-                sacc = fmaf(gv, gv, sacc);
-                if (norm_on && norm_w) gv *= ldf(norm_w + h * P + c);
-                stf(gout + (int64_t)t * a.d_inner + h * P + c, gv);
-            }
-            for (int off = 16; off > 0; off >>= 1) sacc += __shfl_xor_sync(0xffffffffu, sacc, off);
-            if (lane == 0 && ssq) ssq[(int64_t)t * a.H + h] = sacc;
-        }
-    };
-    prepare(0, tid, nall);                                 // first chunk: everybody
+    const int sg = rev ? -1 : 1, x0 = rev ? TC - 1 : 3, z0 = rev ? TC - 1 : 0;      // token i of a chunk is row x0 + sg i of its x tile, z0 + sg i of its z tile
+    if (tid == 0) {
+        for (int i = 0; i < RAW; ++i) mbar_init(&bars[i], 1);
+        abort_word = 0;
+        mbar_fence_init();
+    }
     __syncthreads();
 
-    if (tid >= NS) {
-        // ------------------------------------------------------------------ loader group
-        const int lt = tid - NS;
+    // gated output of chunk ci: one warp per token, lanes over the channels; by warps lw = 0..nwarp-1
+    constexpr int CPL = P / 32;                        // channels per lane
+    float nw[CPL];
+#pragma unroll
+    for (int e = 0; e < CPL; ++e) nw[e] = (norm_on && norm_w) ? ldf(norm_w + h * P + (tid & 31) + 32 * e) : 1.f;
+    auto finish = [&](int ci, int lw, int nwarp, int lane) {
+        const int tau0 = ci * TC, tc = min(TC, L - tau0);
+        const T *zs = reinterpret_cast<const T *>(raw_of(ci) + zoff);
+        const float *ys = xs_of(ci) + TC * P;
+        constexpr int FU = 8 / CPL;                              // tokens in flight per warp
+        for (int i0 = lw; i0 < tc; i0 += FU * nwarp) {
+            float gv[FU][CPL], sacc[FU];
+#pragma unroll
+            for (int u = 0; u < FU; ++u) {
+                const int i = min(i0 + u * nwarp, tc - 1);
+                sacc[u] = 0.f;
+#pragma unroll
+                for (int e = 0; e < CPL; ++e) {
+                    const int c = lane + 32 * e;
+                    gv[u][e] = ys[i * P + c] * silu_f(to_f(zs[(z0 + sg * i) * P + c]));
+                    sacc[u] = fmaf(gv[u][e], gv[u][e], sacc[u]);
+                }
+            }
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) {
+#pragma unroll
+                for (int u = 0; u < FU; ++u) sacc[u] += __shfl_xor_sync(0xffffffffu, sacc[u], off);
+            }
+#pragma unroll
+            for (int u = 0; u < FU; ++u) {
+                const int i = i0 + u * nwarp;
+                if (i >= tc) break;
+                const int t = rev ? L - 1 - (tau0 + i) : tau0 + i;
+#pragma unroll
+                for (int e = 0; e < CPL; ++e) stf(gout + (int64_t)t * a.d_inner + h * P + lane + 32 * e, gv[u][e] * nw[e]);
+                if (lane == 0 && ssq) ssq[(int64_t)t * a.H + h] = sacc[u];
+            }
+        }
+    };
+
+    if (tid >= NS + NP) {
+        // ------------------------------------------------------------------ finishing half of the loader group
+        const int lt = tid - NS - NP;
+        __syncthreads();
         for (int ci = 0; ci < nchunks; ++ci) {
-            if (ci > 0) finish(ci - 1, lt >> 5, NL / 32, lt & 31);
-            asm volatile("bar.sync 1, %0;" ::"n"(NL) : "memory");     // the stage read by finish() is the one prepare() refills
-            if (ci + 1 < nchunks) prepare(ci + 1, lt, NL);
+            if (ci > 0) finish(ci - 1, lt >> 5, NP / 32, lt & 31);
+            __syncthreads();
+        }
+    } else if (tid >= NS) {
+        // ------------------------------------------------------------------ preparing half
+        const int lt = tid - NS;
+        const float Ah = -expf(w.A_log[h]);
+        const float dtb = w.dt_bias[h];
+        // Everything chunk ci needs from memory: a tile of x with the three rows before it in time, one of z (rows outside the sequence become zeros) and
+        // the run of [B' | C'], in physical order.  (16-byte copies by the threads took 1000 clocks a chunk to issue, and held up the
+        // shared-memory reads behind them.)
+        auto fetch = [&](int ci) {
+            if (ci >= nchunks || lt != 0) return;
+            uint8_t *st = raw_of(ci);
+            uint64_t *bar = &bars[ci % RAW];
+            const int tau0 = ci * TC, tc = min(TC, L - tau0), bt = a.zx_tied ? b : dir * a.B + b, t0 = rev ? L - TC - tau0 : tau0;
+            mbar_expect_tx(bar, (uint32_t)((2 * TC + 3) * P * sizeof(T) + tc * 2 * N * 4));
+            tma_load_3d(st + xoff, &map_x, a.d_inner + h * P, rev ? t0 : t0 - 3, bt, bar);
+            tma_load_3d(st + zoff, &map_z, h * P, t0, bt, bar);
+            bulk_load(st, bc + (int64_t)(rev ? L - tau0 - tc : tau0) * 2 * N, tc * 2 * N * 4, bar);
+        };
+        // the carried rows before the sequence (the tile has zeros there)
+        auto carry = [&](int ci) {
+            const int neg = 3 - min(3, ci * TC);               // rows of this chunk's history that are before the sequence
+            if (!conv_in || neg <= 0) return;
+            T *xt = reinterpret_cast<T *>(raw_of(ci) + xoff);
+            for (int u = lt; u < neg * P; u += NP) {
+                const int r = u / P, c = u - r * P, src = k - 1 - neg + r;      // tile row r = token r - neg before the first one
+                if (src >= 0) xt[r * P + c] = conv_in[(int64_t)src * a.conv_ch + h * P + c];
+            }
+            named_sync(1, NP);
+        };
+        auto landed = [&](int ci) { mbar_wait(&bars[ci % RAW], (ci / RAW) & 1, abort_flag, status); };      // (gives up after its limit, then at once: the loop still ends)
+        auto dt_of = [&](int ci) {                         // raw step size of token lt of the chunk (TC <= NP)
+            const int tau = ci * TC + lt;
+            return (lt < TC && tau < L) ? ldf(zx + (int64_t)(rev ? L - 1 - tau : tau) * a.d_in_proj + a.d_inner + a.conv_ch + h) : 0.f;
+        };
+        // conv + SiLU of this head's channels, Delta and decay: task = (channel, run of tokens); with P = 32 or 64 a thread keeps its channel
+        constexpr int nseg = NP / P;
+        const int col = lt % P, cc = h * P + col, seg = lt / P;
+        float wl[4];                                       // wl[m] multiplies the row m steps back in time
+#pragma unroll
+        for (int m = 0; m < 4; ++m) wl[m] = m < k ? ldf(conv_w + (int64_t)cc * k + (k - 1 - m)) : 0.f;
+        const float bias = has_bias ? ldf(conv_b + cc) : 0.f;
+        auto prepare = [&](int ci, float dt_raw) {
+            const int tc = min(TC, L - ci * TC);
+            float *xs = xs_of(ci), *dl = xs + 2 * TC * P, *da = dl + TC;
+            const T *xc = reinterpret_cast<const T *>(raw_of(ci) + xoff) + x0 * P + col;
+            const int sP = sg * P;                             // xc[i * sP] = pre-conv value at token i of the chunk
+            const int len = (tc + nseg - 1) / nseg, i0 = seg * len, i1 = min(tc, i0 + len);
+            if (i0 < i1) {
+                float h1 = to_f(xc[(i0 - 1) * sP]), h2 = to_f(xc[(i0 - 2) * sP]), h3 = to_f(xc[(i0 - 3) * sP]);
+#pragma unroll 4
+                for (int i = i0; i < i1; ++i) {
+                    const float cur = to_f(xc[i * sP]);
+                    float v = fmaf(wl[3], h3, bias);
+                    v = fmaf(wl[2], h2, v); v = fmaf(wl[1], h1, v); v = fmaf(wl[0], cur, v);
+                    xs[i * P + col] = silu_f(v);
+                    h3 = h2; h2 = h1; h1 = cur;
+                }
+            }
+            if (lt < tc) {
+                const float dlt = softplus_f(dt_raw + dtb);
+                dl[lt] = dlt;
+                da[lt] = expf(dlt * Ah);
+            }
+        };
+        fetch(0);
+        fetch(1);
+        float dt_cur = dt_of(0), dt_next = dt_of(1);
+        landed(0);
+        carry(0);
+        prepare(0, dt_cur);
+        __syncthreads();
+        for (int ci = 0; ci < nchunks; ++ci) {
+            fetch(ci + 2);                                 // its stage held chunk ci - 2, finished before the last barrier
+            dt_cur = dt_next;
+            dt_next = dt_of(ci + 2);
+            if (ci + 1 < nchunks) { landed(ci + 1); carry(ci + 1); prepare(ci + 1, dt_cur); }
             __syncthreads();
         }
     } else {
@@ -270,31 +282,55 @@ scan_seq_kernel(const ScanArgs a, const int dir0, const int TC, const int LPC, c
 #pragma unroll
             for (int q = 0; q < 4 * NQ; ++q) hst[q] = 0.f;
         }
+        __syncthreads();
         for (int ci = 0; ci < nchunks; ++ci) {
-            const int s = ci & 1, tc = min(TC, L - ci * TC);
-            const float *xs = xs_of(s), *Bs = xs + 2 * TC * P, *Cs = Bs + TC * N, *dl = Cs + TC * N, *da = dl + TC;
-            float *ys = ys_all + s * TC * P;
-            // h_t = a_t h_{t-1} + Delta_t x_t (x) B_t ;  y_t = h_t C_t + D x_t
-#pragma unroll 2
-            for (int i = 0; i < tc; ++i) {
-                const float av = da[i];
-                const float xv = xs[i * P + p];
-                const float dx = dl[i] * xv;
-                const float4 *B4 = reinterpret_cast<const float4 *>(Bs + i * N);
-                const float4 *C4 = reinterpret_cast<const float4 *>(Cs + i * N);
-                float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;      // four partial sums keep the dependent chain short
+            const int tc = min(TC, L - ci * TC);
+            const float *xs = xs_of(ci), *dl = xs + 2 * TC * P, *da = dl + TC;
+            mbar_wait(&bars[ci % RAW], (ci / RAW) & 1, abort_flag, status);      // (the loaders have waited for it already)
+            const float *BC = reinterpret_cast<const float *>(raw_of(ci)) + (rev ? tc - 1 : 0) * 2 * N;
+            float *ys = xs_of(ci) + TC * P;
+            // h_t = a_t h_{t-1} + Delta_t x_t (x) B_t ;  y_t = h_t C_t + D x_t.  Only h depends on the token before: several tokens' loads and
+            // contractions are in flight together
+            // (all loads of U tokens first: one warp per scheduler has to overlap their latency by itself)
+            constexpr int U = NQ == 1 ? 8 : NQ == 2 ? 4 : NQ == 4 ? 2 : 1;
+            auto tokens = [&](int i, int n) {                  // tokens i .. i + n - 1, n <= U
+                float av[U], xv[U], dx[U], acc[U];
+                float4 bv[U][NQ], cv[U][NQ];
 #pragma unroll
-                for (int q = 0; q < NQ; ++q) {
-                    const float4 bv = B4[q * LPC + j], cv = C4[q * LPC + j];
-                    hst[4 * q + 0] = fmaf(av, hst[4 * q + 0], dx * bv.x); a0 = fmaf(hst[4 * q + 0], cv.x, a0);
-                    hst[4 * q + 1] = fmaf(av, hst[4 * q + 1], dx * bv.y); a1 = fmaf(hst[4 * q + 1], cv.y, a1);
-                    hst[4 * q + 2] = fmaf(av, hst[4 * q + 2], dx * bv.z); a2 = fmaf(hst[4 * q + 2], cv.z, a2);
-                    hst[4 * q + 3] = fmaf(av, hst[4 * q + 3], dx * bv.w); a3 = fmaf(hst[4 * q + 3], cv.w, a3);
+                for (int e = 0; e < U; ++e) {
+                    const int ie = e < n ? i + e : i;
+                    const float4 *B4 = reinterpret_cast<const float4 *>(BC + sg * ie * 2 * N) + j, *C4 = B4 + N / 4;
+                    av[e] = da[ie]; xv[e] = xs[ie * P + p]; dx[e] = dl[ie];
+#pragma unroll
+                    for (int q = 0; q < NQ; ++q) { bv[e][q] = B4[q * LPC]; cv[e][q] = C4[q * LPC]; }
                 }
-                float acc = (a0 + a1) + (a2 + a3);
-                for (int off = LPC >> 1; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-                if (j == 0) ys[i * P + p] = fmaf(Dh, xv, acc);
-            }
+#pragma unroll
+                for (int e = 0; e < U; ++e) {
+                    dx[e] *= xv[e];
+                    if (e >= n) { av[e] = 1.f; dx[e] = 0.f; }
+                    float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;      // four partial sums keep the dependent chain short
+#pragma unroll
+                    for (int q = 0; q < NQ; ++q) {
+                        hst[4 * q + 0] = fmaf(av[e], hst[4 * q + 0], dx[e] * bv[e][q].x); a0 = fmaf(hst[4 * q + 0], cv[e][q].x, a0);
+                        hst[4 * q + 1] = fmaf(av[e], hst[4 * q + 1], dx[e] * bv[e][q].y); a1 = fmaf(hst[4 * q + 1], cv[e][q].y, a1);
+                        hst[4 * q + 2] = fmaf(av[e], hst[4 * q + 2], dx[e] * bv[e][q].z); a2 = fmaf(hst[4 * q + 2], cv[e][q].z, a2);
+                        hst[4 * q + 3] = fmaf(av[e], hst[4 * q + 3], dx[e] * bv[e][q].w); a3 = fmaf(hst[4 * q + 3], cv[e][q].w, a3);
+                    }
+                    acc[e] = (a0 + a1) + (a2 + a3);
+                }
+#pragma unroll
+                for (int off = LPC >> 1; off > 0; off >>= 1) {
+#pragma unroll
+                    for (int e = 0; e < U; ++e) acc[e] += __shfl_xor_sync(0xffffffffu, acc[e], off);
+                }
+                if (j == 0) {
+#pragma unroll
+                    for (int e = 0; e < U; ++e) if (e < n) ys[(i + e) * P + p] = fmaf(Dh, xv[e], acc[e]);
+                }
+            };
+            int i = 0;
+            for (; i + U <= tc; i += U) tokens(i, U);
+            if (i < tc) tokens(i, tc - i);
             __syncthreads();
         }
         if (!rev && a.ssm_out) {
@@ -305,7 +341,29 @@ scan_seq_kernel(const ScanArgs a, const int dir0, const int TC, const int LPC, c
                     make_float4(hst[4 * q], hst[4 * q + 1], hst[4 * q + 2], hst[4 * q + 3]);
         }
     }
-    finish(nchunks - 1, tid >> 5, nall >> 5, tid & 31);    // last chunk: everybody (the loop's last barrier made y visible)
+    finish(nchunks - 1, tid >> 5, blockDim.x >> 5, tid & 31);    // last chunk: everybody (the loop's last barrier made y visible)
+}
+
+// The in_proj output [2 B][L][d_in_proj] in boxes of `rows` x P channels, no swizzle.
+bool make_map_rows(CUtensorMap *m, const ScanArgs &a, int rows) {
+    EncodeTiledFn fn = encode_fn();
+    if (!fn) return false;
+    const cuuint64_t es = es_of(a), d[3] = {(cuuint64_t)a.d_in_proj, (cuuint64_t)a.L, (cuuint64_t)2 * a.B}, st[2] = {a.d_in_proj * es, a.L * a.d_in_proj * es};
+    const cuuint32_t b[3] = {(cuuint32_t)a.P, (cuuint32_t)rows, 1}, e[3] = {1, 1, 1};
+    return fn(m, a.dtype == DM_BF16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<void *>(a.zx), d, st, b, e,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+typedef void (*Kern)(const CUtensorMap, const CUtensorMap, const ScanArgs, const int, const int, const float *, int *);
+template <typename T> Kern kernel_for(int P, int N) {
+    switch (N) {
+        case 16: return P == 32 ? scan_seq_kernel<T, 32, 16> : scan_seq_kernel<T, 64, 16>;
+        case 32: return P == 32 ? scan_seq_kernel<T, 32, 32> : scan_seq_kernel<T, 64, 32>;
+        case 64: return P == 32 ? scan_seq_kernel<T, 32, 64> : scan_seq_kernel<T, 64, 64>;
+        case 128: return P == 32 ? scan_seq_kernel<T, 32, 128> : scan_seq_kernel<T, 64, 128>;
+        case 256: return P == 32 ? scan_seq_kernel<T, 32, 256> : scan_seq_kernel<T, 64, 256>;
+        default: return nullptr;
+    }
 }
 
 }  // namespace
@@ -317,35 +375,37 @@ size_t scan_seq_workspace_bytes(const ScanArgs &a) {
 cudaError_t scan_sequential(const ScanArgs &a, void *ws, cudaStream_t s) {
     if (!ws) return cudaErrorInvalidValue;
     if (a.N % 16 || a.P % 32) return cudaErrorNotSupported;
-    const int NQ = a.N > 128 ? 8 : 4;
-    const int LPC = a.N / (4 * NQ);                     // lanes per channel: 1, 2, 4 or 8
-    const int NS = a.P * LPC;
-    if (LPC < 1 || (LPC & (LPC - 1)) || LPC > 8 || NS > 512 || NS < 32 || a.N != 4 * NQ * LPC) return cudaErrorNotSupported;
+    if (a.P != 32 && a.P != 64) return cudaErrorNotSupported;
+    // 16-byte rows for TMA: true of every workspace and configuration the entry points let through
+    if ((int64_t)a.d_in_proj * es_of(a) % 16 || (int64_t)a.d_inner * es_of(a) % 16 || (int64_t)a.conv_ch * es_of(a) % 16) return cudaErrorNotSupported;
     const int ndir = (a.dir_mask == DM_DIR_BOTH) ? 2 : 1;
     const int dir0 = (a.dir_mask == DM_DIR_REV) ? 1 : 0;
     int TC = a.chunk > 0 ? a.chunk : 32;
     if (TC > a.L) TC = a.L;
+    if (TC > 64) TC = 64;                               // one preparing thread per token's step size
     size_t smem;
     for (;;) {
-        smem = ((size_t)TC * (2 * (2 * a.P + 2 * a.N + 2) + 2 * a.P) + (size_t)(TC + 3) * a.P) * sizeof(float);
-        if (smem <= 160 * 1024 || TC == 1) break;
+        smem = SeqSmem{TC, a.P, a.N, (int)es_of(a)}.total();
+        if (smem <= 200 * 1024 || TC == 1) break;
         TC = (TC + 1) / 2;
     }
-    typedef void (*Kern)(const ScanArgs, const int, const int, const int, const float *);
-    Kern kern;
-    if (a.dtype == DM_BF16) kern = NQ == 8 ? (Kern)scan_seq_kernel<__nv_bfloat16, 8> : (Kern)scan_seq_kernel<__nv_bfloat16, 4>;
-    else kern = NQ == 8 ? (Kern)scan_seq_kernel<float, 8> : (Kern)scan_seq_kernel<float, 4>;
+    const Kern kern = a.dtype == DM_BF16 ? kernel_for<__nv_bfloat16>(a.P, a.N) : kernel_for<float>(a.P, a.N);
+    if (!kern) return cudaErrorNotSupported;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
+    CUtensorMap mx, mz;
+    if (!make_map_rows(&mx, a, TC + 3) || !make_map_rows(&mz, a, TC)) return cudaErrorInvalidValue;
+    int *status = device_status_ptr();
+    if (!status) return cudaErrorUnknown;
     float *bc = static_cast<float *>(ws);
-    const int rows = 32;
-    dim3 pgrid((a.L + rows - 1) / rows, a.B, ndir);
-    if (a.dtype == DM_BF16) bc_prep_kernel<__nv_bfloat16><<<pgrid, 256, 0, s>>>(a, dir0, bc, rows);
-    else bc_prep_kernel<float><<<pgrid, 256, 0, s>>>(a, dir0, bc, rows);
+    const int tasks = (a.L + BC_ROWS - 1) / BC_ROWS * 2 * a.N, bt = tasks >= 256 * 148 ? 256 : 64;        // small CTAs while they do not fill the GPU
+    dim3 pgrid((tasks + bt - 1) / bt, a.B, ndir);
+    if (a.dtype == DM_BF16) bc_prep_kernel<__nv_bfloat16><<<pgrid, bt, 0, s>>>(a, dir0, bc);
+    else bc_prep_kernel<float><<<pgrid, bt, 0, s>>>(a, dir0, bc);
     count_launch();
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     dim3 grid(a.H, ndir, a.B);
-    kern<<<grid, NS + NL, smem, s>>>(a, dir0, TC, LPC, bc);
+    kern<<<grid, a.P * lanes_per_channel(a.N) + loaders(a.P, a.N), smem, s>>>(mx, mz, a, dir0, TC, bc, status);
     count_launch();
     return cudaGetLastError();
 }

@@ -65,6 +65,20 @@ def test_other_state_sizes_fp32(G, dims):
     _check(got, O.bimamba_forward(x, wf, wr, **G.oracle_kwargs(shape)), I.F32)
 
 
+@pytest.mark.parametrize("dtype,P,N,L,chunk", [(I.F32, 32, 16, 97, 1), (I.F32, 64, 16, 70, 2), (I.F32, 32, 32, 33, 5), (I.F32, 64, 64, 200, 64),
+                                               (I.F32, 64, 256, 37, 0), (I.BF16, 32, 256, 75, 0), (I.BF16, 64, 256, 40, 3)])
+def test_sequential_kernel_tiles(G, dtype, P, N, L, chunk):
+    """The sequential kernel's staging: tiles of one token up to the largest, lengths that leave a partial last tile, every kind of
+    lane split; a carried state, so that the rows before the sequence are read."""
+    shape = I.MixerShape(2, L, 2 * P, 2, N, 4, 4)
+    wf, wr, x = _case(shape, dtype, seed=P + L)
+    ssm_in, conv_in = I.make_states(shape, 3, dtype)
+    y, s, c = G.run_block_step(shape, dtype, wf, wr, x, ssm_in, conv_in, chunk=chunk)
+    y_o, s_o, c_o = O.bimamba_block_step(x, wf, wr, ssm_state_in=ssm_in, conv_state_in=conv_in, **G.oracle_kwargs(shape))
+    _check(y, y_o, dtype)
+    assert G.rel_l2(s, s_o) <= (1e-4 if dtype == I.F32 else 1e-2), G.rel_l2(s, s_o)
+
+
 @pytest.mark.parametrize("dims", [(256, 128, 8, 300), (256, 16, 8, 260), (192, 128, 12, 130)])
 def test_bf16_parity_small(G, dims):
     d, N, H, L = dims
