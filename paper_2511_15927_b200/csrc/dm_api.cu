@@ -122,6 +122,8 @@ static int check_weights(const dm_mixer_cfg *c, const dm_dir_weights w[2]) {
 // Up to this many tokens the two directions' out_proj run as one launch that writes an fp32 partial each (summed by a small
 // kernel); above it they are chained, the second adding the first in its epilogue, which moves less memory.
 constexpr int64_t PAIR_OUT_MAX_T = 2048;
+// Up to this many tokens the out_proj launch cuts K over clusters and sums both directions in shared memory (gemm_rows.cu).
+constexpr int64_t SUM_OUT_MAX_T = 128;
 // Up to this many tokens the two directions' in_proj share one launch.  Beyond it two launches are faster: both weight matrices
 // together (70 MB at d_model 2048) no longer stay in L2 while the rows of x stream past them (measured at 16 384 tokens: 1.00 ms
 // for the pair against 0.84 ms for two launches; level at 8192, 15-25 % faster for the 512 tokens of a decoding step).
@@ -249,7 +251,7 @@ static int run_mixer(const dm_mixer_cfg *c, const Dims &m, const dm_dir_weights 
         e = conv_state_update(zx, conv_in, conv_out, c->dtype, m.B, m.L, m.k, m.d_inner, m.conv_ch, m.ldz, s);
         if (e != cudaSuccess) return cuda_fail(e, "conv_state_update");
     }
-    if (!tied && c->dir_mask == DM_DIR_BOTH && m.T <= PAIR_OUT_MAX_T && sum_partials_norm_supports(m.d)) {
+    if (!tied && c->dir_mask == DM_DIR_BOTH && m.T <= PAIR_OUT_MAX_T && m.T > SUM_OUT_MAX_T && sum_partials_norm_supports(m.d)) {
         // short inputs (block decoding): both out_proj in one launch, each into its own fp32 partial (gated by col_scale, not yet scaled by the
         // gated norm); one pass then scales, sums, adds the residual and applies the caller's next norm
         GemmArgs ga[2];
@@ -279,8 +281,8 @@ static int run_mixer(const dm_mixer_cfg *c, const Dims &m, const dm_dir_weights 
             return DM_OK;
         }
     }
-    if (!tied && c->dir_mask == DM_DIR_BOTH && (m.T > PAIR_OUT_MAX_T || c->dtype == DM_F32)) {
-        // long inputs, and fp32 ones that do not fill the GPU: both out_proj and their sum in one launch, each direction's gated-norm scale taken from the sums of squares in the epilogue
+    if (!tied && c->dir_mask == DM_DIR_BOTH && (m.T > PAIR_OUT_MAX_T || m.T <= SUM_OUT_MAX_T || c->dtype == DM_F32)) {
+        // long inputs, a few sequences' blocks, and fp32 inputs that do not fill the GPU: both out_proj and their sum in one launch, each direction's gated-norm scale taken from the sums of squares in the epilogue
         GemmArgs ga[2];
         for (int dir = 0; dir < 2; ++dir) {
             GemmArgs a{};

@@ -41,7 +41,7 @@ struct GemmArgs {
     int64_t ld_cs;           // row pitch of col_scale (0 = N)
     // Row scale from sums of squares instead of row_scale: rsqrt(sum(rs_ssq[r * rs_n .. + rs_n)) * rs_inv + rs_eps); NULL = none
     const float *rs_ssq; int rs_n; float rs_inv, rs_eps;
-    // The next RMSNorm's input (fp32 C, tensor-core kernel for more than 128 rows only): u[r, c] = bf16(C[r, c] * u_w[c]) with row pitch N, and u_ssq[r, j] = sum of
+    // The next RMSNorm's input (fp32 C, tensor-core kernels only): u[r, c] = bf16(C[r, c] * u_w[c]) with row pitch N, and u_ssq[r, j] = sum of
     // C[r, c]^2 over the columns [64 j, 64 j + 64), row pitch ceil(N / 64).  The norm's row scale is left to the product that reads u (rs_ssq); NULL = none
     void *u; const void *u_w; float *u_ssq;
     const int *m_dev;        // device int or NULL: only rows [0, clamp(*m_dev - m_off, 0, M)) are computed (row count known on the device only)
@@ -58,7 +58,7 @@ bool gemm_tcgen05_supports(const GemmArgs &a);
 // of each other: neither reads what the other writes.
 bool gemm_tcgen05_pair_supports(const GemmArgs &a, const GemmArgs &b);
 cudaError_t gemm_tcgen05_pair(const GemmArgs &a, const GemmArgs &b, cudaStream_t s);
-// C = (s_a A_a) B_a^T + (s_b A_b) B_b^T + addend in one pass (s: each problem's row scale; output, addend, column scale and u from b): more than 128 rows.
+// C = (s_a A_a) B_a^T + (s_b A_b) B_b^T + addend in one pass (s: each problem's row scale; output, addend, column scale and u from b).
 bool gemm_tcgen05_sum_supports(const GemmArgs &a, const GemmArgs &b);
 cudaError_t gemm_tcgen05_sum(const GemmArgs &a, const GemmArgs &b, cudaStream_t s);
 // The same pair with each product cut in two along K (fp32 outputs only): the first half of a's product goes to a.C (with its addend and bias),

@@ -218,6 +218,8 @@ inline bool make_map_u(CUtensorMap *m, const void *base, int64_t rows, int64_t c
 // gemm_pair.cu: the two-CTA kernel.  wide: 256 x 256 tiles, else 256 x 128; b, hi: see gemm_tcgen05.cu.  gemm_pair_sum_launch: both products into one output.
 cudaError_t gemm_pair_launch(bool wide, const GemmArgs &a, const GemmArgs *b, float *const *hi, cudaStream_t s);
 cudaError_t gemm_pair_sum_launch(const GemmArgs &a, const GemmArgs &b, cudaStream_t s);
+// gemm_rows.cu: up to 128 rows; sum as in gemm_pair_sum_launch.
+cudaError_t gemm_rows_launch(const GemmArgs &a, const GemmArgs *b, bool sum, cudaStream_t s);
 // Output and addend can go through TMA: 16-byte aligned rows.
 inline bool gemm_pair_tma_io(const GemmArgs &a) {
     return (a.ldc * (int64_t)dtype_size(a.c_dtype)) % 16 == 0 && (!a.addend || a.ld_add % 4 == 0);

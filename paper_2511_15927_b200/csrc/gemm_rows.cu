@@ -1,0 +1,316 @@
+// The GEMM for up to 128 rows (decoding a few sequences): such a product is a read of its weights, so the roles are swapped -- a tile is 128 rows
+// of the weight matrix (the M side of tcgen05.mma) times all the tokens (its N side, 16 to 128), D^T = B A^T -- and what matters is that
+// every SM has weight bytes in flight all the time.  The tiles are cut along K over the CTAs of a cluster until the grid fills the
+// GPU about twice (two CTAs share an SM: while one sets up or finishes, the other one reads); the partial sums go to their owner's shared memory
+// (each CTA of the cluster owns a share of the tokens), which adds them, applies the epilogue and stores them: lanes are
+// consecutive output columns.  sum: the cluster's CTAs are halves over two products (both directions' out_proj) that are added with each product's row scale.
+// Weights from HBM, with tokens as the M side and 128 x 128 tiles before: 32 x 16112 x 1920 18.2 -> 16.3 us, 32 x 1920 x 3840 20.2 -> 8.5 us, 32 x 50304 x 1920
+// 50.6 -> 37.1 us (5.2 TB/s); the rest is start-up: a single token takes 14.5 us where 32 take 16.3.
+//
+// Warp 0 issues the TMA loads, warp 1 the MMAs, the other EW (4 or 8) are the epilogue: one TMEM lane quarter each, tokens shared out between the two
+// warps of a quarter.  Waits and abort as in gemm_pair.cu: every mbarrier wait is bounded, and the CTAs of a cluster leave together.
+#include "gemm_epi.cuh"
+
+namespace dm {
+namespace {
+
+using namespace tc;
+
+constexpr int BF = 128, BK = 64, MAX_STAGES = 8, MAX_CS = 8;
+constexpr uint32_t W_BYTES = BF * BK * 2;
+
+struct __align__(8) Bars {
+    uint64_t full[MAX_STAGES], empty[MAX_STAGES], done;
+    uint32_t tmem_base;
+    int abort;
+    float scale[2][128];           // row scale of this CTA's tokens, per product
+    float red[4][128];             // sums of squares of 32 columns each
+};
+
+struct RowsArgs {
+    EpiArgs p[2];
+    int sum, cs, ks;               // CTAs per cluster, K shares per product
+    int nt, stages, tiles_n;       // nt: tokens rounded up to 16
+    uint32_t tmem_cols;
+};
+
+__device__ __forceinline__ void st_cluster_f32(uint32_t addr, float v) { asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory"); }
+
+// G tokens from t on (n of them exist), one output column: bias, activation, gate, residual, output, the next norm's input.  What does not apply is skipped
+// for all of them at once, and loads come before the arithmetic: a warp has its scheduler almost to itself here, an instruction costs about six clocks.
+template <int G>
+__device__ __forceinline__ void emit(const EpiArgs &ep, int t, int n, int col, bool in, float bias, float uw, float (&v)[G]) {
+    if (!in) {
+#pragma unroll
+        for (int g = 0; g < G; ++g) v[g] = 0.f;
+        return;
+    }
+    float add[G];
+    if (ep.addend) {
+        const float *p = ep.addend + (int64_t)t * ep.ld_add + col;
+#pragma unroll
+        for (int g = 0; g < G; ++g, p += ep.ld_add) add[g] = g < n ? *p : 0.f;
+    }
+    if (ep.col_bias) {
+#pragma unroll
+        for (int g = 0; g < G; ++g) v[g] += bias;
+    }
+    if (col < ep.silu_cols) {
+#pragma unroll
+        for (int g = 0; g < G; ++g) { const float hv = 0.5f * v[g]; v[g] = fmaf(hv, tanh_fast(hv), hv); }      // SiLU(v) = v/2 + v/2 tanh(v/2)
+    }
+    if (ep.gelu) {
+#pragma unroll
+        for (int g = 0; g < G; ++g) { const float x = v[g], hx = 0.5f * x; v[g] = fmaf(hx, tanh_fast(0.7978845608028654f * fmaf(0.044715f * x, x * x, x)), hx); }
+    }
+    if (ep.col_scale) {
+        float cs[G];
+#pragma unroll
+        for (int g = 0; g < G; ++g) cs[g] = g < n ? __ldg(ep.col_scale + (int64_t)((t + g) / ep.cs_rows) * ep.ld_cs + col) : 1.f;
+#pragma unroll
+        for (int g = 0; g < G; ++g) v[g] *= cs[g];
+    }
+    if (ep.addend) {
+#pragma unroll
+        for (int g = 0; g < G; ++g) v[g] += add[g];
+    }
+    if (ep.c_is_f32) {
+        float *p = static_cast<float *>(ep.C) + (int64_t)t * ep.ldc + col;
+#pragma unroll
+        for (int g = 0; g < G; ++g, p += ep.ldc) if (g < n) *p = v[g];
+    } else {
+        __nv_bfloat16 *p = static_cast<__nv_bfloat16 *>(ep.C) + (int64_t)t * ep.ldc + col;
+#pragma unroll
+        for (int g = 0; g < G; ++g, p += ep.ldc) if (g < n) *p = __float2bfloat16_rn(v[g]);
+    }
+    if (ep.u) {
+        __nv_bfloat16 *p = ep.u + (int64_t)t * ep.N + col;
+#pragma unroll
+        for (int g = 0; g < G; ++g, p += ep.N) if (g < n) *p = __float2bfloat16_rn(v[g] * uw);
+    }
+}
+
+template <int EW>
+__global__ void __launch_bounds__(64 + 32 * EW, EW == 4 ? 2 : 1)
+gemm_rows_kernel(const __grid_constant__ CUtensorMap map_x0, const __grid_constant__ CUtensorMap map_w0,
+                 const __grid_constant__ CUtensorMap map_x1, const __grid_constant__ CUtensorMap map_w1,
+                 const __grid_constant__ RowsArgs ra, int *status) {
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t *smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+    const int nt = ra.nt, S = ra.stages, cs = ra.cs, tpc = nt / cs;
+    const uint32_t stage = W_BYTES + (uint32_t)nt * (BK * 2);
+    float *recv = reinterpret_cast<float *>(smem + S * stage);               // [source CTA][own token][BF]  (clusters only)
+    Bars *bars = reinterpret_cast<Bars *>(smem + S * stage + (cs > 1 ? (uint32_t)nt * BF * 4 : 0u));
+    volatile int *abort_flag = &bars->abort;
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int rank = cs > 1 ? (int)cluster_ctarank() : 0, cid = blockIdx.x / cs, tile = cid % ra.tiles_n;
+    const int prod = ra.sum ? rank / ra.ks : cid / ra.tiles_n, kr = rank % ra.ks;
+    const EpiArgs &ep = ra.p[ra.sum ? 1 : prod];                             // output, addend, ...
+    const int M = ep.m_dev ? min(ep.M, max(0, *ep.m_dev - ep.m_off)) : ep.M;
+    const int kblocks = (ep.K + BK - 1) / BK, kb0 = kr * kblocks / ra.ks, nk = (kr + 1) * kblocks / ra.ks - kb0;
+    const int n0 = tile * BF;
+
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < S; ++i) { mbar_init(&bars->full[i], 1); mbar_init(&bars->empty[i], 1); }
+        mbar_init(&bars->done, 1);
+        bars->abort = 0;
+        mbar_fence_init();
+    }
+    if (threadIdx.x == 64) { prefetch_map(prod ? &map_w1 : &map_w0); prefetch_map(prod ? &map_x1 : &map_x0); }
+    if (warp == 1) tmem_alloc(&bars->tmem_base, ra.tmem_cols);
+    __syncwarp();
+    fence_before();
+    if (cs > 1) cluster_sync(); else __syncthreads();                        // (no CTA of a cluster writes to one that has not started)
+    fence_after();
+    const uint32_t tmem = bars->tmem_base;
+
+    bool ok = true;
+    if (warp == 0) {
+        const bool leader = elect_one();
+        const CUtensorMap *mx = prod ? &map_x1 : &map_x0, *mw = prod ? &map_w1 : &map_w0;
+        int s = 0;
+        uint32_t ph = 1;
+        for (int i = 0; i < nk; ++i) {
+            if (!(ok = mbar_wait(&bars->empty[s], ph, abort_flag, status))) break;
+            if (leader) {
+                uint8_t *sw = smem + s * stage;
+                mbar_expect_tx(&bars->full[s], stage);
+                tma_load_2d(sw, mw, (kb0 + i) * BK, n0, &bars->full[s]);
+                tma_load_2d(sw + W_BYTES, mx, (kb0 + i) * BK, 0, &bars->full[s]);
+            }
+            __syncwarp();
+            if (++s == S) { s = 0; ph ^= 1; }
+        }
+        if (!ok) sleep_ns(100000000ull);                                     // aborting: the loads already issued get time to land
+    } else if (warp == 1) {
+        const bool leader = elect_one();
+        const uint32_t idesc = idesc_bf16(BF, nt, 0, 0), d0 = desc_lo_k(smem_u32(smem));
+        int s = 0;
+        uint32_t ph = 0;
+        for (int i = 0; i < nk; ++i) {
+            if (!(ok = mbar_wait(&bars->full[s], ph, abort_flag, status))) break;
+            fence_after();
+            const uint32_t dw = d0 + s * (stage >> 4), dx = dw + (W_BYTES >> 4);
+            if (leader) {
+#pragma unroll
+                for (int k = 0; k < BK / 16; ++k) {
+                    if (i == 0 && k == 0) umma_ss<0>(tmem, dw, dx, idesc); else umma_ss<1>(tmem, dw + 2 * k, dx + 2 * k, idesc);
+                }
+                umma_commit(&bars->empty[s]);
+                if (i == nk - 1) umma_commit(&bars->done);
+            }
+            __syncwarp();
+            if (++s == S) { s = 0; ph ^= 1; }
+        }
+    } else {
+        const int ew = warp - 2, q = warp & 3, f = q * 32 + lane;            // this thread's output column of the tile
+        // row scales of this CTA's tokens, while the products run
+        for (int pi = ra.sum ? 0 : prod; pi <= (ra.sum ? 1 : prod); ++pi) {
+            const EpiArgs &e = ra.p[pi];
+            for (int tl = ew; tl < tpc; tl += EW) {
+                const int t = rank * tpc + tl;
+                float sc = 1.f;
+                if (t < M && e.row_scale) sc = e.row_scale[t];
+                else if (t < M && e.rs_ssq) {
+                    float v = 0.f;
+                    for (int j = lane; j < e.rs_n; j += 32) v += __ldg(e.rs_ssq + (int64_t)t * e.rs_n + j);
+                    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+                    sc = rsqrtf(v * e.rs_inv + e.rs_eps);
+                }
+                if (lane == 0) bars->scale[ra.sum ? pi : 0][tl] = sc;
+            }
+        }
+        named_sync(1, 32 * EW);                                              // the scales are there for all of these warps
+        ok = __all_sync(0xffffffffu, mbar_wait(&bars->done, 0, abort_flag, status));
+        fence_after();
+        if (cs > 1) {                                                        // this CTA's partial sums to the owners of the tokens
+            for (int c0 = 16 * (ew >> 2); c0 < nt && ok; c0 += 4 * EW) {
+                uint32_t r[16];
+                tmem_ld_x16(tmem + ((uint32_t)(q * 32) << 16) + c0, r);
+                tmem_wait_ld();
+                int owner = c0 / tpc, tl = c0 - owner * tpc;
+                uint32_t dst = cluster_addr(recv + (rank * tpc) * BF + f, owner);
+#pragma unroll
+                for (int j = 0; j < 16; ++j) {
+                    st_cluster_f32(dst + tl * (BF * 4), __uint_as_float(r[j]));
+                    if (++tl == tpc && owner + 1 < cs) { tl = 0; ++owner; dst = cluster_addr(recv + (rank * tpc) * BF + f, owner); }
+                }
+            }
+        }
+    }
+    __syncwarp();
+    if (cs > 1) cluster_sync();                                              // every partial sum has arrived; nobody's shared memory is written any more
+    // ---------------------------------------------------------------- the CTA's tokens: sum, epilogue, store
+    if (warp >= 2 && !*abort_flag) {
+        const int ew = warp - 2, q = warp & 3, f = q * 32 + lane, col = n0 + f;
+        const bool in = col < ep.N;
+        const float bias = in && ep.col_bias ? ep.col_bias[col] : 0.f;
+        const float uw = in && ep.u ? __bfloat162float(ep.u_w[col]) : 0.f;
+        auto squares = [&](const auto &v, int tl, int n) {                   // the next norm's sums over this warp's 32 columns
+            if (!ep.u) return;
+#pragma unroll
+            for (int g = 0; g < (int)(sizeof(v) / sizeof(float)); ++g) {
+                float ss = v[g] * v[g];
+#pragma unroll
+                for (int off = 16; off > 0; off >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, off);
+                if (lane == 0 && g < n) bars->red[q][tl + g] = ss;
+            }
+        };
+        if (cs == 1) {
+            for (int c0 = 16 * (ew >> 2); c0 < nt && c0 < M; c0 += 4 * EW) {
+                uint32_t r[16];
+                float v[16];
+                tmem_ld_x16(tmem + ((uint32_t)(q * 32) << 16) + c0, r);
+                tmem_wait_ld();
+#pragma unroll
+                for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(r[j]) * bars->scale[0][c0 + j];
+                emit(ep, c0, min(16, M - c0), col, in, bias, uw, v);
+                squares(v, c0, 16);
+            }
+        } else {
+            const int half = ra.sum ? ra.ks : cs;                            // sources [0, half) are product 0 (or the only one)
+            constexpr int G = 4;
+            for (int tl = G * (ew >> 2); tl < tpc; tl += G * (EW / 4)) {
+                const int t = rank * tpc + tl;
+                if (t >= M) break;
+                float v[G] = {};
+#pragma unroll
+                for (int r = 0; r < MAX_CS; ++r) {
+                    if (r >= cs) break;
+#pragma unroll
+                    for (int g = 0; g < G; ++g) {
+                        const int tg = min(tl + g, tpc - 1);
+                        v[g] = fmaf(recv[(r * tpc + tg) * BF + f], bars->scale[r < half ? 0 : 1][tg], v[g]);
+                    }
+                }
+                emit(ep, t, min(min(G, tpc - tl), M - t), col, in, bias, uw, v);
+                squares(v, tl, tpc - tl);
+            }
+        }
+        if (ep.u) {
+            named_sync(1, 32 * EW);
+            const int parts = (ep.N + 63) / 64;
+            for (int i = threadIdx.x - 64; i < 2 * tpc; i += 32 * EW) {      // (half of the tile, token)
+                const int hf = i / tpc, tl = i - hf * tpc, t = rank * tpc + tl;
+                if (t < M && n0 / 64 + hf < parts) ep.u_ssq[(int64_t)t * parts + n0 / 64 + hf] = bars->red[2 * hf][tl] + bars->red[2 * hf + 1][tl];
+            }
+        }
+    }
+    __syncwarp();
+    fence_before();
+    __syncthreads();
+    if (warp == 1) {
+        fence_after();
+        tmem_dealloc(tmem, ra.tmem_cols);
+    }
+}
+
+}  // namespace
+
+// b == NULL: one product; sum: s_a A_a B_a^T + s_b A_b B_b^T into b's output; else two products of equal sizes side by side.
+cudaError_t gemm_rows_launch(const GemmArgs &a, const GemmArgs *b, bool sum, cudaStream_t s) {
+    RowsArgs ra{};
+    ra.p[0] = epi_of(a);
+    ra.p[1] = b ? epi_of(*b) : ra.p[0];
+    ra.sum = sum ? 1 : 0;
+    ra.nt = (a.M + 15) / 16 * 16;
+    ra.tiles_n = (a.N + BF - 1) / BF;
+    const int items = ra.tiles_n * (b && !sum ? 2 : 1), kblocks = (a.K + BK - 1) / BK, per = sum ? 2 : 1;      // per: products of a cluster
+    const int slots = (ra.nt <= 64 ? 2 : 1) * sm_count();                    // (more tokens: the partial sums of a CTA take 40 KB and more)
+    // K shares: powers of two while the grid fits the GPU at once and a share keeps four steps
+    int ks = 1;
+    while (2 * ks * per <= MAX_CS && items * per * 2 * ks <= slots && kblocks >= 8 * ks && ra.nt % (2 * ks * per) == 0) ks *= 2;
+    ra.ks = ks;
+    ra.cs = ks * per;
+    uint32_t cols = 32;
+    while (cols < (uint32_t)ra.nt) cols *= 2;
+    ra.tmem_cols = cols;
+    const size_t stage = W_BYTES + (size_t)ra.nt * BK * 2, fixed = (ra.cs > 1 ? (size_t)ra.nt * BF * 4 : 0) + sizeof(Bars) + 1024;
+    const int ctas = items * ra.cs;
+    // two CTAs per SM where there are that many and the stages stay at least three deep; else one CTA may use all of the SM, with twice the epilogue warps
+    const bool two = ctas > sm_count() && fixed + 3 * stage <= 113 * 1024;
+    const int stages = (int)(((two ? 113 : 226) * 1024 - fixed) / stage);
+    ra.stages = stages > MAX_STAGES ? MAX_STAGES : stages;
+    const size_t smem = fixed + ra.stages * stage;
+    CUtensorMap mx[2], mw[2];
+    if (!make_map_2d(&mx[0], a.A, a.M, a.K, a.lda, ra.nt) || !make_map_2d(&mw[0], a.B, a.N, a.K, a.ldb, BF)) return cudaErrorInvalidValue;
+    mx[1] = mx[0]; mw[1] = mw[0];
+    if (b && (!make_map_2d(&mx[1], b->A, b->M, b->K, b->lda, ra.nt) || !make_map_2d(&mw[1], b->B, b->N, b->K, b->ldb, BF))) return cudaErrorInvalidValue;
+    auto kern = two ? gemm_rows_kernel<4> : gemm_rows_kernel<8>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
+    if (e != cudaSuccess) return e;
+    int *status = device_status_ptr();
+    if (!status) return cudaErrorUnknown;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(ctas); cfg.blockDim = dim3(two ? 192 : 320); cfg.dynamicSmemBytes = smem; cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = ra.cs; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+    cfg.attrs = at; cfg.numAttrs = 1;
+    e = cudaLaunchKernelEx(&cfg, kern, mx[0], mw[0], mx[1], mw[1], ra, status);
+    count_launch();
+    return e;
+}
+
+}  // namespace dm

@@ -29,6 +29,8 @@ def _rand(shape, seed, dtype, scale=1.0):
                                    (512, 50304 // 16, 128),
                                    # few rows, many columns (ragged rows and columns)
                                    (300, 13000, 192), (512, 17024, 256), (130, 18000, 64),
+                                   # up to 128 rows: K cut over clusters of 2, 4 and 8 CTAs and not at all, one and two CTAs per SM, uneven K shares
+                                   (16, 4200, 2048), (17, 5000, 1096), (48, 300, 4096), (64, 130, 2056), (65, 9000, 1032), (112, 2000, 3000), (128, 1001, 2048),
                                    # the two-CTA kernel around its tiles of 256 rows x 256 or 128 columns: one row or column more, one CTA of a
                                    # pair without rows, K of a single and of one more k-block than the ring of stages holds, several rounds
                                    (257, 128, 64), (256, 129, 72), (384, 250, 456), (385, 40000, 512), (2304, 9480, 136)])
