@@ -119,22 +119,17 @@ __device__ __forceinline__ uint32_t prep_conv_pair(const float (&wl)[2][4], cons
 // softplus(dt + bias) = max(v, 0) + log1p(exp(-|v|)) with the fast exponential and logarithm: log1p by its series where 1 + e
 // would round e away (e < 2^-7: error below e^4 / 4), by log(1 + e) elsewhere.  Relative error of Delta about 1e-6, far inside
 // what the bf16 path needs.
-__device__ __forceinline__ float prep_delta(__nv_bfloat16 dt, float dt_bias) {
-    const float v = __bfloat162float(dt) + dt_bias;
+__device__ __forceinline__ float prep_delta(float dt, float dt_bias) {
+    const float v = dt + dt_bias;
     const float e = __expf(-fabsf(v));
     const float l = e < 0.0078125f ? e * fmaf(e, fmaf(e, 0.33333334f, -0.5f), 1.f) : __logf(1.f + e);
     return fmaxf(v, 0.f) + l;
 }
-// One warp, one head, one 128-token chunk: d[r * ld] = Delta of physical chunk row r.  Writes Lambda (inclusive cumulative
-// Delta A in the direction's time order, log2 units) to dl[0..Q) and Lambda' = Lambda - log2 Delta to dl[Lp..Lp + Q).
-__device__ __forceinline__ void prep_lambda_head(const float *d_col, int ld, float A_log, bool rev, int lane, float *dl, int Lp) {
+// One warp, one head, one 128-token chunk: d[e] = Delta of the token 4 lane + e in the direction's time order.  Writes Lambda (inclusive cumulative
+// Delta A in that order, log2 units) of physical chunk row r to dl[r] and Lambda' = Lambda - log2 Delta to dl[Lp + r].
+__device__ __forceinline__ void prep_lambda_head(const float (&d)[4], float A_log, bool rev, int lane, float *dl, int Lp) {
     const float Ah = -expf(A_log) * 1.4426950408889634f;
-    float d[4], cum[4];
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-        const int tau = 4 * lane + e, r = rev ? Q - 1 - tau : tau;
-        d[e] = d_col[r * ld];
-    }
+    float cum[4];
     cum[0] = d[0] * Ah; cum[1] = fmaf(d[1], Ah, cum[0]); cum[2] = fmaf(d[2], Ah, cum[1]); cum[3] = fmaf(d[3], Ah, cum[2]);
     float run = cum[3];
 #pragma unroll
@@ -154,14 +149,17 @@ __device__ __forceinline__ void prep_lambda_head(const float *d_col, int ld, flo
 }
 
 // --------------------------------------------------------------------------------------------------
-// Launch 1: B', C' (bf16) and Lambda, Lambda' (fp32, log2 units).  A CTA takes one quarter of one physical chunk of one
-// (direction, batch row): 32 of its rows for B' and C', 16 of every 64 heads for the decays.  The work per CTA is a
-// chain of dependent memory round trips, so many small CTAs per SM hide it better than few large ones.
+// Launch 1: B', C' (bf16) and Lambda, Lambda' (fp32, log2 units).  CTAs of two kinds per physical chunk of one (direction, batch row): 64 of its rows
+// of B' and C' (a thread filters one channel pair over 16 rows), or the decays of 64 heads over all 128 rows (a thread takes the 16 heads
+// of one row from two 16-byte loads, a warp then scans a head at a time).  Bound by its chains of round trips, not by its 3 % of the stage's bytes:
+// each kind waits for memory twice.  With both kinds of work one after the other in CTAs of 128 threads, and 2-byte loads of the step sizes, 8 x 2048
+// tokens of 64 heads took 35 us (20 now), 1 x 1024 of 120 heads 23 us (8 now).
 // --------------------------------------------------------------------------------------------------
-constexpr int PREP_PARTS = 4, PREP_THREADS = 128, PREP_HEADS = 64 / PREP_PARTS;
-constexpr int QB = Q / PREP_PARTS;          // tokens per sub-chunk of the short-block kernel = rows of one prep CTA
-constexpr int BCT_LD = N / 2 + 4;           // row pitch (32-bit words) of the prep CTA's B' / C' tile: 16-byte rows, conflict-free ldmatrix
-static_assert(QB == 32, "one prep CTA covers exactly one sub-chunk");
+constexpr int PREP_PARTS = 4;               // sub-chunks of the short-block kernel per chunk
+constexpr int PREP_THREADS = 512, PREP_RUN = 16, PREP_ROWS = PREP_THREADS / N * PREP_RUN, PREP_BC = Q / PREP_ROWS;      // rows per thread, per B', C' unit; units per chunk
+constexpr int QB = Q / PREP_PARTS;          // tokens per sub-chunk of the short-block kernel
+constexpr int BCT_LD = N / 2 + 4;           // row pitch (32-bit words) of the B' / C' tile S is computed from: 16-byte rows, conflict-free ldmatrix
+static_assert(QB == 32 && PREP_ROWS == 2 * QB, "a B', C' unit covers two sub-chunks");
 
 __device__ __forceinline__ void ldmatrix_x4(uint32_t &r0, uint32_t &r1, uint32_t &r2, uint32_t &r3, const void *p) {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];" : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3) : "r"(smem_u32(p)));
@@ -175,82 +173,76 @@ __device__ __forceinline__ void mma_bf16_16816(float (&d)[4], uint32_t a0, uint3
                  : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
-// One unit of prep work, by a group of PREP_THREADS threads (tid = index in the group; `bar` = the group's named barrier): part
-// `part` of chunk pc of (direction, batch row): QB rows of B' and C', PREP_HEADS of every 64 heads for the decays.
-// dsm: the group's [Q][PREP_HEADS + 1] floats.  Sb != NULL (short-block mode, with bct = the group's [2][QB][BCT_LD] words): the unit
-// also writes S[i][j] = C'_i . B'_j over its rows, fp32, to Sb[seq][pc * PREP_PARTS + part][QB][QB].
-// what: PREP_BC = the B', C' (and S) half of the unit, PREP_DECAY = its decays, or both.
-constexpr int PREP_BC = 1, PREP_DECAY = 2;
-__device__ __forceinline__ void prep_unit(const SsdArgs &a, __nv_bfloat16 *__restrict__ Bp, __nv_bfloat16 *__restrict__ Cp, float *__restrict__ dA,
-                                          float *__restrict__ Sb, int dir, int b, int pc, int part, int tid, int bar, float *dsm,
-                                          uint32_t (*bct)[QB][BCT_LD], int what) {
+// Rows [row0, row0 + PREP_ROWS) of B' and C' (row0: physical).  WITH_S (short blocks): also S[i][j] = C'_i . B'_j over each sub-chunk of QB rows, fp32, to
+// Sb[seq][row0 / QB + ..][QB][QB]; bct: [2][PREP_ROWS][BCT_LD] words of shared memory.
+template <bool WITH_S>
+__device__ __forceinline__ void prep_bc(const SsdArgs &a, __nv_bfloat16 *__restrict__ Bp, __nv_bfloat16 *__restrict__ Cp, float *__restrict__ Sb, int dir, int b,
+                                        int row0, uint32_t *bct) {
     const bool rev = dir == 1;
-    const int L = a.L, k = a.k;
+    const int L = a.L, k = a.k, tid = threadIdx.x;
     const ScanDir &w = a.dir[dir];
     const int64_t seq = (int64_t)dir * a.B + b;
     const __nv_bfloat16 *zx = a.zx + ((int64_t)(a.zx_tied ? 0 : dir) * a.B + b) * L * a.d_in_proj;
-    const int r0 = pc * Q;
-    const bool has_bias = (a.flags & DM_FLAG_CONV_BIAS) && w.conv_b;
-
-    // ---- B and C channels: thread = channel pair, over this unit's block of 32 rows; the 35-row window is loaded up front
-    // (a block past the end of the sequence has nothing to write and nobody reads its S)
-    const bool bc_live = (what & PREP_BC) && r0 + part * 32 < L;
-    if (bc_live) {
-        const int cp = tid, rg = part;
-        const bool isC = cp >= N / 2;
-        const int pi = cp & (N / 2 - 1);                                 // pair index inside B or C
-        const bool valid = 2 * pi < a.Nr;                                // beyond the model's d_state: zero padding
-        const int cc = a.d_inner + (isC ? a.Nr : 0) + (valid ? 2 * pi : 0);   // conv channel of the pair's first member
-        const __nv_bfloat16 *cw = static_cast<const __nv_bfloat16 *>(w.conv_w) + (int64_t)cc * k;
-        float wl[2][4];                                                  // wl[e][m]: weight of the row m steps back in time
-#pragma unroll
-        for (int e = 0; e < 2; ++e)
-#pragma unroll
-            for (int m = 0; m < 4; ++m) wl[e][m] = (m < k && valid) ? __bfloat162float(cw[e * k + k - 1 - m]) : 0.f;
-        float bias[2] = {0.f, 0.f};
-        if (has_bias && valid) {
-            bias[0] = __bfloat162float(static_cast<const __nv_bfloat16 *>(w.conv_b)[cc]);
-            bias[1] = __bfloat162float(static_cast<const __nv_bfloat16 *>(w.conv_b)[cc + 1]);
-        }
+    if (row0 >= L) return;                                               // past the end of the sequence: nothing to write, and nobody reads its S
+    const int cp = tid & (N - 1), g = tid / N;                           // channel pair (B then C), run of rows
+    const bool isC = cp >= N / 2;
+    const int pi = cp & (N / 2 - 1);                                     // pair index inside B or C
+    const bool valid = 2 * pi < a.Nr;                                    // beyond the model's d_state: zero padding
+    const int cc = a.d_inner + (isC ? a.Nr : 0) + (valid ? 2 * pi : 0);  // conv channel of the pair's first member
+    const int lo = row0 + g * PREP_RUN;                                  // first physical row of the run
+    const int first = rev ? lo + PREP_RUN - 1 : lo, step = rev ? -1 : 1; // first-in-time row
+    uint32_t raw[PREP_RUN + 3];
+    {
         const uint32_t *col = reinterpret_cast<const uint32_t *>(zx + a.d_inner + cc);      // 4-byte aligned: all widths are even
         const int64_t ld32 = a.d_in_proj / 2;
-        const int first = rev ? r0 + rg * 32 + 31 : r0 + rg * 32, step = rev ? -1 : 1;        // first-in-time row of the block
         const uint32_t *cin = (!rev && a.conv_in) ? reinterpret_cast<const uint32_t *>(a.conv_in + (int64_t)b * (k - 1) * a.conv_ch + cc) : nullptr;
-        uint32_t raw[35];
 #pragma unroll
-        for (int i = 0; i < 35; ++i) {
+        for (int i = 0; i < PREP_RUN + 3; ++i) {
             const int t = first + (i - 3) * step;
             raw[i] = (valid && t >= 0 && t < L) ? __ldg(col + (int64_t)t * ld32) : 0u;
             if (valid && cin && t < 0 && k - 1 + t >= 0) raw[i] = __ldg(cin + (int64_t)(k - 1 + t) * (a.conv_ch / 2));    // carried rows
         }
-        __nv_bfloat16 *dst = (isC ? Cp : Bp) + 2 * pi + seq * L * N;
+    }
+    float wl[2][4], bias[2] = {0.f, 0.f};                                // wl[e][m]: weight of the row m steps back in time
+    {
+        const __nv_bfloat16 *cw = static_cast<const __nv_bfloat16 *>(w.conv_w) + (int64_t)cc * k;
 #pragma unroll
-        for (int i = 0; i < 32; ++i) {
-            const int t = first + i * step;
-            const uint32_t win[4] = {raw[i + 3], raw[i + 2], raw[i + 1], raw[i]};
-            const uint32_t pk = prep_conv_pair(wl, bias, win);
-            if (t < L) *reinterpret_cast<uint32_t *>(dst + (int64_t)t * N) = pk;
-            if (Sb) bct[isC ? 1 : 0][rev ? QB - 1 - i : i][pi] = pk;          // row of the tile = physical row inside the block
+        for (int e = 0; e < 2; ++e)
+#pragma unroll
+            for (int m = 0; m < 4; ++m) wl[e][m] = (m < k && valid) ? __bfloat162float(cw[e * k + k - 1 - m]) : 0.f;
+        if ((a.flags & DM_FLAG_CONV_BIAS) && w.conv_b && valid) {
+            bias[0] = __bfloat162float(static_cast<const __nv_bfloat16 *>(w.conv_b)[cc]);
+            bias[1] = __bfloat162float(static_cast<const __nv_bfloat16 *>(w.conv_b)[cc + 1]);
         }
     }
-    if (Sb && bc_live) {
-        // S = C' B'^T of this block's 32 rows on the legacy tensor path: warp = 16 rows i x 16 columns j, K = d_state
-        named_sync(bar, PREP_THREADS);
-        const int warp = tid >> 5, lane = tid & 31;
-        const int mt = warp & 1, nh = warp >> 1;
+    __nv_bfloat16 *dst = (isC ? Cp : Bp) + 2 * pi + seq * L * N;
+#pragma unroll
+    for (int i = 0; i < PREP_RUN; ++i) {
+        const int t = first + i * step;
+        const uint32_t win[4] = {raw[i + 3], raw[i + 2], raw[i + 1], raw[i]};
+        const uint32_t pk = prep_conv_pair(wl, bias, win);
+        if (t < L) *reinterpret_cast<uint32_t *>(dst + (int64_t)t * N) = pk;
+        if (WITH_S) bct[((isC ? 1 : 0) * PREP_ROWS + t - row0) * BCT_LD + pi] = pk;
+    }
+    if constexpr (WITH_S) {
+        // S = C' B'^T of each sub-chunk on the legacy tensor path: warp = 16 rows i x 16 columns j of one sub-chunk, K = d_state
+        __syncthreads();
+        const int warp = tid >> 5, lane = tid & 31, sub = warp >> 2, mt = warp & 1, nh = (warp >> 1) & 1;
+        if (sub >= PREP_ROWS / QB || row0 + sub * QB >= L) return;
+        const uint32_t *bt = bct + sub * QB * BCT_LD, *ct = bt + PREP_ROWS * BCT_LD;
         float acc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
 #pragma unroll
         for (int k0 = 0; k0 < N; k0 += 16) {
             uint32_t a0, a1, a2, a3;
-            ldmatrix_x4(a0, a1, a2, a3, &bct[1][16 * mt + (lane & 15)][(k0 + (lane >> 4) * 8) / 2]);
+            ldmatrix_x4(a0, a1, a2, a3, ct + (16 * mt + (lane & 15)) * BCT_LD + (k0 + (lane >> 4) * 8) / 2);
 #pragma unroll
             for (int nt = 0; nt < 2; ++nt) {
                 uint32_t b0, b1;
-                ldmatrix_x2(b0, b1, &bct[0][16 * nh + 8 * nt + (lane & 7)][(k0 + ((lane >> 3) & 1) * 8) / 2]);
+                ldmatrix_x2(b0, b1, bt + (16 * nh + 8 * nt + (lane & 7)) * BCT_LD + (k0 + ((lane >> 3) & 1) * 8) / 2);
                 mma_bf16_16816(acc[nt], a0, a1, a2, a3, b0, b1);
             }
         }
-        float *S = Sb + (seq * (a.nch * PREP_PARTS) + pc * PREP_PARTS + part) * (QB * QB);
+        float *S = Sb + (seq * (a.nch * PREP_PARTS) + row0 / QB + sub) * (QB * QB);
         const int gr = lane >> 2, qc = lane & 3;
 #pragma unroll
         for (int nt = 0; nt < 2; ++nt) {
@@ -259,36 +251,51 @@ __device__ __forceinline__ void prep_unit(const SsdArgs &a, __nv_bfloat16 *__res
             *reinterpret_cast<float2 *>(S + (row + 8) * QB + col) = make_float2(acc[nt][2], acc[nt][3]);
         }
     }
-    // ---- Delta, then the inclusive cumulative log-decay of every head in the direction's time order
-    if (!(what & PREP_DECAY)) return;
-    for (int h0 = 0; h0 < a.H; h0 += 64) {
-        named_sync(bar, PREP_THREADS);
-#pragma unroll 4
-        for (int i = 0; i < Q * PREP_HEADS / PREP_THREADS; ++i) {
-            const int idx = tid + PREP_THREADS * i, hh = idx % PREP_HEADS, r = idx / PREP_HEADS, t = r0 + r, h = h0 + part * PREP_HEADS + hh;
-            dsm[r * (PREP_HEADS + 1) + hh] = (t < L && h < a.H) ? prep_delta(zx[(int64_t)t * a.d_in_proj + a.d_inner + a.conv_ch + h], w.dt_bias[h]) : 0.f;
+}
+// Delta and the cumulative log-decays of heads [h0, h0 + 64) over the chunk that starts at row r0; dsm: [64][Q] floats
+__device__ __forceinline__ void prep_decay(const SsdArgs &a, float *__restrict__ dA, int dir, int b, int r0, int h0, float *dsm) {
+    const bool rev = dir == 1;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const ScanDir &w = a.dir[dir];
+    const int64_t seq = (int64_t)dir * a.B + b;
+    {
+        const int row = tid & (Q - 1), hg = tid / Q * 16, t = r0 + row, hb = h0 + hg;
+        // the dt columns start on a 16-byte boundary (all widths are multiples of 8), and the rows are padded to one
+        const __nv_bfloat16 *src = a.zx + (((int64_t)(a.zx_tied ? 0 : dir) * a.B + b) * a.L + t) * a.d_in_proj + a.d_inner + a.conv_ch + hb;
+        uint4 v[2] = {make_uint4(0u, 0u, 0u, 0u), make_uint4(0u, 0u, 0u, 0u)};
+#pragma unroll
+        for (int i = 0; i < 2; ++i) if (t < a.L && hb + 8 * i < a.H) v[i] = __ldg(reinterpret_cast<const uint4 *>(src) + i);
+        float bias[16];
+#pragma unroll
+        for (int j = 0; j < 16; ++j) bias[j] = hb + j < a.H ? __ldg(w.dt_bias + hb + j) : 0.f;
+#pragma unroll
+        for (int j = 0; j < 16; ++j) {
+            const uint32_t word = reinterpret_cast<const uint32_t *>(v)[j >> 1];
+            const float dt = (j & 1) ? bf16_hi(word) : bf16_lo(word);
+            dsm[(hg + j) * Q + row] = t < a.L ? prep_delta(dt, bias[j]) : 0.f;
         }
-        named_sync(bar, PREP_THREADS);
-        const int warp = tid >> 5, lane = tid & 31;
-        for (int hh = warp; hh < PREP_HEADS && h0 + part * PREP_HEADS + hh < a.H; hh += PREP_THREADS / 32) {
-            const int h = h0 + part * PREP_HEADS + hh;
-            prep_lambda_head(dsm + hh, PREP_HEADS + 1, w.A_log[h], rev, lane, dA + ((seq * a.H + h) * 2) * a.Lp + r0, a.Lp);
-        }
+    }
+    __syncthreads();
+#pragma unroll 2
+    for (int hh = warp; hh < 64; hh += PREP_THREADS / 32) {
+        const int h = h0 + hh;
+        if (h >= a.H) break;
+        const float4 q = *reinterpret_cast<const float4 *>(dsm + hh * Q + (rev ? Q - 4 - 4 * lane : 4 * lane));
+        const float d[4] = {rev ? q.w : q.x, rev ? q.z : q.y, rev ? q.y : q.z, rev ? q.x : q.w};
+        prep_lambda_head(d, __ldg(w.A_log + h), rev, lane, dA + ((seq * a.H + h) * 2) * a.Lp + r0, a.Lp);
     }
 }
 
-// grid.x covers the chunks the direction visits first: blockIdx.x / PREP_PARTS is the chunk's index in time order.  With split set (short
-// blocks, where the launch is a handful of CTAs and its latency is what counts) grid.x is twice that: the first half of the CTAs take the
-// B', C', S halves of the units, the second half their decays.
+// grid.x: for every chunk that the direction visits first (in time order), PREP_BC units of B', C' and one of decays per 64 heads
+template <bool WITH_S>
 __global__ void __launch_bounds__(PREP_THREADS)
-ssd_prep_kernel(const SsdArgs a, __nv_bfloat16 *__restrict__ Bp, __nv_bfloat16 *__restrict__ Cp, float *__restrict__ dA, float *__restrict__ Sb,
-                int dir0, int split) {
-    __shared__ float dsm[Q * (PREP_HEADS + 1)];
-    __shared__ __align__(16) uint32_t bct[2][QB][BCT_LD];     // short-block mode: this CTA's rows of B' ([0]) and C' ([1]) as bf16 pairs
-    const int units = split ? gridDim.x / 2 : gridDim.x, u = blockIdx.x % units;
-    const int what = !split ? (PREP_BC | PREP_DECAY) : blockIdx.x < units ? PREP_BC : PREP_DECAY;
-    const int dir = dir0 + blockIdx.z, c = u / PREP_PARTS;
-    prep_unit(a, Bp, Cp, dA, Sb, dir, blockIdx.y, dir == 1 ? a.nch - 1 - c : c, u % PREP_PARTS, threadIdx.x, 0, dsm, bct, what);
+ssd_prep_kernel(const __grid_constant__ SsdArgs a, __nv_bfloat16 *__restrict__ Bp, __nv_bfloat16 *__restrict__ Cp, float *__restrict__ dA, float *__restrict__ Sb, int dir0) {
+    constexpr int S_WORDS = 2 * PREP_ROWS * BCT_LD, D_WORDS = 64 * Q;
+    __shared__ __align__(16) uint32_t sm[WITH_S && S_WORDS > D_WORDS ? S_WORDS : D_WORDS];
+    const int per = PREP_BC + (a.H + 63) / 64, c = blockIdx.x / per, part = blockIdx.x - c * per;
+    const int dir = dir0 + blockIdx.z, pc = dir == 1 ? a.nch - 1 - c : c;
+    if (part < PREP_BC) prep_bc<WITH_S>(a, Bp, Cp, Sb, dir, blockIdx.y, pc * Q + part * PREP_ROWS, sm);
+    else prep_decay(a, dA, dir, blockIdx.y, pc * Q, (part - PREP_BC) * 64, reinterpret_cast<float *>(sm));
 }
 
 // --------------------------------------------------------------------------------------------------
@@ -416,13 +423,16 @@ __device__ __noinline__ void prep_role(const SsdArgs &a, const PrepJob &pj, int 
                 const int hh = idx & 63, r = idx >> 6, t = r0 + r, h = h0 + hh;
                 float d = 0.f;
                 if (t < L && h < a.H)
-                    d = prep_delta((h0 == 0 && dt_vec) ? dtt[idx] : zx[(int64_t)t * a.d_in_proj + a.d_inner + a.conv_ch + h], w.dt_bias[h]);
+                    d = prep_delta(__bfloat162float((h0 == 0 && dt_vec) ? dtt[idx] : zx[(int64_t)t * a.d_in_proj + a.d_inner + a.conv_ch + h]), w.dt_bias[h]);
                 dsm[r * 65 + hh] = d;
             }
             __syncthreads();
             for (int hh = warp; hh < 64 && h0 + hh < a.H; hh += NTHREADS / 32) {
                 const int h = h0 + hh;
-                prep_lambda_head(dsm + hh, 65, w.A_log[h], rev, lane, pj.dA + ((seq * a.H + h) * 2) * a.Lp + r0, a.Lp);
+                float d[4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) d[e] = dsm[(rev ? Q - 1 - 4 * lane - e : 4 * lane + e) * 65 + hh];
+                prep_lambda_head(d, w.A_log[h], rev, lane, pj.dA + ((seq * a.H + h) * 2) * a.Lp + r0, a.Lp);
             }
         }
         // ---- publish the item
@@ -1373,7 +1383,9 @@ cudaError_t scan_ssd(const ScanArgs &a, void *ws, cudaStream_t s) {
     if (pj.sync && g_withhold_prep) pj.nprep = 0;
     cudaError_t e;
     if (pj.sync && (e = cudaMemsetAsync(pj.sync, 0, ((size_t)2 * a.B * l.nch + 1) * sizeof(int), s)) != cudaSuccess) return e;
-    ssd_prep_kernel<<<dim3(n_pre * PREP_PARTS * (blk ? 2 : 1), a.B, ndir), PREP_THREADS, 0, s>>>(k, Bp, Cp, dA, Sb, dir0, blk ? 1 : 0);
+    const dim3 pgrid(n_pre * (PREP_BC + (a.H + 63) / 64), a.B, ndir);
+    if (blk) ssd_prep_kernel<true><<<pgrid, PREP_THREADS, 0, s>>>(k, Bp, Cp, dA, Sb, dir0);
+    else ssd_prep_kernel<false><<<pgrid, PREP_THREADS, 0, s>>>(k, Bp, Cp, dA, Sb, dir0);
     count_launch();
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (blk) {
