@@ -82,6 +82,8 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     fence_before();
     __syncthreads();
     fence_after();
+    pdl_wait();
+    pdl_trigger();
     const uint32_t tmem = bars->tmem_base;
     auto WAIT = [&](uint64_t *bar, uint32_t parity) { return mbar_wait(bar, parity, abort_flag, status); };
 
@@ -314,16 +316,11 @@ cudaError_t attention_forward(const void *qkv, void *out, int B, int Lq, int d, 
     if (!status) return cudaErrorUnknown;
     AttnArgs a{B, Lq, Lk, d, n_heads, cached ? 0 : d, cached ? 0 : 2 * d, static_cast<__nv_bfloat16 *>(out), 1.4426950408889634f / sqrtf((float)dh)};
     const dim3 grid((Lq + 2 * BQ - 1) / (2 * BQ), n_heads, B);
-    cudaError_t e;
-    if (dh == 64) {
-        if ((e = cudaFuncSetAttribute(attention_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg<1>::SMEM)) != cudaSuccess) return e;
-        attention_kernel<1><<<grid, NTHREADS, Cfg<1>::SMEM, s>>>(mq, mk, mv, a, status);
-    } else {
-        if ((e = cudaFuncSetAttribute(attention_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg<2>::SMEM)) != cudaSuccess) return e;
-        attention_kernel<2><<<grid, NTHREADS, Cfg<2>::SMEM, s>>>(mq, mk, mv, a, status);
-    }
-    count_launch();
-    return cudaGetLastError();
+    const uint32_t smem = dh == 64 ? Cfg<1>::SMEM : Cfg<2>::SMEM;
+    auto kern = dh == 64 ? attention_kernel<1> : attention_kernel<2>;
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    return launch_chain(kern, grid, NTHREADS, smem, s, 0, mq, mk, mv, a, status);
 }
 
 }  // namespace dm

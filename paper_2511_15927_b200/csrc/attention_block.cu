@@ -67,6 +67,8 @@ attention_block_kernel(const BlockAttnArgs a, int H, int split) {
     using S = Smem<DH>;
     constexpr int LD = S::LD, U = DH / 8, KS = DH / 16, NO = DH / 8;       // 16-byte pieces per row, K steps of Q K^T, 8-column tiles of O
     extern __shared__ __align__(16) uint8_t sm[];
+    pdl_wait();
+    pdl_trigger();
     const uint32_t base = smem_u32(sm);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, gr = lane >> 2, qc = lane & 3;
     const int rank = blockIdx.x, h = blockIdx.y % H, q0 = blockIdx.y / H * BQ, b = blockIdx.z;
@@ -275,15 +277,7 @@ cudaError_t launch(const BlockAttnArgs &a, int B, int H, cudaStream_t s) {
     while (split < MAX_SPLIT && ctas * split < sm_count() && Lk >= 2 * KT * 2 * split) split *= 2;
     cudaError_t e = cudaFuncSetAttribute(attention_block_kernel<DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Smem<DH>::total);
     if (e != cudaSuccess) return e;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(split, H * qb, B); cfg.blockDim = dim3(NT); cfg.dynamicSmemBytes = Smem<DH>::total; cfg.stream = s;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = split; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-    cfg.attrs = at; cfg.numAttrs = 1;
-    e = cudaLaunchKernelEx(&cfg, attention_block_kernel<DH>, a, H, split);
-    count_launch();
-    return e;
+    return launch_chain(attention_block_kernel<DH>, dim3(split, H * qb, B), NT, Smem<DH>::total, s, split, a, H, split);
 }
 
 }  // namespace

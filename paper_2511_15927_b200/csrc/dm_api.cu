@@ -497,6 +497,7 @@ int dm_check(void *cuda_stream) {
 
 int dm_bimamba_forward(const dm_mixer_cfg *cfg, const dm_dir_weights w[2], const void *x, void *y,
                        void *workspace, size_t workspace_bytes, void *cuda_stream) {
+    chain_begin();
     Dims m;
     int st = check_cfg(cfg, &m);
     if (st != DM_OK) return st;
@@ -511,6 +512,7 @@ int dm_bimamba_forward(const dm_mixer_cfg *cfg, const dm_dir_weights w[2], const
 }
 
 int dm_bimamba_forward_static(const dm_mixer_cfg *cfg, const dm_dir_weights w[2], const void *x, void *y, void *cuda_stream) {
+    chain_begin();
     Dims m;
     int st = check_cfg(cfg, &m);
     if (st != DM_OK) return st;
@@ -532,6 +534,7 @@ int dm_bimamba_block_step(const dm_mixer_cfg *cfg, const dm_dir_weights w[2], co
                           const float *ssm_state_in, const void *conv_state_in,
                           float *ssm_state_out, void *conv_state_out, void *y_blk,
                           void *workspace, size_t workspace_bytes, void *cuda_stream) {
+    chain_begin();
     Dims m;
     int st = check_cfg(cfg, &m);
     if (st != DM_OK) return st;
@@ -567,6 +570,7 @@ static int denoise_impl(const dm_stack_cfg *cfg, const dm_block_cfg *blk, const 
                         const int32_t *tokens, const float *tau, void *logits,
                         int32_t *argmax_out, const dm_layer_state *states, void *workspace, size_t workspace_bytes,
                         void *cuda_stream, const SampleArgs *smp = nullptr, const HybridArgs *hyb = nullptr) {
+    chain_begin();
     Dims m;
     if (!cfg || !weights) return fail(DM_ERR_INVALID_ARG, "cfg or weights is NULL");
     int st = check_cfg(&cfg->mixer, &m);
@@ -868,6 +872,7 @@ int dm_denoise_step_hybrid_block(const dm_stack_cfg *cfg, const dm_block_cfg *bl
 int dm_attention_block_step(int32_t batch, int32_t block_len, int32_t d_model, int32_t n_heads, int32_t dtype, const void *w_qkv,
                             const void *w_o, const void *x_blk, void *k_cache, void *v_cache, int32_t cache_len, int32_t cache_cap,
                             void *y_blk, void *workspace, size_t workspace_bytes, void *cuda_stream) {
+    chain_begin();
     size_t need = 0;
     int st = dm_attention_workspace_bytes(batch, block_len, d_model, dtype, &need);
     if (st != DM_OK) return st;
@@ -908,6 +913,7 @@ int dm_attention_workspace_bytes(int32_t batch, int32_t seqlen, int32_t d_model,
 
 int dm_attention_forward(int32_t batch, int32_t seqlen, int32_t d_model, int32_t n_heads, int32_t dtype, const void *w_qkv,
                          const void *w_o, const void *x, void *y, void *workspace, size_t workspace_bytes, void *cuda_stream) {
+    chain_begin();
     size_t need = 0;
     int st = dm_attention_workspace_bytes(batch, seqlen, d_model, dtype, &need);
     if (st != DM_OK) return st;
@@ -953,6 +959,7 @@ int dm_selftest_wait_timeout(uint32_t limit_us, uint64_t *out, void *cuda_stream
 
 int dm_linear(int dtype, const void *x, const void *w, void *y, int y_dtype, int64_t rows, int32_t in_features,
               int32_t out_features, const float *row_scale, const float *addend, void *cuda_stream) {
+    chain_begin();
     if ((dtype != DM_F32 && dtype != DM_BF16) || (y_dtype != DM_F32 && y_dtype != DM_BF16)) return fail(DM_ERR_INVALID_ARG, "bad dtype");
     if (!x || !w || !y) return fail(DM_ERR_INVALID_ARG, "x, w or y is NULL");
     if (rows <= 0 || rows > (int64_t)1 << 30 || in_features <= 0 || out_features <= 0) return fail(DM_ERR_INVALID_ARG, "sizes must be positive");

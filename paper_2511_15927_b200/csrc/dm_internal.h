@@ -16,6 +16,41 @@ void count_launch(int n = 1);
 // Device status word written by kernels whose bounded waits expire; read and cleared by dm_check().
 int *device_status_ptr();
 
+// Programmatic dependent launch along the chain of kernels that one call of the library enqueues: a kernel starts its set-up (and, in the GEMMs, the loads of its
+// weights) while the one before it is finishing, and waits for that one's completion before it touches anything a kernel of the chain reads or writes.
+//   - Every kernel launched through launch_chain calls pdl_wait() in each thread that accesses such memory, and pdl_trigger() only after it: the next kernel can
+//     then rely on everything before this one being complete, and the weights it reads early were not written by this kernel.
+//   - The first kernel of a call is launched without the attribute (chain_begin): it follows the caller's work in stream order, completely.
+// A decoding pass of 24 layers is 75 to 120 kernels of 4 to 35 us: 1236 -> 974 us for one sequence (hybrid, 2.4 GB of weights), 2449 -> 2302 us for 16; a single
+// layer of 1024 tokens 140 -> 136 us.
+inline thread_local bool g_chain = false;
+inline void chain_begin() { g_chain = false; }
+#ifdef __CUDACC__
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+template <typename... P, typename... A>
+inline cudaError_t launch_chain(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, int cluster, A &&...args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = s;
+    cudaLaunchAttribute at[2];
+    int n = 0;
+    if (cluster > 0) {                       // (0: the kernel's own cluster size)
+        at[n].id = cudaLaunchAttributeClusterDimension;
+        at[n].val.clusterDim.x = cluster; at[n].val.clusterDim.y = 1; at[n].val.clusterDim.z = 1;
+        ++n;
+    }
+    if (g_chain) {
+        at[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[n].val.programmaticStreamSerializationAllowed = 1;
+        ++n;
+    }
+    cfg.attrs = at; cfg.numAttrs = n;
+    g_chain = true;
+    count_launch();
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
+#endif
+
 inline size_t dtype_size(int dtype) { return dtype == DM_BF16 ? 2 : 4; }
 inline size_t align_up(size_t v, size_t a = 256) { return (v + a - 1) / a * a; }
 

@@ -65,6 +65,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_consta
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank();
     const int pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
+    if (ep.m_dev) pdl_wait();                  // (the row count comes from a kernel before this one)
     const int M_eff = ep.m_dev ? min(ep.M, max(0, *ep.m_dev - ep.m_off)) : ep.M;
     const int tiles_m = (M_eff + 2 * BM - 1) / (2 * BM), tiles_n = (ep.N + BN - 1) / BN;
     const int tiles_np = tiles_n * (MODE == SUM ? 1 : epp.nprob);      // separate problems sit side by side along N
@@ -99,6 +100,20 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_consta
             const bool leader = elect_one();
             uint32_t it = 0;
             bool ok = true;
+            // the first stages' share of B (weights) is on its way before the kernel before this one has finished
+            const uint32_t ahead = pair < num_tiles ? min(STAGES, kblocks) : 0;
+            if (leader && ahead > 0) {
+                int tm, cb;
+                tile_at(pair, tm, cb);
+                const int prob = cb / tiles_n, prod = epp.ksplit ? prob >> 1 : prob, n0 = (cb - prob * tiles_n) * BN + (int)rank * (BN / 2);
+                for (uint32_t s = 0; s < ahead; ++s) {
+                    if (rank == 0) mbar_expect_tx(&bars->full[s], 2 * T::STAGE);
+                    tma_load_2d_pair(smem + s * T::STAGE + T::A_BYTES, prod ? &map_b1 : &map_b0, epp.p[prob].k_off + (int)s * BK, n0, cluster_addr(&bars->full[s], 0));
+                }
+            }
+            __syncwarp();
+            pdl_wait();
+            pdl_trigger();
             for (int tile = pair; tile < num_tiles && ok; tile += npairs) {
                 int tm, cb;
                 tile_at(tile, tm, cb);
@@ -112,9 +127,9 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_consta
                         uint8_t *sa = smem + s * T::STAGE, *sb = sa + T::A_BYTES;
                         const uint32_t full = cluster_addr(&bars->full[s], 0);
                         if (leader) {
-                            if (rank == 0) mbar_expect_tx(&bars->full[s], 2 * T::STAGE);        // both CTAs' loads
+                            if (rank == 0 && it >= ahead) mbar_expect_tx(&bars->full[s], 2 * T::STAGE);        // both CTAs' loads
                             tma_load_2d_pair(sa, ma, k_off + kb * BK, m0, full);
-                            tma_load_2d_pair(sb, mb, k_off + kb * BK, n0, full);
+                            if (it >= ahead) tma_load_2d_pair(sb, mb, k_off + kb * BK, n0, full);
                         }
                         __syncwarp();
                     }
@@ -132,6 +147,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_consta
             const uint32_t desc_a0 = desc_lo_k(smem_u32(smem));
             uint32_t it = 0, tcount = 0;
             bool ok = true;
+            pdl_wait();                                        // (the limit of the waits below counts from here)
             const uint32_t products = (uint32_t)(pair < num_tiles ? (num_tiles - 1 - pair) / npairs + 1 : 0) * NSUB;
             for (; tcount < products && ok; ++tcount) {
                 const uint32_t buf = tcount & 1u, bph = (tcount >> 1) & 1u;
@@ -159,6 +175,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_consta
         // ------------------------------------------------------------ epilogue: 8 warps over this CTA's 128 rows
         constexpr int COLS = BN / 2;                           // columns per warp
         const int q = warp & 3, cfirst = ((warp - 2) >> 2) * COLS;       // TMEM lane quarter, first column
+        pdl_wait();
         const uint32_t tlane = tmem_base + ((uint32_t)(q * 32) << 16) + cfirst;
         uint32_t tcount = 0;
         bool ok = true;
@@ -366,9 +383,7 @@ cudaError_t launch(const GemmArgs &a, const GemmArgs *b, float *const *hi, cudaS
     }
     const int64_t tiles = (int64_t)((a.M + 2 * BM - 1) / (2 * BM)) * ((a.N + BN - 1) / BN) * (MODE == SUM ? 1 : epp.nprob);
     const int pairs = sm_count() / 2, grid = 2 * (int)(tiles < pairs ? tiles : pairs);
-    gemm_pair_kernel<BN, MODE><<<grid, NTHREADS, smem, s>>>(ma[0], mb[0], ma[1], mb[1], io, epp, status);
-    count_launch();
-    return cudaGetLastError();
+    return launch_chain(gemm_pair_kernel<BN, MODE>, grid, NTHREADS, smem, s, 0, ma[0], mb[0], ma[1], mb[1], io, epp, status);
 }
 
 bool tma_io(const GemmArgs &a, const GemmArgs *b) { return gemm_pair_tma_io(a) && (!b || (gemm_pair_tma_io(*b) && !a.addend && !b->addend && !a.u && !b->u)); }

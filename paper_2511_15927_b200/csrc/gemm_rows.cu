@@ -107,6 +107,7 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap map_x0, const __grid_consta
     const int rank = cs > 1 ? (int)cluster_ctarank() : 0, cid = blockIdx.x / cs, tile = cid % ra.tiles_n;
     const int prod = ra.sum ? rank / ra.ks : cid / ra.tiles_n, kr = rank % ra.ks;
     const EpiArgs &ep = ra.p[ra.sum ? 1 : prod];                             // output, addend, ...
+    if (ep.m_dev) pdl_wait();                                                // (the row count comes from a kernel before this one)
     const int M = ep.m_dev ? min(ep.M, max(0, *ep.m_dev - ep.m_off)) : ep.M;
     const int kblocks = (ep.K + BK - 1) / BK, kb0 = kr * kblocks / ra.ks, nk = (kr + 1) * kblocks / ra.ks - kb0;
     const int n0 = tile * BF;
@@ -131,12 +132,24 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap map_x0, const __grid_consta
         const CUtensorMap *mx = prod ? &map_x1 : &map_x0, *mw = prod ? &map_w1 : &map_w0;
         int s = 0;
         uint32_t ph = 1;
+        // the weights of the first stages are on their way before the kernel before this one has finished
+        const int ahead = min(S, nk);
+        if (leader)
+            for (int i = 0; i < ahead; ++i) {
+                mbar_expect_tx(&bars->full[i], stage);
+                tma_load_2d(smem + i * stage, mw, (kb0 + i) * BK, n0, &bars->full[i]);
+            }
+        __syncwarp();
+        pdl_wait();
+        pdl_trigger();
         for (int i = 0; i < nk; ++i) {
             if (!(ok = mbar_wait(&bars->empty[s], ph, abort_flag, status))) break;
             if (leader) {
                 uint8_t *sw = smem + s * stage;
-                mbar_expect_tx(&bars->full[s], stage);
-                tma_load_2d(sw, mw, (kb0 + i) * BK, n0, &bars->full[s]);
+                if (i >= ahead) {
+                    mbar_expect_tx(&bars->full[s], stage);
+                    tma_load_2d(sw, mw, (kb0 + i) * BK, n0, &bars->full[s]);
+                }
                 tma_load_2d(sw + W_BYTES, mx, (kb0 + i) * BK, 0, &bars->full[s]);
             }
             __syncwarp();
@@ -145,6 +158,7 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap map_x0, const __grid_consta
         if (!ok) sleep_ns(100000000ull);                                     // aborting: the loads already issued get time to land
     } else if (warp == 1) {
         const bool leader = elect_one();
+        pdl_wait();                                                          // (the limit of the waits below counts from here)
         const uint32_t idesc = idesc_bf16(BF, nt, 0, 0), d0 = desc_lo_k(smem_u32(smem));
         int s = 0;
         uint32_t ph = 0;
@@ -165,6 +179,7 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap map_x0, const __grid_consta
         }
     } else {
         const int ew = warp - 2, q = warp & 3, f = q * 32 + lane;            // this thread's output column of the tile
+        pdl_wait();
         // row scales of this CTA's tokens, while the products run
         for (int pi = ra.sum ? 0 : prod; pi <= (ra.sum ? 1 : prod); ++pi) {
             const EpiArgs &e = ra.p[pi];
@@ -302,15 +317,7 @@ cudaError_t gemm_rows_launch(const GemmArgs &a, const GemmArgs *b, bool sum, cud
     if (e != cudaSuccess) return e;
     int *status = device_status_ptr();
     if (!status) return cudaErrorUnknown;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(ctas); cfg.blockDim = dim3(two ? 192 : 320); cfg.dynamicSmemBytes = smem; cfg.stream = s;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = ra.cs; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-    cfg.attrs = at; cfg.numAttrs = 1;
-    e = cudaLaunchKernelEx(&cfg, kern, mx[0], mw[0], mx[1], mw[1], ra, status);
-    count_launch();
-    return e;
+    return launch_chain(kern, dim3(ctas), dim3(two ? 192 : 320), smem, s, ra.cs, mx[0], mw[0], mx[1], mw[1], ra, status);
 }
 
 }  // namespace dm

@@ -103,6 +103,8 @@ struct F32Problems { GemmArgs p[2]; };
 __global__ void __launch_bounds__(256)
 gemm_f32_kernel(const __grid_constant__ F32Problems pr, const int sum) {
     extern __shared__ __align__(16) float fsm[];
+    pdl_wait();
+    pdl_trigger();
     const int tid = threadIdx.x, g = tid >> 6, t = tid & 63, tx = t & 7, ty = t >> 3;
     const int per = sum ? FG / 2 : FG, prob = sum ? g / per : (int)blockIdx.z, gi = sum ? g % per : g;      // K groups per product
     const GemmArgs &a = pr.p[prob], &o = pr.p[sum ? 1 : prob];
@@ -205,9 +207,7 @@ cudaError_t gemm_f32(const GemmArgs &a, const GemmArgs *b, bool sum, cudaStream_
     }
     cudaError_t e = cudaFuncSetAttribute(gemm_f32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)F32_SMEM);
     if (e != cudaSuccess) return e;
-    gemm_f32_kernel<<<dim3((a.N + FT - 1) / FT, (a.M + FT - 1) / FT, b && !sum ? 2 : 1), 256, F32_SMEM, s>>>(pr, sum ? 1 : 0);
-    count_launch();
-    return cudaGetLastError();
+    return launch_chain(gemm_f32_kernel, dim3((a.N + FT - 1) / FT, (a.M + FT - 1) / FT, b && !sum ? 2 : 1), 256, F32_SMEM, s, 0, pr, sum ? 1 : 0);
 }
 
 cudaError_t gemm_simple(const GemmArgs &a, cudaStream_t s) {

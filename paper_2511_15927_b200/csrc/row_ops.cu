@@ -25,6 +25,8 @@ __device__ __forceinline__ float block_sum(float v, float *red) {
 
 // One warp per row: the lanes read the row's per-head sums side by side, then reduce in a fixed order.
 __global__ void rstd_kernel(const float *__restrict__ ssq, float *__restrict__ rstd, int rows, int H, float inv_n, float eps) {
+    pdl_wait();
+    pdl_trigger();
     const int r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (r >= rows) return;
     float s = 0.f;
@@ -35,6 +37,8 @@ __global__ void rstd_kernel(const float *__restrict__ ssq, float *__restrict__ r
 
 template <typename T>
 __global__ void embed_kernel(const T *__restrict__ embed, const int32_t *__restrict__ tokens, float *__restrict__ r, int d, int vocab) {
+    pdl_wait();
+    pdl_trigger();
     const int64_t t = blockIdx.x;
     int id = tokens[t];
     id = id < 0 ? 0 : (id >= vocab ? vocab - 1 : id);      // ids are validated on the host side of the tests; clamp keeps reads in bounds
@@ -55,6 +59,8 @@ template <> __device__ __forceinline__ void st4<__nv_bfloat16>(__nv_bfloat16 *p,
 template <typename T>
 __global__ void __launch_bounds__(ROW_THREADS)
 rmsnorm_kernel(const float *__restrict__ r, const T *__restrict__ w, T *__restrict__ u, int d, float eps) {
+    pdl_wait();
+    pdl_trigger();
     __shared__ float red[32];
     const int64_t t = blockIdx.x;
     const float *row = r + t * d;
@@ -90,6 +96,8 @@ template <typename T>
 __global__ void __launch_bounds__(ROW_THREADS)
 adaln_kernel(const float *__restrict__ r, const float *__restrict__ gamma, const float *__restrict__ beta, int64_t ld_mod,
              T *__restrict__ u, int L, int d, float eps) {
+    pdl_wait();
+    pdl_trigger();
     __shared__ float red[32];
     const int64_t t = blockIdx.x, b = t / L;
     const float *row = r + t * d, *g = gamma + b * ld_mod, *be = beta + b * ld_mod;
@@ -139,6 +147,8 @@ adaln_kernel(const float *__restrict__ r, const float *__restrict__ gamma, const
 template <typename T>
 __global__ void modulation_kernel(const float *__restrict__ tau, const T *__restrict__ w, const float *__restrict__ bias,
                                   float *__restrict__ mod, int n_out, int d_c) {
+    pdl_wait();
+    pdl_trigger();
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31, b = blockIdx.y;
     if (warp >= n_out) return;
     float s = 0.f;
@@ -196,6 +206,8 @@ __global__ void argmax_kernel(const T *__restrict__ logits, int32_t *__restrict_
 template <typename T>
 __global__ void conv_state_kernel(const T *__restrict__ zx, const T *__restrict__ conv_in, T *__restrict__ conv_out,
                                   int L, int k, int d_inner, int conv_ch, int d_in_proj) {
+    pdl_wait();
+    pdl_trigger();
     const int b = blockIdx.y, r = blockIdx.z;
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= conv_ch) return;
@@ -218,6 +230,8 @@ sum_partials_norm_kernel(const float *__restrict__ p0, const float *__restrict__
                          const float *__restrict__ ssq0, const float *__restrict__ ssq1,
                          int H, float inv_n, float eps_g, const float *addend, int64_t ld_add, TY *y, const TU *__restrict__ w, TU *__restrict__ u,
                          int d, float eps) {
+    pdl_wait();
+    pdl_trigger();
     __shared__ float red[32];
     __shared__ float sc[2];
     const int64_t t = blockIdx.x;
@@ -299,40 +313,30 @@ __global__ void __launch_bounds__(256) combine_kernel(T *__restrict__ g0, const 
 }  // namespace
 
 cudaError_t rstd_from_ssq(const float *ssq, float *rstd, int rows, int H, int d_inner, float eps, cudaStream_t s) {
-    rstd_kernel<<<(rows + 7) / 8, 256, 0, s>>>(ssq, rstd, rows, H, 1.f / (float)d_inner, eps);
-    count_launch();
-    return cudaGetLastError();
+    return launch_chain(rstd_kernel, (rows + 7) / 8, 256, 0, s, 0, ssq, rstd, rows, H, 1.f / (float)d_inner, eps);
 }
 
 cudaError_t embed_gather(const void *embed, int dtype, const int32_t *tokens, float *r, int T, int d, int vocab, cudaStream_t s) {
-    if (dtype == DM_BF16) embed_kernel<<<T, 256, 0, s>>>(static_cast<const __nv_bfloat16 *>(embed), tokens, r, d, vocab);
-    else embed_kernel<<<T, 256, 0, s>>>(static_cast<const float *>(embed), tokens, r, d, vocab);
-    count_launch();
-    return cudaGetLastError();
+    if (dtype == DM_BF16) return launch_chain(embed_kernel<__nv_bfloat16>, T, 256, 0, s, 0, static_cast<const __nv_bfloat16 *>(embed), tokens, r, d, vocab);
+    return launch_chain(embed_kernel<float>, T, 256, 0, s, 0, static_cast<const float *>(embed), tokens, r, d, vocab);
 }
 
 cudaError_t rmsnorm_rows(const float *r, const void *w, void *u, int dtype, int T, int d, float eps, cudaStream_t s) {
-    if (dtype == DM_BF16) rmsnorm_kernel<<<T, 256, 0, s>>>(r, static_cast<const __nv_bfloat16 *>(w), static_cast<__nv_bfloat16 *>(u), d, eps);
-    else rmsnorm_kernel<<<T, 256, 0, s>>>(r, static_cast<const float *>(w), static_cast<float *>(u), d, eps);
-    count_launch();
-    return cudaGetLastError();
+    if (dtype == DM_BF16) return launch_chain(rmsnorm_kernel<__nv_bfloat16>, T, 256, 0, s, 0, r, static_cast<const __nv_bfloat16 *>(w), static_cast<__nv_bfloat16 *>(u), d, eps);
+    return launch_chain(rmsnorm_kernel<float>, T, 256, 0, s, 0, r, static_cast<const float *>(w), static_cast<float *>(u), d, eps);
 }
 
 cudaError_t adaln_rows(const float *r, const float *gamma, const float *beta, int64_t ld_mod, void *u, int dtype, int T, int L, int d,
                        float eps, cudaStream_t s) {
-    if (dtype == DM_BF16) adaln_kernel<<<T, 256, 0, s>>>(r, gamma, beta, ld_mod, static_cast<__nv_bfloat16 *>(u), L, d, eps);
-    else adaln_kernel<<<T, 256, 0, s>>>(r, gamma, beta, ld_mod, static_cast<float *>(u), L, d, eps);
-    count_launch();
-    return cudaGetLastError();
+    if (dtype == DM_BF16) return launch_chain(adaln_kernel<__nv_bfloat16>, T, 256, 0, s, 0, r, gamma, beta, ld_mod, static_cast<__nv_bfloat16 *>(u), L, d, eps);
+    return launch_chain(adaln_kernel<float>, T, 256, 0, s, 0, r, gamma, beta, ld_mod, static_cast<float *>(u), L, d, eps);
 }
 
 cudaError_t modulation_rows(const float *tau, const void *w_cond, const float *b_cond, float *mod, int dtype, int B, int n_out, int d_c,
                             cudaStream_t s) {
     dim3 grid((n_out * 32 + 255) / 256, B);
-    if (dtype == DM_BF16) modulation_kernel<<<grid, 256, 0, s>>>(tau, static_cast<const __nv_bfloat16 *>(w_cond), b_cond, mod, n_out, d_c);
-    else modulation_kernel<<<grid, 256, 0, s>>>(tau, static_cast<const float *>(w_cond), b_cond, mod, n_out, d_c);
-    count_launch();
-    return cudaGetLastError();
+    if (dtype == DM_BF16) return launch_chain(modulation_kernel<__nv_bfloat16>, grid, 256, 0, s, 0, tau, static_cast<const __nv_bfloat16 *>(w_cond), b_cond, mod, n_out, d_c);
+    return launch_chain(modulation_kernel<float>, grid, 256, 0, s, 0, tau, static_cast<const float *>(w_cond), b_cond, mod, n_out, d_c);
 }
 
 cudaError_t argmax_rows(const void *logits, int dtype, int32_t *out, int T, int V, cudaStream_t s) {
@@ -346,13 +350,10 @@ cudaError_t conv_state_update(const void *zx_fwd, const void *conv_in, void *con
                               int k, int d_inner, int conv_ch, int d_in_proj, cudaStream_t s) {
     dim3 grid((conv_ch + 255) / 256, B, k - 1);
     if (dtype == DM_BF16)
-        conv_state_kernel<<<grid, 256, 0, s>>>(static_cast<const __nv_bfloat16 *>(zx_fwd), static_cast<const __nv_bfloat16 *>(conv_in),
+        return launch_chain(conv_state_kernel<__nv_bfloat16>, grid, 256, 0, s, 0, static_cast<const __nv_bfloat16 *>(zx_fwd), static_cast<const __nv_bfloat16 *>(conv_in),
                                                static_cast<__nv_bfloat16 *>(conv_out), L, k, d_inner, conv_ch, d_in_proj);
-    else
-        conv_state_kernel<<<grid, 256, 0, s>>>(static_cast<const float *>(zx_fwd), static_cast<const float *>(conv_in),
+    return launch_chain(conv_state_kernel<float>, grid, 256, 0, s, 0, static_cast<const float *>(zx_fwd), static_cast<const float *>(conv_in),
                                                static_cast<float *>(conv_out), L, k, d_inner, conv_ch, d_in_proj);
-    count_launch();
-    return cudaGetLastError();
 }
 
 bool sum_partials_norm_supports(int d) { return d % 4 == 0 && d <= 4 * ROW_THREADS * ROW_K; }
@@ -363,13 +364,11 @@ cudaError_t sum_partials_norm(const float *p0, const float *p1, const float *q0,
     if (!sum_partials_norm_supports(d) || (q0 == nullptr) != (q1 == nullptr)) return cudaErrorInvalidValue;
     const float inv_n = 1.f / (float)d_inner;
     const int grid = (int)T;
-#define DM_SPN(TY, TU) sum_partials_norm_kernel<TY, TU><<<grid, ROW_THREADS, 0, s>>>(p0, p1, q0, q1, ssq0, ssq1, H, inv_n, eps_g, addend, ld_add, \
+#define DM_SPN(TY, TU) return launch_chain(sum_partials_norm_kernel<TY, TU>, grid, ROW_THREADS, 0, s, 0, p0, p1, q0, q1, ssq0, ssq1, H, inv_n, eps_g, addend, ld_add, \
         static_cast<TY *>(y), static_cast<const TU *>(w), static_cast<TU *>(u), d, eps)
     if (y_dtype == DM_F32) { if (u_dtype == DM_BF16) DM_SPN(float, __nv_bfloat16); else DM_SPN(float, float); }
     else { if (u_dtype == DM_BF16) DM_SPN(__nv_bfloat16, __nv_bfloat16); else DM_SPN(__nv_bfloat16, float); }
 #undef DM_SPN
-    count_launch();
-    return cudaGetLastError();
 }
 
 cudaError_t combine_directions(void *g0, const void *g1, const float *rstd0, const float *rstd1, int dtype, int64_t T, int d_inner, cudaStream_t s) {

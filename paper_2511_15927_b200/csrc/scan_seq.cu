@@ -49,6 +49,8 @@ constexpr int BC_ROWS = 8;
 template <typename T>
 __global__ void __launch_bounds__(256)
 bc_prep_kernel(const ScanArgs a, const int dir0, float *__restrict__ bc) {
+    pdl_wait();
+    pdl_trigger();
     const int N2 = 2 * a.N, L = a.L, k = a.k;
     const int dir = dir0 + blockIdx.z, b = blockIdx.y;
     const bool rev = dir == 1;
@@ -106,6 +108,8 @@ scan_seq_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
     __shared__ uint64_t bars[RAW];                     // raw stage has landed
     __shared__ int abort_word;
     volatile int *abort_flag = &abort_word;
+    pdl_wait();
+    pdl_trigger();
     constexpr int LPC = lanes_per_channel(N), NQ = N / (4 * LPC), NS = P * LPC, NL = loaders(P, N), NP = NL / 2;       // NS: scan threads, NL: loader threads, NP of them preparing
     const int L = a.L, k = a.k;
     const int h = blockIdx.x, b = blockIdx.z;
@@ -400,14 +404,10 @@ cudaError_t scan_sequential(const ScanArgs &a, void *ws, cudaStream_t s) {
     float *bc = static_cast<float *>(ws);
     const int tasks = (a.L + BC_ROWS - 1) / BC_ROWS * 2 * a.N, bt = tasks >= 256 * 148 ? 256 : 64;        // small CTAs while they do not fill the GPU
     dim3 pgrid((tasks + bt - 1) / bt, a.B, ndir);
-    if (a.dtype == DM_BF16) bc_prep_kernel<__nv_bfloat16><<<pgrid, bt, 0, s>>>(a, dir0, bc);
-    else bc_prep_kernel<float><<<pgrid, bt, 0, s>>>(a, dir0, bc);
-    count_launch();
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    e = a.dtype == DM_BF16 ? launch_chain(bc_prep_kernel<__nv_bfloat16>, pgrid, bt, 0, s, 0, a, dir0, bc) : launch_chain(bc_prep_kernel<float>, pgrid, bt, 0, s, 0, a, dir0, bc);
+    if (e != cudaSuccess) return e;
     dim3 grid(a.H, ndir, a.B);
-    kern<<<grid, a.P * lanes_per_channel(a.N) + loaders(a.P, a.N), smem, s>>>(mx, mz, a, dir0, TC, bc, status);
-    count_launch();
-    return cudaGetLastError();
+    return launch_chain(kern, grid, a.P * lanes_per_channel(a.N) + loaders(a.P, a.N), smem, s, 0, mx, mz, a, dir0, TC, bc, status);
 }
 
 }  // namespace dm

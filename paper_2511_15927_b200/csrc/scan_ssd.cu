@@ -290,6 +290,8 @@ __device__ __forceinline__ void prep_decay(const SsdArgs &a, float *__restrict__
 template <bool WITH_S>
 __global__ void __launch_bounds__(PREP_THREADS)
 ssd_prep_kernel(const __grid_constant__ SsdArgs a, __nv_bfloat16 *__restrict__ Bp, __nv_bfloat16 *__restrict__ Cp, float *__restrict__ dA, float *__restrict__ Sb, int dir0) {
+    pdl_wait();
+    pdl_trigger();
     constexpr int S_WORDS = 2 * PREP_ROWS * BCT_LD, D_WORDS = 64 * Q;
     __shared__ __align__(16) uint32_t sm[WITH_S && S_WORDS > D_WORDS ? S_WORDS : D_WORDS];
     const int per = PREP_BC + (a.H + 63) / 64, c = blockIdx.x / per, part = blockIdx.x - c * per;
@@ -470,6 +472,8 @@ ssd_scan_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     int item = blockIdx.x;                     // (batch row, direction, head or head pair), heads fastest
     if (pj.sync) {
+        pdl_wait();                            // (the ticket counter is cleared in stream order)
+        pdl_trigger();
         if (tid == 0) misc->ticket = atomicAdd(pj.sync, 1);
         __syncthreads();
         const int ticket = misc->ticket;
@@ -508,6 +512,8 @@ ssd_scan_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
     fence_before();
     __syncthreads();
     fence_after();
+    pdl_wait();
+    pdl_trigger();
     const uint32_t tmem = misc->tmem_base;
     const uint32_t tlane = tmem + ((uint32_t)((warp & 3) * 32) << 16);     // this warp's TMEM lane quarter
     const float *dA_head = a.dA + (((int64_t)seq * a.H + h) * 2) * a.Lp;
@@ -1073,6 +1079,8 @@ ssd_block_kernel(const SsdArgs a, const __nv_bfloat16 *__restrict__ Bp, const __
     uint4 nwp = make_uint4(0x3F803F80u, 0x3F803F80u, 0x3F803F80u, 0x3F803F80u);      // norm weights of those channels as bf16 pairs (ones when the norm is off)
     if (norm_on && w.norm_w) nwp = __ldg(reinterpret_cast<const uint4 *>(static_cast<const __nv_bfloat16 *>(w.norm_w) + h * PP + ec));
 
+    pdl_wait();
+    pdl_trigger();
     // state accumulators: warp = channels [16 smt, +16) x states [64 snh, +64): tile t covers states 64 snh + 8 t .. + 7;
     // a thread holds rows p = 16 smt + gr (+8), columns n = 64 snh + 8 t + 2 qc (+1)
     const int smt = warp % MT, snh = warp / MT;
@@ -1384,10 +1392,7 @@ cudaError_t scan_ssd(const ScanArgs &a, void *ws, cudaStream_t s) {
     cudaError_t e;
     if (pj.sync && (e = cudaMemsetAsync(pj.sync, 0, ((size_t)2 * a.B * l.nch + 1) * sizeof(int), s)) != cudaSuccess) return e;
     const dim3 pgrid(n_pre * (PREP_BC + (a.H + 63) / 64), a.B, ndir);
-    if (blk) ssd_prep_kernel<true><<<pgrid, PREP_THREADS, 0, s>>>(k, Bp, Cp, dA, Sb, dir0);
-    else ssd_prep_kernel<false><<<pgrid, PREP_THREADS, 0, s>>>(k, Bp, Cp, dA, Sb, dir0);
-    count_launch();
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if ((e = launch_chain(blk ? ssd_prep_kernel<true> : ssd_prep_kernel<false>, pgrid, PREP_THREADS, 0, s, 0, k, Bp, Cp, dA, Sb, dir0)) != cudaSuccess) return e;
     if (blk) {
         // the state is carried in registers when there are several sub-chunks or someone reads it afterwards
         const bool keep = a.L > QB || a.ssm_out != nullptr;
@@ -1397,9 +1402,7 @@ cudaError_t scan_ssd(const ScanArgs &a, void *ws, cudaStream_t s) {
                                      : (keep ? BlockSmem<P / 2>::total : BlockSmem<P / 2>::total_nokeep);
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        kern<<<dim3(a.H, ndir, a.B), 4 * a.P, smem, s>>>(k, Bp, Cp, Sb, dir0);
-        count_launch();
-        return cudaGetLastError();
+        return launch_chain(kern, dim3(a.H, ndir, a.B), 4 * a.P, smem, s, 0, k, Bp, Cp, Sb, dir0);
     }
 
     CUtensorMap mx, mz, mb, mc, mg;
@@ -1427,9 +1430,7 @@ cudaError_t scan_ssd(const ScanArgs &a, void *ws, cudaStream_t s) {
     const uint32_t smem_bytes = pair ? SMEM_BYTES_PAIR : SMEM_BYTES;
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
     if (e != cudaSuccess) return e;
-    kern<<<nscan + pj.nprep, NTHREADS, smem_bytes, s>>>(mx, mz, mb, mc, mg, k, pj, dir0, status);
-    count_launch();
-    return cudaGetLastError();
+    return launch_chain(kern, nscan + pj.nprep, NTHREADS, smem_bytes, s, 0, mx, mz, mb, mc, mg, k, pj, dir0, status);
 }
 
 }  // namespace dm
