@@ -28,25 +28,23 @@
 // Every hand-off is an mbarrier; every wait is bounded.  On expiry the CTA stores DM_ERR_TIMEOUT in the
 // device status word, all roles leave their loops, outstanding TMA traffic is waited for (bounded), TMEM is
 // freed and the CTA returns.
-// Launch 2, short blocks (ssd_block, Q = 32, products with mma.sync from registers): the active block of block-autoregressive
-// decoding is 32 tokens, a quarter of one tcgen05 tile, and a call has thousands of (batch row, head) items of that size;
-// for them the pipeline above is all set-up and tear-down.  ssd_block is a plain CTA of 256 threads per item: it takes the
+// Blocks of up to 32 tokens (the active block of block-autoregressive decoding: a quarter of one tcgen05 tile, and thousands of (batch row, head) items of
+// that size, for which the pipeline above is all set-up and tear-down) take a single launch of their own: scan_step.cu.
+// Launch 2, 33 to 64 tokens (ssd_block, Q = 32, products with mma.sync from registers).  ssd_block is a plain CTA of 256 threads per item: it takes the
 // 32 x 32 matrix S of each sub-chunk from the prep launch (which computes it once per (batch row, direction)), builds W
 // and runs the other three products of the identities above on 16 x 8 x 16 tiles; a state that has to outlive the
 // sub-chunk stays in its fp32 accumulators.  It is also what `chunk = 32` selects at any length.
 #include <cstddef>
 
-#include "dm_internal.h"
-#include "tc_ptx.cuh"
+#include "ssd_common.cuh"
 
 namespace dm {
 namespace {
 
-using namespace tc;
+using namespace ssd;
 
 constexpr int Q = 128;            // tokens per chunk
 constexpr int P = 64;             // headdim
-constexpr int N = 128;            // d_state
 constexpr int HALO = 8;           // conv look-back rows kept with the x tile (8 keeps the tile 1024-byte aligned)
 constexpr int XROWS = Q + HALO;
 constexpr uint32_t T16 = Q * 128;           // bytes of a [128 rows][64 bf16] tile
@@ -89,42 +87,6 @@ struct Misc {
 static_assert(sizeof(Misc) <= 7168, "Misc must fit its slot");
 static_assert(offsetof(Misc, norm_w) % 16 == 0 && offsetof(Misc, wbuf) % 16 == 0 && offsetof(Misc, cbuf) % 16 == 0, "float4 access");
 
-struct SsdArgs {
-    int B, L, H, d_inner, d_in_proj, conv_ch, k, flags, nch, Lp;
-    int Nr;                      // d_state of the model (<= N); B', C' and the state are zero-padded to N
-    int Pr;                      // headdim of the model: P, or P / 2 (the CTA then carries the next head's channels as unused padding)
-    int zx_tied;                 // both directions read the in_proj output of direction 0 (shared projections)
-    __nv_bfloat16 *g;            // [2][B*L][d_inner] gated output (written with plain stores when Pr < P, else through map_g)
-    const __nv_bfloat16 *zx;
-    float *ssq;
-    const float *dA;             // [2][B][H][2][Lp]: Lambda, Lambda' (log2 units)
-    const float *ssm_in; float *ssm_out;
-    const __nv_bfloat16 *conv_in;  // [B][k-1][conv_ch] pre-conv rows before the first token (left-to-right layer), or NULL
-    ScanDir dir[2];
-};
-
-__device__ __forceinline__ float silu_fast(float v) { const float hv = 0.5f * v; return fmaf(hv, tanh_fast(hv), hv); }     // SiLU(v) = v/2 + v/2 tanh(v/2)
-// Arithmetic shared by the two forms of the prep work (the launch of its own below and the prep role inside the scan
-// launch), so that both give the same bits.
-// conv + SiLU of one bf16 channel pair: r[m] = the pre-conv pair m steps back in time, wl[e][m] its weight
-__device__ __forceinline__ uint32_t prep_conv_pair(const float (&wl)[2][4], const float (&bias)[2], const uint32_t (&r)[4]) {
-    float v0 = bias[0], v1 = bias[1];
-#pragma unroll
-    for (int m = 3; m >= 0; --m) {
-        v0 = fmaf(wl[0][m], bf16_lo(r[m]), v0);
-        v1 = fmaf(wl[1][m], bf16_hi(r[m]), v1);
-    }
-    return pack_bf16(silu_fast(v0), silu_fast(v1));
-}
-// softplus(dt + bias) = max(v, 0) + log1p(exp(-|v|)) with the fast exponential and logarithm: log1p by its series where 1 + e
-// would round e away (e < 2^-7: error below e^4 / 4), by log(1 + e) elsewhere.  Relative error of Delta about 1e-6, far inside
-// what the bf16 path needs.
-__device__ __forceinline__ float prep_delta(float dt, float dt_bias) {
-    const float v = dt + dt_bias;
-    const float e = __expf(-fabsf(v));
-    const float l = e < 0.0078125f ? e * fmaf(e, fmaf(e, 0.33333334f, -0.5f), 1.f) : __logf(1.f + e);
-    return fmaxf(v, 0.f) + l;
-}
 // One warp, one head, one 128-token chunk: d[e] = Delta of the token 4 lane + e in the direction's time order.  Writes Lambda (inclusive cumulative
 // Delta A in that order, log2 units) of physical chunk row r to dl[r] and Lambda' = Lambda - log2 Delta to dl[Lp + r].
 __device__ __forceinline__ void prep_lambda_head(const float (&d)[4], float A_log, bool rev, int lane, float *dl, int Lp) {
@@ -157,21 +119,8 @@ __device__ __forceinline__ void prep_lambda_head(const float (&d)[4], float A_lo
 // --------------------------------------------------------------------------------------------------
 constexpr int PREP_PARTS = 4;               // sub-chunks of the short-block kernel per chunk
 constexpr int PREP_THREADS = 512, PREP_RUN = 16, PREP_ROWS = PREP_THREADS / N * PREP_RUN, PREP_BC = Q / PREP_ROWS;      // rows per thread, per B', C' unit; units per chunk
-constexpr int QB = Q / PREP_PARTS;          // tokens per sub-chunk of the short-block kernel
 constexpr int BCT_LD = N / 2 + 4;           // row pitch (32-bit words) of the B' / C' tile S is computed from: 16-byte rows, conflict-free ldmatrix
-static_assert(QB == 32 && PREP_ROWS == 2 * QB, "a B', C' unit covers two sub-chunks");
-
-__device__ __forceinline__ void ldmatrix_x4(uint32_t &r0, uint32_t &r1, uint32_t &r2, uint32_t &r3, const void *p) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];" : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3) : "r"(smem_u32(p)));
-}
-__device__ __forceinline__ void ldmatrix_x2(uint32_t &r0, uint32_t &r1, const void *p) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0, %1}, [%2];" : "=r"(r0), "=r"(r1) : "r"(smem_u32(p)));
-}
-// D (16 x 8, fp32) += A (16 x 16, row-major) B (16 x 8, column-major), bf16 operands
-__device__ __forceinline__ void mma_bf16_16816(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
-                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
+static_assert(QB == Q / PREP_PARTS && PREP_ROWS == 2 * QB, "a B', C' unit covers two sub-chunks");
 
 // Rows [row0, row0 + PREP_ROWS) of B' and C' (row0: physical).  WITH_S (short blocks): also S[i][j] = C'_i . B'_j over each sub-chunk of QB rows, fp32, to
 // Sb[seq][row0 / QB + ..][QB][QB]; bct: [2][PREP_ROWS][BCT_LD] words of shared memory.
@@ -319,12 +268,6 @@ struct PrepJob {
     int nprep, ndir;
     int c0;             // chunks before this one (in time order) come from a prep launch of their own that ran before the scan launch
 };
-// 16-byte asynchronous copy global -> shared; src_bytes = 16, or 0 to fill the destination with zeros (src must still be a valid address)
-__device__ __forceinline__ void cp_async16(void *smem_dst, const void *gsrc, uint32_t src_bytes) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(smem_dst)), "l"(gsrc), "r"(src_bytes) : "memory");
-}
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-
 constexpr int PREP_SEG = 7, PREP_SEG_ROWS = (Q + PREP_SEG - 1) / PREP_SEG;     // row runs per channel pair
 // shared memory of a prep CTA: two stages of { rows [Q + 3][N] words, dt [Q][64] bf16 }, then Delta [Q][65] floats
 constexpr uint32_t PREP_RAW_BYTES = (Q + 3) * N * 4, PREP_DT_BYTES = Q * 64 * 2, PREP_STAGE = PREP_RAW_BYTES + PREP_DT_BYTES;
@@ -1007,39 +950,27 @@ ssd_scan_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
 //           fp32 state stays in the accumulators from one sub-chunk to the next
 // Lambda_0 is Lambda of the token before the sub-chunk inside the same 128-token chunk of the prep launch (0 at its start).
 // --------------------------------------------------------------------------------------------------
-constexpr int NLD = N + 8;             // row pitch (bf16) of the C', B' and state tiles: 16-byte rows, conflict-free ldmatrix
 constexpr int SLD = QB + 4;            // row pitch (fp32) of S
 constexpr int WTL = QB + 8;            // row pitch (bf16) of W
-// The tiles only the state update reads (B', w o x') come last: a launch that carries no state out of its single sub-chunk
-// (KEEP = false: the denoising passes of block decoding) asks for the bytes before them only.  The fp32 y tile reuses the
-// bytes of S and of the raw x rows, both dead once the conv and mask phase is over.
+// The fp32 y tile reuses the bytes of S and of the raw x rows, both dead once the conv and mask phase is over.
 template <int PP> struct BlockSmem {
     static constexpr int XLD = PP + 8;             // row pitch (bf16) of x' and w o x'
     static constexpr size_t ct = 0, ht = ct + QB * NLD * 2, xt = ht + PP * NLD * 2, wt = xt + QB * XLD * 2, ss = wt + QB * WTL * 2,
-                            xr = ss + QB * SLD * 4, lam = xr + (QB + 4) * PP * 2, total_nokeep = lam + (2 * QB + 4) * 4,
-                            bt = total_nokeep, wxt = bt + QB * NLD * 2, total = wxt + QB * XLD * 2, ys = ss;
+                            xr = ss + QB * SLD * 4, lam = xr + (QB + 4) * PP * 2,
+                            bt = lam + (2 * QB + 4) * 4, wxt = bt + QB * NLD * 2, total = wxt + QB * XLD * 2, ys = ss;
     static_assert(ht % 16 == 0 && xt % 16 == 0 && wt % 16 == 0 && ss % 16 == 0 && xr % 16 == 0 && lam % 16 == 0 && bt % 16 == 0 && wxt % 16 == 0, "16-byte tiles");
     static_assert(QB * PP * 4 <= lam - ss, "the y tile fits the bytes of S and the raw x rows");
 };
-__device__ __forceinline__ void ldmatrix_x4_t(uint32_t &r0, uint32_t &r1, uint32_t &r2, uint32_t &r3, const void *p) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];" : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3) : "r"(smem_u32(p)));
-}
-__device__ __forceinline__ void ldmatrix_x2_t(uint32_t &r0, uint32_t &r1, const void *p) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0, %1}, [%2];" : "=r"(r0), "=r"(r1) : "r"(smem_u32(p)));
-}
-
-// KEEP: the fp32 state lives in the accumulators (several sub-chunks, or a state to write out); without it the launch is a
-// single sub-chunk whose state nobody reads, the accumulators and the update's tiles are gone and more CTAs fit an SM.
-template <int PP, bool KEEP>
-__global__ void __launch_bounds__(4 * PP, (KEEP ? 192 : 256) / PP)
+template <int PP>
+__global__ void __launch_bounds__(4 * PP, 192 / PP)
 ssd_block_kernel(const SsdArgs a, const __nv_bfloat16 *__restrict__ Bp, const __nv_bfloat16 *__restrict__ Cp, const float *__restrict__ Sb, int dir0) {
     constexpr int NT = 4 * PP, U8 = PP / 8, MT = PP / 16, XLD = BlockSmem<PP>::XLD, CP2 = PP / 2;
     extern __shared__ __align__(16) uint8_t bsm[];
     __nv_bfloat16 (*Ct)[NLD] = reinterpret_cast<__nv_bfloat16 (*)[NLD]>(bsm + BlockSmem<PP>::ct);      // C' rows [i][n]
-    __nv_bfloat16 (*Bt)[NLD] = reinterpret_cast<__nv_bfloat16 (*)[NLD]>(bsm + BlockSmem<PP>::bt);      // B' rows [j][n]               (KEEP only)
+    __nv_bfloat16 (*Bt)[NLD] = reinterpret_cast<__nv_bfloat16 (*)[NLD]>(bsm + BlockSmem<PP>::bt);      // B' rows [j][n]            
     __nv_bfloat16 (*Ht)[NLD] = reinterpret_cast<__nv_bfloat16 (*)[NLD]>(bsm + BlockSmem<PP>::ht);      // incoming state [p][n]
     __nv_bfloat16 (*Xt)[XLD] = reinterpret_cast<__nv_bfloat16 (*)[XLD]>(bsm + BlockSmem<PP>::xt);      // x' [j][p]
-    __nv_bfloat16 (*WXt)[XLD] = reinterpret_cast<__nv_bfloat16 (*)[XLD]>(bsm + BlockSmem<PP>::wxt);    // w_j x'_j [j][p]              (KEEP only)
+    __nv_bfloat16 (*WXt)[XLD] = reinterpret_cast<__nv_bfloat16 (*)[XLD]>(bsm + BlockSmem<PP>::wxt);    // w_j x'_j [j][p]           
     __nv_bfloat16 (*Wt)[WTL] = reinterpret_cast<__nv_bfloat16 (*)[WTL]>(bsm + BlockSmem<PP>::wt);      // W [i][j]
     __nv_bfloat16 (*xr)[PP] = reinterpret_cast<__nv_bfloat16 (*)[PP]>(bsm + BlockSmem<PP>::xr);        // raw x rows and conv history
     float (*ys)[PP] = reinterpret_cast<float (*)[PP]>(bsm + BlockSmem<PP>::ys);                        // the sub-chunk's y (over S and the raw rows)
@@ -1054,7 +985,7 @@ ssd_block_kernel(const SsdArgs a, const __nv_bfloat16 *__restrict__ Bp, const __
     const ScanDir &w = a.dir[dir];
     const __nv_bfloat16 *zx = a.zx + ((int64_t)(a.zx_tied ? 0 : dir) * a.B + b) * L * a.d_in_proj;
     const float *dA_head = a.dA + ((seq * a.H + h) * 2) * a.Lp;
-    const int nsub = KEEP ? (L + QB - 1) / QB : 1, nsub_all = a.nch * PREP_PARTS;
+    const int nsub = (L + QB - 1) / QB, nsub_all = a.nch * PREP_PARTS;
     const float Dh = (a.flags & DM_FLAG_D_SKIP) ? w.D[h] : 0.f;
     const bool norm_on = (a.flags & DM_FLAG_GATED_RMSNORM) != 0;
 
@@ -1084,9 +1015,9 @@ ssd_block_kernel(const SsdArgs a, const __nv_bfloat16 *__restrict__ Bp, const __
     // state accumulators: warp = channels [16 smt, +16) x states [64 snh, +64): tile t covers states 64 snh + 8 t .. + 7;
     // a thread holds rows p = 16 smt + gr (+8), columns n = 64 snh + 8 t + 2 qc (+1)
     const int smt = warp % MT, snh = warp / MT;
-    float hacc[KEEP ? 8 : 1][4];
+    float hacc[8][4];
     const float *h_in = (!rev && a.ssm_in) ? a.ssm_in + ((int64_t)b * a.H + h) * PP * a.Nr : nullptr;
-    if constexpr (KEEP) {
+    {
 #pragma unroll
         for (int t = 0; t < 8; ++t) {
             const int n = 64 * snh + 8 * t + 2 * qc, p0 = 16 * smt + gr;
@@ -1102,9 +1033,9 @@ ssd_block_kernel(const SsdArgs a, const __nv_bfloat16 *__restrict__ Bp, const __
     for (int si = 0; si < nsub; ++si) {
         const int sub = rev ? nsub - 1 - si : si, r0 = sub * QB;
         const bool have_state = si > 0 || h_in != nullptr;
-        const bool need_update = KEEP && (si + 1 < nsub || (!rev && a.ssm_out != nullptr));
+        const bool need_update = (si + 1 < nsub || (!rev && a.ssm_out != nullptr));
         const int nvalid = min(QB, L - r0);                // tokens of the sub-chunk inside the sequence
-        if (KEEP) __syncthreads();                         // the previous sub-chunk's readers are done with the tiles
+        __syncthreads();                                   // the previous sub-chunk's readers are done with the tiles
         // ---- load
         if (tid < QB) {
             lam[tid] = dA_head[r0 + tid];
@@ -1154,7 +1085,7 @@ ssd_block_kernel(const SsdArgs a, const __nv_bfloat16 *__restrict__ Bp, const __
                     }
                     *reinterpret_cast<uint4 *>(&Ht[p][n0]) = make_uint4(pack_bf16(v0.x, v0.y), pack_bf16(v0.z, v0.w), pack_bf16(v1.x, v1.y), pack_bf16(v1.z, v1.w));
                 }
-            } else if constexpr (KEEP) {
+            } else {
 #pragma unroll
                 for (int t = 0; t < 8; ++t) {              // from the accumulators of the previous sub-chunk
                     const int n = 64 * snh + 8 * t + 2 * qc, p0 = 16 * smt + gr;
@@ -1249,7 +1180,7 @@ ssd_block_kernel(const SsdArgs a, const __nv_bfloat16 *__restrict__ Bp, const __
             }
         }
         // ---- state after the sub-chunk: h <- dec h + (w o x')^T B'
-        if constexpr (KEEP) {
+        {
             if (need_update) {
                 const float dec = ex2f(lam_last - lam0);
 #pragma unroll
@@ -1286,7 +1217,7 @@ ssd_block_kernel(const SsdArgs a, const __nv_bfloat16 *__restrict__ Bp, const __
             }
         }
     }
-    if constexpr (KEEP) {
+    {
         if (!rev && a.ssm_out) {
             float *ho = a.ssm_out + ((int64_t)b * a.H + h) * PP * a.Nr;
 #pragma unroll
@@ -1371,6 +1302,8 @@ cudaError_t scan_ssd(const ScanArgs &a, void *ws, cudaStream_t s) {
     const bool blk = block_mode(a);
     float *Sb = blk ? reinterpret_cast<float *>(base + l.sb) : nullptr;
 
+    if (blk && scan_step_supports(k)) return scan_step(k, a.P, ndir, dir0, s);
+
     // One long sequence leaves SMs without a scan CTA: they take the prep work inside the scan launch (see prep_role), except for
     // the first PRE_CHUNKS chunks of every sequence and direction, which a small prep launch of their own has ready by the time the
     // scan starts (a prep CTA inside the scan launch needs about 20 us for its first chunk; the scan would stand idle that long).
@@ -1394,12 +1327,8 @@ cudaError_t scan_ssd(const ScanArgs &a, void *ws, cudaStream_t s) {
     const dim3 pgrid(n_pre * (PREP_BC + (a.H + 63) / 64), a.B, ndir);
     if ((e = launch_chain(blk ? ssd_prep_kernel<true> : ssd_prep_kernel<false>, pgrid, PREP_THREADS, 0, s, 0, k, Bp, Cp, dA, Sb, dir0)) != cudaSuccess) return e;
     if (blk) {
-        // the state is carried in registers when there are several sub-chunks or someone reads it afterwards
-        const bool keep = a.L > QB || a.ssm_out != nullptr;
-        auto kern = a.P == P ? (keep ? ssd_block_kernel<P, true> : ssd_block_kernel<P, false>)
-                             : (keep ? ssd_block_kernel<P / 2, true> : ssd_block_kernel<P / 2, false>);
-        const size_t smem = a.P == P ? (keep ? BlockSmem<P>::total : BlockSmem<P>::total_nokeep)
-                                     : (keep ? BlockSmem<P / 2>::total : BlockSmem<P / 2>::total_nokeep);
+        auto kern = a.P == P ? ssd_block_kernel<P> : ssd_block_kernel<P / 2>;
+        const size_t smem = a.P == P ? BlockSmem<P>::total : BlockSmem<P / 2>::total;
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         return launch_chain(kern, dim3(a.H, ndir, a.B), 4 * a.P, smem, s, 0, k, Bp, Cp, Sb, dir0);

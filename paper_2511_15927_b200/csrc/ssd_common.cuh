@@ -1,0 +1,83 @@
+// Shared by the chunked scan kernels (scan_ssd.cu, scan_step.cu): arguments, the arithmetic of conv and step size, mma.sync helpers.
+#pragma once
+
+#include "dm_internal.h"
+#include "tc_ptx.cuh"
+
+namespace dm {
+namespace ssd {
+
+using namespace tc;
+
+constexpr int N = 128;                // d_state (a smaller one is zero-padded)
+constexpr int QB = 32;                // tokens per sub-chunk of the short-block kernels
+constexpr int NLD = N + 8;            // row pitch (elements) of C', B' and state tiles: 16-byte rows, conflict-free ldmatrix
+
+struct SsdArgs {
+    int B, L, H, d_inner, d_in_proj, conv_ch, k, flags, nch, Lp;
+    int Nr;                      // d_state of the model (<= N); B', C' and the state are zero-padded to N
+    int Pr;                      // headdim of the model: P, or P / 2 (the CTA then carries the next head's channels as unused padding)
+    int zx_tied;                 // both directions read the in_proj output of direction 0 (shared projections)
+    __nv_bfloat16 *g;            // [2][B*L][d_inner] gated output (written with plain stores when Pr < P, else through map_g)
+    const __nv_bfloat16 *zx;
+    float *ssq;
+    const float *dA;             // [2][B][H][2][Lp]: Lambda, Lambda' (log2 units)
+    const float *ssm_in; float *ssm_out;
+    const __nv_bfloat16 *conv_in;  // [B][k-1][conv_ch] pre-conv rows before the first token (left-to-right layer), or NULL
+    ScanDir dir[2];
+};
+
+__device__ __forceinline__ float silu_fast(float v) { const float hv = 0.5f * v; return fmaf(hv, tanh_fast(hv), hv); }     // SiLU(v) = v/2 + v/2 tanh(v/2)
+// Arithmetic shared by the two forms of the prep work (the launch of its own below and the prep role inside the scan
+// launch), so that both give the same bits.
+// conv + SiLU of one bf16 channel pair: r[m] = the pre-conv pair m steps back in time, wl[e][m] its weight
+__device__ __forceinline__ uint32_t prep_conv_pair(const float (&wl)[2][4], const float (&bias)[2], const uint32_t (&r)[4]) {
+    float v0 = bias[0], v1 = bias[1];
+#pragma unroll
+    for (int m = 3; m >= 0; --m) {
+        v0 = fmaf(wl[0][m], bf16_lo(r[m]), v0);
+        v1 = fmaf(wl[1][m], bf16_hi(r[m]), v1);
+    }
+    return pack_bf16(silu_fast(v0), silu_fast(v1));
+}
+// softplus(dt + bias) = max(v, 0) + log1p(exp(-|v|)) with the fast exponential and logarithm: log1p by its series where 1 + e
+// would round e away (e < 2^-7: error below e^4 / 4), by log(1 + e) elsewhere.  Relative error of Delta about 1e-6, far inside
+// what the bf16 path needs.
+__device__ __forceinline__ float prep_delta(float dt, float dt_bias) {
+    const float v = dt + dt_bias;
+    const float e = __expf(-fabsf(v));
+    const float l = e < 0.0078125f ? e * fmaf(e, fmaf(e, 0.33333334f, -0.5f), 1.f) : __logf(1.f + e);
+    return fmaxf(v, 0.f) + l;
+}
+__device__ __forceinline__ void ldmatrix_x4(uint32_t &r0, uint32_t &r1, uint32_t &r2, uint32_t &r3, const void *p) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];" : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3) : "r"(smem_u32(p)));
+}
+__device__ __forceinline__ void ldmatrix_x2(uint32_t &r0, uint32_t &r1, const void *p) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0, %1}, [%2];" : "=r"(r0), "=r"(r1) : "r"(smem_u32(p)));
+}
+// D (16 x 8, fp32) += A (16 x 16, row-major) B (16 x 8, column-major), bf16 operands
+__device__ __forceinline__ void mma_bf16_16816(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+
+__device__ __forceinline__ void ldmatrix_x4_t(uint32_t &r0, uint32_t &r1, uint32_t &r2, uint32_t &r3, const void *p) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];" : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3) : "r"(smem_u32(p)));
+}
+__device__ __forceinline__ void ldmatrix_x2_t(uint32_t &r0, uint32_t &r1, const void *p) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0, %1}, [%2];" : "=r"(r0), "=r"(r1) : "r"(smem_u32(p)));
+}
+
+// 16-byte asynchronous copy global -> shared; src_bytes = 16, or 0 to fill the destination with zeros (src must still be a valid address)
+__device__ __forceinline__ void cp_async16(void *smem_dst, const void *gsrc, uint32_t src_bytes) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(smem_dst)), "l"(gsrc), "r"(src_bytes) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+}  // namespace ssd
+
+// One block of up to QB tokens per sequence in one launch: see scan_step.cu (which takes 16-byte aligned states).
+bool scan_step_supports(const ssd::SsdArgs &a);
+cudaError_t scan_step(const ssd::SsdArgs &a, int headdim, int ndir, int dir0, cudaStream_t s);
+
+}  // namespace dm

@@ -182,3 +182,23 @@ def test_half_width_heads_single_and_paired(G, H, L):
     y_o, s_o, c_o = O.bimamba_block_step(x, wf, wr, ssm_state_in=ssm_in, conv_state_in=conv_in, **G.oracle_kwargs(blk))
     _check(G, y, y_o)
     assert G.rel_l2(s_out, s_o) <= BF16_REL and G.rel_l2(c_out, c_o) <= BF16_REL
+
+
+@pytest.mark.parametrize("B,H,P,N,L,k", [(2, 8, 64, 128, 1, 4), (1, 8, 64, 128, 32, 2), (64, 24, 64, 16, 31, 4), (64, 24, 32, 128, 32, 4), (3, 8, 32, 16, 5, 3)])
+def test_blocks_of_up_to_32_tokens(G, B, H, P, N, L, k):
+    """The one-launch kernel of short blocks: its smallest and largest block, padded d_state, both head widths, one head per CTA and several (24 heads in groups of
+    7, the last of 3; 64 batch rows take more than one round), with the state committed, read only, and absent."""
+    shape = I.MixerShape(B, L, P * H // 2, 2, N, k, H)
+    assert shape.headdim == P and shape.d_in_proj % 8 == 0
+    wf, wr = I.make_mixer_weights(shape, 60 + L, I.BF16, perturb=True)
+    x = I.make_activations(shape, 60 + L, I.BF16)
+    kw = G.oracle_kwargs(shape)
+    ssm_in, conv_in = I.make_states(shape, 60 + L, I.BF16)
+    y_o, s_o, c_o = O.bimamba_block_step(x, wf, wr, ssm_state_in=ssm_in, conv_state_in=conv_in, **kw)
+    y_g, s_g, c_g = G.run_block_step(shape, I.BF16, wf, wr, x, ssm_in, conv_in)
+    _check(G, y_g, y_o)
+    _check(G, s_g, s_o)
+    _check(G, c_g, c_o)
+    y_r, _, _ = G.run_block_step(shape, I.BF16, wf, wr, x, ssm_in, conv_in, want_state=False)
+    np.testing.assert_array_equal(y_r, y_g)                 # committing the state leaves the output alone
+    _check(G, G.run_forward(shape, I.BF16, wf, wr, x), O.bimamba_forward(x, wf, wr, **kw))
