@@ -119,11 +119,6 @@ static int check_weights(const dm_mixer_cfg *c, const dm_dir_weights w[2]) {
     return DM_OK;
 }
 
-// Up to this many tokens the two directions' out_proj run as one launch that writes an fp32 partial each (summed by a small
-// kernel); above it they are chained, the second adding the first in its epilogue, which moves less memory.
-constexpr int64_t PAIR_OUT_MAX_T = 2048;
-// Up to this many tokens the out_proj launch cuts K over clusters and sums both directions in shared memory (gemm_rows.cu).
-constexpr int64_t SUM_OUT_MAX_T = 128;
 // Up to this many tokens the two directions' in_proj share one launch.  Beyond it two launches are faster: both weight matrices
 // together (70 MB at d_model 2048) no longer stay in L2 while the rows of x stream past them (measured at 16 384 tokens: 1.00 ms
 // for the pair against 0.84 ms for two launches; level at 8192, 15-25 % faster for the 512 tokens of a decoding step).
@@ -141,7 +136,7 @@ static MixerWs mixer_ws(const dm_mixer_cfg *c, const Dims &m) {
     w.g = off;    off += align_up((size_t)2 * m.T * m.d_inner * m.es);
     w.ssq = off;  off += align_up((size_t)2 * m.T * m.H * sizeof(float));
     w.rstd = off; off += align_up((size_t)2 * m.T * sizeof(float));
-    w.ytmp = off; off += align_up((size_t)(m.T <= PAIR_OUT_MAX_T ? 4 : 1) * m.T * m.d * sizeof(float));      // short inputs: up to two fp32 partials per direction
+    w.ytmp = off; off += align_up((size_t)m.T * m.d * sizeof(float));
     ScanArgs sa{};
     sa.B = m.B; sa.L = m.L; sa.d_inner = m.d_inner; sa.H = m.H; sa.P = m.P; sa.N = m.N; sa.k = m.k;
     sa.d_in_proj = m.ldz; sa.conv_ch = m.conv_ch; sa.dtype = c->dtype; sa.flags = c->flags; sa.dir_mask = c->dir_mask; sa.chunk = c->chunk;
@@ -251,38 +246,8 @@ static int run_mixer(const dm_mixer_cfg *c, const Dims &m, const dm_dir_weights 
         e = conv_state_update(zx, conv_in, conv_out, c->dtype, m.B, m.L, m.k, m.d_inner, m.conv_ch, m.ldz, s);
         if (e != cudaSuccess) return cuda_fail(e, "conv_state_update");
     }
-    if (!tied && c->dir_mask == DM_DIR_BOTH && m.T <= PAIR_OUT_MAX_T && m.T > SUM_OUT_MAX_T && sum_partials_norm_supports(m.d)) {
-        // short inputs (block decoding): both out_proj in one launch, each into its own fp32 partial (gated by col_scale, not yet scaled by the
-        // gated norm); one pass then scales, sums, adds the residual and applies the caller's next norm
-        GemmArgs ga[2];
-        for (int dir = 0; dir < 2; ++dir) {
-            GemmArgs a{};
-            a.A = g + (size_t)dir * m.T * m.d_inner * m.es; a.lda = m.d_inner;
-            a.B = w[dir].w_out; a.ldb = m.d_inner;
-            a.in_dtype = c->dtype; a.M = (int)m.T; a.N = m.d; a.K = m.d_inner;
-            a.col_scale = out.col_scale; a.cs_rows = out.cs_rows; a.ld_cs = out.ld_cs;
-            a.C = ytmp + (size_t)dir * m.T * m.d; a.ldc = m.d; a.c_dtype = DM_F32;
-            ga[dir] = a;
-        }
-        if (gemm_tcgen05_pair_supports(ga[0], ga[1])) {
-            {
-                StageTimer tm(DM_STAGE_OUT_PROJ, s);
-                const size_t part = (size_t)m.T * m.d;
-                const bool split = gemm_tcgen05_pair_splitk_pays(ga[0], ga[1]);
-                e = split ? gemm_tcgen05_pair_splitk(ga[0], ga[1], ytmp + 2 * part, ytmp + 3 * part, s) : gemm_tcgen05_pair(ga[0], ga[1], s);
-                if (e != cudaSuccess) return cuda_fail(e, "out_proj");
-                const bool next = out.next_norm_w && out.next_u;
-                e = sum_partials_norm(ytmp, ytmp + part, split ? ytmp + 2 * part : nullptr, split ? ytmp + 3 * part : nullptr, norm_on ? ssq : nullptr, norm_on ? ssq + (size_t)m.T * m.H : nullptr, m.H, m.d_inner,
-                                      c->norm_eps, out.addend, out.ld_add, out.y, out.y_dtype, next ? out.next_norm_w : nullptr, next ? out.next_u : nullptr,
-                                      c->dtype, m.T, m.d, out.next_eps, s);
-                if (next && out.next_done) *out.next_done = true;
-            }
-            if (e != cudaSuccess) return cuda_fail(e, "out_proj sum");
-            return DM_OK;
-        }
-    }
-    if (!tied && c->dir_mask == DM_DIR_BOTH && (m.T > PAIR_OUT_MAX_T || m.T <= SUM_OUT_MAX_T || c->dtype == DM_F32)) {
-        // long inputs, a few sequences' blocks, and fp32 inputs that do not fill the GPU: both out_proj and their sum in one launch, each direction's gated-norm scale taken from the sums of squares in the epilogue
+    if (!tied && c->dir_mask == DM_DIR_BOTH) {
+        // both out_proj and their sum in one launch, each direction's gated-norm scale taken from the sums of squares in the epilogue
         GemmArgs ga[2];
         for (int dir = 0; dir < 2; ++dir) {
             GemmArgs a{};

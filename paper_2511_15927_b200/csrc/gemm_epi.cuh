@@ -16,42 +16,27 @@ struct EpiArgs {
     const int *m_dev; int m_off;
     const float *rs_ssq; int rs_n; float rs_inv, rs_eps;
     __nv_bfloat16 *u; const __nv_bfloat16 *u_w; float *u_ssq;
-    int k_off;       // first element along K of this problem's share (split K: the second half of a product is a problem of its own)
 };
 
-// Up to two products of the same M, N, K in one launch (the two directions' in_proj, or their out_proj on short inputs), each optionally
-// cut in two along K (ksplit: problems 2 i and 2 i + 1 are the halves of product i, each with an output of its own that the caller adds): the tile
-// loop runs over all of them, so that they share one tail round and -- for in_proj, whose A operand is the same x -- the rows of A in L2.
+// Up to two products of the same M, N, K in one launch (the two directions' in_proj or out_proj): the tile loop runs over both, so that they share one tail round and
+// -- for in_proj, whose A operand is the same x -- the rows of A in L2.
 struct EpiPair {
-    EpiArgs p[4];
-    int nprob, ksplit;
+    EpiArgs p[2];
+    int nprob;
     int n_fast;      // tile order: consecutive tiles step along N (the A rows are streamed once, B stays in L2) or along M
 };
 
 inline EpiArgs epi_of(const GemmArgs &a) {
     return EpiArgs{a.C, a.ldc, a.c_dtype == DM_F32 ? 1 : 0, a.row_scale, a.addend, a.ld_add, a.M, a.N, a.K, a.silu_cols,
                    a.col_bias, a.gelu, a.col_scale, a.cs_rows > 0 ? a.cs_rows : 1, a.ld_cs > 0 ? a.ld_cs : (int64_t)a.N, a.m_dev, a.m_off,
-                   a.rs_ssq, a.rs_n, a.rs_inv, a.rs_eps, static_cast<__nv_bfloat16 *>(a.u), static_cast<const __nv_bfloat16 *>(a.u_w), a.u_ssq, 0};
+                   a.rs_ssq, a.rs_n, a.rs_inv, a.rs_eps, static_cast<__nv_bfloat16 *>(a.u), static_cast<const __nv_bfloat16 *>(a.u_w), a.u_ssq};
 }
 
-// The launch's problems: one product, two (b), or two that are each cut in two along K (hi: fp32 outputs of the second halves, same pitch).
-inline EpiPair epi_pair_of(const GemmArgs &a, const GemmArgs *b, float *const *hi) {
+inline EpiPair epi_pair_of(const GemmArgs &a, const GemmArgs *b) {
     EpiPair epp{};
-    if (hi) {
-        const GemmArgs *prod[2] = {&a, b};
-        for (int i = 0; i < 2; ++i) {
-            EpiArgs lo = epi_of(*prod[i]), up = lo;
-            lo.K = up.K = prod[i]->K / 2;
-            up.k_off = lo.K;
-            up.C = hi[i]; up.addend = nullptr; up.col_bias = nullptr;
-            epp.p[2 * i] = lo; epp.p[2 * i + 1] = up;
-        }
-        epp.nprob = 4; epp.ksplit = 1;
-    } else {
-        epp.p[0] = epi_of(a);
-        epp.p[1] = b ? epi_of(*b) : epp.p[0];
-        epp.nprob = b ? 2 : 1;
-    }
+    epp.p[0] = epi_of(a);
+    epp.p[1] = b ? epi_of(*b) : epp.p[0];
+    epp.nprob = b ? 2 : 1;
     epp.n_fast = a.M > a.N ? 1 : 0;
     return epp;
 }
@@ -195,6 +180,86 @@ __device__ __forceinline__ void epi_add_store(const EpiArgs &ep, const EpiRow &e
     }
 }
 
+constexpr uint32_t STG_BYTES = 32 * 128;     // staging of one epilogue warp
+// Tensor maps of the outputs (boxes of 32 rows x 128 bytes), the addend and the next norm's input.
+struct IoMaps { CUtensorMap c[2], add, u; };
+
+// How one epilogue warp's 32 rows reach memory: 32 rows x 128 bytes at a time through 4 KB of shared memory and TMA.
+// Staging: 16-byte piece j of row `lane` sits at lane * 128 + ((j ^ (lane & 7)) << 4), the 128-byte swizzle of the maps.
+struct EpiOut {
+    uint8_t *stg;
+    int lane;
+    uint64_t *add_bar;
+    volatile int *abort_flag;
+    int *status;
+    uint32_t add_count;
+    __device__ __forceinline__ uint4 *piece(int j) const { return reinterpret_cast<uint4 *>(stg + lane * 128 + ((j ^ (lane & 7)) << 4)); }
+    __device__ __forceinline__ void free() const {             // the previous store has read the staging bytes
+        if (lane == 0) bulk_wait_read0();
+        __syncwarp();
+    }
+    __device__ __forceinline__ void store(const CUtensorMap &map, int x, int y) const {
+        fence_proxy_async();
+        __syncwarp();
+        if (lane == 0) { tma_store_2d(&map, stg, x, y); bulk_commit(); }
+    }
+    __device__ __forceinline__ void add_fetch(const CUtensorMap &map, int x, int y) const {      // 32 rows x 32 columns of the addend on their way into the staging bytes
+        free();
+        if (lane == 0) { mbar_expect_tx(add_bar, STG_BYTES); tma_load_2d(stg, &map, x, y, add_bar); }
+    }
+    __device__ __forceinline__ bool add_take(float *v) {       // v[0..32) += this lane's row
+        const bool r = __all_sync(0xffffffffu, mbar_wait(add_bar, add_count++ & 1u, abort_flag, status));
+        if (r) {
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const uint4 a4 = *piece(j);
+                v[4 * j] += __uint_as_float(a4.x); v[4 * j + 1] += __uint_as_float(a4.y); v[4 * j + 2] += __uint_as_float(a4.z); v[4 * j + 3] += __uint_as_float(a4.w);
+            }
+        }
+        __syncwarp();
+        return r;
+    }
+    // One 32-column group of results (columns n0 + c0 .., n0 a multiple of 64): to the output, and to the next norm's input where that is asked for.  ss: the row's sum of
+    // squares over the current 64 columns.
+    __device__ __forceinline__ void emit(const EpiArgs &pe, const CUtensorMap &map_c, const CUtensorMap &map_u, int n0, int c0, int row0, int row, bool row_ok, const float *v, float &ss) const {
+        const int col = n0 + c0;
+        if (pe.c_is_f32) {
+            free();
+#pragma unroll
+            for (int j = 0; j < 8; ++j) *piece(j) = make_uint4(__float_as_uint(v[4 * j]), __float_as_uint(v[4 * j + 1]), __float_as_uint(v[4 * j + 2]), __float_as_uint(v[4 * j + 3]));
+            store(map_c, col, row0);
+        } else {
+            if (!(c0 & 32)) free();
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                *piece((c0 & 32) / 8 + j) = make_uint4(pack_bf16(v[8 * j], v[8 * j + 1]), pack_bf16(v[8 * j + 2], v[8 * j + 3]),
+                                                      pack_bf16(v[8 * j + 4], v[8 * j + 5]), pack_bf16(v[8 * j + 6], v[8 * j + 7]));
+            if ((c0 & 32) || col + 32 >= pe.N) store(map_c, n0 + (c0 & ~63), row0);
+        }
+        if (pe.u) {                                            // 32 rows x 64 bytes, the 64-byte swizzle of its map
+            free();
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const bool in = col + 8 * j < pe.N;            // N is a multiple of 8
+                const uint4 w4 = in ? __ldg(reinterpret_cast<const uint4 *>(pe.u_w + col + 8 * j)) : make_uint4(0u, 0u, 0u, 0u);
+                const float *x = v + 8 * j;
+                *reinterpret_cast<uint4 *>(stg + lane * 64 + ((j ^ ((lane >> 1) & 3)) << 4)) =
+                    make_uint4(pack_bf16(x[0] * bf16_lo(w4.x), x[1] * bf16_hi(w4.x)), pack_bf16(x[2] * bf16_lo(w4.y), x[3] * bf16_hi(w4.y)),
+                               pack_bf16(x[4] * bf16_lo(w4.z), x[5] * bf16_hi(w4.z)), pack_bf16(x[6] * bf16_lo(w4.w), x[7] * bf16_hi(w4.w)));
+                if (in) {
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) ss = fmaf(x[e], x[e], ss);
+                }
+            }
+            store(map_u, col, row0);
+            if ((c0 & 32) || col + 32 >= pe.N) {
+                if (row_ok) pe.u_ssq[(int64_t)row * ((pe.N + 63) / 64) + col / 64] = ss;
+                ss = 0.f;
+            }
+        }
+    }
+};
+
 // 2-D bf16 tensor [rows, cols] with row pitch ld elements; box = [box_rows, 64 columns], 128-byte swizzle.
 inline bool make_map_2d(CUtensorMap *m, const void *base, int64_t rows, int64_t cols, int64_t ld, int box_rows) {
     const uint64_t dims[2] = {(uint64_t)cols, (uint64_t)rows};
@@ -215,9 +280,12 @@ inline bool make_map_u(CUtensorMap *m, const void *base, int64_t rows, int64_t c
 
 }  // namespace tc
 
-// gemm_pair.cu: the two-CTA kernel.  wide: 256 x 256 tiles, else 256 x 128; b, hi: see gemm_tcgen05.cu.  gemm_pair_sum_launch: both products into one output.
-cudaError_t gemm_pair_launch(bool wide, const GemmArgs &a, const GemmArgs *b, float *const *hi, cudaStream_t s);
+// gemm_pair.cu: the two-CTA kernel.  wide: 256 x 256 tiles, else 256 x 128; b: a second product of the same sizes.  gemm_pair_sum_launch: both products into one output.
+cudaError_t gemm_pair_launch(bool wide, const GemmArgs &a, const GemmArgs *b, cudaStream_t s);
 cudaError_t gemm_pair_sum_launch(const GemmArgs &a, const GemmArgs &b, cudaStream_t s);
+// gemm_cluster.cu: the same with each tile's K spread over a cluster, for few tiles.
+bool gemm_cluster_sum_pays(const GemmArgs &a);
+cudaError_t gemm_cluster_sum_launch(const GemmArgs &a, const GemmArgs &b, cudaStream_t s);
 // gemm_rows.cu: up to 128 rows; sum as in gemm_pair_sum_launch.
 cudaError_t gemm_rows_launch(const GemmArgs &a, const GemmArgs *b, bool sum, cudaStream_t s);
 // Output and addend can go through TMA: 16-byte aligned rows.

@@ -22,7 +22,6 @@ using namespace tc;
 constexpr int BM = 128, BK = 64;             // rows of A per CTA and row block, K step
 constexpr int NTHREADS = 64 + 8 * 32;
 constexpr int MAX_STAGES = 8;
-constexpr uint32_t STG_BYTES = 32 * 128;     // staging of one epilogue warp
 
 // 256 rows x BN columns per pair.  Stage of one CTA: 128 rows of A and BN / 2 rows of B.
 template <int BN> struct Tile {
@@ -36,9 +35,6 @@ struct __align__(8) Bars {
     uint32_t tmem_base;
     int abort;
 };
-
-// Tensor maps of the outputs (boxes of 32 rows x 128 bytes), the addend and the next norm's input.
-struct IoMaps { CUtensorMap c[4], add, u; };
 
 // How a tile leaves the kernel:
 //   DIRECT  every lane reads and writes its own row: for outputs whose rows do not start on 16-byte boundaries
@@ -105,10 +101,10 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_consta
             if (leader && ahead > 0) {
                 int tm, cb;
                 tile_at(pair, tm, cb);
-                const int prob = cb / tiles_n, prod = epp.ksplit ? prob >> 1 : prob, n0 = (cb - prob * tiles_n) * BN + (int)rank * (BN / 2);
+                const int prob = cb / tiles_n, n0 = (cb - prob * tiles_n) * BN + (int)rank * (BN / 2);
                 for (uint32_t s = 0; s < ahead; ++s) {
                     if (rank == 0) mbar_expect_tx(&bars->full[s], 2 * T::STAGE);
-                    tma_load_2d_pair(smem + s * T::STAGE + T::A_BYTES, prod ? &map_b1 : &map_b0, epp.p[prob].k_off + (int)s * BK, n0, cluster_addr(&bars->full[s], 0));
+                    tma_load_2d_pair(smem + s * T::STAGE + T::A_BYTES, prob ? &map_b1 : &map_b0, (int)s * BK, n0, cluster_addr(&bars->full[s], 0));
                 }
             }
             __syncwarp();
@@ -119,8 +115,8 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_consta
                 tile_at(tile, tm, cb);
                 const int prob0 = cb / tiles_n, m0 = tm * 2 * BM + (int)rank * BM, n0 = (cb - prob0 * tiles_n) * BN + (int)rank * (BN / 2);
                 for (int sub = 0; sub < NSUB && ok; ++sub) {
-                    const int prob = prob0 + sub, prod = epp.ksplit ? prob >> 1 : prob, k_off = epp.p[prob].k_off;
-                    const CUtensorMap *ma = prod ? &map_a1 : &map_a0, *mb = prod ? &map_b1 : &map_b0;
+                    const int prob = prob0 + sub;
+                    const CUtensorMap *ma = prob ? &map_a1 : &map_a0, *mb = prob ? &map_b1 : &map_b0;
                     for (int kb = 0; kb < kblocks; ++kb, ++it) {
                         const uint32_t s = it % STAGES, ph = (it / STAGES) & 1u;
                         if (!(ok = mbar_wait(&bars->empty[s], ph ^ 1u, abort_flag, status))) break;
@@ -128,8 +124,8 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_consta
                         const uint32_t full = cluster_addr(&bars->full[s], 0);
                         if (leader) {
                             if (rank == 0 && it >= ahead) mbar_expect_tx(&bars->full[s], 2 * T::STAGE);        // both CTAs' loads
-                            tma_load_2d_pair(sa, ma, k_off + kb * BK, m0, full);
-                            if (it >= ahead) tma_load_2d_pair(sb, mb, k_off + kb * BK, n0, full);
+                            tma_load_2d_pair(sa, ma, kb * BK, m0, full);
+                            if (it >= ahead) tma_load_2d_pair(sb, mb, kb * BK, n0, full);
                         }
                         __syncwarp();
                     }
@@ -189,35 +185,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_consta
             fence_after();
             return r;
         };
-        // staging: 16-byte piece j of row `lane` sits at lane * 128 + ((j ^ (lane & 7)) << 4), the 128-byte swizzle of the maps
-        uint8_t *stg = smem + STAGES * T::STAGE + (warp - 2) * STG_BYTES;
-        uint32_t add_count = 0;
-        auto piece = [&](int j) { return reinterpret_cast<uint4 *>(stg + lane * 128 + ((j ^ (lane & 7)) << 4)); };
-        auto stg_free = [&] {                                  // the previous store has read the staging bytes
-            if (lane == 0) bulk_wait_read0();
-            __syncwarp();
-        };
-        auto stg_store = [&](const CUtensorMap *map, int x, int y) {
-            fence_proxy_async();
-            __syncwarp();
-            if (lane == 0) { tma_store_2d(map, stg, x, y); bulk_commit(); }
-        };
-        auto add_fetch = [&](int x, int y) {                   // 32 rows x 32 columns of the addend on their way into the staging bytes
-            stg_free();
-            if (lane == 0) { mbar_expect_tx(&bars->add_full[warp - 2], STG_BYTES); tma_load_2d(stg, &io.add, x, y, &bars->add_full[warp - 2]); }
-        };
-        auto add_take = [&](float *v) -> bool {                // v[0..32) += this lane's row
-            const bool r = __all_sync(0xffffffffu, mbar_wait(&bars->add_full[warp - 2], add_count++ & 1u, abort_flag, status));
-            if (r) {
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    const uint4 a4 = *piece(j);
-                    v[4 * j] += __uint_as_float(a4.x); v[4 * j + 1] += __uint_as_float(a4.y); v[4 * j + 2] += __uint_as_float(a4.z); v[4 * j + 3] += __uint_as_float(a4.w);
-                }
-            }
-            __syncwarp();
-            return r;
-        };
+        EpiOut out{smem + STAGES * T::STAGE + (warp - 2) * STG_BYTES, lane, &bars->add_full[warp - 2], abort_flag, status, 0};
         for (int tile = pair; tile < num_tiles && ok; tile += npairs, tcount += NSUB) {
             int tm, cb;
             tile_at(tile, tm, cb);
@@ -229,46 +197,9 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_consta
             const float sc = row_ok ? epi_row_scale(pe, row) : 1.f;
             const EpiRow er(pe, row_ok ? row : 0);
             const bool add = MODE != DIRECT && pe.addend && live;
-            if (MODE == TMA && add) add_fetch(n0, row0);       // the first columns' addend arrives while the products run
-            // one 32-column group of results: to the output, and to the next norm's input where that is asked for
+            if (MODE == TMA && add) out.add_fetch(io.add, n0, row0);       // the first columns' addend arrives while the products run
             float ss = 0.f;
-            auto emit = [&](int c0, const float *v) {
-                const int col = n0 + c0;
-                if (pe.c_is_f32) {
-                    stg_free();
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) *piece(j) = make_uint4(__float_as_uint(v[4 * j]), __float_as_uint(v[4 * j + 1]), __float_as_uint(v[4 * j + 2]), __float_as_uint(v[4 * j + 3]));
-                    stg_store(&io.c[prob], col, row0);
-                } else {
-                    if (!(c0 & 32)) stg_free();
-#pragma unroll
-                    for (int j = 0; j < 4; ++j)
-                        *piece((c0 & 32) / 8 + j) = make_uint4(pack_bf16(v[8 * j], v[8 * j + 1]), pack_bf16(v[8 * j + 2], v[8 * j + 3]),
-                                                              pack_bf16(v[8 * j + 4], v[8 * j + 5]), pack_bf16(v[8 * j + 6], v[8 * j + 7]));
-                    if ((c0 & 32) || col + 32 >= pe.N) stg_store(&io.c[prob], n0 + (c0 & ~63), row0);
-                }
-                if (pe.u) {                                    // 32 rows x 64 bytes, the 64-byte swizzle of its map
-                    stg_free();
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const bool in = col + 8 * j < pe.N;    // N is a multiple of 8
-                        const uint4 w4 = in ? __ldg(reinterpret_cast<const uint4 *>(pe.u_w + col + 8 * j)) : make_uint4(0u, 0u, 0u, 0u);
-                        const float *x = v + 8 * j;
-                        *reinterpret_cast<uint4 *>(stg + lane * 64 + ((j ^ ((lane >> 1) & 3)) << 4)) =
-                            make_uint4(pack_bf16(x[0] * bf16_lo(w4.x), x[1] * bf16_hi(w4.x)), pack_bf16(x[2] * bf16_lo(w4.y), x[3] * bf16_hi(w4.y)),
-                                       pack_bf16(x[4] * bf16_lo(w4.z), x[5] * bf16_hi(w4.z)), pack_bf16(x[6] * bf16_lo(w4.w), x[7] * bf16_hi(w4.w)));
-                        if (in) {
-#pragma unroll
-                            for (int e = 0; e < 8; ++e) ss = fmaf(x[e], x[e], ss);
-                        }
-                    }
-                    stg_store(&io.u, col, row0);
-                    if ((c0 & 32) || col + 32 >= pe.N) {
-                        if (row_ok) pe.u_ssq[(int64_t)row * ((pe.N + 63) / 64) + col / 64] = ss;
-                        ss = 0.f;
-                    }
-                }
-            };
+            auto emit = [&](int c0, const float *v) { out.emit(pe, io.c[prob], io.u, n0, c0, row0, row, row_ok, v, ss); };
             if constexpr (MODE == SUM) {
                 const EpiArgs &p0 = epp.p[0];
                 const float sc0 = row_ok ? epi_row_scale(p0, row) : 1.f;
@@ -277,7 +208,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_consta
 #pragma unroll
                 for (int c0 = 0; c0 < COLS; c0 += 32) {
                     const bool some = n0 + c0 < pe.N;
-                    if (add && some) add_fetch(n0 + c0, row0);
+                    if (add && some) out.add_fetch(io.add, n0 + c0, row0);
                     uint32_t r[32];
                     tmem_ld_x32(tlane + (tcount & 1u) * BN + c0, r);
                     tmem_wait_ld();
@@ -285,7 +216,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_consta
 #pragma unroll
                     for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]) * sc0;
                     if (some) epi_pre<false>(p0, er, n0 + c0, v);
-                    if (add && some && ok) ok = add_take(v);
+                    if (add && some && ok) ok = out.add_take(v);
 #pragma unroll
                     for (int j = 0; j < 32; ++j) held[c0 + j] = v[j];
                 }
@@ -333,8 +264,8 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_consta
                         epi_add_store(pe, er, row, col, v);
                     } else {
                         if (add) {
-                            if (c0 > 0) add_fetch(col, row0);
-                            if (!(ok = add_take(v))) break;
+                            if (c0 > 0) out.add_fetch(io.add, col, row0);
+                            if (!(ok = out.add_take(v))) break;
                         }
                         emit(c0, v);
                     }
@@ -357,7 +288,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_consta
 }
 
 template <int BN, int MODE>
-cudaError_t launch(const GemmArgs &a, const GemmArgs *b, float *const *hi, cudaStream_t s) {
+cudaError_t launch(const GemmArgs &a, const GemmArgs *b, cudaStream_t s) {
     using T = Tile<BN>;
     CUtensorMap ma[2], mb[2];
     if (!make_map_2d(&ma[0], a.A, a.M, a.K, a.lda, BM) || !make_map_2d(&mb[0], a.B, a.N, a.K, a.ldb, BN / 2)) return cudaErrorInvalidValue;
@@ -369,7 +300,7 @@ cudaError_t launch(const GemmArgs &a, const GemmArgs *b, float *const *hi, cudaS
     if (e != cudaSuccess) return e;
     int *status = device_status_ptr();
     if (!status) return cudaErrorUnknown;
-    const EpiPair epp = epi_pair_of(a, b, hi);
+    const EpiPair epp = epi_pair_of(a, b);
     IoMaps io;
     memset(&io, 0, sizeof(io));
     if (MODE != DIRECT) {
@@ -390,11 +321,11 @@ bool tma_io(const GemmArgs &a, const GemmArgs *b) { return gemm_pair_tma_io(a) &
 
 }  // namespace
 
-cudaError_t gemm_pair_launch(bool wide, const GemmArgs &a, const GemmArgs *b, float *const *hi, cudaStream_t s) {
-    if (tma_io(a, b)) return wide ? launch<256, TMA>(a, b, hi, s) : launch<128, TMA>(a, b, hi, s);
-    return wide ? launch<256, DIRECT>(a, b, hi, s) : launch<128, DIRECT>(a, b, hi, s);
+cudaError_t gemm_pair_launch(bool wide, const GemmArgs &a, const GemmArgs *b, cudaStream_t s) {
+    if (tma_io(a, b)) return wide ? launch<256, TMA>(a, b, s) : launch<128, TMA>(a, b, s);
+    return wide ? launch<256, DIRECT>(a, b, s) : launch<128, DIRECT>(a, b, s);
 }
 
-cudaError_t gemm_pair_sum_launch(const GemmArgs &a, const GemmArgs &b, cudaStream_t s) { return launch<256, SUM>(a, &b, nullptr, s); }
+cudaError_t gemm_pair_sum_launch(const GemmArgs &a, const GemmArgs &b, cudaStream_t s) { return launch<256, SUM>(a, &b, s); }
 
 }  // namespace dm

@@ -1,7 +1,8 @@
 // bf16 x bf16 -> fp32 GEMM on the 5th-generation tensor cores, for the dense projections:
 //     C[m, n] = row_scale[m] * sum_k A[m, k] * B[n, k] + addend[m, n]
-// This file chooses the kernel and its tile: gemm_rows.cu for up to 128 rows (reading the weights is all such a product does), gemm_pair.cu for more.
-// Both: operands staged by TMA with the 128-byte swizzle, accumulators in TMEM, mbarrier pipelines.
+// This file chooses the kernel and its tile: gemm_rows.cu for up to 128 rows (reading the weights is all such a product does), gemm_pair.cu for more, and gemm_cluster.cu for
+// a sum of two products whose tiles are few.
+// All: operands staged by TMA with the 128-byte swizzle, accumulators in TMEM, mbarrier pipelines.
 #include "gemm_epi.cuh"
 
 namespace dm {
@@ -9,7 +10,7 @@ namespace {
 
 using namespace tc;
 
-constexpr int BM = 128, BK = 64;
+constexpr int BM = 128;
 
 int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }
 
@@ -21,9 +22,9 @@ bool pair_wide_tile(const GemmArgs &a, int nprob) {
     return a.N > 128 && 10 * r256 <= 7 * r128;
 }
 
-cudaError_t dispatch(const GemmArgs &a, const GemmArgs *b, float *const *hi, cudaStream_t s) {
+cudaError_t dispatch(const GemmArgs &a, const GemmArgs *b, cudaStream_t s) {
     if (a.M <= BM) return gemm_rows_launch(a, b, false, s);
-    return gemm_pair_launch(pair_wide_tile(a, hi ? 4 : b ? 2 : 1), a, b, hi, s);
+    return gemm_pair_launch(pair_wide_tile(a, b ? 2 : 1), a, b, s);
 }
 
 }  // namespace
@@ -44,7 +45,7 @@ bool gemm_tcgen05_supports(const GemmArgs &a) {
 
 cudaError_t gemm_tcgen05(const GemmArgs &a, cudaStream_t s) {
     if (!gemm_tcgen05_supports(a)) return cudaErrorNotSupported;
-    return dispatch(a, nullptr, nullptr, s);
+    return dispatch(a, nullptr, s);
 }
 
 bool gemm_tcgen05_pair_supports(const GemmArgs &a, const GemmArgs &b) {
@@ -54,7 +55,7 @@ bool gemm_tcgen05_pair_supports(const GemmArgs &a, const GemmArgs &b) {
 
 cudaError_t gemm_tcgen05_pair(const GemmArgs &a, const GemmArgs &b, cudaStream_t s) {
     if (!gemm_tcgen05_pair_supports(a, b)) return cudaErrorNotSupported;
-    return dispatch(a, &b, nullptr, s);
+    return dispatch(a, &b, s);
 }
 
 bool gemm_tcgen05_sum_supports(const GemmArgs &a, const GemmArgs &b) {
@@ -63,22 +64,8 @@ bool gemm_tcgen05_sum_supports(const GemmArgs &a, const GemmArgs &b) {
 
 cudaError_t gemm_tcgen05_sum(const GemmArgs &a, const GemmArgs &b, cudaStream_t s) {
     if (!gemm_tcgen05_sum_supports(a, b)) return cudaErrorNotSupported;
-    return a.M <= BM ? gemm_rows_launch(a, &b, true, s) : gemm_pair_sum_launch(a, b, s);
-}
-
-// Few rows and a long K (the out_proj pair of block decoding): whole products fill less than half of the SMs.  Halving K instead doubles
-// the number of tiles of the same shape.
-bool gemm_tcgen05_pair_splitk_pays(const GemmArgs &a, const GemmArgs &b) {
-    if (!gemm_tcgen05_pair_supports(a, b) || a.M <= BM || a.c_dtype != DM_F32 || a.K % (2 * BK) || a.gelu || b.gelu || a.silu_cols || b.silu_cols) return false;
-    const int64_t tiles = ceil_div(a.M, BM) * ceil_div(a.N, 256) * 2;
-    return a.N > 128 && 2 * tiles <= sm_count();
-}
-
-cudaError_t gemm_tcgen05_pair_splitk(const GemmArgs &a, const GemmArgs &b, float *a_hi, float *b_hi, cudaStream_t s) {
-    if (!gemm_tcgen05_pair_splitk_pays(a, b) || !a_hi || !b_hi || ((reinterpret_cast<uintptr_t>(a_hi) | reinterpret_cast<uintptr_t>(b_hi)) & 15u))
-        return cudaErrorNotSupported;
-    float *const hi[2] = {a_hi, b_hi};
-    return dispatch(a, &b, hi, s);
+    if (a.M <= BM) return gemm_rows_launch(a, &b, true, s);
+    return gemm_cluster_sum_pays(b) ? gemm_cluster_sum_launch(a, b, s) : gemm_pair_sum_launch(a, b, s);
 }
 
 }  // namespace dm

@@ -205,10 +205,10 @@ __device__ __forceinline__ void tma_load_2d_pair(void *smem_dst, const CUtensorM
         "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
         ::"r"(smem_u32(smem_dst)), "l"(map), "r"(x), "r"(y), "r"(cluster_bar) : "memory");
 }
-// Arrives on the barrier at this offset in both CTAs of the pair when the MMAs issued so far have completed.
-__device__ __forceinline__ void umma_commit_2cta(uint64_t *bar) {
+// Arrives on the barrier at this offset in both CTAs of the pair when the MMAs issued so far have completed (lead: the pair's first CTA in its cluster).
+__device__ __forceinline__ void umma_commit_2cta(uint64_t *bar, uint32_t lead = 0) {
     asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
-                 ::"r"(smem_u32(bar)), "h"((uint16_t)3) : "memory");
+                 ::"r"(smem_u32(bar)), "h"((uint16_t)(3u << lead)) : "memory");
 }
 __device__ __forceinline__ void tmem_alloc_2cta(uint32_t *smem_slot, uint32_t cols) {   // one whole warp of each CTA
     asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(smem_slot)), "r"(cols) : "memory");

@@ -62,6 +62,13 @@ def test_denoise_step_summed_out_proj(G, d, H, B, L, d_ff):
     assert G.rel_l2(got, want) <= 1e-2, G.rel_l2(got, want)
 
 
+@pytest.mark.parametrize("d,H,B,L,d_ff", [(288, 9, 1, 129, 0), (192, 6, 1, 256, 384), (1024, 32, 2, 1000, 0), (320, 10, 17, 256, 0)])
+def test_denoise_step_out_proj_over_clusters(G, d, H, B, L, d_ff):
+    """Few 256 x 256 tiles: the summed out_proj cuts a tile over 4 or 2 pairs of CTAs.  An odd number of k-blocks and a last column tile of 32 columns; columns that
+    end inside the tile's shares, with a gate; 32 tiles (two pairs each); 34 tiles (more than one round of clusters: the kernel of long inputs)."""
+    test_denoise_step_summed_out_proj(G, d, H, B, L, d_ff)
+
+
 @pytest.mark.parametrize("dtype", [I.F32, I.BF16])
 def test_denoise_step_block_mode(G, dtype):
     d, N, H, V, layers = 64, 16, 4, 120, 2
