@@ -20,7 +20,8 @@ namespace {
 
 using namespace ssd;
 
-constexpr int HG_MAX = 7;              // heads per CTA
+// heads per CTA at most (their decays are kept)
+template <bool COMMIT> constexpr int HG_MAX = COMMIT ? 16 : 7;
 constexpr int KG = N / 16;             // 16-wide groups of states
 constexpr int XR = QB + 4;             // rows of a raw tile: three of history, one unused
 constexpr int SLD = QB + 4;            // row pitch (fp32) of S
@@ -28,12 +29,15 @@ constexpr int WTL = QB + 8;            // row pitch (bf16) of W
 // CTAs per SM
 template <int PP, bool COMMIT> constexpr int RES = PP == 64 ? (COMMIT ? 2 : 3) : (COMMIT ? 3 : 4);
 
+// Heads per CTA and CTAs per batch row of either direction
+struct StepSplit { int hg[2], groups[2]; };
+
 template <int PP, bool COMMIT> struct StepSmem {
     static constexpr int XLD = PP + 8;             // row pitch (bf16) of x' and w o x'
     static constexpr int XRAW = XR * PP * 2, NRAW = 2 * N / PP;            // a raw tile of PP channels; tiles of B and C
     static constexpr int STATE = KG * PP * 16 * 4;                         // [16-state group][p][16]; the raw B, C tiles before that
     static constexpr int st = 0, xr = st + (STATE > NRAW * XRAW ? STATE : NRAW * XRAW), ct = xr + XRAW, bt = ct + QB * NLD * 2, ss = bt + QB * NLD * 2, xt = ss + QB * SLD * 4,
-                         wt = xt + QB * XLD * 2, ys = wt + QB * WTL * 2, lam = ys + QB * PP * 4, bars = lam + HG_MAX * 2 * QB * 4, wxt = bars + 64, total = wxt + (COMMIT ? QB * XLD * 2 : 0);
+                         wt = xt + QB * XLD * 2, ys = wt + QB * WTL * 2, lam = ys + QB * PP * 4, bars = lam + HG_MAX<COMMIT> * 2 * QB * 4, wxt = bars + 64, total = wxt + (COMMIT ? QB * XLD * 2 : 0);
     static_assert(xr % 128 == 0 && XRAW % 128 == 0, "TMA tiles");
     static_assert(ct % 16 == 0 && bt % 16 == 0 && ss % 16 == 0 && xt % 16 == 0 && wt % 16 == 0 && ys % 16 == 0 && lam % 16 == 0 && wxt % 16 == 0, "16-byte tiles");
 };
@@ -44,8 +48,7 @@ __device__ __forceinline__ void prefetch_3d(const CUtensorMap *map, int x, int y
 
 template <int PP, bool COMMIT>
 __global__ void __launch_bounds__(4 * PP, RES<PP, COMMIT>)
-ssd_step_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_s, const __grid_constant__ SsdArgs a, const int ndir, const int dir0,
-                const int hg, const int groups, const int round, int *status) {
+ssd_step_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_s, const __grid_constant__ SsdArgs a, const StepSplit sp, int *status) {
     using M = StepSmem<PP, COMMIT>;
     constexpr int NT = 4 * PP, U8 = PP / 8, MT = PP / 16, XLD = M::XLD, CP2 = PP / 2;
     extern __shared__ __align__(128) uint8_t sm[];
@@ -63,10 +66,9 @@ ssd_step_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
     volatile int *abort_flag = reinterpret_cast<volatile int *>(bar_bc + 3);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, gr = lane >> 2, qc = lane & 3;
-    // CTA -> (group of heads, batch row, direction).  A left-to-right CTA also reads (and with COMMIT writes) states, so the directions alternate from CTA to CTA and,
-    // `round` (SMs) CTAs later, start with the other one: the CTAs of an SM are then of both kinds
-    const int i0 = blockIdx.x, dsel = ndir == 2 ? (i0 ^ (i0 / round)) & 1 : 0, rest = ndir == 2 ? i0 >> 1 : i0;
-    const int h0 = rest % groups * hg, nh = min(hg, a.H - h0), b = rest / groups, dir = dir0 + dsel;
+    // CTA -> (batch row, direction, group of heads)
+    const int per = sp.groups[0] + sp.groups[1], b = blockIdx.x / per, j = blockIdx.x - b * per, dir = j >= sp.groups[0];
+    const int hg = dir ? sp.hg[1] : sp.hg[0], h0 = (dir ? j - sp.groups[0] : j) * hg, nh = min(hg, a.H - h0);
     const bool rev = dir == 1;
     const int L = a.L, k = a.k;
     const int64_t seq = (int64_t)dir * a.B + b;
@@ -166,6 +168,7 @@ ssd_step_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
         if (have_state)
             for (int i = 0; i < nh; ++i) prefetch_3d(&map_s, 0, (b * a.H + h0 + i) * PP, 0);
     }
+    const float dtb0 = warp < nh ? w.dt_bias[h0 + warp] : 0.f, al0 = warp < nh ? w.A_log[h0 + warp] : 0.f;      // (its first head's)
     pdl_wait();
     pdl_trigger();
     if (tid == 0) {
@@ -178,8 +181,8 @@ ssd_step_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
     if (warp < nh) {
         for (int hd = warp; hd < nh; hd += NT / 32) {
             const int h = h0 + hd, r = rev ? QB - 1 - lane : lane;
-            const float d = r < L ? prep_delta(__bfloat162float(zx[(int64_t)r * a.d_in_proj + a.d_inner + a.conv_ch + h]), w.dt_bias[h]) : 0.f;
-            float cum = d * (-expf(w.A_log[h]) * 1.4426950408889634f);
+            const float d = r < L ? prep_delta(__bfloat162float(zx[(int64_t)r * a.d_in_proj + a.d_inner + a.conv_ch + h]), hd == warp ? dtb0 : w.dt_bias[h]) : 0.f;
+            float cum = d * (-expf(hd == warp ? al0 : w.A_log[h]) * 1.4426950408889634f);
 #pragma unroll
             for (int off = 1; off < 32; off <<= 1) {
                 const float up = __shfl_up_sync(0xffffffffu, cum, off);
@@ -389,14 +392,29 @@ cudaError_t launch(const SsdArgs &a, int ndir, int dir0, cudaStream_t s) {
     }
     cudaError_t e = cudaFuncSetAttribute(ssd_step_kernel<PP, COMMIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, M::total);
     if (e != cudaSuccess) return e;
-    // as many CTAs as are resident at once, so that what the heads share is computed as seldom as one round allows
-    const int seqs = ndir * a.B, slots = sm_count() * RES<PP, COMMIT>;
-    int groups = slots / seqs;
-    groups = groups < 1 ? 1 : groups > a.H ? a.H : groups;
-    int hg = (a.H + groups - 1) / groups;
-    hg = hg > HG_MAX ? HG_MAX : hg;
-    groups = (a.H + hg - 1) / hg;
-    return launch_chain(ssd_step_kernel<PP, COMMIT>, dim3(groups * seqs), 4 * PP, M::total, s, 0, mx, ms, a, ndir, dir0, hg, groups, sm_count() & ~1, status);
+    // As many CTAs as are resident at once, so that what the heads share is computed as seldom as one round allows, and shared out between the directions by what a head costs:
+    // a left-to-right one reads its state, and with COMMIT writes it (16 sequences of 64 heads: 4.0 us against 2.8, and 4.2 against 1.9; with equal shares the SMs that happened to
+    // get left-to-right CTAs only finished at 27 and 43 us, the others at 19 and 18;
+    // one layer with the state committed 103 -> 96 us, 24 layers 2191 -> 2118 us).
+    StepSplit sp{};
+    const int slots = sm_count() * RES<PP, COMMIT> / a.B, cap = HG_MAX<COMMIT>;
+    const int cost[2] = {!a.ssm_in && !COMMIT ? 10 : COMMIT ? 22 : 14, 10};
+    auto groups_of = [&](int hg) { return (a.H + hg - 1) / hg; };
+    if (ndir == 1) {
+        const int most = slots < 1 ? 1 : slots > a.H ? a.H : slots, hg = groups_of(most);
+        sp.hg[dir0] = hg > cap ? cap : hg;
+    } else {
+        int best = 0;
+        for (int f = 1; f <= cap; ++f) {                 // heads per left-to-right CTA
+            const int left = slots - groups_of(f);
+            if (left < 1) continue;
+            const int r = groups_of(left > a.H ? a.H : left), t = f * cost[0] > r * cost[1] ? f * cost[0] : r * cost[1];
+            if (r <= cap && (!best || t < best)) { best = t; sp.hg[0] = f; sp.hg[1] = r; }
+        }
+        if (!best) { sp.hg[1] = cap; sp.hg[0] = cap * cost[1] / cost[0]; }      // more than one round
+    }
+    for (int d = 0; d < 2; ++d) sp.groups[d] = sp.hg[d] ? groups_of(sp.hg[d]) : 0;
+    return launch_chain(ssd_step_kernel<PP, COMMIT>, dim3((sp.groups[0] + sp.groups[1]) * a.B), 4 * PP, M::total, s, 0, mx, ms, a, sp, status);
 }
 
 }  // namespace
