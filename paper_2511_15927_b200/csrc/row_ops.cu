@@ -42,7 +42,18 @@ __global__ void embed_kernel(const T *__restrict__ embed, const int32_t *__restr
     const int64_t t = blockIdx.x;
     int id = tokens[t];
     id = id < 0 ? 0 : (id >= vocab ? vocab - 1 : id);      // ids are validated on the host side of the tests; clamp keeps reads in bounds
-    for (int c = threadIdx.x; c < d; c += blockDim.x) r[t * d + c] = ldf(embed + (int64_t)id * d + c);
+    const T *e = embed + (int64_t)id * d;
+    constexpr int PER = 16 / (int)sizeof(T);                // channels per 16-byte load, where the rows allow it
+    if (d % PER == 0 && (reinterpret_cast<uintptr_t>(embed) & 15u) == 0) {
+        for (int c = threadIdx.x * PER; c < d; c += blockDim.x * PER) {
+            const uint4 v = __ldg(reinterpret_cast<const uint4 *>(e + c));
+            const T *x = reinterpret_cast<const T *>(&v);
+#pragma unroll
+            for (int i = 0; i < PER; i += 4) *reinterpret_cast<float4 *>(r + t * d + c + i) = make_float4(ldf(x + i), ldf(x + i + 1), ldf(x + i + 2), ldf(x + i + 3));
+        }
+    } else {
+        for (int c = threadIdx.x; c < d; c += blockDim.x) r[t * d + c] = ldf(e + c);
+    }
 }
 
 // The two row kernels below keep the token's channels in registers between the statistics and the output (one read
@@ -54,6 +65,15 @@ template <> __device__ __forceinline__ void st4<float>(float *p, float a, float 
 template <> __device__ __forceinline__ void st4<__nv_bfloat16>(__nv_bfloat16 *p, float a, float b, float c, float d) {
     __nv_bfloat162 lo = __floats2bfloat162_rn(a, b), hi = __floats2bfloat162_rn(c, d);
     *reinterpret_cast<uint2 *>(p) = make_uint2(*reinterpret_cast<uint32_t *>(&lo), *reinterpret_cast<uint32_t *>(&hi));
+}
+
+// eight consecutive channels, the first a multiple of 8
+template <typename T> __device__ __forceinline__ void st8(T *p, float a, float b, float c, float d, float e, float f, float g, float h);
+template <> __device__ __forceinline__ void st8<float>(float *p, float a, float b, float c, float d, float e, float f, float g, float h) { st4(p, a, b, c, d); st4(p + 4, e, f, g, h); }
+template <> __device__ __forceinline__ void st8<__nv_bfloat16>(__nv_bfloat16 *p, float a, float b, float c, float d, float e, float f, float g, float h) {
+    const __nv_bfloat162 v[4] = {__floats2bfloat162_rn(a, b), __floats2bfloat162_rn(c, d), __floats2bfloat162_rn(e, f), __floats2bfloat162_rn(g, h)};
+    const uint32_t *w = reinterpret_cast<const uint32_t *>(v);
+    *reinterpret_cast<uint4 *>(p) = make_uint4(w[0], w[1], w[2], w[3]);
 }
 
 template <typename T>
@@ -142,19 +162,104 @@ adaln_kernel(const float *__restrict__ r, const float *__restrict__ gamma, const
     }
 }
 
-// mod[b, j] = bias[j] + sum_c w[j, c] tau[b, c]: the modulation vectors of one layer (App. A.1: (gamma, beta) = W_cond tau).
-// One warp per output element.
+// The same with a warp per row, its channels in the lanes' registers (8 (lane + 32 k) .. +7, k < K8): every load of a row is in flight at once and the statistics need no
+// block barrier.  Bound by the stream of rows (4 bytes in, 2 out per channel).  8192 rows of 1920: 34 us with a block per row, 24 us.  For d up to 2048 in whole groups of 8; the
+// kernel above takes the rest (a wider row no longer fits a warp's registers).
+constexpr int AW_K8 = 8, AW_ROWS = 4;
 template <typename T>
-__global__ void modulation_kernel(const float *__restrict__ tau, const T *__restrict__ w, const float *__restrict__ bias,
-                                  float *__restrict__ mod, int n_out, int d_c) {
+__global__ void __launch_bounds__(32 * AW_ROWS)
+adaln_warp_kernel(const float *__restrict__ r, const float *__restrict__ gamma, const float *__restrict__ beta, int64_t ld_mod, T *__restrict__ u, int T_rows, int L, int d, float eps) {
     pdl_wait();
     pdl_trigger();
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31, b = blockIdx.y;
-    if (warp >= n_out) return;
+    const int lane = threadIdx.x & 31;
+    const int64_t t = (int64_t)blockIdx.x * AW_ROWS + (threadIdx.x >> 5);
+    if (t >= T_rows) return;
+    const float *row = r + t * d, *g = gamma + t / L * ld_mod, *be = beta + t / L * ld_mod;
+    float4 v[2 * AW_K8];
     float s = 0.f;
-    for (int c = lane; c < d_c; c += 32) s = fmaf(ldf(w + (int64_t)warp * d_c + c), tau[(int64_t)b * d_c + c], s);
+#pragma unroll
+    for (int k = 0; k < AW_K8; ++k) {
+        const int c = 8 * (lane + 32 * k);
+        v[2 * k] = v[2 * k + 1] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (c < d) { v[2 * k] = *reinterpret_cast<const float4 *>(row + c); v[2 * k + 1] = *reinterpret_cast<const float4 *>(row + c + 4); }
+    }
+#pragma unroll
+    for (int k = 0; k < 2 * AW_K8; ++k) s += (v[k].x + v[k].y) + (v[k].z + v[k].w);
     for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-    if (lane == 0) mod[(int64_t)b * n_out + warp] = s + (bias ? bias[warp] : 0.f);
+    const float mu = s / (float)d;
+    float q = 0.f;
+#pragma unroll
+    for (int k = 0; k < AW_K8; ++k) {
+        if (8 * (lane + 32 * k) >= d) break;
+#pragma unroll
+        for (int e = 2 * k; e < 2 * k + 2; ++e) {
+            v[e].x -= mu; v[e].y -= mu; v[e].z -= mu; v[e].w -= mu;
+            q = fmaf(v[e].x, v[e].x, q); q = fmaf(v[e].y, v[e].y, q); q = fmaf(v[e].z, v[e].z, q); q = fmaf(v[e].w, v[e].w, q);
+        }
+    }
+    for (int off = 16; off > 0; off >>= 1) q += __shfl_xor_sync(0xffffffffu, q, off);
+    const float rs = rsqrtf(q / (float)d + eps);
+#pragma unroll
+    for (int k = 0; k < AW_K8; ++k) {
+        const int c = 8 * (lane + 32 * k);
+        if (c >= d) break;
+        const float4 g0 = __ldg(reinterpret_cast<const float4 *>(g + c)), g1 = __ldg(reinterpret_cast<const float4 *>(g + c + 4));
+        const float4 b0 = __ldg(reinterpret_cast<const float4 *>(be + c)), b1 = __ldg(reinterpret_cast<const float4 *>(be + c + 4));
+        const float4 x = v[2 * k], y = v[2 * k + 1];
+        st8(u + t * d + c, fmaf(g0.x, x.x * rs, b0.x), fmaf(g0.y, x.y * rs, b0.y), fmaf(g0.z, x.z * rs, b0.z), fmaf(g0.w, x.w * rs, b0.w),
+            fmaf(g1.x, y.x * rs, b1.x), fmaf(g1.y, y.y * rs, b1.y), fmaf(g1.z, y.z * rs, b1.z), fmaf(g1.w, y.w * rs, b1.w));
+    }
+}
+
+// mod[b, j] = bias[j] + sum_c w[j, c] tau[b, c]: the modulation vectors of one layer (App. A.1: (gamma, beta) = W_cond tau).
+// A warp computes MOD_R consecutive outputs of MOD_B sequences: a weight is read once for all of them, the first MOD_C columns before the kernel before this one has
+// finished.  Bound by latency: 8 sequences, 11520 outputs of 128 columns (3 MB of weights): 8 us; with a warp per output element, whose lanes did 4
+// products between five shuffles, 15 us.
+constexpr int MOD_R = 4, MOD_B = 8, MOD_C = 128;
+template <typename T>
+__global__ void __launch_bounds__(256)
+modulation_kernel(const float *__restrict__ tau, const T *__restrict__ w, const float *__restrict__ bias, float *__restrict__ mod, int n_out, int d_c, int B) {
+    const int j0 = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * MOD_R, lane = threadIdx.x & 31, b0 = blockIdx.y * MOD_B;
+    float wv[MOD_C / 32][MOD_R];
+#pragma unroll
+    for (int i = 0; i < MOD_C / 32; ++i)
+#pragma unroll
+        for (int r = 0; r < MOD_R; ++r) wv[i][r] = j0 + r < n_out && 32 * i + lane < d_c ? ldf(w + (int64_t)(j0 + r) * d_c + 32 * i + lane) : 0.f;
+    pdl_wait();
+    pdl_trigger();
+    if (j0 >= n_out) return;
+    float acc[MOD_R * MOD_B];
+#pragma unroll
+    for (int i = 0; i < MOD_R * MOD_B; ++i) acc[i] = 0.f;
+    auto column = [&](int c, const float (&x)[MOD_R]) {
+#pragma unroll
+        for (int b = 0; b < MOD_B; ++b) {
+            const float t = b0 + b < B && c < d_c ? __ldg(tau + (int64_t)(b0 + b) * d_c + c) : 0.f;
+#pragma unroll
+            for (int r = 0; r < MOD_R; ++r) acc[r * MOD_B + b] = fmaf(x[r], t, acc[r * MOD_B + b]);
+        }
+    };
+#pragma unroll
+    for (int i = 0; i < MOD_C / 32; ++i) column(32 * i + lane, wv[i]);
+    for (int c = MOD_C + lane; c < d_c + lane; c += 32) {          // (every lane takes every step: the sums below are the warp's)
+        float x[MOD_R];
+#pragma unroll
+        for (int r = 0; r < MOD_R; ++r) x[r] = j0 + r < n_out && c < d_c ? ldf(w + (int64_t)(j0 + r) * d_c + c) : 0.f;
+        column(c, x);
+    }
+    // sums over the lanes, halving the number of values a lane holds at each step: lane l ends with value l
+    static_assert(MOD_R * MOD_B == 32, "one value per lane");
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        const bool up = lane & off;
+#pragma unroll
+        for (int i = 0; i < off; ++i) {
+            const float other = __shfl_xor_sync(0xffffffffu, up ? acc[i] : acc[i + off], off);
+            acc[i] = (up ? acc[i + off] : acc[i]) + other;
+        }
+    }
+    const int j = j0 + lane / MOD_B, b = b0 + lane % MOD_B;
+    if (j < n_out && b < B) mod[(int64_t)b * n_out + j] = acc[0] + (bias ? bias[j] : 0.f);
 }
 
 template <typename T>
@@ -271,15 +376,21 @@ cudaError_t rmsnorm_rows(const float *r, const void *w, void *u, int dtype, int 
 
 cudaError_t adaln_rows(const float *r, const float *gamma, const float *beta, int64_t ld_mod, void *u, int dtype, int T, int L, int d,
                        float eps, cudaStream_t s) {
+    const bool al = !((reinterpret_cast<uintptr_t>(r) | reinterpret_cast<uintptr_t>(gamma) | reinterpret_cast<uintptr_t>(beta) | reinterpret_cast<uintptr_t>(u)) & 15u);
+    if (d % 8 == 0 && ld_mod % 4 == 0 && d <= 8 * 32 * AW_K8 && al) {
+        const int grid = (T + AW_ROWS - 1) / AW_ROWS;
+        if (dtype == DM_BF16) return launch_chain(adaln_warp_kernel<__nv_bfloat16>, grid, 32 * AW_ROWS, 0, s, 0, r, gamma, beta, ld_mod, static_cast<__nv_bfloat16 *>(u), T, L, d, eps);
+        return launch_chain(adaln_warp_kernel<float>, grid, 32 * AW_ROWS, 0, s, 0, r, gamma, beta, ld_mod, static_cast<float *>(u), T, L, d, eps);
+    }
     if (dtype == DM_BF16) return launch_chain(adaln_kernel<__nv_bfloat16>, T, 256, 0, s, 0, r, gamma, beta, ld_mod, static_cast<__nv_bfloat16 *>(u), L, d, eps);
     return launch_chain(adaln_kernel<float>, T, 256, 0, s, 0, r, gamma, beta, ld_mod, static_cast<float *>(u), L, d, eps);
 }
 
 cudaError_t modulation_rows(const float *tau, const void *w_cond, const float *b_cond, float *mod, int dtype, int B, int n_out, int d_c,
                             cudaStream_t s) {
-    dim3 grid((n_out * 32 + 255) / 256, B);
-    if (dtype == DM_BF16) return launch_chain(modulation_kernel<__nv_bfloat16>, grid, 256, 0, s, 0, tau, static_cast<const __nv_bfloat16 *>(w_cond), b_cond, mod, n_out, d_c);
-    return launch_chain(modulation_kernel<float>, grid, 256, 0, s, 0, tau, static_cast<const float *>(w_cond), b_cond, mod, n_out, d_c);
+    const dim3 grid((n_out + 8 * MOD_R - 1) / (8 * MOD_R), (B + MOD_B - 1) / MOD_B);
+    if (dtype == DM_BF16) return launch_chain(modulation_kernel<__nv_bfloat16>, grid, 256, 0, s, 0, tau, static_cast<const __nv_bfloat16 *>(w_cond), b_cond, mod, n_out, d_c, B);
+    return launch_chain(modulation_kernel<float>, grid, 256, 0, s, 0, tau, static_cast<const float *>(w_cond), b_cond, mod, n_out, d_c, B);
 }
 
 cudaError_t argmax_rows(const void *logits, int dtype, int32_t *out, int T, int V, cudaStream_t s) {

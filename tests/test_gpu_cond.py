@@ -79,6 +79,21 @@ def test_conditioned_step_block_mode(G, dtype):
     assert G.rel_l2(got_blk, want_blk) <= tol
 
 
+@pytest.mark.parametrize("dtype,d,d_c", [(I.F32, 48, 20), (I.BF16, 48, 170), (I.BF16, 2048, 32), (I.BF16, 2080, 128)])
+def test_conditioned_step_row_widths(G, dtype, d, d_c):
+    """AdaLN with a warp per row: rows that leave lanes without channels, the widest row it takes, one that goes to the block-per-row kernel; 21 rows over three
+    sequences, so that a block's rows belong to two of them.  Timestep widths within, at and past the columns the modulation kernel reads ahead; fewer sequences than
+    it takes at once."""
+    shape = I.MixerShape(3, 7, d, 2, 16, 4, d // 16)
+    sw = I.make_stack_weights(shape, 1, 64, seed=9, dtype=dtype, perturb=True)
+    I.add_block_weights(sw, shape, 64, d_c, seed=9, dtype=dtype)
+    tau = I.make_timestep_embedding(3, d_c, seed=9)
+    tok = I.make_tokens(3, 7, 63, 63, seed=9)
+    want = O.denoise_step_cond(tok, tau, sw, **G.oracle_kwargs(shape))
+    got, _, _ = G.run_denoise(shape, dtype, sw, tok, 64, want_argmax=False, tau=tau, d_ff=64)
+    assert G.rel_l2(got, want) <= (1e-4 if dtype == I.F32 else 1e-2), G.rel_l2(got, want)
+
+
 def test_conditioned_step_argument_checks(G):
     from paper_2511_15927_b200 import binding as dm
     shape = I.MixerShape(1, 8, 64, 2, 16, 4, 4)
