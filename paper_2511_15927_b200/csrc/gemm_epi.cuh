@@ -281,6 +281,7 @@ inline bool make_map_u(CUtensorMap *m, const void *base, int64_t rows, int64_t c
 }  // namespace tc
 
 // gemm_pair.cu: the two-CTA kernel.  wide: 256 x 256 tiles, else 256 x 128; b: a second product of the same sizes.  gemm_pair_sum_launch: both products into one output.
+int gemm_pair_cost(bool wide, const GemmArgs &a, int nprob);      // of the launch's rounds, for the choice of the tile
 cudaError_t gemm_pair_launch(bool wide, const GemmArgs &a, const GemmArgs *b, cudaStream_t s);
 cudaError_t gemm_pair_sum_launch(const GemmArgs &a, const GemmArgs &b, cudaStream_t s);
 // gemm_cluster.cu: the same with each tile's K spread over a cluster, for few tiles.

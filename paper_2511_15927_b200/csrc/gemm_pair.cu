@@ -25,9 +25,56 @@ constexpr int MAX_STAGES = 8;
 
 // 256 rows x BN columns per pair.  Stage of one CTA: 128 rows of A and BN / 2 rows of B.
 template <int BN> struct Tile {
-    static constexpr uint32_t A_BYTES = BM * BK * 2, B_BYTES = BN / 2 * BK * 2, STAGE = A_BYTES + B_BYTES;
+    static constexpr uint32_t A_BYTES = BM * BK * 2, B_BYTES = BN / 2 * BK * 2, STAGE = A_BYTES + B_BYTES, NARROW = A_BYTES + B_BYTES / 2;     // (NARROW: of a narrow tile)
     static constexpr int STAGES = BN == 128 ? 8 : 6;
     static constexpr uint32_t TMEM_COLS = 2 * BN;               // two accumulator buffers
+};
+
+// Operands of up to two problems: A in boxes of 128 rows, B in boxes of BN / 2 rows, and (256-column tiles) of 64 for the narrow ones.
+struct OpMaps { CUtensorMap a[2], b[2], bn[2]; };
+
+// The tiles of a launch, in the order in which the pairs take them: tile i goes to pair i % npairs.  Tiles are 256 rows x BN columns; with BN = 256 a last column tile of at most 128 columns is
+// narrow (256 x 128: 0.74 of a wide tile's time, see gemm_tcgen05.cu), and so are the halves into which the wide tiles of an incomplete last round are cut where that ends
+// earlier.  Narrow ones come last.  (16384 x 1024, 256 wide tiles for 74 pairs: 222 wide and 68 halves, 3.74 rounds instead of 4.  One layer of 1024 tokens,
+// in_proj 252 tiles of which 8 are 120 columns wide: 129.5 -> 128.2 us; 24 conditioned layers of 8192 tokens, under the power limit: 28.02 -> 27.89 ms.)
+struct TileAt { int mb, prob, n0; bool narrow; };
+template <int BN> struct Tiles {
+    int tiles_m, wn, wn_all, whole, halves, total, n_fast;     // row tiles; wide columns per problem, over all problems; uncut wide tiles; halves; all tiles
+    int cost;                                                  // of the launch, in hundredths of a round of 256-column tiles
+    __host__ __device__ Tiles(int M, int N, int nprob, int npairs, int n_fast) : n_fast(n_fast) {
+        const int rem = N % BN, strip = BN == 256 && rem > 0 && rem <= 128;
+        tiles_m = (M + 2 * BM - 1) / (2 * BM);
+        wn = N / BN + (rem > 0 && !strip);
+        wn_all = wn * nprob;
+        const int wide = tiles_m * wn_all, narrow = strip ? tiles_m * nprob : 0;
+        int cut = 0;
+        const int r = wide % npairs, more = r > 0 ? narrow - (npairs - r) : narrow;      // narrow tiles that find no pair idle in the last round of wide ones
+        int last = (r > 0 ? 100 : 0) + (more > 0 ? 74 * ((more + npairs - 1) / npairs) : 0);
+        if (BN == 256 && r > 0) {
+            const int cut_up = 74 * ((2 * r + narrow + npairs - 1) / npairs);
+            if (cut_up < last) { cut = r; last = cut_up; }
+        }
+        cost = BN == 256 ? 100 * (wide / npairs) + last : 74 * ((wide + npairs - 1) / npairs);
+        whole = wide - cut;
+        halves = 2 * cut;
+        total = whole + halves + narrow;
+    }
+    __device__ __forceinline__ TileAt at(int i) const {
+        TileAt t;
+        int w = i, half = 0;
+        t.narrow = BN == 256 && i >= whole;
+        if (BN == 256 && i >= whole + halves) {                // the last columns
+            const int j = i - whole - halves;
+            t.prob = j / tiles_m; t.mb = j - t.prob * tiles_m; t.n0 = wn * BN;
+            return t;
+        }
+        if (t.narrow) { w = whole + ((i - whole) >> 1); half = (i - whole) & 1; }
+        t.mb = n_fast ? w / wn_all : w % tiles_m;
+        const int cb = n_fast ? w % wn_all : w / tiles_m;
+        t.prob = cb / wn;
+        t.n0 = (cb - t.prob * wn) * BN + half * (BN / 2);
+        return t;
+    }
 };
 
 struct __align__(8) Bars {
@@ -47,9 +94,7 @@ struct __align__(8) Bars {
 enum { DIRECT = 0, TMA = 1, SUM = 2 };
 template <int BN, int MODE>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
-gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant__ CUtensorMap map_b0,
-                 const __grid_constant__ CUtensorMap map_a1, const __grid_constant__ CUtensorMap map_b1,
-                 const __grid_constant__ IoMaps io, const __grid_constant__ EpiPair epp, int *status) {
+gemm_pair_kernel(const __grid_constant__ OpMaps op, const __grid_constant__ IoMaps io, const __grid_constant__ EpiPair epp, int *status) {
     using T = Tile<BN>;
     constexpr int STAGES = T::STAGES;
     const EpiArgs &ep = epp.p[0];              // sizes are common to all problems
@@ -63,14 +108,9 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_consta
     const int pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
     if (ep.m_dev) pdl_wait();                  // (the row count comes from a kernel before this one)
     const int M_eff = ep.m_dev ? min(ep.M, max(0, *ep.m_dev - ep.m_off)) : ep.M;
-    const int tiles_m = (M_eff + 2 * BM - 1) / (2 * BM), tiles_n = (ep.N + BN - 1) / BN;
-    const int tiles_np = tiles_n * (MODE == SUM ? 1 : epp.nprob);      // separate problems sit side by side along N
-    const int num_tiles = tiles_m * tiles_np;
     constexpr int NSUB = MODE == SUM ? 2 : 1;                  // products per tile
-    auto tile_at = [&](int tile, int &mb, int &cb) {
-        mb = epp.n_fast ? tile / tiles_np : tile % tiles_m;
-        cb = epp.n_fast ? tile % tiles_np : tile / tiles_m;
-    };
+    const Tiles<BN> tiles(M_eff, ep.N, MODE == SUM ? 1 : epp.nprob, npairs, epp.n_fast);       // separate problems sit side by side along N
+    const int num_tiles = tiles.total;
     const int kblocks = (ep.K + BK - 1) / BK;
 
     if (threadIdx.x == 0) {
@@ -81,8 +121,8 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_consta
         mbar_fence_init();
     }
     if (threadIdx.x == 64) {                   // the maps are on their way while the barriers and TMEM are set up
-        prefetch_map(&map_a0); prefetch_map(&map_b0);
-        if (epp.nprob > 1) { prefetch_map(&map_a1); prefetch_map(&map_b1); }
+        prefetch_map(&op.a[0]); prefetch_map(&op.b[0]);
+        if (epp.nprob > 1) { prefetch_map(&op.a[1]); prefetch_map(&op.b[1]); }
     }
     if (warp == 1) tmem_alloc_2cta(&bars->tmem_base, T::TMEM_COLS);
     fence_before();
@@ -99,31 +139,29 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_consta
             // the first stages' share of B (weights) is on its way before the kernel before this one has finished
             const uint32_t ahead = pair < num_tiles ? min(STAGES, kblocks) : 0;
             if (leader && ahead > 0) {
-                int tm, cb;
-                tile_at(pair, tm, cb);
-                const int prob = cb / tiles_n, n0 = (cb - prob * tiles_n) * BN + (int)rank * (BN / 2);
+                const TileAt t = tiles.at(pair);
+                const int n0 = t.n0 + (int)rank * (t.narrow ? BN / 4 : BN / 2);
                 for (uint32_t s = 0; s < ahead; ++s) {
-                    if (rank == 0) mbar_expect_tx(&bars->full[s], 2 * T::STAGE);
-                    tma_load_2d_pair(smem + s * T::STAGE + T::A_BYTES, prob ? &map_b1 : &map_b0, (int)s * BK, n0, cluster_addr(&bars->full[s], 0));
+                    if (rank == 0) mbar_expect_tx(&bars->full[s], t.narrow ? 2 * T::NARROW : 2 * T::STAGE);
+                    tma_load_2d_pair(smem + s * T::STAGE + T::A_BYTES, t.narrow ? &op.bn[t.prob] : &op.b[t.prob], (int)s * BK, n0, cluster_addr(&bars->full[s], 0));
                 }
             }
             __syncwarp();
             pdl_wait();
             pdl_trigger();
             for (int tile = pair; tile < num_tiles && ok; tile += npairs) {
-                int tm, cb;
-                tile_at(tile, tm, cb);
-                const int prob0 = cb / tiles_n, m0 = tm * 2 * BM + (int)rank * BM, n0 = (cb - prob0 * tiles_n) * BN + (int)rank * (BN / 2);
+                const TileAt t = tiles.at(tile);
+                const int m0 = t.mb * 2 * BM + (int)rank * BM, n0 = t.n0 + (int)rank * (t.narrow ? BN / 4 : BN / 2);
                 for (int sub = 0; sub < NSUB && ok; ++sub) {
-                    const int prob = prob0 + sub;
-                    const CUtensorMap *ma = prob ? &map_a1 : &map_a0, *mb = prob ? &map_b1 : &map_b0;
+                    const int prob = t.prob + sub;
+                    const CUtensorMap *ma = &op.a[prob], *mb = t.narrow ? &op.bn[prob] : &op.b[prob];
                     for (int kb = 0; kb < kblocks; ++kb, ++it) {
                         const uint32_t s = it % STAGES, ph = (it / STAGES) & 1u;
                         if (!(ok = mbar_wait(&bars->empty[s], ph ^ 1u, abort_flag, status))) break;
                         uint8_t *sa = smem + s * T::STAGE, *sb = sa + T::A_BYTES;
                         const uint32_t full = cluster_addr(&bars->full[s], 0);
                         if (leader) {
-                            if (rank == 0 && it >= ahead) mbar_expect_tx(&bars->full[s], 2 * T::STAGE);        // both CTAs' loads
+                            if (rank == 0 && it >= ahead) mbar_expect_tx(&bars->full[s], t.narrow ? 2 * T::NARROW : 2 * T::STAGE);        // both CTAs' loads
                             tma_load_2d_pair(sa, ma, kb * BK, m0, full);
                             if (it >= ahead) tma_load_2d_pair(sb, mb, kb * BK, n0, full);
                         }
@@ -139,40 +177,41 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_consta
         // about 80, which held every k-block at 600 clocks where its products take 512)
         if (rank == 0) {
             const bool leader = elect_one();
-            constexpr uint32_t idesc = idesc_bf16(2 * BM, BN, 0, 0);
             const uint32_t desc_a0 = desc_lo_k(smem_u32(smem));
             uint32_t it = 0, tcount = 0;
             bool ok = true;
             pdl_wait();                                        // (the limit of the waits below counts from here)
-            const uint32_t products = (uint32_t)(pair < num_tiles ? (num_tiles - 1 - pair) / npairs + 1 : 0) * NSUB;
-            for (; tcount < products && ok; ++tcount) {
-                const uint32_t buf = tcount & 1u, bph = (tcount >> 1) & 1u;
-                if (!(ok = mbar_wait(&bars->tmem_empty[buf], bph ^ 1u, abort_flag, status))) break;
-                fence_after();
-                const uint32_t d_tmem = tmem_base + buf * BN;
-                for (int kb = 0; kb < kblocks; ++kb, ++it) {
-                    const uint32_t s = it % STAGES, ph = (it / STAGES) & 1u;
-                    if (!(ok = mbar_wait(&bars->full[s], ph, abort_flag, status))) break;
+            for (int tile = pair; tile < num_tiles && ok; tile += npairs) {
+                const uint32_t idesc = tiles.at(tile).narrow ? idesc_bf16(2 * BM, BN / 2, 0, 0) : idesc_bf16(2 * BM, BN, 0, 0);
+                for (int sub = 0; sub < NSUB && ok; ++sub, ++tcount) {
+                    const uint32_t buf = tcount & 1u, bph = (tcount >> 1) & 1u;
+                    if (!(ok = mbar_wait(&bars->tmem_empty[buf], bph ^ 1u, abort_flag, status))) break;
                     fence_after();
-                    const uint32_t da = desc_a0 + s * (T::STAGE >> 4), db = da + (T::A_BYTES >> 4);
-                    if (leader) {
-#pragma unroll
-                        for (int k = 0; k < BK / 16; ++k)          // 32 bytes along K per MMA: +2 in 16-byte units
-                            umma_ss_2cta(d_tmem, da + 2 * k, db + 2 * k, idesc, (kb | k) != 0);
-                        umma_commit_2cta(&bars->empty[s]);         // frees the stage in both CTAs when these MMAs have read it
+                    const uint32_t d_tmem = tmem_base + buf * BN;
+                    for (int kb = 0; kb < kblocks; ++kb, ++it) {
+                        const uint32_t s = it % STAGES, ph = (it / STAGES) & 1u;
+                        if (!(ok = mbar_wait(&bars->full[s], ph, abort_flag, status))) break;
+                        fence_after();
+                        const uint32_t da = desc_a0 + s * (T::STAGE >> 4), db = da + (T::A_BYTES >> 4);
+                        if (leader) {
+    #pragma unroll
+                            for (int k = 0; k < BK / 16; ++k)          // 32 bytes along K per MMA: +2 in 16-byte units
+                                umma_ss_2cta(d_tmem, da + 2 * k, db + 2 * k, idesc, (kb | k) != 0);
+                            umma_commit_2cta(&bars->empty[s]);         // frees the stage in both CTAs when these MMAs have read it
+                        }
+                        __syncwarp();
                     }
+                    if (ok && leader) umma_commit_2cta(&bars->tmem_full[buf]);
                     __syncwarp();
                 }
-                if (ok && leader) umma_commit_2cta(&bars->tmem_full[buf]);
-                __syncwarp();
             }
         }
     } else {
         // ------------------------------------------------------------ epilogue: 8 warps over this CTA's 128 rows
-        constexpr int COLS = BN / 2;                           // columns per warp
-        const int q = warp & 3, cfirst = ((warp - 2) >> 2) * COLS;       // TMEM lane quarter, first column
+        constexpr int COLS = BN / 2;                           // columns per warp (of a narrow tile: half of them)
+        const int q = warp & 3, ch = (warp - 2) >> 2;          // TMEM lane quarter, half of the columns
         pdl_wait();
-        const uint32_t tlane = tmem_base + ((uint32_t)(q * 32) << 16) + cfirst;
+        const uint32_t tquarter = tmem_base + ((uint32_t)(q * 32) << 16);
         uint32_t tcount = 0;
         bool ok = true;
         auto drained = [&](uint32_t buf) {                     // this warp has taken the buffer out of TMEM
@@ -187,11 +226,11 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_consta
         };
         EpiOut out{smem + STAGES * T::STAGE + (warp - 2) * STG_BYTES, lane, &bars->add_full[warp - 2], abort_flag, status, 0};
         for (int tile = pair; tile < num_tiles && ok; tile += npairs, tcount += NSUB) {
-            int tm, cb;
-            tile_at(tile, tm, cb);
-            const int prob = MODE == SUM ? 1 : cb / tiles_n;
+            const TileAt t = tiles.at(tile);
+            const int prob = MODE == SUM ? 1 : t.prob, cols = t.narrow ? COLS / 2 : COLS;
             const EpiArgs &pe = epp.p[prob];                   // this tile's problem: its output, scales and addend
-            const int row0 = tm * 2 * BM + (int)rank * BM + q * 32, row = row0 + lane, n0 = (MODE == SUM ? cb : cb - prob * tiles_n) * BN + cfirst;
+            const uint32_t tlane = tquarter + ch * cols;
+            const int row0 = t.mb * 2 * BM + (int)rank * BM + q * 32, row = row0 + lane, n0 = t.n0 + ch * cols;
             const bool row_ok = row < M_eff;
             const bool live = row0 < M_eff && n0 < pe.N;       // some of this warp's part of the tile exists
             const float sc = row_ok ? epi_row_scale(pe, row) : 1.f;
@@ -207,6 +246,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_consta
                 if (!(ok = ready(tcount))) break;
 #pragma unroll
                 for (int c0 = 0; c0 < COLS; c0 += 32) {
+                    if (c0 >= cols) break;
                     const bool some = n0 + c0 < pe.N;
                     if (add && some) out.add_fetch(io.add, n0 + c0, row0);
                     uint32_t r[32];
@@ -224,6 +264,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_consta
                 if (!ok || !(ok = ready(tcount + 1))) break;
 #pragma unroll
                 for (int c0 = 0; c0 < COLS; c0 += 32) {
+                    if (c0 >= cols) break;
 #pragma unroll
                     for (int c1 = c0; c1 < c0 + 32; c1 += 16) {
                         uint32_t r[16];
@@ -243,17 +284,17 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_consta
                             for (int j = 0; j < 16; ++j) held[c1 + j] = fmaf(__uint_as_float(r[j]), sc, held[c1 + j]);
                         }
                     }
-                    if (c0 == COLS - 32) drained((tcount + 1) & 1u);
+                    if (c0 == cols - 32) drained((tcount + 1) & 1u);
                     if (live && n0 + c0 < pe.N) emit(c0, held + c0);
                 }
             } else {
                 if (!(ok = ready(tcount))) break;
 #pragma unroll 1
-                for (int c0 = 0; c0 < COLS; c0 += 32) {
+                for (int c0 = 0; c0 < cols; c0 += 32) {
                     uint32_t r[32];
                     tmem_ld_x32(tlane + (tcount & 1u) * BN + c0, r);
                     tmem_wait_ld();
-                    if (c0 == COLS - 32) drained(tcount & 1u);
+                    if (c0 == cols - 32) drained(tcount & 1u);
                     const int col = n0 + c0;
                     if (!live || col >= pe.N || (MODE == DIRECT && !row_ok)) continue;
                     float v[32];
@@ -290,10 +331,13 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_consta
 template <int BN, int MODE>
 cudaError_t launch(const GemmArgs &a, const GemmArgs *b, cudaStream_t s) {
     using T = Tile<BN>;
-    CUtensorMap ma[2], mb[2];
-    if (!make_map_2d(&ma[0], a.A, a.M, a.K, a.lda, BM) || !make_map_2d(&mb[0], a.B, a.N, a.K, a.ldb, BN / 2)) return cudaErrorInvalidValue;
-    ma[1] = ma[0]; mb[1] = mb[0];
-    if (b && (!make_map_2d(&ma[1], b->A, b->M, b->K, b->lda, BM) || !make_map_2d(&mb[1], b->B, b->N, b->K, b->ldb, BN / 2))) return cudaErrorInvalidValue;
+    OpMaps op;
+    memset(&op, 0, sizeof(op));
+    for (int i = 0; i < (b ? 2 : 1); ++i) {
+        const GemmArgs &p = i ? *b : a;
+        if (!make_map_2d(&op.a[i], p.A, p.M, p.K, p.lda, BM) || !make_map_2d(&op.b[i], p.B, p.N, p.K, p.ldb, BN / 2)) return cudaErrorInvalidValue;
+        if (BN == 256 && !make_map_2d(&op.bn[i], p.B, p.N, p.K, p.ldb, BN / 4)) return cudaErrorInvalidValue;
+    }
     constexpr size_t smem = T::STAGES * (size_t)T::STAGE + (MODE == DIRECT ? 0 : 8 * STG_BYTES) + sizeof(Bars) + 1024;
     static_assert(smem <= 232448, "shared memory budget");
     cudaError_t e = cudaFuncSetAttribute(gemm_pair_kernel<BN, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -312,14 +356,18 @@ cudaError_t launch(const GemmArgs &a, const GemmArgs *b, cudaStream_t s) {
         if (p.addend && !make_map_f32_2d(&io.add, p.addend, p.M, p.N, p.ld_add, 32)) return cudaErrorInvalidValue;
         if (p.u && !make_map_u(&io.u, p.u, p.M, p.N)) return cudaErrorInvalidValue;
     }
-    const int64_t tiles = (int64_t)((a.M + 2 * BM - 1) / (2 * BM)) * ((a.N + BN - 1) / BN) * (MODE == SUM ? 1 : epp.nprob);
-    const int pairs = sm_count() / 2, grid = 2 * (int)(tiles < pairs ? tiles : pairs);
-    return launch_chain(gemm_pair_kernel<BN, MODE>, grid, NTHREADS, smem, s, 0, ma[0], mb[0], ma[1], mb[1], io, epp, status);
+    const int pairs = sm_count() / 2, tiles = Tiles<BN>(a.M, a.N, MODE == SUM ? 1 : epp.nprob, pairs, epp.n_fast).total, grid = 2 * (tiles < pairs ? tiles : pairs);
+    return launch_chain(gemm_pair_kernel<BN, MODE>, grid, NTHREADS, smem, s, 0, op, io, epp, status);
 }
 
 bool tma_io(const GemmArgs &a, const GemmArgs *b) { return gemm_pair_tma_io(a) && (!b || (gemm_pair_tma_io(*b) && !a.addend && !b->addend && !a.u && !b->u)); }
 
 }  // namespace
+
+int gemm_pair_cost(bool wide, const GemmArgs &a, int nprob) {
+    const int pairs = sm_count() / 2;
+    return wide ? Tiles<256>(a.M, a.N, nprob, pairs, 0).cost : Tiles<128>(a.M, a.N, nprob, pairs, 0).cost;
+}
 
 cudaError_t gemm_pair_launch(bool wide, const GemmArgs &a, const GemmArgs *b, cudaStream_t s) {
     if (tma_io(a, b)) return wide ? launch<256, TMA>(a, b, s) : launch<128, TMA>(a, b, s);

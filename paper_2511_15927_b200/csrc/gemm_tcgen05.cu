@@ -12,15 +12,9 @@ using namespace tc;
 
 constexpr int BM = 128;
 
-int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }
-
 // Tile width of the pair kernel, by rounds of CTA pairs.  A k-block of a 256 x 256 tile takes 0.31 us, of a 256 x 128 one 0.23 us (its operands, 24 KB
-// per CTA, then arrive at 15 TB/s over all SMs: what L2 delivers, while its products take half of that time), so a narrow round counts 0.7.
-bool pair_wide_tile(const GemmArgs &a, int nprob) {
-    const int64_t pairs = sm_count() / 2, tm = ceil_div(a.M, 256);
-    const int64_t r256 = ceil_div(tm * ceil_div(a.N, 256) * nprob, pairs), r128 = ceil_div(tm * ceil_div(a.N, 128) * nprob, pairs);
-    return a.N > 128 && 10 * r256 <= 7 * r128;
-}
+// per CTA, then arrive at 15 TB/s over all SMs: what L2 delivers, while its products take half of that time), so a narrow round counts 0.74.
+bool pair_wide_tile(const GemmArgs &a, int nprob) { return a.N > 128 && gemm_pair_cost(true, a, nprob) <= gemm_pair_cost(false, a, nprob); }
 
 cudaError_t dispatch(const GemmArgs &a, const GemmArgs *b, cudaStream_t s) {
     if (a.M <= BM) return gemm_rows_launch(a, b, false, s);

@@ -66,3 +66,10 @@ def test_linear_epilogue_scale_addend_inplace(dm, dtype, shape):
     dm.dm_check(0)
     want = sc[:, None].astype(np.float64) * O.out_proj(x, w) + add
     np.testing.assert_allclose(yd.cpu().numpy().astype(np.float64), want, rtol=1e-5, atol=1e-5)
+
+
+@pytest.mark.parametrize("M,N,K", [(6400, 768, 72), (6300, 840, 136), (9728, 2048, 64), (2048, 9728, 456), (600, 24960, 64)])
+def test_linear_mixed_tile_widths(dm, M, N, K):
+    """The two-CTA kernel with tiles of two widths: an incomplete last round cut into halves (rows or columns first in the tile order), a last column tile of 72 columns,
+    both, with ragged rows; a column strip whose tiles start in the last round of wide ones."""
+    test_linear_parity(dm, I.BF16, M, N, K)

@@ -62,6 +62,12 @@ def test_denoise_step_summed_out_proj(G, d, H, B, L, d_ff):
     assert G.rel_l2(got, want) <= 1e-2, G.rel_l2(got, want)
 
 
+@pytest.mark.parametrize("d,H,B,L,d_ff", [(320, 10, 75, 255, 0)])
+def test_denoise_step_summed_out_proj_mixed_tiles(G, d, H, B, L, d_ff):
+    """75 wide tiles and a 64-column strip of as many: one wide tile is left for the last round and cut in two."""
+    test_denoise_step_summed_out_proj(G, d, H, B, L, d_ff)
+
+
 @pytest.mark.parametrize("d,H,B,L,d_ff", [(288, 9, 1, 129, 0), (192, 6, 1, 256, 384), (1024, 32, 2, 1000, 0), (320, 10, 17, 256, 0)])
 def test_denoise_step_out_proj_over_clusters(G, d, H, B, L, d_ff):
     """Few 256 x 256 tiles: the summed out_proj cuts a tile over 4 or 2 pairs of CTAs.  An odd number of k-blocks and a last column tile of 32 columns; columns that
