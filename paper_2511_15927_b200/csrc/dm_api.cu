@@ -165,8 +165,7 @@ struct PendingNorm {
 struct MixerOut {
     void *y; int y_dtype; const float *addend; int64_t ld_add;
     const float *col_scale = nullptr; int cs_rows = 0; int64_t ld_cs = 0;   // per-sequence gate on the mixer's output (App. A.1), or NULL
-    // The caller's next step is u = RMSNorm(y; next_norm_w).  A mixer that sums its directions in a pass of its own applies it there; one that sums them inside
-    // the out_proj launch leaves y * next_norm_w in u and the rows' sums of squares in next_ssq ([T][ceil(d / 64)]), the scale pending.  *next_done: u is there.
+    // The caller's next step is u = RMSNorm(y; next_norm_w).  An out_proj launch that completes y leaves y * next_norm_w in u and the rows' sums of squares in next_ssq ([T][ceil(d / 64)]), the scale pending.  *next_done: u is there.
     const void *next_norm_w = nullptr; void *next_u = nullptr; float next_eps = 0.f; bool *next_done = nullptr;
     float *next_ssq = nullptr; PendingNorm *pending = nullptr;
     bool fuse_norm(GemmArgs &a, int d) const {         // asks the product that completes y for u
@@ -321,7 +320,7 @@ static int check_ws(const void *ws, size_t have, size_t need) {
 }
 
 struct StackWs {
-    size_t r, u, ussq, logits, mixer, mod, hmid, idx, count, ug, qkv, att, total;
+    size_t r, u, ussq, logits, mixer, mod, hmid, idx, count, ug, ugssq, qkv, att, total;
     int logits_rows;
 };
 
@@ -339,11 +338,12 @@ static StackWs stack_ws(const dm_stack_cfg *c, const Dims &m, const dm_block_cfg
         w.mod = off; off += align_up((size_t)m.B * 6 * m.d * sizeof(float));
         w.hmid = off; off += align_up((size_t)m.T * blk->d_ff * m.es);
     }
-    w.idx = w.count = w.ug = off;
+    w.idx = w.count = w.ug = w.ugssq = off;
     if (sampler) {
         w.idx = off; off += align_up((size_t)m.T * sizeof(int32_t));
         w.count = off; off += align_up(sizeof(int));
         w.ug = off; off += align_up((size_t)m.T * m.d * m.es);
+        w.ugssq = off; off += align_up((size_t)m.T * ((m.d + 63) / 64) * sizeof(float));
     }
     w.qkv = w.att = off;
     if (hybrid) {
@@ -630,8 +630,7 @@ static int denoise_impl(const dm_stack_cfg *cfg, const dm_block_cfg *blk, const 
             // what follows this layer's mixer is the next layer's (or the final) RMSNorm of r
             out.next_norm_w = i + 1 < cfg->n_layers ? weights->layers[i + 1].norm_w : weights->final_norm_w;
             out.next_u = u; out.next_eps = cfg->rms_eps; out.next_done = &u_ready;
-            // (the sampler gathers rows of the final norm: they are normalised in a pass of their own)
-            out.next_ssq = smp && i + 1 == cfg->n_layers ? nullptr : reinterpret_cast<float *>(ws + l.ussq);
+            out.next_ssq = reinterpret_cast<float *>(ws + l.ussq);
         }
         const PendingNorm in_norm = u_norm;
         u_ready = false; u_norm = PendingNorm{};
@@ -684,6 +683,11 @@ static int denoise_impl(const dm_stack_cfg *cfg, const dm_block_cfg *blk, const 
         const dm_sample_cfg &q = *smp->cfg;
         if ((e = select_drawn(tokens, smp->u_keep, q.keep_prob, q.mask_id, smp->tokens_out, idx, count, (int)m.T, s)) != cudaSuccess) return cuda_fail(e, "select");
         if ((e = gather_rows(u, idx, count, ug, dtype, (int)m.T, m.d, s)) != cudaSuccess) return cuda_fail(e, "gather");
+        if (u_norm.ssq) {                         // the final norm's scale is pending: the rows' sums of squares go along
+            float *gs = reinterpret_cast<float *>(ws + l.ugssq);
+            if ((e = gather_rows(u_norm.ssq, idx, count, gs, DM_F32, (int)m.T, u_norm.n, s)) != cudaSuccess) return cuda_fail(e, "gather");
+            u_norm.ssq = gs;
+        }
         for (int64_t t0 = 0; t0 < m.T; t0 += l.logits_rows) {
             const int rows = (int)((m.T - t0) < l.logits_rows ? (m.T - t0) : l.logits_rows);
             GemmArgs a{};
@@ -692,6 +696,7 @@ static int denoise_impl(const dm_stack_cfg *cfg, const dm_block_cfg *blk, const 
             a.C = ws + l.logits; a.ldc = cfg->vocab;
             a.in_dtype = dtype; a.c_dtype = dtype; a.M = rows; a.N = cfg->vocab; a.K = m.d;
             a.m_dev = count; a.m_off = (int)t0;
+            u_norm.apply(a, t0);
             if ((e = gemm(a, s)) != cudaSuccess) return cuda_fail(e, "vocab projection");
             if ((e = draw_rows(a.C, cfg->vocab, dtype, idx, count, (int)t0, rows, smp->u_cat, q.mask_id, q.vocab_real, smp->tokens_out, s)) != cudaSuccess)
                 return cuda_fail(e, "draw");
