@@ -1,13 +1,14 @@
 // The GEMM for up to 128 rows (decoding a few sequences): such a product is a read of its weights, so the roles are swapped -- a tile is 128 rows
 // of the weight matrix (the M side of tcgen05.mma) times all the tokens (its N side, 16 to 128), D^T = B A^T -- and what matters is that
-// every SM has weight bytes in flight all the time.  The tiles are cut along K over the CTAs of a cluster until the grid fills the
-// GPU about twice (two CTAs share an SM: while one sets up or finishes, the other one reads); the partial sums go to their owner's shared memory
+// every SM has weight bytes in flight all the time.  Where the tiles are few they are cut along K over the CTAs of a cluster; the partial sums go to their owner's shared memory
 // (each CTA of the cluster owns a share of the tokens), which adds them, applies the epilogue and stores them: lanes are
 // consecutive output columns.  sum: the cluster's CTAs are halves over two products (both directions' out_proj) that are added with each product's row scale.
 // Weights from HBM, with tokens as the M side and 128 x 128 tiles before: 32 x 16112 x 1920 18.2 -> 16.3 us, 32 x 1920 x 3840 20.2 -> 8.5 us, 32 x 50304 x 1920
-// 50.6 -> 37.1 us (5.2 TB/s); the rest is start-up: a single token takes 14.5 us where 32 take 16.3.
+// 50.6 -> 37.1 us (5.2 TB/s).  Inside a pass over 24 layers (one sequence, hybrid), where every kernel's instructions have left the chip since its last launch: 942 us, 925 us with
+// the weights marked as read once (the instructions then stay in L2), 902 us with a warp that runs the epilogue's code ahead of time, 849 us with 126 uncut tiles
+// in place of 252 halves of K (the exchange costs 2 us and a CTA already fills its SM's share of the bandwidth).
 //
-// Warp 0 issues the TMA loads, warp 1 the MMAs, the other EW (4 or 8) are the epilogue: one TMEM lane quarter each, tokens shared out between the two
+// Warp 0 issues the TMA loads, warp 1 the MMAs, the next EW (4 or 8) are the epilogue and a last one brings its code: one TMEM lane quarter each, tokens shared out between the two
 // warps of a quarter.  Waits and abort as in gemm_pair.cu: every mbarrier wait is bounded, and the CTAs of a cluster leave together.
 #include "gemm_epi.cuh"
 
@@ -91,7 +92,7 @@ __device__ __forceinline__ void emit(const EpiArgs &ep, int t, int n, int col, b
 }
 
 template <int EW>
-__global__ void __launch_bounds__(64 + 32 * EW, EW == 4 ? 2 : 1)
+__global__ void __launch_bounds__(96 + 32 * EW, EW == 4 ? 2 : 1)
 gemm_rows_kernel(const __grid_constant__ CUtensorMap map_x0, const __grid_constant__ CUtensorMap map_w0,
                  const __grid_constant__ CUtensorMap map_x1, const __grid_constant__ CUtensorMap map_w1,
                  const __grid_constant__ RowsArgs ra, int *status) {
@@ -130,6 +131,7 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap map_x0, const __grid_consta
     if (warp == 0) {
         const bool leader = elect_one();
         const CUtensorMap *mx = prod ? &map_x1 : &map_x0, *mw = prod ? &map_w1 : &map_w0;
+        const uint64_t once = l2_evict_first();
         int s = 0;
         uint32_t ph = 1;
         // the weights of the first stages are on their way before the kernel before this one has finished
@@ -137,7 +139,7 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap map_x0, const __grid_consta
         if (leader)
             for (int i = 0; i < ahead; ++i) {
                 mbar_expect_tx(&bars->full[i], stage);
-                tma_load_2d(smem + i * stage, mw, (kb0 + i) * BK, n0, &bars->full[i]);
+                tma_load_2d_hint(smem + i * stage, mw, (kb0 + i) * BK, n0, &bars->full[i], once);
             }
         __syncwarp();
         pdl_wait();
@@ -148,7 +150,7 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap map_x0, const __grid_consta
                 uint8_t *sw = smem + s * stage;
                 if (i >= ahead) {
                     mbar_expect_tx(&bars->full[s], stage);
-                    tma_load_2d(sw, mw, (kb0 + i) * BK, n0, &bars->full[s]);
+                    tma_load_2d_hint(sw, mw, (kb0 + i) * BK, n0, &bars->full[s], once);
                 }
                 tma_load_2d(sw + W_BYTES, mx, (kb0 + i) * BK, 0, &bars->full[s]);
             }
@@ -178,99 +180,111 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap map_x0, const __grid_consta
             if (++s == S) { s = 0; ph ^= 1; }
         }
     } else {
-        const int ew = warp - 2, q = warp & 3, f = q * 32 + lane;            // this thread's output column of the tile
-        pdl_wait();
-        // row scales of this CTA's tokens, while the products run
-        for (int pi = ra.sum ? 0 : prod; pi <= (ra.sum ? 1 : prod); ++pi) {
-            const EpiArgs &e = ra.p[pi];
-            for (int tl = ew; tl < tpc; tl += EW) {
-                const int t = rank * tpc + tl;
+        const int ew = warp - 2, q = warp & 3, f = q * 32 + lane, col = n0 + f;      // this thread's output column of the tile
+        const bool in = col < ep.N;
+        const float bias = in && ep.col_bias ? ep.col_bias[col] : 0.f;
+        const float uw = in && ep.u ? __bfloat162float(ep.u_w[col]) : 0.f;
+        // The last warp does the same without a token (real = false: no wait, no load of activations, no store), as soon as the CTA starts: it brings the instructions.  They come from memory --
+        // the weights of a pass have gone through L2 since the last launch --, all SMs wait for each line of them, and after the products nothing would hide that.
+        const bool real = ew < EW;
+        {
+            if (real) pdl_wait();
+            const int Mp = real ? M : 0;
+            // row scales of this CTA's tokens, while the products run: a warp per (product, token)
+            const int first = ra.sum ? 0 : prod, items = (ra.sum ? 2 : 1) * tpc;
+            for (int i = real ? ew : items - 1; i < items; i += EW) {
+                const int pi = i / tpc, tl = i - pi * tpc, t = rank * tpc + tl;
+                const EpiArgs &e = ra.p[first + pi];
                 float sc = 1.f;
-                if (t < M && e.row_scale) sc = e.row_scale[t];
-                else if (t < M && e.rs_ssq) {
+                if (t < Mp && e.row_scale) sc = e.row_scale[t];
+                else if (e.rs_ssq) {
                     float v = 0.f;
-                    for (int j = lane; j < e.rs_n; j += 32) v += __ldg(e.rs_ssq + (int64_t)t * e.rs_n + j);
+                    for (int j = lane; j < e.rs_n; j += 32) v += t < Mp ? __ldg(e.rs_ssq + (int64_t)t * e.rs_n + j) : 0.f;
                     for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
                     sc = rsqrtf(v * e.rs_inv + e.rs_eps);
                 }
-                if (lane == 0) bars->scale[ra.sum ? pi : 0][tl] = sc;
+                if (lane == 0 && real) bars->scale[pi][tl] = sc;
             }
-        }
-        named_sync(1, 32 * EW);                                              // the scales are there for all of these warps
-        ok = __all_sync(0xffffffffu, mbar_wait(&bars->done, 0, abort_flag, status));
-        fence_after();
-        if (cs > 1) {                                                        // this CTA's partial sums to the owners of the tokens
-            for (int c0 = 16 * (ew >> 2); c0 < nt && ok; c0 += 4 * EW) {
-                uint32_t r[16];
-                tmem_ld_x16(tmem + ((uint32_t)(q * 32) << 16) + c0, r);
-                tmem_wait_ld();
-                int owner = c0 / tpc, tl = c0 - owner * tpc;
-                uint32_t dst = cluster_addr(recv + (rank * tpc) * BF + f, owner);
+            if (real) {
+                named_sync(1, 32 * EW);                                      // the scales are there for all of these warps
+                ok = __all_sync(0xffffffffu, mbar_wait(&bars->done, 0, abort_flag, status));
+                fence_after();
+            }
+            if (cs > 1) {                                                    // this CTA's partial sums to the owners of the tokens
+                for (int c0 = real ? 16 * (ew >> 2) : 0; c0 < nt && ok; c0 += 4 * EW) {
+                    uint32_t r[16];
+                    tmem_ld_x16(tmem + ((uint32_t)(q * 32) << 16) + c0, r);
+                    tmem_wait_ld();
+                    int owner = c0 / tpc, tl = c0 - owner * tpc;
+                    uint32_t dst = cluster_addr(recv + (rank * tpc) * BF + f, owner);
 #pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    st_cluster_f32(dst + tl * (BF * 4), __uint_as_float(r[j]));
-                    if (++tl == tpc && owner + 1 < cs) { tl = 0; ++owner; dst = cluster_addr(recv + (rank * tpc) * BF + f, owner); }
+                    for (int j = 0; j < 16; ++j) {
+                        if (real) st_cluster_f32(dst + tl * (BF * 4), __uint_as_float(r[j]));
+                        if (++tl == tpc && owner + 1 < cs) { tl = 0; ++owner; dst = cluster_addr(recv + (rank * tpc) * BF + f, owner); }
+                    }
+                    if (!real) break;
+                }
+                __syncwarp();
+                if (real) cluster_sync();                                    // every partial sum has arrived; nobody's shared memory is written any more
+            }
+            // ------------------------------------------------------------ the CTA's tokens: sum, epilogue, store
+            const bool go = !real || !*abort_flag;
+            auto squares = [&](const auto &v, int tl, int n) {               // the next norm's sums over this warp's 32 columns
+                if (!ep.u) return;
+#pragma unroll
+                for (int g = 0; g < (int)(sizeof(v) / sizeof(float)); ++g) {
+                    float ss = v[g] * v[g];
+#pragma unroll
+                    for (int off = 16; off > 0; off >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, off);
+                    if (lane == 0 && g < n && real) bars->red[q][tl + g] = ss;
+                }
+            };
+            if (cs == 1) {
+                for (int c0 = real ? 16 * (ew >> 2) : 0; c0 < nt && c0 < M && go; c0 += 4 * EW) {
+                    uint32_t r[16];
+                    float v[16];
+                    tmem_ld_x16(tmem + ((uint32_t)(q * 32) << 16) + c0, r);
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(r[j]) * bars->scale[0][c0 + j];
+                    emit(ep, c0, min(16, Mp - c0), col, in, bias, uw, v);
+                    squares(v, c0, 16);
+                    if (!real) break;
+                }
+            } else {
+                const int half = ra.sum ? ra.ks : cs;                        // sources [0, half) are product 0 (or the only one)
+                constexpr int G = 4;
+                for (int tl = real ? G * (ew >> 2) : 0; tl < tpc && go; tl += G * (EW / 4)) {
+                    const int t = rank * tpc + tl;
+                    if (t >= M) break;
+                    float v[G] = {};
+#pragma unroll
+                    for (int r = 0; r < MAX_CS; ++r) {
+                        if (r >= cs) break;
+#pragma unroll
+                        for (int g = 0; g < G; ++g) {
+                            const int tg = min(tl + g, tpc - 1);
+                            v[g] = fmaf(recv[(r * tpc + tg) * BF + f], bars->scale[r < half ? 0 : 1][tg], v[g]);
+                        }
+                    }
+                    emit(ep, t, min(min(G, tpc - tl), Mp - t), col, in, bias, uw, v);
+                    squares(v, tl, tpc - tl);
+                    if (!real) break;
+                }
+            }
+            if (ep.u && go) {
+                if (real) named_sync(1, 32 * EW);
+                const int parts = (ep.N + 63) / 64;
+                for (int i = real ? threadIdx.x - 64 : lane; i < 2 * tpc; i += 32 * EW) {  // (half of the tile, token)
+                    const int hf = i / tpc, tl = i - hf * tpc, t = rank * tpc + tl;
+                    if (t < Mp && n0 / 64 + hf < parts) ep.u_ssq[(int64_t)t * parts + n0 / 64 + hf] = bars->red[2 * hf][tl] + bars->red[2 * hf + 1][tl];
                 }
             }
         }
     }
-    __syncwarp();
-    if (cs > 1) cluster_sync();                                              // every partial sum has arrived; nobody's shared memory is written any more
-    // ---------------------------------------------------------------- the CTA's tokens: sum, epilogue, store
-    if (warp >= 2 && !*abort_flag) {
-        const int ew = warp - 2, q = warp & 3, f = q * 32 + lane, col = n0 + f;
-        const bool in = col < ep.N;
-        const float bias = in && ep.col_bias ? ep.col_bias[col] : 0.f;
-        const float uw = in && ep.u ? __bfloat162float(ep.u_w[col]) : 0.f;
-        auto squares = [&](const auto &v, int tl, int n) {                   // the next norm's sums over this warp's 32 columns
-            if (!ep.u) return;
-#pragma unroll
-            for (int g = 0; g < (int)(sizeof(v) / sizeof(float)); ++g) {
-                float ss = v[g] * v[g];
-#pragma unroll
-                for (int off = 16; off > 0; off >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, off);
-                if (lane == 0 && g < n) bars->red[q][tl + g] = ss;
-            }
-        };
-        if (cs == 1) {
-            for (int c0 = 16 * (ew >> 2); c0 < nt && c0 < M; c0 += 4 * EW) {
-                uint32_t r[16];
-                float v[16];
-                tmem_ld_x16(tmem + ((uint32_t)(q * 32) << 16) + c0, r);
-                tmem_wait_ld();
-#pragma unroll
-                for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(r[j]) * bars->scale[0][c0 + j];
-                emit(ep, c0, min(16, M - c0), col, in, bias, uw, v);
-                squares(v, c0, 16);
-            }
-        } else {
-            const int half = ra.sum ? ra.ks : cs;                            // sources [0, half) are product 0 (or the only one)
-            constexpr int G = 4;
-            for (int tl = G * (ew >> 2); tl < tpc; tl += G * (EW / 4)) {
-                const int t = rank * tpc + tl;
-                if (t >= M) break;
-                float v[G] = {};
-#pragma unroll
-                for (int r = 0; r < MAX_CS; ++r) {
-                    if (r >= cs) break;
-#pragma unroll
-                    for (int g = 0; g < G; ++g) {
-                        const int tg = min(tl + g, tpc - 1);
-                        v[g] = fmaf(recv[(r * tpc + tg) * BF + f], bars->scale[r < half ? 0 : 1][tg], v[g]);
-                    }
-                }
-                emit(ep, t, min(min(G, tpc - tl), M - t), col, in, bias, uw, v);
-                squares(v, tl, tpc - tl);
-            }
-        }
-        if (ep.u) {
-            named_sync(1, 32 * EW);
-            const int parts = (ep.N + 63) / 64;
-            for (int i = threadIdx.x - 64; i < 2 * tpc; i += 32 * EW) {      // (half of the tile, token)
-                const int hf = i / tpc, tl = i - hf * tpc, t = rank * tpc + tl;
-                if (t < M && n0 / 64 + hf < parts) ep.u_ssq[(int64_t)t * parts + n0 / 64 + hf] = bars->red[2 * hf][tl] + bars->red[2 * hf + 1][tl];
-            }
-        }
+    if ((warp < 2 || warp == 2 + EW) && cs > 1) {
+        __syncwarp();
+        cluster_sync();                                                      // (the epilogue warps' turn is after their sums are sent)
     }
     __syncwarp();
     fence_before();
@@ -293,9 +307,10 @@ cudaError_t gemm_rows_launch(const GemmArgs &a, const GemmArgs *b, bool sum, cud
     ra.tiles_n = (a.N + BF - 1) / BF;
     const int items = ra.tiles_n * (b && !sum ? 2 : 1), kblocks = (a.K + BK - 1) / BK, per = sum ? 2 : 1;      // per: products of a cluster
     const int slots = (ra.nt <= 64 ? 2 : 1) * sm_count();                    // (more tokens: the partial sums of a CTA take 40 KB and more)
-    // K shares: powers of two while the grid fits the GPU at once and a share keeps four steps
+    // K shares: powers of two while less than three fifths of the SMs have a CTA (beyond that the exchange costs more than the idle SMs: 90 and 126 CTAs beat 180 and 252), the grid fits
+    // the GPU at once and a share keeps four steps
     int ks = 1;
-    while (2 * ks * per <= MAX_CS && items * per * 2 * ks <= slots && kblocks >= 8 * ks && ra.nt % (2 * ks * per) == 0) ks *= 2;
+    while (items * per * ks < sm_count() * 3 / 5 && 2 * ks * per <= MAX_CS && items * per * 2 * ks <= slots && kblocks >= 8 * ks && ra.nt % (2 * ks * per) == 0) ks *= 2;
     ra.ks = ks;
     ra.cs = ks * per;
     uint32_t cols = 32;
@@ -303,8 +318,8 @@ cudaError_t gemm_rows_launch(const GemmArgs &a, const GemmArgs *b, bool sum, cud
     ra.tmem_cols = cols;
     const size_t stage = W_BYTES + (size_t)ra.nt * BK * 2, fixed = (ra.cs > 1 ? (size_t)ra.nt * BF * 4 : 0) + sizeof(Bars) + 1024;
     const int ctas = items * ra.cs;
-    // two CTAs per SM where there are that many and the stages stay at least three deep; else one CTA may use all of the SM, with twice the epilogue warps
-    const bool two = ctas > sm_count() && fixed + 3 * stage <= 113 * 1024;
+    // two CTAs per SM where there are that many and the stages stay at least three deep (four without partial sums: 128 x 50304 x 1920 lost 6 us with three); else one CTA may use all of the SM, with twice the epilogue warps
+    const bool two = ctas > sm_count() && fixed + (ra.cs == 1 ? 4 : 3) * stage <= 113 * 1024;
     const int stages = (int)(((two ? 113 : 226) * 1024 - fixed) / stage);
     ra.stages = stages > MAX_STAGES ? MAX_STAGES : stages;
     const size_t smem = fixed + ra.stages * stage;
@@ -317,7 +332,7 @@ cudaError_t gemm_rows_launch(const GemmArgs &a, const GemmArgs *b, bool sum, cud
     if (e != cudaSuccess) return e;
     int *status = device_status_ptr();
     if (!status) return cudaErrorUnknown;
-    return launch_chain(kern, dim3(ctas), dim3(two ? 192 : 320), smem, s, ra.cs, mx[0], mw[0], mx[1], mw[1], ra, status);
+    return launch_chain(kern, dim3(ctas), dim3(two ? 224 : 352), smem, s, ra.cs, mx[0], mw[0], mx[1], mw[1], ra, status);
 }
 
 }  // namespace dm

@@ -73,3 +73,9 @@ def test_linear_mixed_tile_widths(dm, M, N, K):
     """The two-CTA kernel with tiles of two widths: an incomplete last round cut into halves (rows or columns first in the tile order), a last column tile of 72 columns,
     both, with ragged rows; a column strip whose tiles start in the last round of wide ones."""
     test_linear_parity(dm, I.BF16, M, N, K)
+
+
+@pytest.mark.parametrize("M,N,K", [(32, 11264, 520), (33, 11392, 520), (128, 18900, 200), (100, 25000, 136), (5, 25000, 136)])
+def test_linear_few_rows_uncut_tiles(dm, M, N, K):
+    """Up to 128 rows around the line where K is no longer cut (88 and 89 tiles), one tile per SM, and more tiles than SMs with one and two CTAs on each."""
+    test_linear_parity(dm, I.BF16, M, N, K)
