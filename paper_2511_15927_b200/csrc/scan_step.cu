@@ -1,7 +1,7 @@
 // Fused conv + scan + gate for one block of up to 32 tokens per sequence (the active block of block-autoregressive decoding, Sec. 4.3): one launch, products
 // on mma.sync m16n8k16 tiles, with the identities of scan_ssd.cu over a single sub-chunk.
-// A CTA of 4 * PP threads takes several heads of one (batch row, direction), one after the other.  What the heads share -- B' and C' (conv + SiLU), S = C' B'^T,
-// and the decays, all from the raw in_proj rows -- it computes once; per head:
+// A CTA of 4 * PP threads takes several tiles (PP channels: a head, or two of 32) of one (batch row, direction), one after the other.  What the heads share -- B' and C' (conv + SiLU), S = C' B'^T,
+// and the decays, all from the raw in_proj rows -- it computes once; per tile:
 //   conv    x' = SiLU(conv(x)) as bf16 [j][p] (COMMIT: also w_j x'_j);  W_ij = S_ij 2^(Lambda_i - Lambda'_j) [+ D on the diagonal] for j not after i, else 0
 //   y       Yb = C' h^T (K = d_state; the B operand is packed from the fp32 state in shared memory), rows scaled by 2^Lambda_i, then += W x' into
 //           the same accumulators: warp = 16 tokens x 16 channels
@@ -20,24 +20,25 @@ namespace {
 
 using namespace ssd;
 
-// heads per CTA at most (their decays are kept)
+// tiles (of PP channels: a head, or two of half that width) per CTA at most: the decays of their heads are kept
 template <bool COMMIT> constexpr int HG_MAX = COMMIT ? 16 : 7;
 constexpr int KG = N / 16;             // 16-wide groups of states
 constexpr int XR = QB + 4;             // rows of a raw tile: three of history, one unused
 constexpr int SLD = QB + 4;            // row pitch (fp32) of S
 constexpr int WTL = QB + 8;            // row pitch (bf16) of W
 // CTAs per SM
-template <int PP, bool COMMIT> constexpr int RES = PP == 64 ? (COMMIT ? 2 : 3) : (COMMIT ? 3 : 4);
+template <int PP, int HW, bool COMMIT> constexpr int RES = PP == 32 ? (COMMIT ? 3 : 4) : COMMIT || HW == 32 ? 2 : 3;
 
-// Heads per CTA and CTAs per batch row of either direction
+// Tiles per CTA and CTAs per batch row of either direction
 struct StepSplit { int hg[2], groups[2]; };
 
-template <int PP, bool COMMIT> struct StepSmem {
+template <int PP, int HW, bool COMMIT> struct StepSmem {
+    static constexpr int HPT = PP / HW;            // heads per tile
     static constexpr int XLD = PP + 8;             // row pitch (bf16) of x' and w o x'
     static constexpr int XRAW = XR * PP * 2, NRAW = 2 * N / PP;            // a raw tile of PP channels; tiles of B and C
     static constexpr int STATE = KG * PP * 16 * 4;                         // [16-state group][p][16]; the raw B, C tiles before that
     static constexpr int st = 0, xr = st + (STATE > NRAW * XRAW ? STATE : NRAW * XRAW), ct = xr + XRAW, bt = ct + QB * NLD * 2, ss = bt + QB * NLD * 2, xt = ss + QB * SLD * 4,
-                         wt = xt + QB * XLD * 2, ys = wt + QB * WTL * 2, lam = ys + QB * PP * 4, bars = lam + HG_MAX<COMMIT> * 2 * QB * 4, wxt = bars + 64, total = wxt + (COMMIT ? QB * XLD * 2 : 0);
+                         wt = xt + QB * XLD * 2, ys = wt + HPT * QB * WTL * 2, lam = ys + QB * PP * 4, bars = lam + HG_MAX<COMMIT> * HPT * 2 * QB * 4, wxt = bars + 64, total = wxt + (COMMIT ? QB * XLD * 2 : 0);
     static_assert(xr % 128 == 0 && XRAW % 128 == 0, "TMA tiles");
     static_assert(ct % 16 == 0 && bt % 16 == 0 && ss % 16 == 0 && xt % 16 == 0 && wt % 16 == 0 && ys % 16 == 0 && lam % 16 == 0 && wxt % 16 == 0, "16-byte tiles");
 };
@@ -46,21 +47,21 @@ __device__ __forceinline__ void prefetch_3d(const CUtensorMap *map, int x, int y
     asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];" ::"l"(map), "r"(x), "r"(y), "r"(z) : "memory");
 }
 
-template <int PP, bool COMMIT>
-__global__ void __launch_bounds__(4 * PP, RES<PP, COMMIT>)
+template <int PP, int HW, bool COMMIT>
+__global__ void __launch_bounds__(4 * PP, RES<PP, HW, COMMIT>)
 ssd_step_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_s, const __grid_constant__ SsdArgs a, const StepSplit sp, int *status) {
-    using M = StepSmem<PP, COMMIT>;
-    constexpr int NT = 4 * PP, U8 = PP / 8, MT = PP / 16, XLD = M::XLD, CP2 = PP / 2;
+    using M = StepSmem<PP, HW, COMMIT>;
+    constexpr int HPT = M::HPT, NT = 4 * PP, U8 = PP / 8, MT = PP / 16, XLD = M::XLD, CP2 = PP / 2;
     extern __shared__ __align__(128) uint8_t sm[];
     __nv_bfloat16 (*Ct)[NLD] = reinterpret_cast<__nv_bfloat16 (*)[NLD]>(sm + M::ct);      // C' rows [i][n], columns permuted (see perm)
     __nv_bfloat16 (*Bt)[NLD] = reinterpret_cast<__nv_bfloat16 (*)[NLD]>(sm + M::bt);      // B' rows [j][n], likewise
     float (*Ss)[SLD] = reinterpret_cast<float (*)[SLD]>(sm + M::ss);
     __nv_bfloat16 (*Xt)[XLD] = reinterpret_cast<__nv_bfloat16 (*)[XLD]>(sm + M::xt);      // x' [j][p]
     __nv_bfloat16 (*WXt)[XLD] = reinterpret_cast<__nv_bfloat16 (*)[XLD]>(sm + M::wxt);    // w_j x'_j [j][p]   (COMMIT)
-    __nv_bfloat16 (*Wt)[WTL] = reinterpret_cast<__nv_bfloat16 (*)[WTL]>(sm + M::wt);      // W [i][j]
+    __nv_bfloat16 (*Wt)[QB][WTL] = reinterpret_cast<__nv_bfloat16 (*)[QB][WTL]>(sm + M::wt);      // W [i][j] of either head of the tile
     float (*ys)[PP] = reinterpret_cast<float (*)[PP]>(sm + M::ys);
     float (*lams)[2][QB] = reinterpret_cast<float (*)[2][QB]>(sm + M::lam);               // Lambda, Lambda' of every head
-    const float *Hs = reinterpret_cast<const float *>(sm + M::st);                        // incoming state: group g, channel p at (g * PP + p) * 16
+    const float *Hs = reinterpret_cast<const float *>(sm + M::st);                        // incoming state of the tile: group g, channel p at (g * PP + p) * 16
     const __nv_bfloat16 *xraw = reinterpret_cast<const __nv_bfloat16 *>(sm + M::xr);
     uint64_t *bar_bc = reinterpret_cast<uint64_t *>(sm + M::bars), *bar_x = bar_bc + 1, *bar_s = bar_bc + 2;
     volatile int *abort_flag = reinterpret_cast<volatile int *>(bar_bc + 3);
@@ -68,7 +69,7 @@ ssd_step_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, gr = lane >> 2, qc = lane & 3;
     // CTA -> (batch row, direction, group of heads)
     const int per = sp.groups[0] + sp.groups[1], b = blockIdx.x / per, j = blockIdx.x - b * per, dir = j >= sp.groups[0];
-    const int hg = dir ? sp.hg[1] : sp.hg[0], h0 = (dir ? j - sp.groups[0] : j) * hg, nh = min(hg, a.H - h0);
+    const int hg = dir ? sp.hg[1] : sp.hg[0], h0 = (dir ? j - sp.groups[0] : j) * hg, nh = min(hg, a.H / HPT - h0);       // h0, nh: tiles
     const bool rev = dir == 1;
     const int L = a.L, k = a.k;
     const int64_t seq = (int64_t)dir * a.B + b;
@@ -128,11 +129,12 @@ ssd_step_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
     // per-head registers: taps and carried rows of the thread's conv pair, gate and norm weights of its epilogue channels, D
     const int cp2 = tid % CP2, rg = tid / CP2;         // conv: channel pair, group of four rows
     const int ei = tid / U8, ec = (tid % U8) * 8;      // epilogue: token, first of 8 channels
-    struct Head { Taps t; uint4 z, nw; float D; uint32_t c[3]; };
+    struct Head { Taps t; uint4 z, nw; float D[HPT]; uint32_t c[3]; };
     auto weights_of = [&](Head &q, int h) {
         q.t = taps_of(h * PP + 2 * cp2);
         q.nw = norm_on ? __ldg(reinterpret_cast<const uint4 *>(static_cast<const __nv_bfloat16 *>(w.norm_w) + h * PP + ec)) : make_uint4(0x3F803F80u, 0x3F803F80u, 0x3F803F80u, 0x3F803F80u);
-        q.D = has_d ? __ldg(w.D + h) : 0.f;
+#pragma unroll
+        for (int e = 0; e < HPT; ++e) q.D[e] = has_d ? __ldg(w.D + h * HPT + e) : 0.f;
     };
     auto rows_of = [&](Head &q, int h) {               // (z holds SiLU(z): the in_proj epilogue applied it)
         q.z = ei < L ? __ldg(reinterpret_cast<const uint4 *>(zx + (int64_t)ei * a.d_in_proj + h * PP + ec)) : make_uint4(0u, 0u, 0u, 0u);
@@ -148,7 +150,7 @@ ssd_step_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
     };
     auto fetch_state = [&](int h) {                    // one thread
         mbar_expect_tx(bar_s, M::STATE);
-        tma_load_3d(sm + M::st, &map_s, 0, (b * a.H + h) * PP, 0, bar_s);
+        tma_load_3d(sm + M::st, &map_s, 0, (b * (a.H / HPT) + h) * PP, 0, bar_s);
     };
     // column of state n in the tiles of B' and C': within 16, a lane's operand values (2 q, 2 q + 1, 8 + 2 q, 9 + 2 q) are the states 4 q .. 4 q + 3
     auto perm = [](int n) { return (n & ~15) + ((n & 2) << 2) + ((n & 12) >> 1) + (n & 1); };
@@ -166,9 +168,9 @@ ssd_step_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
         *abort_flag = 0;
         mbar_fence_init();
         if (have_state)
-            for (int i = 0; i < nh; ++i) prefetch_3d(&map_s, 0, (b * a.H + h0 + i) * PP, 0);
+            for (int i = 0; i < nh; ++i) prefetch_3d(&map_s, 0, (b * (a.H / HPT) + h0 + i) * PP, 0);
     }
-    const float dtb0 = warp < nh ? w.dt_bias[h0 + warp] : 0.f, al0 = warp < nh ? w.A_log[h0 + warp] : 0.f;      // (its first head's)
+    const float dtb0 = warp < nh * HPT ? w.dt_bias[h0 * HPT + warp] : 0.f, al0 = warp < nh * HPT ? w.A_log[h0 * HPT + warp] : 0.f;      // (its first head's)
     pdl_wait();
     pdl_trigger();
     if (tid == 0) {
@@ -178,9 +180,9 @@ ssd_step_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
         fetch_x(h0);
     }
     // decays: a warp per head, lane = token in time order; Lambda of physical row r, log2 units (rows past the sequence have Delta = 0)
-    if (warp < nh) {
-        for (int hd = warp; hd < nh; hd += NT / 32) {
-            const int h = h0 + hd, r = rev ? QB - 1 - lane : lane;
+    if (warp < nh * HPT) {
+        for (int hd = warp; hd < nh * HPT; hd += NT / 32) {
+            const int h = h0 * HPT + hd, r = rev ? QB - 1 - lane : lane;
             const float d = r < L ? prep_delta(__bfloat162float(zx[(int64_t)r * a.d_in_proj + a.d_inner + a.conv_ch + h]), hd == warp ? dtb0 : w.dt_bias[h]) : 0.f;
             float cum = d * (-expf(hd == warp ? al0 : w.A_log[h]) * 1.4426950408889634f);
 #pragma unroll
@@ -228,44 +230,47 @@ ssd_step_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
     }
     // ================================================================ the heads
     for (int hd = 0; hd < nh; ++hd) {
-        const int h = h0 + hd;
-        const float *lam = lams[hd][0], *lamp = lams[hd][1];
+        const int h = h0 + hd;                                          // tile
+        const float (*lm)[2][QB] = &lams[hd * HPT];                     // Lambda, Lambda' of its heads
         if (hd + 1 < nh) { weights_of(nxt, h + 1); rows_of(nxt, h + 1); }
         mbar_wait(bar_x, hd & 1, abort_flag, status);
         // ---- conv: thread = channel pair, four rows
         {
             const uint32_t *xr = reinterpret_cast<const uint32_t *>(xraw) + rofs * (PP / 2) + cp2;
-            const float last = COMMIT ? lam[QB - 1] : 0.f;
+            const float (&lh)[2][QB] = lm[2 * cp2 / HW];
+            const float last = COMMIT ? lh[0][QB - 1] : 0.f;
             filter(cur.t, 4 * rg, 4, [&](int i) { return xr[i * (PP / 2)]; }, [&](int m) { return cur.c[m - 1]; }, [&](int i, f32x2 o) {
                 *reinterpret_cast<uint32_t *>(&Xt[i][2 * cp2]) = f2_to_bf2(o);
                 if (COMMIT && update) {
-                    const float wj = ex2f(last - lamp[i]);                 // rows past the sequence: 2^-inf = 0
+                    const float wj = ex2f(last - lh[1][i]);                 // rows past the sequence: 2^-inf = 0
                     *reinterpret_cast<uint32_t *>(&WXt[i][2 * cp2]) = f2_to_bf2(mul2(o, pk2(wj, wj)));
                 }
             });
         }
         if (hd == 0) __syncthreads();                                   // S is there
         // ---- mask: thread = (row i, four columns)
+#pragma unroll
+        for (int e = 0; e < HPT; ++e)
         for (int u = tid; u < QB * QB / 4; u += NT) {
             const int i = u >> 3, j0 = (u & 7) * 4;
-            const float li = lam[i];
-            const float4 s4 = *reinterpret_cast<const float4 *>(&Ss[i][j0]), lp4 = *reinterpret_cast<const float4 *>(lamp + j0);
+            const float li = lm[e][0][i];
+            const float4 s4 = *reinterpret_cast<const float4 *>(&Ss[i][j0]), lp4 = *reinterpret_cast<const float4 *>(&lm[e][1][j0]);
             const float sv[4] = {s4.x, s4.y, s4.z, s4.w}, lpv[4] = {lp4.x, lp4.y, lp4.z, lp4.w};
             float wv[4];
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 const int jj = j0 + q;
                 const bool ok = rev ? jj >= i : jj <= i;                // (rows past the sequence: Lambda' = inf)
-                wv[q] = fmaf(sv[q], ex2f(ok ? li - lpv[q] : -INFINITY), i == jj ? cur.D : 0.f);      // 2^-inf = 0: no branch around the exponential
+                wv[q] = fmaf(sv[q], ex2f(ok ? li - lpv[q] : -INFINITY), i == jj ? cur.D[e] : 0.f);      // 2^-inf = 0: no branch around the exponential
             }
-            *reinterpret_cast<uint2 *>(&Wt[i][j0]) = make_uint2(pack_bf16(wv[0], wv[1]), pack_bf16(wv[2], wv[3]));
+            *reinterpret_cast<uint2 *>(&Wt[e][i][j0]) = make_uint2(pack_bf16(wv[0], wv[1]), pack_bf16(wv[2], wv[3]));
         }
         if (have_state) mbar_wait(bar_s, hd & 1, abort_flag, status);
         __syncthreads();
         if (tid == 0 && hd + 1 < nh) fetch_x(h + 1);
         // ---- y: warp = tokens [16 ymt, +16) x channels [16 ynh, +16)
         {
-            const int ymt = warp & 1, ynh = warp >> 1;
+            const int ymt = warp & 1, ynh = warp >> 1, sub = 16 * ynh / HW;
             float acc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
             if (have_state) {
                 const float *hp = Hs + (16 * ynh + gr) * 16 + 4 * qc;
@@ -279,14 +284,14 @@ ssd_step_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
                         mma_bf16_16816(acc[nt], a0, a1, a2, a3, pack_bf16(v.x, v.y), pack_bf16(v.z, v.w));
                     }
                 }
-                const float e0 = ex2f(lam[16 * ymt + gr]), e1 = ex2f(lam[16 * ymt + gr + 8]);
+                const float e0 = ex2f(lm[sub][0][16 * ymt + gr]), e1 = ex2f(lm[sub][0][16 * ymt + gr + 8]);
 #pragma unroll
                 for (int nt = 0; nt < 2; ++nt) { acc[nt][0] *= e0; acc[nt][1] *= e0; acc[nt][2] *= e1; acc[nt][3] *= e1; }
             }
 #pragma unroll
             for (int k0 = 0; k0 < QB; k0 += 16) {
                 uint32_t a0, a1, a2, a3, b0, b1, b2, b3;
-                ldmatrix_x4(a0, a1, a2, a3, &Wt[16 * ymt + (lane & 15)][k0 + (lane >> 4) * 8]);
+                ldmatrix_x4(a0, a1, a2, a3, &Wt[sub][16 * ymt + (lane & 15)][k0 + (lane >> 4) * 8]);
                 ldmatrix_x4_t(b0, b1, b2, b3, &Xt[k0 + (lane & 15)][16 * ynh + (lane >> 4) * 8]);
                 mma_bf16_16816(acc[0], a0, a1, a2, a3, b0, b1);
                 mma_bf16_16816(acc[1], a0, a1, a2, a3, b2, b3);
@@ -301,7 +306,7 @@ ssd_step_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
         if (COMMIT && update) {
             // ---- state after the block: channels [16 smt, +16) x states [64 snh, +64) per warp; a lane's values of a 16-state group are four consecutive states
             const int smt = warp % MT, snh = warp / MT, p0 = 16 * smt + gr;
-            const float dec = ex2f(lam[QB - 1]);
+            const float dec = ex2f(lm[16 * smt / HW][0][QB - 1]);
             float acc[8][4];
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
@@ -326,7 +331,7 @@ ssd_step_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
                     mma_bf16_16816(acc[2 * u + 1], a0, a1, a2, a3, b2, b3);
                 }
             }
-            float *ho = a.ssm_out + (((int64_t)b * a.H + h) * PP + p0) * a.Nr + 4 * qc;
+            float *ho = a.ssm_out + (((int64_t)b * (a.H / HPT) + h) * PP + p0) * a.Nr + 4 * qc;
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 const int n = 64 * snh + 16 * u;
@@ -348,11 +353,11 @@ ssd_step_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
 #pragma unroll
             for (int e = 0; e < 8; ++e) { g[e] = yv[e] * zf[e]; sq = fmaf(g[e], g[e], sq); g[e] *= nw[e]; }
 #pragma unroll
-            for (int off = 1; off < U8; off <<= 1) sq += __shfl_xor_sync(0xffffffffu, sq, off);
+            for (int off = 1; off < U8 / HPT; off <<= 1) sq += __shfl_xor_sync(0xffffffffu, sq, off);
             if (ei < L) {
                 *reinterpret_cast<uint4 *>(a.g + (seq * L + ei) * a.d_inner + h * PP + ec) =
                     make_uint4(pack_bf16(g[0], g[1]), pack_bf16(g[2], g[3]), pack_bf16(g[4], g[5]), pack_bf16(g[6], g[7]));
-                if (a.ssq && ec == 0) a.ssq[(seq * L + ei) * a.H + h] = sq;
+                if (a.ssq && ec % HW == 0) a.ssq[(seq * L + ei) * a.H + h * HPT + ec / HW] = sq;
             }
         }
         cur = nxt;
@@ -373,10 +378,11 @@ bool make_map_plain(CUtensorMap *m, CUtensorMapDataType t, int es, const void *b
                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int PP, bool COMMIT>
+template <int PP, int HW, bool COMMIT>
 cudaError_t launch(const SsdArgs &a, int ndir, int dir0, cudaStream_t s) {
-    using M = StepSmem<PP, COMMIT>;
-    static_assert((M::total + 1024) * RES<PP, COMMIT> <= 233472, "the CTAs of an SM fit its shared memory");
+    using M = StepSmem<PP, HW, COMMIT>;
+    const int tiles = a.H / M::HPT;
+    static_assert((M::total + 1024) * RES<PP, HW, COMMIT> <= 233472, "the CTAs of an SM fit its shared memory");
     int *status = device_status_ptr();
     if (!status) return cudaErrorUnknown;
     CUtensorMap mx, ms{};
@@ -386,35 +392,35 @@ cudaError_t launch(const SsdArgs &a, int ndir, int dir0, cudaStream_t s) {
         if (!make_map_plain(&mx, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, a.zx, d, st, box)) return cudaErrorInvalidValue;
     }
     if (a.ssm_in) {                                  // [16-state group][row][16]
-        const cuuint64_t d[3] = {16, (cuuint64_t)a.B * a.H * PP, (cuuint64_t)a.Nr / 16}, st[2] = {(cuuint64_t)a.Nr, 16};
+        const cuuint64_t d[3] = {16, (cuuint64_t)a.B * tiles * PP, (cuuint64_t)a.Nr / 16}, st[2] = {(cuuint64_t)a.Nr, 16};
         const cuuint32_t box[3] = {16, PP, KG};
         if (!make_map_plain(&ms, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, a.ssm_in, d, st, box)) return cudaErrorInvalidValue;
     }
-    cudaError_t e = cudaFuncSetAttribute(ssd_step_kernel<PP, COMMIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, M::total);
+    cudaError_t e = cudaFuncSetAttribute(ssd_step_kernel<PP, HW, COMMIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, M::total);
     if (e != cudaSuccess) return e;
     // As many CTAs as are resident at once, so that what the heads share is computed as seldom as one round allows, and shared out between the directions by what a head costs:
     // a left-to-right one reads its state, and with COMMIT writes it (16 sequences of 64 heads: 4.0 us against 2.8, and 4.2 against 1.9; with equal shares the SMs that happened to
     // get left-to-right CTAs only finished at 27 and 43 us, the others at 19 and 18;
     // one layer with the state committed 103 -> 96 us, 24 layers 2191 -> 2118 us).
     StepSplit sp{};
-    const int slots = sm_count() * RES<PP, COMMIT> / a.B, cap = HG_MAX<COMMIT>;
+    const int slots = sm_count() * RES<PP, HW, COMMIT> / a.B, cap = HG_MAX<COMMIT>;
     const int cost[2] = {!a.ssm_in && !COMMIT ? 10 : COMMIT ? 22 : 14, 10};
-    auto groups_of = [&](int hg) { return (a.H + hg - 1) / hg; };
+    auto groups_of = [&](int hg) { return (tiles + hg - 1) / hg; };
     if (ndir == 1) {
-        const int most = slots < 1 ? 1 : slots > a.H ? a.H : slots, hg = groups_of(most);
+        const int most = slots < 1 ? 1 : slots > tiles ? tiles : slots, hg = groups_of(most);
         sp.hg[dir0] = hg > cap ? cap : hg;
     } else {
         int best = 0;
         for (int f = 1; f <= cap; ++f) {                 // heads per left-to-right CTA
             const int left = slots - groups_of(f);
             if (left < 1) continue;
-            const int r = groups_of(left > a.H ? a.H : left), t = f * cost[0] > r * cost[1] ? f * cost[0] : r * cost[1];
+            const int r = groups_of(left > tiles ? tiles : left), t = f * cost[0] > r * cost[1] ? f * cost[0] : r * cost[1];
             if (r <= cap && (!best || t < best)) { best = t; sp.hg[0] = f; sp.hg[1] = r; }
         }
         if (!best) { sp.hg[1] = cap; sp.hg[0] = cap * cost[1] / cost[0]; }      // more than one round
     }
     for (int d = 0; d < 2; ++d) sp.groups[d] = sp.hg[d] ? groups_of(sp.hg[d]) : 0;
-    return launch_chain(ssd_step_kernel<PP, COMMIT>, dim3((sp.groups[0] + sp.groups[1]) * a.B), 4 * PP, M::total, s, 0, mx, ms, a, sp, status);
+    return launch_chain(ssd_step_kernel<PP, HW, COMMIT>, dim3((sp.groups[0] + sp.groups[1]) * a.B), 4 * PP, M::total, s, 0, mx, ms, a, sp, status);
 }
 
 }  // namespace
@@ -425,8 +431,10 @@ bool scan_step_supports(const ssd::SsdArgs &a) {
 
 cudaError_t scan_step(const ssd::SsdArgs &a, int headdim, int ndir, int dir0, cudaStream_t s) {
     const bool commit = a.ssm_out != nullptr;
-    if (headdim == 64) return commit ? launch<64, true>(a, ndir, dir0, s) : launch<64, false>(a, ndir, dir0, s);
-    return commit ? launch<32, true>(a, ndir, dir0, s) : launch<32, false>(a, ndir, dir0, s);
+    if (headdim == 64) return commit ? launch<64, 64, true>(a, ndir, dir0, s) : launch<64, 64, false>(a, ndir, dir0, s);
+    // heads of 32: two to a tile, so that eight warps share the work that all heads have in common (24 layers, 120 heads, one sequence: 848 -> 794 us, four: 689 -> 656 us in 16 layers)
+    if (a.H % 2 == 0) return commit ? launch<64, 32, true>(a, ndir, dir0, s) : launch<64, 32, false>(a, ndir, dir0, s);
+    return commit ? launch<32, 32, true>(a, ndir, dir0, s) : launch<32, 32, false>(a, ndir, dir0, s);
 }
 
 }  // namespace dm

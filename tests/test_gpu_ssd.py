@@ -184,12 +184,12 @@ def test_half_width_heads_single_and_paired(G, H, L):
     assert G.rel_l2(s_out, s_o) <= BF16_REL and G.rel_l2(c_out, c_o) <= BF16_REL
 
 
-@pytest.mark.parametrize("B,H,P,N,L,k", [(2, 8, 64, 128, 1, 4), (1, 8, 64, 128, 32, 2), (64, 24, 64, 16, 31, 4), (64, 24, 32, 128, 32, 4), (3, 8, 32, 16, 5, 3)])
+@pytest.mark.parametrize("B,H,P,N,L,k", [(2, 8, 64, 128, 1, 4), (1, 8, 64, 128, 32, 2), (64, 24, 64, 16, 31, 4), (64, 24, 32, 128, 32, 4), (3, 8, 32, 16, 5, 3), (2, 7, 32, 32, 32, 4)])
 def test_blocks_of_up_to_32_tokens(G, B, H, P, N, L, k):
-    """The one-launch kernel of short blocks: its smallest and largest block, padded d_state, both head widths, one head per CTA and several (24 heads in groups of
+    """The one-launch kernel of short blocks: its smallest and largest block, padded d_state, both head widths (32: two heads a tile, and one where their number is odd), one head per CTA and several (24 heads in groups of
     7, the last of 3; 64 batch rows take more than one round), with the state committed, read only, and absent."""
     shape = I.MixerShape(B, L, P * H // 2, 2, N, k, H)
-    assert shape.headdim == P and shape.d_in_proj % 8 == 0
+    assert shape.headdim == P
     wf, wr = I.make_mixer_weights(shape, 60 + L, I.BF16, perturb=True)
     x = I.make_activations(shape, 60 + L, I.BF16)
     kw = G.oracle_kwargs(shape)
