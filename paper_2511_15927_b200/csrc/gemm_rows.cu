@@ -10,6 +10,8 @@
 //
 // Warp 0 issues the TMA loads, warp 1 the MMAs, the next EW (4 or 8) are the epilogue and a last one brings its code: one TMEM lane quarter each, tokens shared out between the two
 // warps of a quarter.  Waits and abort as in gemm_pair.cu: every mbarrier wait is bounded, and the CTAs of a cluster leave together.
+#include <array>
+
 #include "gemm_epi.cuh"
 
 namespace dm {
@@ -297,6 +299,26 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap map_x0, const __grid_consta
 
 }  // namespace
 
+// Clusters of 2^i CTAs that are resident at once with one CTA per SM (of eight: 15 on 148 SMs; the GPU's parts hold uneven numbers of SMs).
+static int resident_clusters(int cs) {
+    static const std::array<int, 4> n = [] {
+        std::array<int, 4> r{};
+        const int smem = 226 * 1024;
+        if (cudaFuncSetAttribute(gemm_rows_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return r;
+        for (int i = 0; i < 4; ++i) {
+            cudaLaunchConfig_t cfg{};
+            cfg.gridDim = dim3(1 << i); cfg.blockDim = dim3(352); cfg.dynamicSmemBytes = smem;
+            cudaLaunchAttribute at;
+            at.id = cudaLaunchAttributeClusterDimension;
+            at.val.clusterDim.x = 1 << i; at.val.clusterDim.y = 1; at.val.clusterDim.z = 1;
+            cfg.attrs = &at; cfg.numAttrs = 1;
+            if (cudaOccupancyMaxActiveClusters(&r[i], gemm_rows_kernel<8>, &cfg) != cudaSuccess) r[i] = 0;
+        }
+        return r;
+    }();
+    return n[cs == 8 ? 3 : cs == 4 ? 2 : cs == 2 ? 1 : 0];
+}
+
 // b == NULL: one product; sum: s_a A_a B_a^T + s_b A_b B_b^T into b's output; else two products of equal sizes side by side.
 cudaError_t gemm_rows_launch(const GemmArgs &a, const GemmArgs *b, bool sum, cudaStream_t s) {
     RowsArgs ra{};
@@ -311,15 +333,24 @@ cudaError_t gemm_rows_launch(const GemmArgs &a, const GemmArgs *b, bool sum, cud
     // the GPU at once and a share keeps four steps
     int ks = 1;
     while (items * per * ks < sm_count() * 3 / 5 && 2 * ks * per <= MAX_CS && items * per * 2 * ks <= slots && kblocks >= 8 * ks && ra.nt % (2 * ks * per) == 0) ks *= 2;
-    ra.ks = ks;
-    ra.cs = ks * per;
     uint32_t cols = 32;
     while (cols < (uint32_t)ra.nt) cols *= 2;
     ra.tmem_cols = cols;
-    const size_t stage = W_BYTES + (size_t)ra.nt * BK * 2, fixed = (ra.cs > 1 ? (size_t)ra.nt * BF * 4 : 0) + sizeof(Bars) + 1024;
+    // Two CTAs per SM where not all clusters are resident with one and the stages stay at least three deep (four without partial sums: 128 x 50304 x 1920 lost 6 us with three);
+    // else one CTA may use all of the SM, with twice the epilogue warps, and a cut of K that does not fit one round is halved.  (16 clusters of eight CTAs, the summed
+    // out_proj of d_model 2048, ran in two rounds: 24 layers of 32 tokens 1003 -> 846 us, one layer of 100 tokens 53 -> 47 us.)
+    const size_t stage = W_BYTES + (size_t)ra.nt * BK * 2;
+    size_t fixed;
+    bool two;
+    for (;; ks /= 2) {
+        ra.ks = ks;
+        ra.cs = ks * per;
+        fixed = (ra.cs > 1 ? (size_t)ra.nt * BF * 4 : 0) + sizeof(Bars) + 1024;
+        const bool fits = items <= resident_clusters(ra.cs);
+        two = !fits && fixed + (ra.cs == 1 ? 4 : 3) * stage <= 113 * 1024;
+        if (fits || two || ks == 1) break;
+    }
     const int ctas = items * ra.cs;
-    // two CTAs per SM where there are that many and the stages stay at least three deep (four without partial sums: 128 x 50304 x 1920 lost 6 us with three); else one CTA may use all of the SM, with twice the epilogue warps
-    const bool two = ctas > sm_count() && fixed + (ra.cs == 1 ? 4 : 3) * stage <= 113 * 1024;
     const int stages = (int)(((two ? 113 : 226) * 1024 - fixed) / stage);
     ra.stages = stages > MAX_STAGES ? MAX_STAGES : stages;
     const size_t smem = fixed + ra.stages * stage;

@@ -101,6 +101,13 @@ def test_short_input_out_proj_paths_bf16(G, B, L, d, H):
     _check(got0, O.bimamba_forward(x, wf, wr, **G.oracle_kwargs(shape, flags=dm_flags_no_norm())), I.BF16)
 
 
+@pytest.mark.parametrize("B,L", [(1, 32), (2, 50)])
+def test_few_rows_out_proj_rounds_bf16(G, B, L):
+    """The summed out_proj of d_model 2048 for up to 128 rows: 16 clusters of eight CTAs are more than fit one CTA to an SM, so that two share one (32 tokens) or the
+    cut of K is halved (100 tokens, whose partial sums leave no room for two)."""
+    test_short_input_out_proj_paths_bf16(G, B, L, 2048, 64)
+
+
 def dm_flags_no_norm():
     from paper_2511_15927_b200 import binding as dm
     return dm.DM_FLAGS_DEFAULT & ~dm.DM_FLAG_GATED_RMSNORM
