@@ -68,6 +68,25 @@ def test_linear_epilogue_scale_addend_inplace(dm, dtype, shape):
     np.testing.assert_allclose(yd.cpu().numpy().astype(np.float64), want, rtol=1e-5, atol=1e-5)
 
 
+@pytest.mark.parametrize("y_dtype", [I.BF16, I.F32])
+@pytest.mark.parametrize("M,N", [(100, 300), (128, 64), (129, 32), (129, 64), (129, 100), (300, 300), (256, 520), (333, 40), (2304, 1096)])
+def test_linear_separate_addend(dm, y_dtype, M, N):
+    """An addend that is not the output, both output types: every epilogue of the tensor-core kernels (up to 128 rows; rows of 16-byte pieces, whole and cut short
+    inside a group of 64 columns and of 32; rows that are not)."""
+    from paper_2511_15927_b200.torch_io import dev, dm_dtype, tdtype
+    K = 136
+    x = _rand((M, K), 7, I.BF16); w = _rand((N, K), 8, I.BF16, 0.05)
+    sc = np.random.default_rng(9).uniform(0.5, 2.0, M).astype(np.float32)
+    add = np.random.default_rng(10).standard_normal((M, N)).astype(np.float32)
+    xd, wd, scd, addd = dev(x, I.BF16), dev(w, I.BF16), dev(sc), dev(add)
+    yd = torch.full((M, N), float("nan"), device="cuda", dtype=tdtype(y_dtype))
+    dm.dm_linear(dm.DM_BF16, xd.data_ptr(), wd.data_ptr(), yd.data_ptr(), dm_dtype(y_dtype), M, K, N, scd.data_ptr(), addd.data_ptr(), torch.cuda.current_stream().cuda_stream)
+    dm.dm_check(0)
+    want = sc[:, None].astype(np.float64) * O.out_proj(x, w) + add
+    # bf16: half a unit in the last place (2^-9 of the value) beside the fp32 sums' error
+    np.testing.assert_allclose(yd.double().cpu().numpy(), want, rtol=2.0 ** -8 if y_dtype == I.BF16 else 1e-5, atol=1e-5)
+
+
 @pytest.mark.parametrize("M,N,K", [(6400, 768, 72), (6300, 840, 136), (9728, 2048, 64), (2048, 9728, 456), (600, 24960, 64)])
 def test_linear_mixed_tile_widths(dm, M, N, K):
     """The two-CTA kernel with tiles of two widths: an incomplete last round cut into halves (rows or columns first in the tile order), a last column tile of 72 columns,

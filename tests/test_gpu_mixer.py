@@ -108,6 +108,12 @@ def test_few_rows_out_proj_rounds_bf16(G, B, L):
     test_short_input_out_proj_paths_bf16(G, B, L, 2048, 64)
 
 
+@pytest.mark.parametrize("B,L,d,H", [(1, 201, 96, 3), (1, 77, 96, 3), (3, 683, 160, 5), (2, 1001, 480, 15)])
+def test_out_proj_with_ragged_sums_of_squares_bf16(G, B, L, d, H):
+    """B L H not a multiple of 4: the right-to-left layer's sums of squares do not start on a 16-byte boundary."""
+    test_short_input_out_proj_paths_bf16(G, B, L, d, H)
+
+
 def dm_flags_no_norm():
     from paper_2511_15927_b200 import binding as dm
     return dm.DM_FLAGS_DEFAULT & ~dm.DM_FLAG_GATED_RMSNORM
