@@ -402,11 +402,12 @@ cudaError_t scan_sequential(const ScanArgs &a, void *ws, cudaStream_t s) {
     int *status = device_status_ptr();
     if (!status) return cudaErrorUnknown;
     float *bc = static_cast<float *>(ws);
-    const int tasks = (a.L + BC_ROWS - 1) / BC_ROWS * 2 * a.N, bt = tasks >= 256 * 148 ? 256 : 64;        // small CTAs while they do not fill the GPU
+    const int tasks = (a.L + BC_ROWS - 1) / BC_ROWS * 2 * a.N, bt = tasks >= 256 * sm_count() ? 256 : 64;        // small CTAs while they do not fill the GPU
     dim3 pgrid((tasks + bt - 1) / bt, a.B, ndir);
     e = a.dtype == DM_BF16 ? launch_chain(bc_prep_kernel<__nv_bfloat16>, pgrid, bt, 0, s, 0, a, dir0, bc) : launch_chain(bc_prep_kernel<float>, pgrid, bt, 0, s, 0, a, dir0, bc);
     if (e != cudaSuccess) return e;
     dim3 grid(a.H, ndir, a.B);
+    chain_spread((int64_t)pgrid.x * pgrid.y * pgrid.z, sm_count());
     return launch_chain(kern, grid, a.P * lanes_per_channel(a.N) + loaders(a.P, a.N), smem, s, 0, mx, mz, a, dir0, TC, bc, status);
 }
 

@@ -1331,6 +1331,7 @@ cudaError_t scan_ssd(const ScanArgs &a, void *ws, cudaStream_t s) {
         const size_t smem = a.P == P ? BlockSmem<P>::total : BlockSmem<P / 2>::total;
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
+        chain_spread((int64_t)pgrid.x * pgrid.y * pgrid.z, sm_count());
         return launch_chain(kern, dim3(a.H, ndir, a.B), 4 * a.P, smem, s, 0, k, Bp, Cp, Sb, dir0);
     }
 

@@ -179,6 +179,11 @@ def test_chunk_size_invariance_bf16(G, L, P):
         assert e.value.status == dm.DM_ERR_UNSUPPORTED
 
 
+def test_short_chunks_after_a_prep_grid_that_fills_the_gpu_bf16(G):
+    """chunk = 32 over a length whose prep launch has more CTAs than there are SMs: the scan then follows it without overlap."""
+    test_chunk_size_invariance_bf16(G, 4100, 64)
+
+
 def test_run_to_run_determinism(G):
     shape = I.MixerShape(2, 200, 128, 2, 128, 4, 4)
     wf, wr, x = _case(shape, I.BF16, seed=8)
