@@ -1,6 +1,6 @@
 // Bidirectional multi-head attention for the hybrid variant (Sec. 3.3: one attention mixer every N mixer blocks):
 //     O_h = softmax(Q_h K_h^T / sqrt(d_h)) V_h        full (non-causal), no position encoding, d_h = 64 or 80.
-// One CTA per (256 queries, head, sequence), as two streams of 128 queries that share the key and value tiles; the running-maximum form
+// One CTA per (256 queries, head, sequence), as two streams (NS = 2) of 128 queries that share the key and value tiles; the running-maximum form
 // of the softmax, so the L x L score matrix never leaves the SM:
 //     warp 0       TMA loads: the two Q tiles once, K and V tiles through a ring
 //     warp 1       issues, per key tile and stream, S = Q K^T (both operands K-major in shared memory, fp32 accumulator in TMEM) and
@@ -17,8 +17,12 @@
 // channels 0..63 and the 64 columns from channel 64 on, of which the products use the first 16 (the rest belongs to the next head, or is
 // the zero fill beyond the tensor, and is never read): one more K step of 16 for S, one more product of 16 columns for O.  Key tiles of 96 there:
 // S, P and O of two streams then fit the 512 TMEM columns.
+// The last CTA of a sequence may have queries for its first stream only: the second one then issues and computes nothing.
+// Up to 128 queries per sequence, more (head, sequence) pairs than SMs: CTAs of one stream, key tiles of 64, two to an SM, so that one's set-up and latencies are covered by the other.
+// 16 sequences, 16 heads of 64, a block of 100 after 2048 keys, projections included: 97 us with both streams running, 80 without the empty one, 68 with one stream
+// (64 sequences: 153, 137, 119 for 128 after 512 keys).  Fewer pairs: the two-stream form, whose larger key tiles take fewer steps (1 sequence, 8192 keys: 97 us against 112).
 // Every wait is bounded; on expiry the CTA stores DM_ERR_TIMEOUT in the device status word and leaves.
-// Few queries (block decoding) go to attention_block.cu.
+// Few queries (block decoding) go to attention_block.cu where block_pays says so.
 #include "dm_internal.h"
 #include "tc_ptx.cuh"
 
@@ -26,16 +30,16 @@ namespace dm {
 using namespace tc;
 namespace {
 
-constexpr int BQ = 128, SUB = 64, NTHREADS = 384;           // SUB: columns of a sub-tile (128 bytes: one swizzle atom)
+constexpr int BQ = 128, SUB = 64;                           // SUB: columns of a sub-tile (128 bytes: one swizzle atom)
 constexpr float RESCALE_LOG2 = 8.f;
 
-// NT: sub-tiles per operand tile; 1 = heads of 64 channels, 2 = heads of 80
-template <int NT> struct Cfg {
-    static constexpr int DH = NT == 1 ? 64 : 80, BK = NT == 1 ? 128 : 96, STAGES = NT == 1 ? 4 : 3;
+// NT: sub-tiles per operand tile; 1 = heads of 64 channels, 2 = heads of 80.  NS: query streams
+template <int NT, int NS> struct Cfg {
+    static constexpr int DH = NT == 1 ? 64 : 80, BK = NS == 1 ? 64 : NT == 1 ? 128 : 96, STAGES = NT == 1 ? 4 : NS == 1 ? 2 : 3, NTHREADS = 128 + 128 * NS;
     static constexpr uint32_t QTILE = BQ * 128, KTILE = BK * 128, Q_BYTES = NT * QTILE, KV_BYTES = NT * KTILE;
-    static constexpr uint32_t OFF_K = 2 * Q_BYTES, OFF_V = OFF_K + STAGES * KV_BYTES, OFF_BAR = OFF_V + STAGES * KV_BYTES, SMEM = OFF_BAR + 1024 + 1024;
-    static constexpr uint32_t TM_P = 2 * BK, TM_O = TM_P + BK;               // S of stream s at s BK, its P at TM_P + s BK / 2, its O at TM_O + s DH
-    static_assert(TM_O + 2 * DH <= 512 && SMEM <= 232448, "TMEM and shared memory budget");
+    static constexpr uint32_t OFF_K = NS * Q_BYTES, OFF_V = OFF_K + STAGES * KV_BYTES, OFF_BAR = OFF_V + STAGES * KV_BYTES, SMEM = OFF_BAR + 1024 + 1024;
+    static constexpr uint32_t TM_P = NS * BK, TM_O = TM_P + NS * BK / 2, TM_COLS = 256 * NS;      // S of stream s at s BK, its P at TM_P + s BK / 2, its O at TM_O + s DH
+    static_assert(TM_O + NS * DH <= TM_COLS && SMEM * (3 - NS) <= 232448, "TMEM and shared memory budget");
 };
 
 struct Bars {
@@ -51,19 +55,19 @@ struct AttnArgs {
     float scale_log2;            // log2(e) / sqrt(d_h)
 };
 
-template <int NT>
-__global__ void __launch_bounds__(NTHREADS, 1)
+template <int NT, int NS>
+__global__ void __launch_bounds__(Cfg<NT, NS>::NTHREADS, 3 - NS)
 attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                  const __grid_constant__ CUtensorMap map_v, const AttnArgs a, int *status) {
-    using C = Cfg<NT>;
+    using C = Cfg<NT, NS>;
     constexpr int DH = C::DH, BK = C::BK, STAGES = C::STAGES;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
     Bars *bars = reinterpret_cast<Bars *>(smem + C::OFF_BAR);
     volatile int *abort_flag = &bars->abort;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int q0 = blockIdx.x * 2 * BQ, h = blockIdx.y, b = blockIdx.z;
-    const int n_kv = (a.Lk + BK - 1) / BK;
+    const int q0 = blockIdx.x * NS * BQ, h = blockIdx.y, b = blockIdx.z;
+    const int n_kv = (a.Lk + BK - 1) / BK, ns = NS == 2 && a.Lq - q0 > BQ ? 2 : 1;      // streams that have queries
 
     if (tid == 0) {
         mbar_init(&bars->q_full, 1);
@@ -78,7 +82,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         bars->abort = 0;
         mbar_fence_init();
     }
-    if (warp == 1) tmem_alloc(&bars->tmem_base, 512);
+    if (warp == 1) tmem_alloc(&bars->tmem_base, C::TM_COLS);
     fence_before();
     __syncthreads();
     fence_after();
@@ -90,9 +94,8 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     if (warp == 0) {
         // ------------------------------------------------------------ TMA producer
         if (lane == 0) {
-            mbar_expect_tx(&bars->q_full, 2 * C::Q_BYTES);
-#pragma unroll
-            for (int i = 0; i < 2; ++i)
+            mbar_expect_tx(&bars->q_full, ns * C::Q_BYTES);
+            for (int i = 0; i < ns; ++i)
 #pragma unroll
                 for (int u = 0; u < NT; ++u) tma_load_3d(smem + i * C::Q_BYTES + u * C::QTILE, &map_q, h * DH + u * SUB, q0 + i * BQ, b, &bars->q_full);
             int issued_k = 0, issued_v = 0;
@@ -131,7 +134,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
                 for (int kk = 1; kk < 4; ++kk) umma_ss<1>(ts, dQ + 2 * kk, dK + 2 * kk, I_S);
                 if constexpr (NT == 2) umma_ss<1>(ts, dQ + (C::QTILE >> 4), dK + (C::KTILE >> 4), I_S);      // channels 64..79: one K step of the second sub-tiles
                 umma_commit(&bars->s_full[s]);
-                if (s == 1) umma_commit(&bars->k_empty[j % STAGES]);
+                if (s == ns - 1) umma_commit(&bars->k_empty[j % STAGES]);
             }
             __syncwarp();
             return true;
@@ -151,19 +154,19 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
                     for (int kk = 1; kk < BK / 16; ++kk) umma_ts<1>(to + 64, tp + 8 * kk, dV2 + kk * 128, I_O16);
                 }
                 umma_commit(&bars->o_done[s]);            // phase j: O holds tiles 0..j and P(j) has been read
-                if (s == 1) umma_commit(&bars->v_empty[j % STAGES]);
+                if (s == ns - 1) umma_commit(&bars->v_empty[j % STAGES]);
             }
             __syncwarp();
             return true;
         };
-        bool ok = WAIT(&bars->q_full, 0) && WAIT(&bars->k_full[0], 0) && issue_s(0, 0) && issue_s(0, 1);
+        bool ok = WAIT(&bars->q_full, 0) && WAIT(&bars->k_full[0], 0) && issue_s(0, 0) && (ns < 2 || issue_s(0, 1));
         for (int j = 0; j < n_kv && ok; ++j) {
             const bool more = j + 1 < n_kv;
             if (more) ok = WAIT(&bars->k_full[(j + 1) % STAGES], ((j + 1) / STAGES) & 1);
             ok = ok && WAIT(&bars->v_full[j % STAGES], (j / STAGES) & 1);
-            for (int s = 0; s < 2 && ok; ++s) ok = (!more || issue_s(j + 1, s)) && issue_pv(j, s);
+            for (int s = 0; s < ns && ok; ++s) ok = (!more || issue_s(j + 1, s)) && issue_pv(j, s);
         }
-    } else if (warp >= 4) {
+    } else if (warp >= 4 && warp < 4 + 4 * ns) {
         // ------------------------------------------------------------ softmax, O scaling, output
         const int s = (warp - 4) >> 2;                            // stream
         const int q = warp & 3;                                   // TMEM lane quarter of this warp
@@ -261,7 +264,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     __syncthreads();
     if (warp == 1) {
         fence_after();
-        tmem_dealloc(tmem, 512);
+        tmem_dealloc(tmem, C::TM_COLS);
     }
 }
 
@@ -281,6 +284,15 @@ bool attention_supports(int dtype, int d, int n_heads) {
     return dtype == DM_BF16 && n_heads > 0 && (d == n_heads * 64 || d == n_heads * 80) && encode_fn() != nullptr;
 }
 
+// Few queries: which kernel.  attention_block.cu splits the keys of a (head, sequence) over the GPU, but its products run on mma.sync, for blocks of 32 queries that each read all keys; the
+// kernel above takes 128 queries at the price of 33, with a CTA per pair.  Measured, projections included (block kernel / this one), by pairs, 148 SMs:
+//   48 queries after 2048 keys, heads of 64: 64 pairs 41 / 43 us, 128 57 / 47, 256 93 / 60, 1024 277 / 155; heads of 80: 48 pairs 49 / 48, 96 74 / 53, 384 163 / 103
+//   32 queries, 512 pairs of 64: 66 / 60 us after 512 keys, 105 / 101 after 2048, 259 / 269 after 8192; 384 pairs of 80: 65 / 59, 108 / 104, 278 / 274
+static bool block_pays(int64_t pairs, int Lq, int Lk) {
+    if (Lq > ATTN_BLOCK_MAX_Q) return false;
+    return Lq > 32 ? 8 * pairs < 5 * sm_count() : pairs <= 2 * sm_count() || Lk > 4096;
+}
+
 // qkv [B*Lq, 3 d] bf16 (columns [Q | K | V], heads contiguous inside each), out [B*Lq, d] bf16.
 // k_cache == NULL: keys and values are the K and V columns of qkv (Lk = Lq).  Otherwise the block's keys and values are
 // first appended at rows [cache_len, cache_len + Lq) of k_cache, v_cache [B, cache_cap, d], and the queries attend to the
@@ -290,11 +302,13 @@ cudaError_t attention_forward(const void *qkv, void *out, int B, int Lq, int d, 
     if (!attention_supports(DM_BF16, d, n_heads) || B <= 0 || Lq <= 0 || B > 65535 || n_heads > 65535) return cudaErrorNotSupported;
     const bool cached = k_cache != nullptr;
     if (cached && (!v_cache || cache_len < 0 || cache_len + Lq > cache_cap)) return cudaErrorInvalidValue;
-    if (Lq <= ATTN_BLOCK_MAX_Q) return attention_block(qkv, out, B, Lq, d, n_heads, k_cache, v_cache, cache_len, cache_cap, s);
     const int Lk = cached ? cache_len + Lq : Lq;
+    const int64_t pairs = (int64_t)B * n_heads;
+    if (block_pays(pairs, Lq, Lk)) return attention_block(qkv, out, B, Lq, d, n_heads, k_cache, v_cache, cache_len, cache_cap, s);
+    const int streams = Lq <= BQ && pairs > sm_count() ? 1 : 2;
     CUtensorMap mq, mk, mv;
     const int dh = d / n_heads;
-    const uint32_t box[3] = {(uint32_t)SUB, (uint32_t)BQ, 1}, box_kv[3] = {(uint32_t)SUB, (uint32_t)(dh == 64 ? Cfg<1>::BK : Cfg<2>::BK), 1};
+    const uint32_t box[3] = {(uint32_t)SUB, (uint32_t)BQ, 1}, box_kv[3] = {(uint32_t)SUB, (uint32_t)(streams == 1 ? Cfg<1, 1>::BK : dh == 64 ? Cfg<1, 2>::BK : Cfg<2, 2>::BK), 1};
     {
         const uint64_t dims[3] = {(uint64_t)3 * d, (uint64_t)Lq, (uint64_t)B};
         const uint64_t str[2] = {(uint64_t)3 * d, (uint64_t)Lq * 3 * d};
@@ -315,12 +329,14 @@ cudaError_t attention_forward(const void *qkv, void *out, int B, int Lq, int d, 
     int *status = device_status_ptr();
     if (!status) return cudaErrorUnknown;
     AttnArgs a{B, Lq, Lk, d, n_heads, cached ? 0 : d, cached ? 0 : 2 * d, static_cast<__nv_bfloat16 *>(out), 1.4426950408889634f / sqrtf((float)dh)};
-    const dim3 grid((Lq + 2 * BQ - 1) / (2 * BQ), n_heads, B);
-    const uint32_t smem = dh == 64 ? Cfg<1>::SMEM : Cfg<2>::SMEM;
-    auto kern = dh == 64 ? attention_kernel<1> : attention_kernel<2>;
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    return launch_chain(kern, grid, NTHREADS, smem, s, 0, mq, mk, mv, a, status);
+    const dim3 grid((Lq + streams * BQ - 1) / (streams * BQ), n_heads, B);
+    auto go = [&](auto kern, uint32_t threads, uint32_t smem) {
+        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        return e != cudaSuccess ? e : launch_chain(kern, grid, threads, smem, s, 0, mq, mk, mv, a, status);
+    };
+    if (streams == 1)
+        return dh == 64 ? go(attention_kernel<1, 1>, Cfg<1, 1>::NTHREADS, Cfg<1, 1>::SMEM) : go(attention_kernel<2, 1>, Cfg<2, 1>::NTHREADS, Cfg<2, 1>::SMEM);
+    return dh == 64 ? go(attention_kernel<1, 2>, Cfg<1, 2>::NTHREADS, Cfg<1, 2>::SMEM) : go(attention_kernel<2, 2>, Cfg<2, 2>::NTHREADS, Cfg<2, 2>::SMEM);
 }
 
 }  // namespace dm

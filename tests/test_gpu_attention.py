@@ -220,6 +220,37 @@ def test_attention_block_splits(G, dh, H, G_len, prefix):
     assert torch.isnan(kc[:, n:]).all() and torch.isnan(vc[:, n:]).all()
 
 
+@pytest.mark.parametrize("dh,H,B,G_len,prefix", [
+    (64, 8, 12, 33, 100), (80, 4, 24, 64, 31),             # more than 32 queries, 96 pairs: two streams, the second without a query
+    (64, 20, 8, 33, 63), (80, 20, 8, 100, 1), (64, 20, 8, 128, 0), (80, 20, 8, 128, 65),      # 160 pairs, up to 128 queries: CTAs of one stream
+    (64, 20, 8, 129, 0), (64, 2, 2, 128, 150), (80, 2, 1, 300, 20),                             # the second stream with one query; without; in the last CTA only
+    (64, 38, 8, 32, 40), (80, 38, 8, 1, 64)])              # up to 32 queries, 304 pairs: no longer the few-query kernel
+def test_attention_streams(G, dh, H, B, G_len, prefix):
+    """The forms of the tensor-core kernel at the lines between them, key tiles cut short, with a key/value cache (beyond the valid keys: NaN)."""
+    from paper_2511_15927_b200 import binding as dm
+    d, cap = dh * H, prefix + G_len + 3
+    x, wq, wo = _case(B, G_len, H, 300 + prefix, 1.0, dh=dh)
+    r = np.random.default_rng(prefix)
+    k0 = I.round_to_bf16(r.standard_normal((B, prefix, d), dtype=np.float32))
+    v0 = I.round_to_bf16(r.standard_normal((B, prefix, d), dtype=np.float32))
+    pad = np.full((B, cap - prefix, d), np.nan, np.float32)
+    kc, vc = G.dev(np.concatenate([k0, pad], 1), I.BF16), G.dev(np.concatenate([v0, pad], 1), I.BF16)
+    xd, wqd, wod = G.dev(x, I.BF16), G.dev(wq, I.BF16), G.dev(wo, I.BF16)
+    yd = torch.empty_like(xd)
+    nb = dm.dm_attention_workspace_bytes(B, G_len, d, dm.DM_BF16)
+    ws = G.workspace(nb)
+    st = torch.cuda.current_stream().cuda_stream
+    dm.dm_attention_block_step(B, G_len, d, H, dm.DM_BF16, wqd.data_ptr(), wod.data_ptr(), xd.data_ptr(), kc.data_ptr(), vc.data_ptr(), prefix, cap,
+                               yd.data_ptr(), ws.data_ptr(), nb, st)
+    dm.dm_check(st)
+    want, _, _ = O.attention_block_step(x, wq, wo, H, k0.astype(np.float64), v0.astype(np.float64))
+    got = yd.float().cpu().numpy().astype(np.float64)
+    assert np.all(np.isfinite(got)) and G.rel_l2(got, want) <= BF16_REL and G.max_abs(got, want) <= BF16_ABS, (G.rel_l2(got, want), G.max_abs(got, want))
+    if prefix == 0:
+        full = _run(G, x, wq, wo, H)
+        assert G.rel_l2(full, want) <= BF16_REL and G.max_abs(full, want) <= BF16_ABS
+
+
 def test_hybrid_stack_block_mode(G):
     """Prefix pass commits Mamba states and key/value caches, the next block starts from them (Sec. 4.3)."""
     from paper_2511_15927_b200 import binding as dm
