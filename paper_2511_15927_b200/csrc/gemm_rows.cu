@@ -297,6 +297,157 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap map_x0, const __grid_consta
     }
 }
 
+// The same for more uncut tiles than two to an SM (the vocabulary's projection): every CTA takes each gridDim.x-th tile, with two accumulator buffers, so that a tile's epilogue runs
+// under the next one's products and the ring of stages never empties.  Bound by the weights' way from HBM.  A CTA per tile / this kernel: 128 x 50304 x 1024 37.8 / 26.2 us, 128 x 50304 x 2048
+// 51.3 / 41.2, 64 x 50304 x 1024 28.1 / 23.7, 16 rows 24.0 / 20.9 (4.9 TB/s).  A kernel of its own: as an option of the one above its loop cost the launches of a decoding pass 1 to 2 us each.
+// Warps 0 and 1 as above, the next EW are the epilogue.  (No next norm's input: nothing that wide is normed.)
+struct __align__(8) LoopBars {
+    uint64_t full[MAX_STAGES], empty[MAX_STAGES], done[2], drained[2];
+    uint32_t tmem_base;
+    int abort;
+    float scale[2][128];           // row scale of every token, per product
+};
+
+template <int EW>
+__global__ void __launch_bounds__(64 + 32 * EW, EW == 4 ? 2 : 1)
+gemm_rows_loop_kernel(const __grid_constant__ CUtensorMap map_x0, const __grid_constant__ CUtensorMap map_w0,
+                      const __grid_constant__ CUtensorMap map_x1, const __grid_constant__ CUtensorMap map_w1,
+                      const __grid_constant__ RowsArgs ra, const int items, int *status) {
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t *smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+    const int nt = ra.nt, S = ra.stages, nprob = items / ra.tiles_n;
+    const uint32_t stage = W_BYTES + (uint32_t)nt * (BK * 2);
+    LoopBars *bars = reinterpret_cast<LoopBars *>(smem + S * stage);
+    volatile int *abort_flag = &bars->abort;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const EpiArgs &e0 = ra.p[0];                                             // (sizes are common to both products)
+    if (e0.m_dev) pdl_wait();                                                // (the row count comes from a kernel before this one)
+    const int M = e0.m_dev ? min(e0.M, max(0, *e0.m_dev - e0.m_off)) : e0.M;
+    const int kblocks = (e0.K + BK - 1) / BK;
+
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < S; ++i) { mbar_init(&bars->full[i], 1); mbar_init(&bars->empty[i], 1); }
+        for (int i = 0; i < 2; ++i) { mbar_init(&bars->done[i], 1); mbar_init(&bars->drained[i], EW); }
+        bars->abort = 0;
+        mbar_fence_init();
+    }
+    if (threadIdx.x == 64) { prefetch_map(&map_w0); prefetch_map(&map_x0); }
+    if (warp == 1) tmem_alloc(&bars->tmem_base, 2 * ra.tmem_cols);
+    __syncwarp();
+    fence_before();
+    __syncthreads();
+    fence_after();
+    const uint32_t tmem = bars->tmem_base;
+
+    bool ok = true;
+    if (warp == 0) {
+        const bool leader = elect_one();
+        const uint64_t once = l2_evict_first();
+        int s = 0;
+        uint32_t ph = 1;
+        // the weights of the first stages are on their way before the kernel before this one has finished
+        const int ahead = min(S, kblocks);
+        if (leader)
+            for (int i = 0; i < ahead; ++i) {
+                mbar_expect_tx(&bars->full[i], stage);
+                tma_load_2d_hint(smem + i * stage, (int)blockIdx.x < ra.tiles_n ? &map_w0 : &map_w1, i * BK, (int)blockIdx.x % ra.tiles_n * BF, &bars->full[i], once);
+            }
+        __syncwarp();
+        pdl_wait();
+        pdl_trigger();
+        for (int item = blockIdx.x; item < items && ok; item += gridDim.x) {
+            const bool second = item >= ra.tiles_n;
+            const CUtensorMap *mx = second ? &map_x1 : &map_x0, *mw = second ? &map_w1 : &map_w0;
+            const int n0 = (second ? item - ra.tiles_n : item) * BF;
+            for (int i = 0; i < kblocks; ++i) {
+                if (!(ok = mbar_wait(&bars->empty[s], ph, abort_flag, status))) break;
+                if (leader) {
+                    uint8_t *sw = smem + s * stage;
+                    if (item != (int)blockIdx.x || i >= ahead) {
+                        mbar_expect_tx(&bars->full[s], stage);
+                        tma_load_2d_hint(sw, mw, i * BK, n0, &bars->full[s], once);
+                    }
+                    tma_load_2d(sw + W_BYTES, mx, i * BK, 0, &bars->full[s]);
+                }
+                __syncwarp();
+                if (++s == S) { s = 0; ph ^= 1; }
+            }
+        }
+        if (!ok) sleep_ns(100000000ull);                                     // aborting: the loads already issued get time to land
+    } else if (warp == 1) {
+        const bool leader = elect_one();
+        pdl_wait();                                                          // (the limit of the waits below counts from here)
+        const uint32_t idesc = idesc_bf16(BF, nt, 0, 0), d0 = desc_lo_k(smem_u32(smem));
+        int s = 0, n = 0;
+        uint32_t ph = 0;
+        for (int item = blockIdx.x; item < items && ok; item += gridDim.x, ++n) {
+            if (n > 1 && !(ok = mbar_wait(&bars->drained[n & 1], ((n >> 1) - 1) & 1, abort_flag, status))) break;
+            fence_after();
+            const uint32_t d_tmem = tmem + (n & 1) * ra.tmem_cols;
+            for (int i = 0; i < kblocks; ++i) {
+                if (!(ok = mbar_wait(&bars->full[s], ph, abort_flag, status))) break;
+                fence_after();
+                const uint32_t dw = d0 + s * (stage >> 4), dx = dw + (W_BYTES >> 4);
+                if (leader) {
+#pragma unroll
+                    for (int k = 0; k < BK / 16; ++k) {
+                        if (i == 0 && k == 0) umma_ss<0>(d_tmem, dw, dx, idesc); else umma_ss<1>(d_tmem, dw + 2 * k, dx + 2 * k, idesc);
+                    }
+                    umma_commit(&bars->empty[s]);
+                    if (i == kblocks - 1) umma_commit(&bars->done[n & 1]);
+                }
+                __syncwarp();
+                if (++s == S) { s = 0; ph ^= 1; }
+            }
+        }
+    } else {
+        const int ew = warp - 2, q = warp & 3, f = q * 32 + lane;             // f: this thread's output column of the tile
+        pdl_wait();
+        for (int i = ew; i < nprob * nt; i += EW) {                          // row scales, while the products run: a warp per (product, token)
+            const int pi = i / nt, t = i - pi * nt;
+            const EpiArgs &e = ra.p[pi];
+            float sc = 1.f;
+            if (t < M && e.row_scale) sc = e.row_scale[t];
+            else if (e.rs_ssq) {
+                float v = 0.f;
+                for (int j = lane; j < e.rs_n; j += 32) v += t < M ? __ldg(e.rs_ssq + (int64_t)t * e.rs_n + j) : 0.f;
+                for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+                sc = rsqrtf(v * e.rs_inv + e.rs_eps);
+            }
+            if (lane == 0) bars->scale[pi][t] = sc;
+        }
+        named_sync(1, 32 * EW);                                              // the scales are there for all of these warps
+        int n = 0;
+        for (int item = blockIdx.x; item < items; item += gridDim.x, ++n) {
+            const int prod = item >= ra.tiles_n ? 1 : 0, col = (item - prod * ra.tiles_n) * BF + f;
+            const EpiArgs &ep = ra.p[prod];
+            const bool in = col < ep.N;
+            const float bias = in && ep.col_bias ? ep.col_bias[col] : 0.f;
+            if (!__all_sync(0xffffffffu, mbar_wait(&bars->done[n & 1], (n >> 1) & 1, abort_flag, status))) break;
+            fence_after();
+            for (int c0 = 16 * (ew >> 2); c0 < nt && c0 < M; c0 += 4 * EW) {
+                uint32_t r[16];
+                float v[16];
+                tmem_ld_x16(tmem + (n & 1) * ra.tmem_cols + ((uint32_t)(q * 32) << 16) + c0, r);
+                tmem_wait_ld();
+#pragma unroll
+                for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(r[j]) * bars->scale[prod][c0 + j];
+                emit(ep, c0, min(16, M - c0), col, in, bias, 0.f, v);
+            }
+            fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&bars->drained[n & 1]);
+        }
+    }
+    __syncwarp();
+    fence_before();
+    __syncthreads();
+    if (warp == 1) {
+        fence_after();
+        tmem_dealloc(tmem, 2 * ra.tmem_cols);
+    }
+}
+
 }  // namespace
 
 // Clusters of 2^i CTAs that are resident at once with one CTA per SM (of eight: 15 on 148 SMs; the GPU's parts hold uneven numbers of SMs).
@@ -336,21 +487,23 @@ cudaError_t gemm_rows_launch(const GemmArgs &a, const GemmArgs *b, bool sum, cud
     uint32_t cols = 32;
     while (cols < (uint32_t)ra.nt) cols *= 2;
     ra.tmem_cols = cols;
-    // Two CTAs per SM where not all clusters are resident with one and the stages stay at least three deep (four without partial sums: 128 x 50304 x 1920 lost 6 us with three);
+    // Two CTAs per SM where not all clusters are resident with one and the stages stay at least three deep (128 x 25000 x 1920: 25.5 us, 32.4 in two rounds of one CTA; four where tiles are taken
+    // in turn: 128 x 50304 x 2048 41.2 us with one CTA of seven stages per SM, 44.5 with two of three);
     // else one CTA may use all of the SM, with twice the epilogue warps, and a cut of K that does not fit one round is halved.  (16 clusters of eight CTAs, the summed
     // out_proj of d_model 2048, ran in two rounds: 24 layers of 32 tokens 1003 -> 846 us, one layer of 100 tokens 53 -> 47 us.)
     const size_t stage = W_BYTES + (size_t)ra.nt * BK * 2;
+    const bool loop = ks * per == 1 && items > 2 * sm_count() && !a.u && !(b && b->u);
     size_t fixed;
     bool two;
     for (;; ks /= 2) {
         ra.ks = ks;
         ra.cs = ks * per;
-        fixed = (ra.cs > 1 ? (size_t)ra.nt * BF * 4 : 0) + sizeof(Bars) + 1024;
+        fixed = (ra.cs > 1 ? (size_t)ra.nt * BF * 4 : 0) + (loop ? sizeof(LoopBars) : sizeof(Bars)) + 1024;
         const bool fits = items <= resident_clusters(ra.cs);
-        two = !fits && fixed + (ra.cs == 1 ? 4 : 3) * stage <= 113 * 1024;
+        two = !fits && fixed + (loop ? 4 : 3) * stage <= 113 * 1024;
         if (fits || two || ks == 1) break;
     }
-    const int ctas = items * ra.cs;
+    const int ctas = loop ? (two ? 2 : 1) * sm_count() : items * ra.cs;
     const int stages = (int)(((two ? 113 : 226) * 1024 - fixed) / stage);
     ra.stages = stages > MAX_STAGES ? MAX_STAGES : stages;
     const size_t smem = fixed + ra.stages * stage;
@@ -358,11 +511,16 @@ cudaError_t gemm_rows_launch(const GemmArgs &a, const GemmArgs *b, bool sum, cud
     if (!make_map_2d(&mx[0], a.A, a.M, a.K, a.lda, ra.nt) || !make_map_2d(&mw[0], a.B, a.N, a.K, a.ldb, BF)) return cudaErrorInvalidValue;
     mx[1] = mx[0]; mw[1] = mw[0];
     if (b && (!make_map_2d(&mx[1], b->A, b->M, b->K, b->lda, ra.nt) || !make_map_2d(&mw[1], b->B, b->N, b->K, b->ldb, BF))) return cudaErrorInvalidValue;
-    auto kern = two ? gemm_rows_kernel<4> : gemm_rows_kernel<8>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
-    if (e != cudaSuccess) return e;
     int *status = device_status_ptr();
     if (!status) return cudaErrorUnknown;
+    if (loop) {
+        auto kern = two ? gemm_rows_loop_kernel<4> : gemm_rows_loop_kernel<8>;
+        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
+        return e != cudaSuccess ? e : launch_chain(kern, dim3(ctas), dim3(two ? 192 : 320), smem, s, 0, mx[0], mw[0], mx[1], mw[1], ra, items, status);
+    }
+    auto kern = two ? gemm_rows_kernel<4> : gemm_rows_kernel<8>;
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
+    if (e != cudaSuccess) return e;
     return launch_chain(kern, dim3(ctas), dim3(two ? 224 : 352), smem, s, ra.cs, mx[0], mw[0], mx[1], mw[1], ra, status);
 }
 

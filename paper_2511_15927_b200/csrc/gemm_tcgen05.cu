@@ -1,6 +1,6 @@
 // bf16 x bf16 -> fp32 GEMM on the 5th-generation tensor cores, for the dense projections:
 //     C[m, n] = row_scale[m] * sum_k A[m, k] * B[n, k] + addend[m, n]
-// This file chooses the kernel and its tile: gemm_rows.cu for up to 128 rows (reading the weights is all such a product does), gemm_pair.cu for more, and gemm_cluster.cu for
+// This file chooses the kernel and its tile: gemm_rows.cu for up to 128 rows (reading the weights is nearly all such a product does), gemm_pair.cu for more, and gemm_cluster.cu for
 // a sum of two products whose tiles are few.
 // All: operands staged by TMA with the 128-byte swizzle, accumulators in TMEM, mbarrier pipelines.
 #include "gemm_epi.cuh"
@@ -16,8 +16,17 @@ constexpr int BM = 128;
 // per CTA, then arrive at 15 TB/s over all SMs: what L2 delivers, while its products take half of that time), so a narrow round counts 0.74.
 bool pair_wide_tile(const GemmArgs &a, int nprob) { return a.N > 128 && gemm_pair_cost(true, a, nprob) <= gemm_pair_cost(false, a, nprob); }
 
+// Which kernel for up to 128 rows.  gemm_rows.cu is the faster reader of weights, but what it does per row -- a row's scale from its sums of squares, one round trip to memory after the other,
+// and its stores -- shows where the products are short.  K up to 768, more than 80 rows with such scales or 96 without: few-row kernel / pair kernel 128 x 2000 x 512 12.5 / 10.4 us, 12 decoding
+// layers of 96 tokens 344 / 298 us at d_model 512, 377 / 300 at 256; K = 1024: level at 128 rows, 10.4 / 12.5 us at 80.  More tiles than two to an SM go to its looping form at any K
+// (128 x 50304 x 512: 18.5 / 22.7 us).
+bool few_rows(const GemmArgs &a, int nprob) {
+    if (a.M > BM) return false;
+    return a.M <= (a.rs_ssq ? 80 : 96) || a.K > 768 || (int64_t)((a.N + BM - 1) / BM) * nprob > 2 * sm_count();
+}
+
 cudaError_t dispatch(const GemmArgs &a, const GemmArgs *b, cudaStream_t s) {
-    if (a.M <= BM) return gemm_rows_launch(a, b, false, s);
+    if (few_rows(a, b ? 2 : 1)) return gemm_rows_launch(a, b, false, s);
     return gemm_pair_launch(pair_wide_tile(a, b ? 2 : 1), a, b, s);
 }
 

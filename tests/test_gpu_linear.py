@@ -98,3 +98,15 @@ def test_linear_mixed_tile_widths(dm, M, N, K):
 def test_linear_few_rows_uncut_tiles(dm, M, N, K):
     """Up to 128 rows around the line where K is no longer cut (88 and 89 tiles), one tile per SM, and more tiles than SMs with one and two CTAs on each."""
     test_linear_parity(dm, I.BF16, M, N, K)
+
+
+@pytest.mark.parametrize("M,N,K", [(5, 38016, 72), (64, 38016, 520), (80, 40000, 1032), (81, 37889, 72), (128, 38100, 456)])
+def test_linear_few_rows_tiles_in_turn(dm, M, N, K):
+    """Up to 128 rows and more tiles than two to an SM: each CTA takes several, in two accumulator buffers; three rounds for some CTAs; rows that are not 16-byte pieces."""
+    test_linear_parity(dm, I.BF16, M, N, K)
+
+
+@pytest.mark.parametrize("M,N,K", [(96, 300, 768), (97, 300, 768), (97, 300, 776), (128, 20000, 776), (97, 19000, 72)])
+def test_linear_few_rows_kernel_choice(dm, M, N, K):
+    """The lines between the few-row kernel and the two-CTA one: 96 rows, K of 768; more tiles than SMs with more than 80 rows (three stages to a CTA)."""
+    test_linear_parity(dm, I.BF16, M, N, K)

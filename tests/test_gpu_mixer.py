@@ -114,6 +114,15 @@ def test_out_proj_with_ragged_sums_of_squares_bf16(G, B, L, d, H):
     test_short_input_out_proj_paths_bf16(G, B, L, d, H)
 
 
+@pytest.mark.parametrize("L", [40, 128])
+def test_wide_in_proj_few_rows_bf16(G, L):
+    """Both directions' in_proj of 9600 inner channels (2 x 152 tiles) for up to 128 rows: CTAs whose tiles belong to both products."""
+    shape = I.MixerShape(1, L, 192, 50, 16, 4, 150)
+    wf, wr, x = _case(shape, I.BF16, seed=21)
+    got = G.run_forward(shape, I.BF16, wf, wr, x)
+    _check(got, O.bimamba_forward(x, wf, wr, **G.oracle_kwargs(shape)), I.BF16)
+
+
 def dm_flags_no_norm():
     from paper_2511_15927_b200 import binding as dm
     return dm.DM_FLAGS_DEFAULT & ~dm.DM_FLAG_GATED_RMSNORM

@@ -81,6 +81,22 @@ def test_reverse_step_against_oracle(G, dtype, N, d, H, V, vocab_real, cond):
     _check_draws(tok, out, ref_logits, u_keep, u_cat, keep_prob, mask_id, vocab_real, slack=np.expm1(2 * eps) + 2e-5)
     assert (out[drawn] == want[drawn]).mean() > 0.5           # and most draws coincide outright
 
+
+@pytest.mark.parametrize("L", [40, 64])
+def test_reverse_step_few_rows_many_tiles(G, L):
+    """Up to 128 rows of a vocabulary whose column tiles are more than are resident at once, the number of drawn rows known on the device only."""
+    shape, V, mask_id, keep_prob = I.MixerShape(2, L, 64, 2, 16, 4, 2), 38016, 38000, 0.6
+    sw = I.make_stack_weights(shape, 1, V, seed=17, dtype=I.BF16, perturb=True)
+    tok = I.make_tokens(2, L, mask_id, mask_id, seed=17)
+    r = np.random.default_rng(17)
+    u_keep, u_cat = r.random((2, L), dtype=np.float32), r.random((2, L), dtype=np.float32)
+    out = G.run_sample_step(shape, I.BF16, sw, tok, V, u_keep, u_cat, keep_prob, mask_id, mask_id + 1)
+    logits, _, _ = G.run_denoise(shape, I.BF16, sw, tok, V, want_argmax=False)
+    want = O.denoise_step(tok, sw, **G.oracle_kwargs(shape))
+    assert G.rel_l2(logits, want) <= 1e-2, G.rel_l2(logits, want)
+    assert 5 < _check_draws(tok, out, logits, u_keep, u_cat, keep_prob, mask_id, mask_id + 1, slack=2e-4) < 2 * L
+
+
 def test_keep_everything_or_nothing_and_determinism(G):
     shape = I.MixerShape(2, 40, 64, 2, 16, 4, 4)
     V, mask_id = 120, 100
