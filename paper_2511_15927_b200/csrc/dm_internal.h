@@ -6,6 +6,8 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include <initializer_list>
+
 #include "dm_bimamba.h"
 
 namespace dm {
@@ -88,6 +90,27 @@ struct GemmArgs {
     const int *m_dev;        // device int or NULL: only rows [0, clamp(*m_dev - m_off, 0, M)) are computed (row count known on the device only)
     int m_off;
 };
+// What the tensor-core kernels take: bf16 operands in 16-byte rows (TMA), and 16-byte alignment of what their epilogues read as vectors.
+inline bool gemm_tensor_ok(const GemmArgs &a) {
+    auto off16 = [](const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) != 0; };
+    if (a.in_dtype != DM_BF16 || a.M <= 0 || a.N <= 0 || a.K <= 0 || a.lda % 8 || a.ldb % 8) return false;
+    if (off16(a.A) || off16(a.B) || off16(a.C) || off16(a.addend) || off16(a.col_bias)) return false;
+    if (a.col_scale && (off16(a.col_scale) || (a.ld_cs > 0 ? a.ld_cs : (int64_t)a.N) % 4)) return false;
+    if (a.rs_ssq && a.rs_n % 4 == 0 && off16(a.rs_ssq)) return false;       // (read as float4 where a row holds whole ones, one by one elsewhere)
+    return true;
+}
+// Output and addend can go through TMA: 16-byte aligned rows, and no bf16 output with an addend (EpiOut in gemm_epi.cuh keeps the first 32 of 64 bf16 columns in the staging bytes
+// until the other 32 are there, and the addend of those arrives in the same bytes).
+inline bool gemm_tma_io(const GemmArgs &a) {
+    if (a.addend && (a.c_dtype != DM_F32 || a.ld_add % 4)) return false;
+    return (a.ldc * (int64_t)dtype_size(a.c_dtype)) % 16 == 0;
+}
+// The sum of two products in one launch.
+inline bool gemm_sum_ok(const GemmArgs &a, const GemmArgs &b) {
+    for (const GemmArgs *p : {&a, &b})
+        if (!gemm_tensor_ok(*p) || p->m_dev) return false;
+    return a.M == b.M && a.N == b.N && a.K == b.K && gemm_tma_io(b);
+}
 cudaError_t gemm_simple(const GemmArgs &a, cudaStream_t s);
 // fp32 products that do not fill the GPU: n of them (same sizes) in one launch, or both into b's output (sum).
 bool gemm_f32_supports(const GemmArgs &a, int n);

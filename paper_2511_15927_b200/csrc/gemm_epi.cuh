@@ -289,11 +289,5 @@ bool gemm_cluster_sum_pays(const GemmArgs &a);
 cudaError_t gemm_cluster_sum_launch(const GemmArgs &a, const GemmArgs &b, cudaStream_t s);
 // gemm_rows.cu: up to 128 rows; sum as in gemm_pair_sum_launch.
 cudaError_t gemm_rows_launch(const GemmArgs &a, const GemmArgs *b, bool sum, cudaStream_t s);
-// Output and addend can go through TMA: 16-byte aligned rows, and no bf16 output with an addend (EpiOut keeps the first 32 of 64 bf16 columns in the staging bytes until
-// the other 32 are there, and the addend of those arrives in the same bytes).
-inline bool gemm_pair_tma_io(const GemmArgs &a) {
-    if (a.addend && (a.c_dtype != DM_F32 || a.ld_add % 4)) return false;
-    return (a.ldc * (int64_t)dtype_size(a.c_dtype)) % 16 == 0;
-}
 
 }  // namespace dm

@@ -360,7 +360,7 @@ cudaError_t launch(const GemmArgs &a, const GemmArgs *b, cudaStream_t s) {
     return launch_chain(gemm_pair_kernel<BN, MODE>, grid, NTHREADS, smem, s, 0, op, io, epp, status);
 }
 
-bool tma_io(const GemmArgs &a, const GemmArgs *b) { return gemm_pair_tma_io(a) && (!b || (gemm_pair_tma_io(*b) && !a.addend && !b->addend && !a.u && !b->u)); }
+bool tma_io(const GemmArgs &a, const GemmArgs *b) { return gemm_tma_io(a) && (!b || (gemm_tma_io(*b) && !a.addend && !b->addend && !a.u && !b->u)); }
 
 }  // namespace
 

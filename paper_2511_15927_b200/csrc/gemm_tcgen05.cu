@@ -33,16 +33,8 @@ cudaError_t dispatch(const GemmArgs &a, const GemmArgs *b, cudaStream_t s) {
 }  // namespace
 
 bool gemm_tcgen05_supports(const GemmArgs &a) {
-    if (a.in_dtype != DM_BF16) return false;
-    if (a.M <= 0 || a.N <= 0 || a.K <= 0) return false;
-    if ((a.lda % 8) || (a.ldb % 8)) return false;                                   // TMA: 16-byte row pitch
-    if ((reinterpret_cast<uintptr_t>(a.A) & 15u) || (reinterpret_cast<uintptr_t>(a.B) & 15u)) return false;
-    if (reinterpret_cast<uintptr_t>(a.C) & 15u) return false;
-    if (a.addend && (reinterpret_cast<uintptr_t>(a.addend) & 15u)) return false;
-    if (a.col_bias && (reinterpret_cast<uintptr_t>(a.col_bias) & 15u)) return false;
-    if (a.col_scale && ((reinterpret_cast<uintptr_t>(a.col_scale) & 15u) || ((a.ld_cs > 0 ? a.ld_cs : (int64_t)a.N) & 3))) return false;
-    if (a.rs_ssq && (reinterpret_cast<uintptr_t>(a.rs_ssq) & 15u)) return false;
-    if (a.u && (a.c_dtype != DM_F32 || !gemm_pair_tma_io(a) || ((reinterpret_cast<uintptr_t>(a.u) | reinterpret_cast<uintptr_t>(a.u_w)) & 15u) || (a.N % 8))) return false;
+    if (!gemm_tensor_ok(a)) return false;
+    if (a.u && (a.c_dtype != DM_F32 || !gemm_tma_io(a) || ((reinterpret_cast<uintptr_t>(a.u) | reinterpret_cast<uintptr_t>(a.u_w)) & 15u) || (a.N % 8))) return false;
     return encode_fn() != nullptr;
 }
 
@@ -61,9 +53,7 @@ cudaError_t gemm_tcgen05_pair(const GemmArgs &a, const GemmArgs &b, cudaStream_t
     return dispatch(a, &b, s);
 }
 
-bool gemm_tcgen05_sum_supports(const GemmArgs &a, const GemmArgs &b) {
-    return gemm_tcgen05_supports(b) && gemm_tcgen05_supports(a) && a.M == b.M && a.N == b.N && a.K == b.K && !a.m_dev && !b.m_dev && gemm_pair_tma_io(b);
-}
+bool gemm_tcgen05_sum_supports(const GemmArgs &a, const GemmArgs &b) { return gemm_sum_ok(a, b) && gemm_tcgen05_supports(a) && gemm_tcgen05_supports(b); }
 
 cudaError_t gemm_tcgen05_sum(const GemmArgs &a, const GemmArgs &b, cudaStream_t s) {
     if (!gemm_tcgen05_sum_supports(a, b)) return cudaErrorNotSupported;

@@ -90,13 +90,13 @@ def test_bf16_parity_small(G, dims):
 
 @pytest.mark.parametrize("B,L,d,H", [(1, 1500, 1024, 32), (3, 400, 512, 16), (2, 60, 256, 8)])
 def test_short_input_out_proj_paths_bf16(G, B, L, d, H):
-    """Up to 2048 tokens the two out_proj run as one launch into fp32 partials that one pass scales and sums: 1500 tokens at d_model 1024
-    fill the GPU with whole products (256 tiles), the two smaller cases cut each product in two along K (four partials)."""
+    """Both directions' out_proj in one launch at three sizes: 1500 tokens at d_model 1024 (24 tiles of 256 x 256), 1200 at 512 and, on the kernel for up to 128 rows, 120 at 256;
+    with and without the gated norm's row scales."""
     shape = I.MixerShape(B, L, d, 2, 128, 4, H)
     wf, wr, x = _case(shape, I.BF16, seed=9)
     got = G.run_forward(shape, I.BF16, wf, wr, x)
     _check(got, O.bimamba_forward(x, wf, wr, **G.oracle_kwargs(shape)), I.BF16)
-    # without the gated norm the partials are summed unscaled
+    # without the gated norm the products are summed unscaled
     got0 = G.run_forward(shape, I.BF16, wf, wr, x, flags=dm_flags_no_norm())
     _check(got0, O.bimamba_forward(x, wf, wr, **G.oracle_kwargs(shape, flags=dm_flags_no_norm())), I.BF16)
 
@@ -110,8 +110,17 @@ def test_few_rows_out_proj_rounds_bf16(G, B, L):
 
 @pytest.mark.parametrize("B,L,d,H", [(1, 201, 96, 3), (1, 77, 96, 3), (3, 683, 160, 5), (2, 1001, 480, 15)])
 def test_out_proj_with_ragged_sums_of_squares_bf16(G, B, L, d, H):
-    """B L H not a multiple of 4: the right-to-left layer's sums of squares do not start on a 16-byte boundary."""
-    test_short_input_out_proj_paths_bf16(G, B, L, d, H)
+    """B L H not a multiple of 4: the right-to-left layer's sums of squares do not start on a 16-byte boundary.  in_proj, scan (prep in a launch of its own) and one out_proj."""
+    from paper_2511_15927_b200 import binding as dm
+    shape = I.MixerShape(B, L, d, 2, 128, 4, H)
+    wf, wr, x = _case(shape, I.BF16, seed=9)
+    before = dm.dm_kernel_launch_count()
+    got = G.run_forward(shape, I.BF16, wf, wr, x)
+    assert dm.dm_kernel_launch_count() - before == 4
+    _check(got, O.bimamba_forward(x, wf, wr, **G.oracle_kwargs(shape)), I.BF16)
+    # each direction alone (its row scales from a pass of their own)
+    fwd, rev = (G.run_forward(shape, I.BF16, wf, wr, x, dir_mask=m) for m in (dm.DM_DIR_FWD, dm.DM_DIR_REV))
+    _check(fwd + rev, O.bimamba_forward(x, wf, wr, **G.oracle_kwargs(shape)), I.BF16)
 
 
 @pytest.mark.parametrize("L", [40, 128])

@@ -45,10 +45,20 @@ def test_denoise_step_full_sequence(G, dtype, N, d, H, layers, V):
     np.testing.assert_array_equal(amax, amax2)
 
 
-@pytest.mark.parametrize("d,H,B,L,d_ff", [(160, 5, 3, 683, 0), (64, 2, 1, 2049, 0), (320, 10, 2, 1100, 640)])
+def _launches_with_summed_out_proj(B, L, layers, cond):
+    """Kernels of a stack pass whose out_proj is one launch per layer that also writes the next norm's input (sequences of more than 64 tokens): in_proj (one launch for both
+    directions up to 4096 tokens), prep, scan, out_proj; around them the embedding, the first norm and the vocabulary -- or, with a conditioned block, its modulation, two AdaLN and
+    two products, and the final norm.  A layer whose directions are not summed in one launch takes three more (row scales, a second product, the norm)."""
+    per_layer = (1 if B * L <= 4096 else 2) + 3 + (5 if cond else 0)
+    return 3 + layers * per_layer
+
+
+@pytest.mark.parametrize("d,H,B,L,d_ff", [(160, 5, 3, 683, 0), (64, 2, 1, 2049, 0), (320, 10, 2, 1100, 640), (320, 10, 10, 500, 640)])
 def test_denoise_step_summed_out_proj(G, d, H, B, L, d_ff):
-    """Above 2048 tokens both directions' out_proj run as one launch that also writes the next norm's input: ragged rows, widths
-    that end inside the 64-column parts of its sums of squares (and inside a 256-column tile); with a gate on the sum."""
+    """Both directions' out_proj run as one launch that also writes the next norm's input: ragged rows, widths that end inside the 64-column parts of its sums of squares (and inside
+    a 256-column tile), B L H not a multiple of 4 (the second direction's sums of squares then start off a 16-byte boundary); with a gate on the sum.  The second and the last case
+    have no form on clusters (64 columns; 40 tiles of 256 x 256, more than clusters of four CTAs fit 148 SMs): the kernel of long inputs, with a column strip."""
+    from paper_2511_15927_b200 import binding as dm
     shape = I.MixerShape(B, L, d, 2, 32, 4, H)
     sw = I.make_stack_weights(shape, 3, 96, seed=7, dtype=I.BF16, perturb=True)
     tau = None
@@ -58,7 +68,9 @@ def test_denoise_step_summed_out_proj(G, d, H, B, L, d_ff):
     tok = I.make_tokens(B, L, 95, 95, seed=7)
     kw = G.oracle_kwargs(shape)
     want = O.denoise_step_cond(tok, tau, sw, **kw) if d_ff else O.denoise_step(tok, sw, **kw)
+    before = dm.dm_kernel_launch_count()
     got, _, _ = G.run_denoise(shape, I.BF16, sw, tok, 96, want_argmax=False, tau=tau, d_ff=d_ff)
+    assert dm.dm_kernel_launch_count() - before == _launches_with_summed_out_proj(B, L, 3, d_ff > 0)
     assert G.rel_l2(got, want) <= 1e-2, G.rel_l2(got, want)
 
 
@@ -71,7 +83,7 @@ def test_denoise_step_summed_out_proj_mixed_tiles(G, d, H, B, L, d_ff):
 @pytest.mark.parametrize("d,H,B,L,d_ff", [(288, 9, 1, 129, 0), (192, 6, 1, 256, 384), (1024, 32, 2, 1000, 0), (320, 10, 17, 256, 0)])
 def test_denoise_step_out_proj_over_clusters(G, d, H, B, L, d_ff):
     """Few 256 x 256 tiles: the summed out_proj cuts a tile over 4 or 2 pairs of CTAs.  An odd number of k-blocks and a last column tile of 32 columns; columns that
-    end inside the tile's shares, with a gate; 32 tiles (two pairs each); 34 tiles (more than one round of clusters: the kernel of long inputs)."""
+    end inside the tile's shares, with a gate; 32 tiles (two pairs each); 34 tiles (more than one round of clusters where 33 are resident)."""
     test_denoise_step_summed_out_proj(G, d, H, B, L, d_ff)
 
 
