@@ -105,10 +105,10 @@ inline bool gemm_tma_io(const GemmArgs &a) {
     if (a.addend && (a.c_dtype != DM_F32 || a.ld_add % 4)) return false;
     return (a.ldc * (int64_t)dtype_size(a.c_dtype)) % 16 == 0;
 }
-// The sum of two products in one launch.
+// The sum of two products in one launch: its epilogues know scales and the addend, no bias and no activation.
 inline bool gemm_sum_ok(const GemmArgs &a, const GemmArgs &b) {
     for (const GemmArgs *p : {&a, &b})
-        if (!gemm_tensor_ok(*p) || p->m_dev) return false;
+        if (!gemm_tensor_ok(*p) || p->m_dev || p->col_bias || p->gelu || p->silu_cols) return false;
     return a.M == b.M && a.N == b.N && a.K == b.K && gemm_tma_io(b);
 }
 cudaError_t gemm_simple(const GemmArgs &a, cudaStream_t s);
