@@ -364,8 +364,9 @@ int dm_selftest_wait_timeout(uint32_t limit_us, uint64_t *out, void *cuda_stream
  * whose scan would do its prep work inside the scan launch (one long sequence: fewer scan CTAs than SMs, more than eight chunks)
  * launches the scan without the CTAs of that role: the flags its load warps wait for from the ninth chunk on are never raised,
  * the waits run out after their regular limit (2 s), and every role of every CTA has to leave through the abort path -- loads in
- * flight waited for, TMEM freed.  The call itself returns DM_OK; dm_check then reports DM_ERR_TIMEOUT; y is unspecified.  Nothing
- * faults or hangs.  Process-wide; switch it off again. */
+ * flight waited for, TMEM freed.  A call on the sequential scan (fp32, or d_state 256) of more than two chunks leaves out the
+ * copies of every CTA's third chunk, with the same consequences.  The call itself returns DM_OK; dm_check then reports
+ * DM_ERR_TIMEOUT; y is unspecified.  Nothing faults or hangs.  Process-wide; switch it off again. */
 int dm_selftest_withhold_prep(int on);
 
 /* Number of kernels this library has launched from this process since load (for benchmarks). */

@@ -103,7 +103,7 @@ struct SeqSmem {
 // P channels and N states of a head; LPC = lanes per channel, NQ = float4 groups of state per lane
 template <typename T, int P, int N>
 __global__ void __launch_bounds__(P * lanes_per_channel(N) + loaders(P, N))
-scan_seq_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_z, const __grid_constant__ ScanArgs a, const int dir0, const int TC, const float *__restrict__ bc_all, int *status) {
+scan_seq_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_z, const __grid_constant__ ScanArgs a, const int dir0, const int TC, const int hold, const float *__restrict__ bc_all, int *status) {
     extern __shared__ __align__(128) uint8_t smem[];
     __shared__ uint64_t bars[RAW];                     // raw stage has landed
     __shared__ int abort_word;
@@ -199,8 +199,9 @@ scan_seq_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
         // Everything chunk ci needs from memory: a tile of x with the three rows before it in time, one of z (rows outside the sequence become zeros) and
         // the run of [B' | C'], in physical order.  (16-byte copies by the threads took 1000 clocks a chunk to issue, and held up the
         // shared-memory reads behind them.)
+        bool ok = true;                                    // no wait of this thread has given up: afterwards no copies are started
         auto fetch = [&](int ci) {
-            if (ci >= nchunks || lt != 0) return;
+            if (ci >= nchunks || lt != 0 || !ok || ci == hold) return;      // (hold: left out, for the self-test)
             uint8_t *st = raw_of(ci);
             uint64_t *bar = &bars[ci % RAW];
             const int tau0 = ci * TC, tc = min(TC, L - tau0), bt = a.zx_tied ? b : dir * a.B + b, t0 = rev ? L - TC - tau0 : tau0;
@@ -220,7 +221,7 @@ scan_seq_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
             }
             named_sync(1, NP);
         };
-        auto landed = [&](int ci) { mbar_wait(&bars[ci % RAW], (ci / RAW) & 1, abort_flag, status); };      // (gives up after its limit, then at once: the loop still ends)
+        auto landed = [&](int ci) { ok = mbar_wait(&bars[ci % RAW], (ci / RAW) & 1, abort_flag, status) && ok; };      // (gives up after its limit, then at once: the loop still ends)
         auto dt_of = [&](int ci) {                         // raw step size of token lt of the chunk (TC <= NP)
             const int tau = ci * TC + lt;
             return (lt < TC && tau < L) ? ldf(zx + (int64_t)(rev ? L - 1 - tau : tau) * a.d_in_proj + a.d_inner + a.conv_ch + h) : 0.f;
@@ -262,13 +263,17 @@ scan_seq_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
         carry(0);
         prepare(0, dt_cur);
         __syncthreads();
+        int gave_up = ok ? nchunks : 0;                    // chunk whose wait did: it and the one after it may still be on their way
         for (int ci = 0; ci < nchunks; ++ci) {
             fetch(ci + 2);                                 // its stage held chunk ci - 2, finished before the last barrier
             dt_cur = dt_next;
             dt_next = dt_of(ci + 2);
-            if (ci + 1 < nchunks) { landed(ci + 1); carry(ci + 1); prepare(ci + 1, dt_cur); }
+            if (ci + 1 < nchunks) { landed(ci + 1); if (!ok) gave_up = min(gave_up, ci + 1); carry(ci + 1); prepare(ci + 1, dt_cur); }
             __syncthreads();
         }
+        // after a wait that gave up: no copy of this CTA may still be in flight when it leaves
+        if (lt == 0 && !ok)
+            for (int c = gave_up; c < min(nchunks, gave_up + 2); ++c) mbar_wait_quiet(&bars[c % RAW], (c / RAW) & 1, 100000000ull);
     } else {
         // ------------------------------------------------------------------ scan group
         const int p = tid / LPC, j = tid - p * LPC;
@@ -358,7 +363,7 @@ bool make_map_rows(CUtensorMap *m, const ScanArgs &a, int rows) {
               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-typedef void (*Kern)(const CUtensorMap, const CUtensorMap, const ScanArgs, const int, const int, const float *, int *);
+typedef void (*Kern)(const CUtensorMap, const CUtensorMap, const ScanArgs, const int, const int, const int, const float *, int *);
 template <typename T> Kern kernel_for(int P, int N) {
     switch (N) {
         case 16: return P == 32 ? scan_seq_kernel<T, 32, 16> : scan_seq_kernel<T, 64, 16>;
@@ -408,7 +413,7 @@ cudaError_t scan_sequential(const ScanArgs &a, void *ws, cudaStream_t s) {
     if (e != cudaSuccess) return e;
     dim3 grid(a.H, ndir, a.B);
     chain_spread((int64_t)pgrid.x * pgrid.y * pgrid.z, sm_count());
-    return launch_chain(kern, grid, a.P * lanes_per_channel(a.N) + loaders(a.P, a.N), smem, s, 0, mx, mz, a, dir0, TC, bc, status);
+    return launch_chain(kern, grid, a.P * lanes_per_channel(a.N) + loaders(a.P, a.N), smem, s, 0, mx, mz, a, dir0, TC, scan_selftest_withheld() ? 2 : -1, bc, status);
 }
 
 }  // namespace dm

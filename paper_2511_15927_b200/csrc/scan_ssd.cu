@@ -1267,6 +1267,7 @@ bool shape_ok(const ScanArgs &a) {
 // ninth chunk run out and every role of every CTA leaves through the abort path (dm_selftest_withhold_prep).
 static int g_withhold_prep = 0;
 void scan_ssd_selftest_withhold(int on) { g_withhold_prep = on ? 1 : 0; }
+bool scan_selftest_withheld() { return g_withhold_prep != 0; }
 
 bool scan_ssd_chunk_ok(int dtype, int d_state, int chunk) {
     return !(dtype == DM_BF16 && d_state <= N) || chunk == 0 || chunk == QB || chunk == Q;

@@ -68,6 +68,31 @@ def test_the_scan_kernel_leaves_through_its_abort_path_when_its_prep_never_comes
     assert G.rel_l2(got, O.bimamba_forward(x, wf, wr, **G.oracle_kwargs(shape))) <= 1e-2
 
 
+def test_the_sequential_scan_leaves_when_a_copy_never_comes(G):
+    """The sequential scan: with the copies of each CTA's third chunk left out, the waits for them run out (2 s) while the fourth chunk's are under way; no further copies are started, the
+    ones under way are waited for, and the loops end.  DM_ERR_TIMEOUT once, and the same call is correct again afterwards."""
+    import time
+    import torch
+    from oracle import bimamba_oracle as O
+    from paper_2511_15927_b200 import binding as dm
+    for dtype, shape, chunk in ((I.F32, I.MixerShape(2, 300, 64, 2, 16, 4, 4), 0), (I.BF16, I.MixerShape(1, 90, 128, 2, 256, 4, 4), 8)):
+        wf, wr = I.make_mixer_weights(shape, 5, dtype)
+        x = I.make_activations(shape, 5, dtype)
+        dm.dm_check(torch.cuda.current_stream().cuda_stream)
+        dm.dm_selftest_withhold_prep(True)
+        try:
+            t0 = time.time()
+            with pytest.raises(dm.DmError) as e:
+                G.run_forward(shape, dtype, wf, wr, x, chunk=chunk)
+            waited = time.time() - t0
+        finally:
+            dm.dm_selftest_withhold_prep(False)
+        assert e.value.status == dm.DM_ERR_TIMEOUT
+        assert 1.5 < waited < 20.0
+        got = G.run_forward(shape, dtype, wf, wr, x, chunk=chunk)
+        assert G.rel_l2(got, O.bimamba_forward(x, wf, wr, **G.oracle_kwargs(shape))) <= (1e-4 if dtype == I.F32 else 1e-2)
+
+
 def test_selftest_argument_checks(G):
     from paper_2511_15927_b200 import binding as dm
     before = dm.dm_kernel_launch_count()
