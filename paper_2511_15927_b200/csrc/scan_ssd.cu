@@ -1008,7 +1008,7 @@ ssd_block_kernel(const SsdArgs a, const __nv_bfloat16 *__restrict__ Bp, const __
     }
     const int ei = tid / U8, ec = (tid % U8) * 8;      // epilogue: token row of the sub-chunk, first of 8 channels
     uint4 nwp = make_uint4(0x3F803F80u, 0x3F803F80u, 0x3F803F80u, 0x3F803F80u);      // norm weights of those channels as bf16 pairs (ones when the norm is off)
-    if (norm_on && w.norm_w) nwp = __ldg(reinterpret_cast<const uint4 *>(static_cast<const __nv_bfloat16 *>(w.norm_w) + h * PP + ec));
+    if (norm_on && w.norm_w) nwp = ld8_bf16(static_cast<const __nv_bfloat16 *>(w.norm_w) + h * PP + ec);
 
     pdl_wait();
     pdl_trigger();

@@ -425,7 +425,11 @@ cudaError_t launch(const SsdArgs &a, int ndir, int dir0, cudaStream_t s) {
 
 }  // namespace
 
+// (norm weights that are not 16-byte aligned go to the prep launch and ssd_block_kernel: reading them either way here cost 1 % of a decoding pass of 16 sequences)
 bool scan_step_supports(const ssd::SsdArgs &a) {
+    if (a.flags & DM_FLAG_GATED_RMSNORM)
+        for (const ScanDir &d : a.dir)
+            if (reinterpret_cast<uintptr_t>(d.norm_w) & 15u) return false;
     return a.L <= QB && !((reinterpret_cast<uintptr_t>(a.ssm_in) | reinterpret_cast<uintptr_t>(a.ssm_out)) & 15u) && (int64_t)a.B * a.H * 64 < (1ll << 31);
 }
 

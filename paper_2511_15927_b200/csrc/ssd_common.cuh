@@ -68,6 +68,16 @@ __device__ __forceinline__ void ldmatrix_x2_t(uint32_t &r0, uint32_t &r1, const 
     asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0, %1}, [%2];" : "=r"(r0), "=r"(r1) : "r"(smem_u32(p)));
 }
 
+// Eight consecutive bf16 of a read-only array, two to a word; at any address (callers' weight vectors carry no alignment rule)
+__device__ __forceinline__ uint4 ld8_bf16(const __nv_bfloat16 *p) {
+    if ((reinterpret_cast<uintptr_t>(p) & 15u) == 0) return __ldg(reinterpret_cast<const uint4 *>(p));
+    const unsigned short *q = reinterpret_cast<const unsigned short *>(p);
+    uint32_t w[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) w[i] = (uint32_t)__ldg(q + 2 * i) | ((uint32_t)__ldg(q + 2 * i + 1) << 16);
+    return make_uint4(w[0], w[1], w[2], w[3]);
+}
+
 // 16-byte asynchronous copy global -> shared; src_bytes = 16, or 0 to fill the destination with zeros (src must still be a valid address)
 __device__ __forceinline__ void cp_async16(void *smem_dst, const void *gsrc, uint32_t src_bytes) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(smem_dst)), "l"(gsrc), "r"(src_bytes) : "memory");
@@ -76,7 +86,7 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 
 }  // namespace ssd
 
-// One block of up to QB tokens per sequence in one launch: see scan_step.cu (which takes 16-byte aligned states).
+// One block of up to QB tokens per sequence in one launch: see scan_step.cu (which takes 16-byte aligned states and norm weights).
 bool scan_step_supports(const ssd::SsdArgs &a);
 cudaError_t scan_step(const ssd::SsdArgs &a, int headdim, int ndir, int dir0, cudaStream_t s);
 

@@ -132,6 +132,34 @@ def test_wide_in_proj_few_rows_bf16(G, L):
     _check(got, O.bimamba_forward(x, wf, wr, **G.oracle_kwargs(shape)), I.BF16)
 
 
+@pytest.mark.parametrize("L,N,chunk", [(20, 128, 0), (48, 64, 0), (140, 128, 0), (140, 128, 32), (40, 256, 0)])
+def test_vectors_without_alignment_bf16(G, L, N, chunk):
+    """Norm weights and conv parameters that start on any element: only the matrices are required to be aligned.  Every scan kernel."""
+    import torch
+    from paper_2511_15927_b200 import binding as dm
+    shape = I.MixerShape(2, L, 128, 2, N, 4, 4)
+    wf, wr, x = _case(shape, I.BF16, seed=33)
+    cfg = G.cfg_of(shape, I.BF16, chunk=chunk)
+    xd = G.dev(x, I.BF16)
+    ws = G.workspace(dm.dm_bimamba_workspace_bytes(cfg))
+    st = torch.cuda.current_stream().cuda_stream
+    want = O.bimamba_forward(x, wf, wr, **G.oracle_kwargs(shape))
+    for shift in (0, 1, 4):
+        dw = []
+        for w in (wf, wr):
+            t = G.dev_dir_weights(w, I.BF16)
+            for k in ("norm_w", "conv_w", "conv_b"):
+                buf = torch.empty(t[k].numel() + 8, device="cuda", dtype=t[k].dtype)
+                view = buf[shift:shift + t[k].numel()]
+                view.copy_(t[k].flatten())
+                t[k] = view
+            dw.append(t)
+        y = torch.empty_like(xd)
+        dm.dm_bimamba_forward(cfg, tuple(dm.make_dir_weights(t) for t in dw), xd.data_ptr(), y.data_ptr(), ws.data_ptr(), ws.numel(), st)
+        dm.dm_check(st)
+        _check(y.float().cpu().numpy().astype(np.float64), want, I.BF16)
+
+
 def dm_flags_no_norm():
     from paper_2511_15927_b200 import binding as dm
     return dm.DM_FLAGS_DEFAULT & ~dm.DM_FLAG_GATED_RMSNORM
