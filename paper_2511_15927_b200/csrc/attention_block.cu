@@ -36,19 +36,6 @@ struct BlockAttnArgs {
     float scale_log2;                    // log2(e) / sqrt(DH)
 };
 
-__device__ __forceinline__ void ldsm_x4(uint32_t (&r)[4], uint32_t addr) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
-}
-__device__ __forceinline__ void ldsm_x4_t(uint32_t (&r)[4], uint32_t addr) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
-}
-__device__ __forceinline__ void mma16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
-                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-__device__ __forceinline__ void copy16(uint32_t dst, const void *src, uint32_t bytes) {      // 0 bytes: fill with zeros
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
-}
 __device__ __forceinline__ float ld_cluster_f32(uint32_t cluster_addr) {
     float v;
     asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(cluster_addr) : "memory");
@@ -91,8 +78,8 @@ attention_block_kernel(const BlockAttnArgs a, int H, int split) {
             for (int i = 0; i < PIECES; ++i) {
                 if (KT * U % NT != 0 && i == PIECES - 1 && prow[i] >= KT) break;
                 const uint32_t off = (prow[i] * LD + pcol[i]) * 2, g = (uint32_t)(prow[i] * a.d + pcol[i]);
-                copy16(ks + off, pk + g, 16);
-                copy16(ks + S::TILE + off, pv + g, 16);
+                cp_async16(ks + off, pk + g, 16);
+                cp_async16(ks + S::TILE + off, pv + g, 16);
             }
             return;
         }
@@ -104,8 +91,8 @@ attention_block_kernel(const BlockAttnArgs a, int H, int split) {
             if (key < a.len) { pk = kc + (int64_t)key * a.d + pcol[i]; pv = vc + (int64_t)key * a.d + pcol[i]; }
             else if (key < Lk) { pk = own + (int64_t)(key - a.len) * 3 * a.d + a.d + pcol[i]; pv = pk + a.d; }
             const uint32_t nb = key < Lk ? 16 : 0, off = (prow[i] * LD + pcol[i]) * 2;
-            copy16(ks + off, pk, nb);
-            copy16(ks + S::TILE + off, pv, nb);
+            cp_async16(ks + off, pk, nb);
+            cp_async16(ks + S::TILE + off, pv, nb);
         }
     };
     auto commit = [] { asm volatile("cp.async.commit_group;" ::: "memory"); };
@@ -114,7 +101,7 @@ attention_block_kernel(const BlockAttnArgs a, int H, int split) {
     for (int u = tid; u < BQ * U; u += NT) {
         const int r = u / U, c = (u - r * U) * 8;
         const bool ok = q0 + r < a.Lq;
-        copy16(base + S::q + (r * LD + c) * 2, ok ? own + (int64_t)(q0 + r) * 3 * a.d + c : own, ok ? 16 : 0);
+        cp_async16(base + S::q + (r * LD + c) * 2, ok ? own + (int64_t)(q0 + r) * 3 * a.d + c : own, ok ? 16 : 0);
     }
 #pragma unroll
     for (int i = 0; i < STAGES - 1; ++i) {
@@ -145,7 +132,7 @@ attention_block_kernel(const BlockAttnArgs a, int H, int split) {
         commit();
         if (t == t0) {
 #pragma unroll
-            for (int k = 0; k < KS; ++k) ldsm_x4(qf[k], base + S::q + ((16 * mt + (lane & 15)) * LD + 16 * k + (lane >> 4) * 8) * 2);
+            for (int k = 0; k < KS; ++k) ldmatrix_x4(qf[k][0], qf[k][1], qf[k][2], qf[k][3], base + S::q + ((16 * mt + (lane & 15)) * LD + 16 * k + (lane >> 4) * 8) * 2);
         }
         const uint32_t ks = base + S::kv + st * 2 * S::TILE + WK * kg * LD * 2, vs = ks + S::TILE;
         // S = Q K^T: 16 queries x WK keys
@@ -159,9 +146,9 @@ attention_block_kernel(const BlockAttnArgs a, int H, int split) {
 #pragma unroll
             for (int n2 = 0; n2 < WK / 16; ++n2) {
                 uint32_t kb[4];                    // keys 0-7 of the 16: channels 16 k + (0-7, 8-15); keys 8-15 likewise
-                ldsm_x4(kb, ks + ((16 * n2 + (lane & 7) + (lane >> 4) * 8) * LD + 16 * k + ((lane >> 3) & 1) * 8) * 2);
-                mma16816(s[2 * n2], qf[k], kb[0], kb[1]);
-                mma16816(s[2 * n2 + 1], qf[k], kb[2], kb[3]);
+                ldmatrix_x4(kb[0], kb[1], kb[2], kb[3], ks + ((16 * n2 + (lane & 7) + (lane >> 4) * 8) * LD + 16 * k + ((lane >> 3) & 1) * 8) * 2);
+                mma_bf16_16816(s[2 * n2], qf[k][0], qf[k][1], qf[k][2], qf[k][3], kb[0], kb[1]);
+                mma_bf16_16816(s[2 * n2 + 1], qf[k][0], qf[k][1], qf[k][2], qf[k][3], kb[2], kb[3]);
             }
         const int kleft = Lk - t * KT - WK * kg;    // valid keys of this warp's share
         if (kleft < WK) {
@@ -203,13 +190,13 @@ attention_block_kernel(const BlockAttnArgs a, int H, int split) {
 #pragma unroll
             for (int n2 = 0; n2 < NO / 2; ++n2) {
                 uint32_t vb[4];                    // 16 keys x channels 16 n2 + (0-7, 8-15), transposed
-                ldsm_x4_t(vb, vs + ((16 * k2 + (lane & 15)) * LD + 16 * n2 + (lane >> 4) * 8) * 2);
-                mma16816(o[2 * n2], pf, vb[0], vb[1]);
-                mma16816(o[2 * n2 + 1], pf, vb[2], vb[3]);
+                ldmatrix_x4_t(vb[0], vb[1], vb[2], vb[3], vs + ((16 * k2 + (lane & 15)) * LD + 16 * n2 + (lane >> 4) * 8) * 2);
+                mma_bf16_16816(o[2 * n2], pf[0], pf[1], pf[2], pf[3], vb[0], vb[1]);
+                mma_bf16_16816(o[2 * n2 + 1], pf[0], pf[1], pf[2], pf[3], vb[2], vb[3]);
             }
         }
     }
-    asm volatile("cp.async.wait_all;" ::: "memory");
+    cp_async_wait_all();
     __syncthreads();                               // the ring is free: its bytes take the partial results
     float *ow = reinterpret_cast<float *>(sm + S::ow), *mw = reinterpret_cast<float *>(sm + S::mw), *lw = reinterpret_cast<float *>(sm + S::lw);
     float *oc = reinterpret_cast<float *>(sm + S::oc), *mc = reinterpret_cast<float *>(sm + S::mc), *lc = reinterpret_cast<float *>(sm + S::lc);

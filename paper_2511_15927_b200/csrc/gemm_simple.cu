@@ -121,8 +121,8 @@ gemm_f32_kernel(const __grid_constant__ F32Problems pr, const int sum) {
             const int r = u / (FK / 4), c = (u % (FK / 4)) * 4, left = K - k0 - c;
             const uint32_t nb = left >= 4 ? 16u : left > 0 ? 4u * left : 0u;
             const uint32_t na = m0 + r < M ? nb : 0u, nbb = n0 + r < N ? nb : 0u;
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(tc::smem_u32(as + r * FLD + c)), "l"(na ? A + (int64_t)(m0 + r) * a.lda + k0 + c : A), "r"(na) : "memory");
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(tc::smem_u32(bs + r * FLD + c)), "l"(nbb ? B + (int64_t)(n0 + r) * a.ldb + k0 + c : B), "r"(nbb) : "memory");
+            tc::cp_async16(as + r * FLD + c, na ? A + (int64_t)(m0 + r) * a.lda + k0 + c : A, na);
+            tc::cp_async16(bs + r * FLD + c, nbb ? B + (int64_t)(n0 + r) * a.ldb + k0 + c : B, nbb);
         }
     };
     float acc[4][4] = {};
@@ -154,7 +154,7 @@ gemm_f32_kernel(const __grid_constant__ F32Problems pr, const int sum) {
         if (i + 2 < mine) fetch(i + 2);
         asm volatile("cp.async.commit_group;" ::: "memory");
     }
-    asm volatile("cp.async.wait_all;" ::: "memory");
+    tc::cp_async_wait_all();
     __syncthreads();
     float *red = fsm;                                          // [FG][FT][FT + 1]
 #pragma unroll

@@ -1,6 +1,7 @@
 // Small row-wise kernels around the mixer: embedding gather, RMSNorm, the gated norm's rstd, arg-max
 // over the vocabulary, the carried conv state.  All are bandwidth-trivial next to the GEMMs and the scan.
 #include "dm_internal.h"
+#include "tc_ptx.cuh"
 
 namespace dm {
 namespace {
@@ -411,7 +412,8 @@ cudaError_t conv_state_update(const void *zx_fwd, const void *conv_in, void *con
 }
 
 cudaError_t combine_directions(void *g0, const void *g1, const float *rstd0, const float *rstd1, int dtype, int64_t T, int d_inner, cudaStream_t s) {
-    const int blocks = (int)(T < 148 * 8 ? T : 148 * 8);
+    const int64_t most = 8 * (int64_t)tc::sm_count();
+    const int blocks = (int)(T < most ? T : most);
     const size_t es = dtype_size(dtype);
     const bool vec = ((size_t)d_inner * es) % 16 == 0 && ((reinterpret_cast<uintptr_t>(g0) | reinterpret_cast<uintptr_t>(g1)) & 15u) == 0;
     if (dtype == DM_BF16) {
