@@ -119,10 +119,10 @@ static int check_weights(const dm_mixer_cfg *c, const dm_dir_weights w[2]) {
     return DM_OK;
 }
 
-// Up to this many tokens the two directions' in_proj share one launch.  Beyond it two launches are faster: both weight matrices
-// together (70 MB at d_model 2048) no longer stay in L2 while the rows of x stream past them (measured at 16 384 tokens: 1.00 ms
-// for the pair against 0.84 ms for two launches; level at 8192, 15-25 % faster for the 512 tokens of a decoding step).
-constexpr int64_t PAIR_IN_MAX_T = 4096;
+// Both directions' in_proj share one launch up to this many tokens, or at any length while both weight matrices are small enough to stay in L2 beside the rows of x that stream past them.
+// A layer with one launch / two, one sequence: 1024 tokens at d_model 1024, 1920, 2048: 68 / 75, 120 / 130, 120 / 126 us; 5000 tokens: 221 / 229, 466 / 473, 455 / 459; 16384 tokens: 605 / 611
+// (17 MB of weights), 1458 / 1412 (62 MB), 1439 / 1371 (70 MB).  In between, 6 x 2048 tokens: d_model 1280 (28 MB) 525 / 530, 1536 (40 MB) 666 / 663.
+constexpr int64_t PAIR_IN_MAX_T = 6144, PAIR_IN_L2_BYTES = 32 << 20;
 
 // Workspace layout of one mixer call.
 struct MixerWs {
@@ -224,7 +224,7 @@ static int run_mixer(const dm_mixer_cfg *c, const Dims &m, const dm_dir_weights 
             ga[n++] = a;
         }
         StageTimer tm(DM_STAGE_IN_PROJ, s);
-        if (n == 2 && m.T <= PAIR_IN_MAX_T && gemm_tcgen05_pair_supports(ga[0], ga[1])) {
+        if (n == 2 && (m.T <= PAIR_IN_MAX_T || 2 * (int64_t)m.d_in_proj * m.d * (int64_t)m.es <= PAIR_IN_L2_BYTES) && gemm_tcgen05_pair_supports(ga[0], ga[1])) {
             // both directions in one launch: x is fetched once for the two, and there is one tail round instead of two
             if ((e = gemm_tcgen05_pair(ga[0], ga[1], s)) != cudaSuccess) return cuda_fail(e, "in_proj");
         } else if (n == 2 && gemm_f32_supports(ga[0], 2) && gemm_f32_supports(ga[1], 2)) {

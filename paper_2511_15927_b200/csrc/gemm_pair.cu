@@ -1,4 +1,4 @@
-// The GEMM of gemm_tcgen05.cu for more than 128 rows, on pairs of CTAs (tcgen05 cta_group::2): the two SMs of a pair work on one 256-row
+// The GEMM for more than 128 rows (the choice is in gemm_tcgen05.cu), on pairs of CTAs (tcgen05 cta_group::2): the two SMs of a pair work on one 256-row
 // tile, each holding half of its rows of A and of its accumulators, and each loading half of B -- the tensor cores read the other half
 // out of the partner's shared memory.  Per product that is two thirds of the operand traffic (L2 to shared memory) of a single CTA's 128 x 256
 // tile.  Bound by the tensor cores under the power limit on large products (about 1.3 GHz in a long run): 16384 x 8512 x 2048 in 438 us =
@@ -9,7 +9,7 @@
 // report to the first CTA's barrier; warp 1 of the first CTA issues the MMAs of the pair; warps 2-9 drain this CTA's accumulators.
 // Tile order: the larger operand is streamed from HBM once, the other one stays in L2 (n_fast: consecutive tiles step along N).
 //
-// Waits and abort as in gemm_tcgen05.cu: every mbarrier wait is bounded, in both CTAs; the CTAs of a pair leave together.
+// Every mbarrier wait is bounded, in both CTAs; on expiry the CTA stores DM_ERR_TIMEOUT in the device status word, lets its loads land and frees TMEM; the CTAs of a pair leave together.
 #include <cstring>
 
 #include "gemm_epi.cuh"
@@ -35,8 +35,9 @@ struct OpMaps { CUtensorMap a[2], b[2], bn[2]; };
 
 // The tiles of a launch, in the order in which the pairs take them: tile i goes to pair i % npairs.  Tiles are 256 rows x BN columns; with BN = 256 a last column tile of at most 128 columns is
 // narrow (256 x 128: 0.74 of a wide tile's time, see gemm_tcgen05.cu), and so are the halves into which the wide tiles of an incomplete last round are cut where that ends
-// earlier.  Narrow ones come last.  (16384 x 1024, 256 wide tiles for 74 pairs: 222 wide and 68 halves, 3.74 rounds instead of 4.  One layer of 1024 tokens,
-// in_proj 252 tiles of which 8 are 120 columns wide: 129.5 -> 128.2 us; 24 conditioned layers of 8192 tokens, under the power limit: 28.02 -> 27.89 ms.)
+// earlier.  Narrow ones come last.  (16384 x 1024, 256 wide tiles for 74 pairs: 222 wide and 68 halves, 3.74 rounds instead of 4.  All tiles of one width / these, one layer: 1 x 1024
+// tokens at d_model 1920 124 / 120 us, 3 x 1111 343 / 330; 1 x 6000 at 1024 270 / 259; 8 x 1024 at 2048 731 / 719; 4 conditioned layers of 3 x 700 at 1920 1571 / 1528.  Level or up to 1 % slower
+// where the rounds come out even, as 8 x 2048.)
 struct TileAt { int mb, prob, n0; bool narrow; };
 template <int BN> struct Tiles {
     int tiles_m, wn, wn_all, whole, halves, total, n_fast;     // row tiles; wide columns per problem, over all problems; uncut wide tiles; halves; all tiles

@@ -401,7 +401,9 @@ cudaError_t launch(const SsdArgs &a, int ndir, int dir0, cudaStream_t s) {
     // As many CTAs as are resident at once, so that what the heads share is computed as seldom as one round allows, and shared out between the directions by what a head costs:
     // a left-to-right one reads its state, and with COMMIT writes it (16 sequences of 64 heads: 4.0 us against 2.8, and 4.2 against 1.9; with equal shares the SMs that happened to
     // get left-to-right CTAs only finished at 27 and 43 us, the others at 19 and 18;
-    // one layer with the state committed 103 -> 96 us, 24 layers 2191 -> 2118 us).
+    // one layer with the state committed 103 -> 96 us, 24 layers 2191 -> 2118 us).  The same costs serve smaller states and 32-wide heads: with equal ones a committed layer of 16 sequences took
+    // 56 us instead of 51 at d_state 16 and 97 instead of 87 with 120 heads of 32, with ones scaled to the state's bytes 56 at d_state 16; without a commit all are level (24 sequences of 64
+    // heads: equal shares 110 us, these 115).
     StepSplit sp{};
     const int slots = sm_count() * RES<PP, HW, COMMIT> / a.B, cap = HG_MAX<COMMIT>;
     const int cost[2] = {!a.ssm_in && !COMMIT ? 10 : COMMIT ? 22 : 14, 10};

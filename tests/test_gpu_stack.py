@@ -45,12 +45,11 @@ def test_denoise_step_full_sequence(G, dtype, N, d, H, layers, V):
     np.testing.assert_array_equal(amax, amax2)
 
 
-def _launches_with_summed_out_proj(B, L, layers, cond):
+def _launches_with_summed_out_proj(layers, cond):
     """Kernels of a stack pass whose out_proj is one launch per layer that also writes the next norm's input (sequences of more than 64 tokens): in_proj (one launch for both
-    directions up to 4096 tokens), prep, scan, out_proj; around them the embedding, the first norm and the vocabulary -- or, with a conditioned block, its modulation, two AdaLN and
+    directions at these widths), prep, scan, out_proj; around them the embedding, the first norm and the vocabulary -- or, with a conditioned block, its modulation, two AdaLN and
     two products, and the final norm.  A layer whose directions are not summed in one launch takes three more (row scales, a second product, the norm)."""
-    per_layer = (1 if B * L <= 4096 else 2) + 3 + (5 if cond else 0)
-    return 3 + layers * per_layer
+    return 3 + layers * (4 + (5 if cond else 0))
 
 
 @pytest.mark.parametrize("d,H,B,L,d_ff", [(160, 5, 3, 683, 0), (64, 2, 1, 2049, 0), (320, 10, 2, 1100, 640), (320, 10, 10, 500, 640)])
@@ -70,7 +69,7 @@ def test_denoise_step_summed_out_proj(G, d, H, B, L, d_ff):
     want = O.denoise_step_cond(tok, tau, sw, **kw) if d_ff else O.denoise_step(tok, sw, **kw)
     before = dm.dm_kernel_launch_count()
     got, _, _ = G.run_denoise(shape, I.BF16, sw, tok, 96, want_argmax=False, tau=tau, d_ff=d_ff)
-    assert dm.dm_kernel_launch_count() - before == _launches_with_summed_out_proj(B, L, 3, d_ff > 0)
+    assert dm.dm_kernel_launch_count() - before == _launches_with_summed_out_proj(3, d_ff > 0)
     assert G.rel_l2(got, want) <= 1e-2, G.rel_l2(got, want)
 
 
