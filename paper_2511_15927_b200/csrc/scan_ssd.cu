@@ -1308,12 +1308,15 @@ cudaError_t scan_ssd(const ScanArgs &a, void *ws, cudaStream_t s) {
     // One long sequence leaves SMs without a scan CTA: they take the prep work inside the scan launch (see prep_role), except for
     // the first PRE_CHUNKS chunks of every sequence and direction, which a small prep launch of their own has ready by the time the
     // scan starts (a prep CTA inside the scan launch needs about 20 us for its first chunk; the scan would stand idle that long).
-    constexpr int PRE_CHUNKS = 8;
+    // From FUSE_CHUNKS chunks on: prep in a launch of its own / inside, one layer, 64 heads of 64 (20 SMs left over): 2048 tokens 197 / 202 us, 8192 710 / 708, 16384 1388 / 1369, 32768
+    // 2789 / 2753; 120 heads of 32: 201 / 207, 743 / 737, 1430 / 1412, 2929 / 2843.  Two and more sequences: the SMs left over do not keep up with 2 B chains of chunks (2 x 8192, 32 heads
+    // 467 / 507 us, 4 x 8192, 16 heads 416 / 572).
+    constexpr int PRE_CHUNKS = 8, FUSE_CHUNKS = 64;
     const bool pair = a.P == P / 2 && a.H % 2 == 0;        // two half-width heads per scan CTA
     const int nscan = (pair ? a.H / 2 : a.H) * ndir * a.B;
     PrepJob pj{Bp, Cp, dA, nullptr, 0, ndir, 0};
     int n_pre = l.nch;                              // chunks (in time order) done by the prep launch
-    if (!blk && nscan < sm_count() && a.N % 8 == 0 && l.nch > PRE_CHUNKS) {
+    if (!blk && nscan < sm_count() && a.N % 8 == 0 && l.nch > PRE_CHUNKS && (g_withhold_prep || (a.B == 1 && l.nch >= FUSE_CHUNKS))) {
         const int n_items = ndir * a.B * (l.nch - PRE_CHUNKS);
         pj.nprep = n_items < sm_count() - nscan ? n_items : sm_count() - nscan;
         if (ndir == 2) pj.nprep &= ~1;                             // even: every prep CTA then stays with one direction

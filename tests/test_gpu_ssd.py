@@ -202,3 +202,19 @@ def test_blocks_of_up_to_32_tokens(G, B, H, P, N, L, k):
     y_r, _, _ = G.run_block_step(shape, I.BF16, wf, wr, x, ssm_in, conv_in, want_state=False)
     np.testing.assert_array_equal(y_r, y_g)                 # committing the state leaves the output alone
     _check(G, G.run_forward(shape, I.BF16, wf, wr, x), O.bimamba_forward(x, wf, wr, **kw))
+
+
+@pytest.mark.parametrize("H,P,N,L,k", [(2, 64, 128, 8064, 4), (2, 64, 64, 8065, 3), (4, 32, 16, 8197, 4)])
+def test_prep_inside_the_scan_launch(G, H, P, N, L, k):
+    """One sequence at the line (63 chunks: a prep launch of its own; 64 and 65: the chunks from the ninth on are prepared inside the scan launch), a last chunk of one token and of five, carried state in
+    and out, padded d_state, two 32-wide heads to a CTA."""
+    shape = I.MixerShape(1, L, P * H // 2, 2, N, k, H)
+    wf, wr = I.make_mixer_weights(shape, 70, I.BF16, perturb=True)
+    x = I.make_activations(shape, 70, I.BF16)
+    kw = G.oracle_kwargs(shape)
+    ssm_in, conv_in = I.make_states(shape, 70, I.BF16)
+    y_o, s_o, c_o = O.bimamba_block_step(x, wf, wr, ssm_state_in=ssm_in, conv_state_in=conv_in, **kw)
+    y_g, s_g, c_g = G.run_block_step(shape, I.BF16, wf, wr, x, ssm_in, conv_in)
+    _check(G, y_g, y_o)
+    _check(G, s_g, s_o)
+    _check(G, c_g, c_o)
