@@ -99,11 +99,9 @@ inline bool gemm_tensor_ok(const GemmArgs &a) {
     if (a.rs_ssq && a.rs_n % 4 == 0 && off16(a.rs_ssq)) return false;       // (read as float4 where a row holds whole ones, one by one elsewhere)
     return true;
 }
-// Output and addend can go through TMA: 16-byte aligned rows, and no bf16 output with an addend (EpiOut in gemm_epi.cuh keeps the first 32 of 64 bf16 columns in the staging bytes
-// until the other 32 are there, and the addend of those arrives in the same bytes).
+// Output and addend can go through TMA: 16-byte aligned rows.
 inline bool gemm_tma_io(const GemmArgs &a) {
-    if (a.addend && (a.c_dtype != DM_F32 || a.ld_add % 4)) return false;
-    return (a.ldc * (int64_t)dtype_size(a.c_dtype)) % 16 == 0;
+    return (a.ldc * (int64_t)dtype_size(a.c_dtype)) % 16 == 0 && (!a.addend || a.ld_add % 4 == 0);
 }
 // The sum of two products in one launch: its epilogues know scales and the addend, no bias and no activation.
 inline bool gemm_sum_ok(const GemmArgs &a, const GemmArgs &b) {

@@ -181,7 +181,7 @@ __device__ __forceinline__ void epi_add_store(const EpiArgs &ep, const EpiRow &e
 }
 
 constexpr uint32_t STG_BYTES = 32 * 128;     // staging of one epilogue warp
-// Tensor maps of the outputs (boxes of 32 rows x 128 bytes), the addend and the next norm's input.
+// Tensor maps of the outputs (boxes of 32 rows x 128 bytes; 64 of a bf16 one with an addend), the addend and the next norm's input (64 bytes).
 struct IoMaps { CUtensorMap c[2], add, u; };
 
 // How one epilogue warp's 32 rows reach memory: 32 rows x 128 bytes at a time through 4 KB of shared memory and TMA.
@@ -194,6 +194,7 @@ struct EpiOut {
     int *status;
     uint32_t add_count;
     __device__ __forceinline__ uint4 *piece(int j) const { return reinterpret_cast<uint4 *>(stg + lane * 128 + ((j ^ (lane & 7)) << 4)); }
+    __device__ __forceinline__ uint4 *half_piece(int j) const { return reinterpret_cast<uint4 *>(stg + lane * 64 + ((j ^ ((lane >> 1) & 3)) << 4)); }     // of 32 rows x 64 bytes, the 64-byte swizzle
     __device__ __forceinline__ void free() const {             // the previous store has read the staging bytes
         if (lane == 0) bulk_wait_read0();
         __syncwarp();
@@ -220,13 +221,20 @@ struct EpiOut {
         return r;
     }
     // One 32-column group of results (columns n0 + c0 .., n0 a multiple of 64): to the output, and to the next norm's input where that is asked for.  ss: the row's sum of
-    // squares over the current 64 columns.
+    // squares over the current 64 columns.  ADD: an addend of later columns may be fetched into the staging bytes in between, so a bf16 output with one leaves 32 columns at a time.
+    template <bool ADD>
     __device__ __forceinline__ void emit(const EpiArgs &pe, const CUtensorMap &map_c, const CUtensorMap &map_u, int n0, int c0, int row0, int row, bool row_ok, const float *v, float &ss) const {
         const int col = n0 + c0;
         if (pe.c_is_f32) {
             free();
 #pragma unroll
             for (int j = 0; j < 8; ++j) *piece(j) = make_uint4(__float_as_uint(v[4 * j]), __float_as_uint(v[4 * j + 1]), __float_as_uint(v[4 * j + 2]), __float_as_uint(v[4 * j + 3]));
+            store(map_c, col, row0);
+        } else if (ADD && pe.addend) {
+            free();
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                *half_piece(j) = make_uint4(pack_bf16(v[8 * j], v[8 * j + 1]), pack_bf16(v[8 * j + 2], v[8 * j + 3]), pack_bf16(v[8 * j + 4], v[8 * j + 5]), pack_bf16(v[8 * j + 6], v[8 * j + 7]));
             store(map_c, col, row0);
         } else {
             if (!(c0 & 32)) free();
@@ -236,14 +244,14 @@ struct EpiOut {
                                                       pack_bf16(v[8 * j + 4], v[8 * j + 5]), pack_bf16(v[8 * j + 6], v[8 * j + 7]));
             if ((c0 & 32) || col + 32 >= pe.N) store(map_c, n0 + (c0 & ~63), row0);
         }
-        if (pe.u) {                                            // 32 rows x 64 bytes, the 64-byte swizzle of its map
+        if (pe.u) {
             free();
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 const bool in = col + 8 * j < pe.N;            // N is a multiple of 8
                 const uint4 w4 = in ? __ldg(reinterpret_cast<const uint4 *>(pe.u_w + col + 8 * j)) : make_uint4(0u, 0u, 0u, 0u);
                 const float *x = v + 8 * j;
-                *reinterpret_cast<uint4 *>(stg + lane * 64 + ((j ^ ((lane >> 1) & 3)) << 4)) =
+                *half_piece(j) =
                     make_uint4(pack_bf16(x[0] * bf16_lo(w4.x), x[1] * bf16_hi(w4.x)), pack_bf16(x[2] * bf16_lo(w4.y), x[3] * bf16_hi(w4.y)),
                                pack_bf16(x[4] * bf16_lo(w4.z), x[5] * bf16_hi(w4.z)), pack_bf16(x[6] * bf16_lo(w4.w), x[7] * bf16_hi(w4.w)));
                 if (in) {
@@ -268,14 +276,20 @@ inline bool make_map_2d(CUtensorMap *m, const void *base, int64_t rows, int64_t 
     return make_map_bf16(m, base, 2, dims, strides, box);
 }
 
-// The next norm's input: box = 32 rows x 32 columns, 64-byte swizzle.
-inline bool make_map_u(CUtensorMap *m, const void *base, int64_t rows, int64_t cols) {
+// bf16 tensor in boxes of 32 rows x 32 columns, 64-byte swizzle: the next norm's input, a bf16 output with an addend.
+inline bool make_map_half(CUtensorMap *m, const void *base, int64_t rows, int64_t cols, int64_t ld) {
     EncodeTiledFn fn = encode_fn();
     if (!fn) return false;
-    const cuuint64_t d[2] = {(cuuint64_t)cols, (cuuint64_t)rows}, st[1] = {(cuuint64_t)cols * 2};
+    const cuuint64_t d[2] = {(cuuint64_t)cols, (cuuint64_t)rows}, st[1] = {(cuuint64_t)ld * 2};
     const cuuint32_t b[2] = {32, 32}, e[2] = {1, 1};
     return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(base), d, st, b, e, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B,
               CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// The output as EpiOut::emit<add> stores it
+inline bool make_map_out(CUtensorMap *m, const EpiArgs &p, bool add) {
+    if (p.c_is_f32) return make_map_f32_2d(m, p.C, p.M, p.N, p.ldc, 32);
+    return add && p.addend ? make_map_half(m, p.C, p.M, p.N, p.ldc) : make_map_2d(m, p.C, p.M, p.N, p.ldc, 32);
 }
 
 }  // namespace tc

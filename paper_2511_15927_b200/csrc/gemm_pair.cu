@@ -239,7 +239,7 @@ gemm_pair_kernel(const __grid_constant__ OpMaps op, const __grid_constant__ IoMa
             const bool add = MODE != DIRECT && pe.addend && live;
             if (MODE == TMA && add) out.add_fetch(io.add, n0, row0);       // the first columns' addend arrives while the products run
             float ss = 0.f;
-            auto emit = [&](int c0, const float *v) { out.emit(pe, io.c[prob], io.u, n0, c0, row0, row, row_ok, v, ss); };
+            auto emit = [&](int c0, const float *v) { out.template emit<MODE != SUM>(pe, io.c[prob], io.u, n0, c0, row0, row, row_ok, v, ss); };
             if constexpr (MODE == SUM) {
                 const EpiArgs &p0 = epp.p[0];
                 const float sc0 = row_ok ? epi_row_scale(p0, row) : 1.f;
@@ -351,11 +351,11 @@ cudaError_t launch(const GemmArgs &a, const GemmArgs *b, cudaStream_t s) {
     if (MODE != DIRECT) {
         for (int i = MODE == SUM ? 1 : 0; i < epp.nprob; ++i) {
             const EpiArgs &p = epp.p[i];
-            if (!(p.c_is_f32 ? make_map_f32_2d(&io.c[i], p.C, p.M, p.N, p.ldc, 32) : make_map_2d(&io.c[i], p.C, p.M, p.N, p.ldc, 32))) return cudaErrorInvalidValue;
+            if (!make_map_out(&io.c[i], p, MODE != SUM)) return cudaErrorInvalidValue;
         }
         const EpiArgs &p = epp.p[MODE == SUM ? 1 : 0];         // (separate problems in one launch have no addend here: see tma_io)
         if (p.addend && !make_map_f32_2d(&io.add, p.addend, p.M, p.N, p.ld_add, 32)) return cudaErrorInvalidValue;
-        if (p.u && !make_map_u(&io.u, p.u, p.M, p.N)) return cudaErrorInvalidValue;
+        if (p.u && !make_map_half(&io.u, p.u, p.M, p.N, p.N)) return cudaErrorInvalidValue;
     }
     const int pairs = sm_count() / 2, tiles = Tiles<BN>(a.M, a.N, MODE == SUM ? 1 : epp.nprob, pairs, epp.n_fast).total, grid = 2 * (tiles < pairs ? tiles : pairs);
     return launch_chain(gemm_pair_kernel<BN, MODE>, grid, NTHREADS, smem, s, 0, op, io, epp, status);

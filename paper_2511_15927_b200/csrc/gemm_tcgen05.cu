@@ -19,10 +19,10 @@ bool pair_wide_tile(const GemmArgs &a, int nprob) { return a.N > 128 && gemm_pai
 // Which kernel for up to 128 rows.  gemm_rows.cu is the faster reader of weights, but what it does per row -- a row's scale from its sums of squares, one round trip to memory after the other,
 // and its stores -- shows where the products are short.  K up to 768, more than 80 rows with such scales or 96 without: few-row kernel / pair kernel 128 x 2000 x 512 12.5 / 10.4 us, 12 decoding
 // layers of 96 tokens 344 / 298 us at d_model 512, 377 / 300 at 256; K = 1024: level at 128 rows, 10.4 / 12.5 us at 80.  More tiles than two to an SM go to its looping form at any K
-// (128 x 50304 x 512: 18.5 / 22.7 us).
+// (128 x 50304 x 512: 18.5 / 22.7 us); so do outputs that the pair kernel cannot store through TMA (100 x 300 x 512, bf16 rows of 600 bytes with an addend: 12.5 / 24 us).
 bool few_rows(const GemmArgs &a, int nprob) {
     if (a.M > BM) return false;
-    return a.M <= (a.rs_ssq ? 80 : 96) || a.K > 768 || (int64_t)((a.N + BM - 1) / BM) * nprob > 2 * sm_count();
+    return a.M <= (a.rs_ssq ? 80 : 96) || a.K > 768 || !gemm_tma_io(a) || (int64_t)((a.N + BM - 1) / BM) * nprob > 2 * sm_count();
 }
 
 cudaError_t dispatch(const GemmArgs &a, const GemmArgs *b, cudaStream_t s) {
