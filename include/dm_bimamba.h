@@ -362,7 +362,7 @@ int dm_selftest_wait_timeout(uint32_t limit_us, uint64_t *out, void *cuda_stream
 
 /* Self-test switch for the same failure path inside the tensor-core scan (no counterpart in the paper).  While on, a mixer call
  * whose scan can do its prep work inside the scan launch (fewer scan CTAs than SMs, more than eight chunks; outside the test one
- * sequence of 64 chunks or more does) launches the scan without the CTAs of that role: the flags its load warps wait for from the ninth chunk on are never raised,
+ * sequence of 32 chunks or more does) launches the scan without the CTAs of that role: the flags its load warps wait for from the ninth chunk on are never raised,
  * the waits run out after their regular limit (2 s), and every role of every CTA has to leave through the abort path -- loads in
  * flight waited for, TMEM freed.  A call on the sequential scan (fp32, or d_state 256) of more than two chunks leaves out the
  * copies of every CTA's third chunk, with the same consequences.  The call itself returns DM_OK; dm_check then reports

@@ -27,11 +27,11 @@ int *device_status_ptr();
 // layer of 1024 tokens 140 -> 136 us.
 inline thread_local bool g_chain = false;
 inline void chain_begin() { g_chain = false; }
-// Before the launch of a kernel whose few CTAs each run long and could share an SM: behind a grid of `ahead` CTAs that covers the GPU it is launched without overlap.  Ahead of time its CTAs
+// Before the launch of a kernel of few CTAs that each run long and could share an SM: behind a grid of `ahead` CTAs that covers the GPU it is launched without overlap.  Ahead of time its CTAs
 // would be packed onto the SMs that have the most room at that moment and stay there: chunk-32 scan of 1 x 4096 tokens, 32 heads, behind 192 prep CTAs 674 us, 472 us spread out;
 // fp32 layer of 1 x 8192 tokens, 8 heads, 830 and 589 us.  Behind a grid that leaves SMs empty the overlap does no harm (1 x 1024: 113 us either way).
-inline void chain_spread(int64_t ahead, int sms) {
-    if (ahead > sms) chain_begin();
+inline void chain_spread(int64_t ahead, int64_t ctas, int sms) {
+    if (ahead > sms && ctas < 2 * sms) chain_begin();
 }
 #ifdef __CUDACC__
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
@@ -103,11 +103,11 @@ inline bool gemm_tensor_ok(const GemmArgs &a) {
 inline bool gemm_tma_io(const GemmArgs &a) {
     return (a.ldc * (int64_t)dtype_size(a.c_dtype)) % 16 == 0 && (!a.addend || a.ld_add % 4 == 0);
 }
-// The sum of two products in one launch: its epilogues know scales and the addend, no bias and no activation.
+// The sum of two products in one launch: its epilogues know scales and, for fp32 outputs, the addend; no bias and no activation.
 inline bool gemm_sum_ok(const GemmArgs &a, const GemmArgs &b) {
     for (const GemmArgs *p : {&a, &b})
         if (!gemm_tensor_ok(*p) || p->m_dev || p->col_bias || p->gelu || p->silu_cols) return false;
-    return a.M == b.M && a.N == b.N && a.K == b.K && gemm_tma_io(b);
+    return a.M == b.M && a.N == b.N && a.K == b.K && gemm_tma_io(b) && !(b.addend && b.c_dtype == DM_BF16);
 }
 cudaError_t gemm_simple(const GemmArgs &a, cudaStream_t s);
 // fp32 products that do not fill the GPU: n of them (same sizes) in one launch, or both into b's output (sum).

@@ -187,7 +187,7 @@ gemm_cluster_sum_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid
             }
             epi_pre<false>(pe, er, col, v);
             if (pe.addend) ok = out.add_take(v);
-            if (ok) out.emit<true>(pe, io.c[1], io.u, n0, c0, row0, row, row_ok, v, ss);
+            if (ok) out.emit<false>(pe, io.c[1], io.u, n0, c0, row0, row, row_ok, v, ss);
         }
         if (lane == 0) bulk_wait_read0();      // (what the stores wrote is complete when the launch is)
     }
@@ -227,7 +227,7 @@ cudaError_t launch(const GemmArgs &a, const GemmArgs &b, cudaStream_t s) {
     IoMaps io;
     memset(&io, 0, sizeof(io));
     const EpiArgs &p = epp.p[1];
-    if (!make_map_out(&io.c[1], p, true)) return cudaErrorInvalidValue;
+    if (!make_map_out(&io.c[1], p, false)) return cudaErrorInvalidValue;
     if (p.addend && !make_map_f32_2d(&io.add, p.addend, p.M, p.N, p.ld_add, 32)) return cudaErrorInvalidValue;
     if (p.u && !make_map_half(&io.u, p.u, p.M, p.N, p.N)) return cudaErrorInvalidValue;
     cudaError_t e = cudaFuncSetAttribute(gemm_cluster_sum_kernel<NP, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Tile<BN>::SMEM);

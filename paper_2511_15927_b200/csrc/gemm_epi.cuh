@@ -181,7 +181,7 @@ __device__ __forceinline__ void epi_add_store(const EpiArgs &ep, const EpiRow &e
 }
 
 constexpr uint32_t STG_BYTES = 32 * 128;     // staging of one epilogue warp
-// Tensor maps of the outputs (boxes of 32 rows x 128 bytes; 64 of a bf16 one with an addend), the addend and the next norm's input (64 bytes).
+// Tensor maps of the outputs (boxes of 32 rows x 128 bytes; 64 of a bf16 one stored in halves), the addend and the next norm's input (64 bytes).
 struct IoMaps { CUtensorMap c[2], add, u; };
 
 // How one epilogue warp's 32 rows reach memory: 32 rows x 128 bytes at a time through 4 KB of shared memory and TMA.
@@ -221,8 +221,8 @@ struct EpiOut {
         return r;
     }
     // One 32-column group of results (columns n0 + c0 .., n0 a multiple of 64): to the output, and to the next norm's input where that is asked for.  ss: the row's sum of
-    // squares over the current 64 columns.  ADD: an addend of later columns may be fetched into the staging bytes in between, so a bf16 output with one leaves 32 columns at a time.
-    template <bool ADD>
+    // squares over the current 64 columns.  HALF: a bf16 output 32 columns at a time, because an addend's next columns are fetched into the staging bytes in between.
+    template <bool HALF>
     __device__ __forceinline__ void emit(const EpiArgs &pe, const CUtensorMap &map_c, const CUtensorMap &map_u, int n0, int c0, int row0, int row, bool row_ok, const float *v, float &ss) const {
         const int col = n0 + c0;
         if (pe.c_is_f32) {
@@ -230,7 +230,7 @@ struct EpiOut {
 #pragma unroll
             for (int j = 0; j < 8; ++j) *piece(j) = make_uint4(__float_as_uint(v[4 * j]), __float_as_uint(v[4 * j + 1]), __float_as_uint(v[4 * j + 2]), __float_as_uint(v[4 * j + 3]));
             store(map_c, col, row0);
-        } else if (ADD && pe.addend) {
+        } else if (HALF) {
             free();
 #pragma unroll
             for (int j = 0; j < 4; ++j)
@@ -286,10 +286,10 @@ inline bool make_map_half(CUtensorMap *m, const void *base, int64_t rows, int64_
               CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// The output as EpiOut::emit<add> stores it
-inline bool make_map_out(CUtensorMap *m, const EpiArgs &p, bool add) {
+// The output as EpiOut::emit<half> stores it
+inline bool make_map_out(CUtensorMap *m, const EpiArgs &p, bool half) {
     if (p.c_is_f32) return make_map_f32_2d(m, p.C, p.M, p.N, p.ldc, 32);
-    return add && p.addend ? make_map_half(m, p.C, p.M, p.N, p.ldc) : make_map_2d(m, p.C, p.M, p.N, p.ldc, 32);
+    return half ? make_map_half(m, p.C, p.M, p.N, p.ldc) : make_map_2d(m, p.C, p.M, p.N, p.ldc, 32);
 }
 
 }  // namespace tc

@@ -92,7 +92,8 @@ struct __align__(8) Bars {
 //   SUM     TMA, and the two problems are summed (s_0 A_0 B_0^T + s_1 A_1 B_1^T into problem 1's output): a pair runs both on a tile, one after the other in the
 //           two accumulator buffers; the epilogue warps take the first product out of TMEM into registers (128 per thread, scaled by its
 //           rows' factor, the addend added) while the second one runs, so the sum costs no pass over memory and the buffers still alternate
-enum { DIRECT = 0, TMA = 1, SUM = 2 };
+//   TMA_HALF  TMA for a bf16 output with an addend, 32 columns at a time (a form of its own: as a branch it cost the projections of a layer 1 %)
+enum { DIRECT = 0, TMA = 1, SUM = 2, TMA_HALF = 3 };
 template <int BN, int MODE>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
 gemm_pair_kernel(const __grid_constant__ OpMaps op, const __grid_constant__ IoMaps io, const __grid_constant__ EpiPair epp, int *status) {
@@ -237,9 +238,9 @@ gemm_pair_kernel(const __grid_constant__ OpMaps op, const __grid_constant__ IoMa
             const float sc = row_ok ? epi_row_scale(pe, row) : 1.f;
             const EpiRow er(pe, row_ok ? row : 0);
             const bool add = MODE != DIRECT && pe.addend && live;
-            if (MODE == TMA && add) out.add_fetch(io.add, n0, row0);       // the first columns' addend arrives while the products run
+            if ((MODE == TMA || MODE == TMA_HALF) && add) out.add_fetch(io.add, n0, row0);       // the first columns' addend arrives while the products run
             float ss = 0.f;
-            auto emit = [&](int c0, const float *v) { out.template emit<MODE != SUM>(pe, io.c[prob], io.u, n0, c0, row0, row, row_ok, v, ss); };
+            auto emit = [&](int c0, const float *v) { out.template emit<MODE == TMA_HALF>(pe, io.c[prob], io.u, n0, c0, row0, row, row_ok, v, ss); };
             if constexpr (MODE == SUM) {
                 const EpiArgs &p0 = epp.p[0];
                 const float sc0 = row_ok ? epi_row_scale(p0, row) : 1.f;
@@ -351,7 +352,7 @@ cudaError_t launch(const GemmArgs &a, const GemmArgs *b, cudaStream_t s) {
     if (MODE != DIRECT) {
         for (int i = MODE == SUM ? 1 : 0; i < epp.nprob; ++i) {
             const EpiArgs &p = epp.p[i];
-            if (!make_map_out(&io.c[i], p, MODE != SUM)) return cudaErrorInvalidValue;
+            if (!make_map_out(&io.c[i], p, MODE == TMA_HALF)) return cudaErrorInvalidValue;
         }
         const EpiArgs &p = epp.p[MODE == SUM ? 1 : 0];         // (separate problems in one launch have no addend here: see tma_io)
         if (p.addend && !make_map_f32_2d(&io.add, p.addend, p.M, p.N, p.ld_add, 32)) return cudaErrorInvalidValue;
@@ -371,7 +372,10 @@ int gemm_pair_cost(bool wide, const GemmArgs &a, int nprob) {
 }
 
 cudaError_t gemm_pair_launch(bool wide, const GemmArgs &a, const GemmArgs *b, cudaStream_t s) {
-    if (tma_io(a, b)) return wide ? launch<256, TMA>(a, b, s) : launch<128, TMA>(a, b, s);
+    if (tma_io(a, b)) {
+        if (a.addend && a.c_dtype == DM_BF16) return wide ? launch<256, TMA_HALF>(a, b, s) : launch<128, TMA_HALF>(a, b, s);
+        return wide ? launch<256, TMA>(a, b, s) : launch<128, TMA>(a, b, s);
+    }
     return wide ? launch<256, DIRECT>(a, b, s) : launch<128, DIRECT>(a, b, s);
 }
 

@@ -412,7 +412,7 @@ cudaError_t scan_sequential(const ScanArgs &a, void *ws, cudaStream_t s) {
     e = a.dtype == DM_BF16 ? launch_chain(bc_prep_kernel<__nv_bfloat16>, pgrid, bt, 0, s, 0, a, dir0, bc) : launch_chain(bc_prep_kernel<float>, pgrid, bt, 0, s, 0, a, dir0, bc);
     if (e != cudaSuccess) return e;
     dim3 grid(a.H, ndir, a.B);
-    chain_spread((int64_t)pgrid.x * pgrid.y * pgrid.z, sm_count());
+    chain_spread((int64_t)pgrid.x * pgrid.y * pgrid.z, (int64_t)a.H * ndir * a.B, sm_count());
     return launch_chain(kern, grid, a.P * lanes_per_channel(a.N) + loaders(a.P, a.N), smem, s, 0, mx, mz, a, dir0, TC, scan_selftest_withheld() ? 2 : -1, bc, status);
 }
 

@@ -1308,10 +1308,10 @@ cudaError_t scan_ssd(const ScanArgs &a, void *ws, cudaStream_t s) {
     // One long sequence leaves SMs without a scan CTA: they take the prep work inside the scan launch (see prep_role), except for
     // the first PRE_CHUNKS chunks of every sequence and direction, which a small prep launch of their own has ready by the time the
     // scan starts (a prep CTA inside the scan launch needs about 20 us for its first chunk; the scan would stand idle that long).
-    // From FUSE_CHUNKS chunks on: prep in a launch of its own / inside, one layer, 64 heads of 64 (20 SMs left over): 2048 tokens 197 / 202 us, 8192 710 / 708, 16384 1388 / 1369, 32768
-    // 2789 / 2753; 120 heads of 32: 201 / 207, 743 / 737, 1430 / 1412, 2929 / 2843.  Two and more sequences: the SMs left over do not keep up with 2 B chains of chunks (2 x 8192, 32 heads
-    // 467 / 507 us, 4 x 8192, 16 heads 416 / 572).
-    constexpr int PRE_CHUNKS = 8, FUSE_CHUNKS = 64;
+    // From FUSE_CHUNKS chunks on.  Prep in a launch of its own / inside, one layer: 2048 tokens, 64 heads of 64 (20 SMs left over) 197 / 202 us, 32 heads 105 / 109, 120 heads of 32 201 / 207; 4000 to
+    // 8000 tokens level to 1 % apart, the second better once clocks are at the power limit (64 heads, 6000 tokens: 640 / 632); 16384 1388 / 1369, 32768 2789 / 2753.  Two and more sequences: the
+    // SMs left over do not keep up with 2 B chains of chunks (2 x 8192, 32 heads 467 / 507 us, 4 x 8192, 16 heads 416 / 572).
+    constexpr int PRE_CHUNKS = 8, FUSE_CHUNKS = 32;
     const bool pair = a.P == P / 2 && a.H % 2 == 0;        // two half-width heads per scan CTA
     const int nscan = (pair ? a.H / 2 : a.H) * ndir * a.B;
     PrepJob pj{Bp, Cp, dA, nullptr, 0, ndir, 0};
@@ -1335,7 +1335,7 @@ cudaError_t scan_ssd(const ScanArgs &a, void *ws, cudaStream_t s) {
         const size_t smem = a.P == P ? BlockSmem<P>::total : BlockSmem<P / 2>::total;
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        chain_spread((int64_t)pgrid.x * pgrid.y * pgrid.z, sm_count());
+        chain_spread((int64_t)pgrid.x * pgrid.y * pgrid.z, (int64_t)a.H * ndir * a.B, sm_count());
         return launch_chain(kern, dim3(a.H, ndir, a.B), 4 * a.P, smem, s, 0, k, Bp, Cp, Sb, dir0);
     }
 

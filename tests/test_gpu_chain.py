@@ -91,7 +91,7 @@ def _stack(G, kind, shape, layers=3, V=304):
 
 
 CASES = {
-    "mixer_long": lambda G: _mixer(G, I.BF16, I.MixerShape(1, 8100, 128, 2, 128, 4, 4)),               # prep partly inside the scan launch
+    "mixer_long": lambda G: _mixer(G, I.BF16, I.MixerShape(1, 4100, 128, 2, 128, 4, 4)),               # prep partly inside the scan launch
     "mixer_1k_pairs": lambda G: _mixer(G, I.BF16, I.MixerShape(2, 700, 512, 2, 128, 4, 32)),
     "mixer_chunk32": lambda G: _mixer(G, I.BF16, I.MixerShape(1, 2100, 128, 2, 16, 4, 4), chunk=32),
     "mixer_tied": lambda G: _mixer(G, I.BF16, I.MixerShape(2, 200, 256, 2, 64, 4, 8), flags=15),

@@ -204,9 +204,9 @@ def test_blocks_of_up_to_32_tokens(G, B, H, P, N, L, k):
     _check(G, G.run_forward(shape, I.BF16, wf, wr, x), O.bimamba_forward(x, wf, wr, **kw))
 
 
-@pytest.mark.parametrize("H,P,N,L,k", [(2, 64, 128, 8064, 4), (2, 64, 64, 8065, 3), (4, 32, 16, 8197, 4)])
+@pytest.mark.parametrize("H,P,N,L,k", [(2, 64, 128, 3968, 4), (2, 64, 64, 3969, 3), (4, 32, 16, 4101, 4)])
 def test_prep_inside_the_scan_launch(G, H, P, N, L, k):
-    """One sequence at the line (63 chunks: a prep launch of its own; 64 and 65: the chunks from the ninth on are prepared inside the scan launch), a last chunk of one token and of five, carried state in
+    """One sequence at the line (31 chunks: a prep launch of its own; 32 and 33: the chunks from the ninth on are prepared inside the scan launch), a last chunk of one token and of five, carried state in
     and out, padded d_state, two 32-wide heads to a CTA."""
     shape = I.MixerShape(1, L, P * H // 2, 2, N, k, H)
     wf, wr = I.make_mixer_weights(shape, 70, I.BF16, perturb=True)
