@@ -199,9 +199,11 @@ scan_seq_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
         // Everything chunk ci needs from memory: a tile of x with the three rows before it in time, one of z (rows outside the sequence become zeros) and
         // the run of [B' | C'], in physical order.  (16-byte copies by the threads took 1000 clocks a chunk to issue, and held up the
         // shared-memory reads behind them.)
-        bool ok = true;                                    // no wait of this thread has given up: afterwards no copies are started
+        bool ok = true;
+        int limit = nchunks;                               // copies are started for the chunks below it
         auto fetch = [&](int ci) {
-            if (ci >= nchunks || lt != 0 || !ok || ci == hold) return;      // (hold: left out, for the self-test)
+            if (ci >= limit || lt != 0) return;
+            if (ci == hold) return;                        // (left out, for the self-test)
             uint8_t *st = raw_of(ci);
             uint64_t *bar = &bars[ci % RAW];
             const int tau0 = ci * TC, tc = min(TC, L - tau0), bt = a.zx_tied ? b : dir * a.B + b, t0 = rev ? L - TC - tau0 : tau0;
@@ -263,17 +265,17 @@ scan_seq_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
         carry(0);
         prepare(0, dt_cur);
         __syncthreads();
-        int gave_up = ok ? nchunks : 0;                    // chunk whose wait did: it and the one after it may still be on their way
+        if (!ok) limit = 0;                                // a wait of this thread has given up: no more copies
         for (int ci = 0; ci < nchunks; ++ci) {
             fetch(ci + 2);                                 // its stage held chunk ci - 2, finished before the last barrier
             dt_cur = dt_next;
             dt_next = dt_of(ci + 2);
-            if (ci + 1 < nchunks) { landed(ci + 1); if (!ok) gave_up = min(gave_up, ci + 1); carry(ci + 1); prepare(ci + 1, dt_cur); }
+            if (ci + 1 < nchunks) { landed(ci + 1); if (!ok) limit = min(limit, ci + 1); carry(ci + 1); prepare(ci + 1, dt_cur); }
             __syncthreads();
         }
         // after a wait that gave up: no copy of this CTA may still be in flight when it leaves
         if (lt == 0 && !ok)
-            for (int c = gave_up; c < min(nchunks, gave_up + 2); ++c) mbar_wait_quiet(&bars[c % RAW], (c / RAW) & 1, 100000000ull);
+            for (int c = limit; c < min(nchunks, limit + 2); ++c) mbar_wait_quiet(&bars[c % RAW], (c / RAW) & 1, 100000000ull);
     } else {
         // ------------------------------------------------------------------ scan group
         const int p = tid / LPC, j = tid - p * LPC;
