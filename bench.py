@@ -833,7 +833,7 @@ def main():
                   "traffic": ncu_traffic("scan", shape, dtype, T), "peak_source": peaks["source"] + " (copy bandwidth)"}
 
     def gemm_entry(name, tf, ms):
-        return {"kernel": name + " GEMM (one launch per direction)", "bound": "tensor", "achieved": tf, "peak": tpk, "unit": "TFLOP/s",
+        return {"kernel": name + (" GEMM (both directions, one launch or two)" if name == "in_proj" else " GEMM (both directions summed in one launch)"), "bound": "tensor", "achieved": tf, "peak": tpk, "unit": "TFLOP/s",
                 "frac": tf / tpk, "frac_of_sustained": tf / peaks["bf16_tflops_sustained"], "ms": ms,
                 "traffic": ncu_traffic(name, shape, dtype, T), "peak_source": tsrc}
     dominant = max(("in_proj", inp_ms), ("scan", scan_ms), ("out_proj", outp_ms), key=lambda kv: kv[1])[0]

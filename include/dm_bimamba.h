@@ -373,8 +373,8 @@ int dm_selftest_withhold_prep(int on);
 uint64_t dm_kernel_launch_count(void);
 
 /* Measurement aid (no counterpart in the paper).  While enabled, every mixer call records CUDA event
- * pairs on its stream around its three stages: in_proj (one span per direction), the fused
- * conv+scan+gate launch, out_proj (one span per direction).  dm_profile_read waits for the recorded
+ * pairs on its stream around its three stages: in_proj, the fused conv+scan+gate launches, out_proj (one span each;
+ * where the directions are not summed in one launch, one per direction).  dm_profile_read waits for the recorded
  * events, writes the summed device time in milliseconds and the number of spans per stage into the HOST
  * arrays ms[DM_STAGE_COUNT], spans[DM_STAGE_COUNT], and forgets them.  Not for use during stream capture. */
 enum { DM_STAGE_IN_PROJ = 0, DM_STAGE_SCAN = 1, DM_STAGE_OUT_PROJ = 2, DM_STAGE_COUNT = 3 };
