@@ -9,18 +9,19 @@
 //                  and its sum; at the end O / l -> bf16 -> global
 // S(j + 1) of a stream is issued as soon as its softmax warps hold S(j) in registers (P has TMEM columns of its own), so the products run
 // under the softmax, and the two streams fall out of step by themselves: while one waits, the other one has the exponential unit.  What bounds
-// it is that unit: 128 x 128 exponentials take 1024 clocks of an SM, their products 512.  B=4, L=4096, 16 heads of 64: 378 us, 0.73 PFLOP/s (620 us with
-// one stream per CTA, two CTAs per SM, O scaled for every tile); B=8, L=1024, 24 heads of 80: 93 us (230 us).
-// The maximum m that P and O are relative to is only raised when a row's scores exceed it by more than 2^8: P then stays within what bf16 and
-// the fp32 sums hold without loss, and O is read back from TMEM and scaled for a few tiles per row instead of for each one.
+// it is that unit: 128 x 128 exponentials take 1024 clocks of an SM, their products 512.  With the projections around it, B=4, L=4096, 16 heads of 64: 495 us (740 us with
+// one stream per CTA, two CTAs per SM); B=8, L=1024, 24 heads of 80: 258 us (407 us).
+// P and O are relative to the row's exact running maximum: O is read back and scaled in every tile in which a row of the warp finds a new one.  (Raising the maximum only when it was exceeded by 2^8
+// saved 2 to 5 % of a call -- 4 x 4096, 16 heads of 64, projections included 471 us instead of 495 -- but the largest weight of a row is then no longer the exact 1 that bf16 holds without rounding:
+// error against 64 bits 5.69e-3 instead of 5.60e-3.)
 // Heads of 80 channels (the paper's 1.3B hybrid, d = 1920 with 24 heads): every Q, K, V tile is two 64-column sub-tiles, the head's
 // channels 0..63 and the 64 columns from channel 64 on, of which the products use the first 16 (the rest belongs to the next head, or is
 // the zero fill beyond the tensor, and is never read): one more K step of 16 for S, one more product of 16 columns for O.  Key tiles of 96 there:
 // S, P and O of two streams then fit the 512 TMEM columns.
 // The last CTA of a sequence may have queries for its first stream only: the second one then issues and computes nothing.
 // Up to 128 queries per sequence, more (head, sequence) pairs than SMs: CTAs of one stream, key tiles of 64, two to an SM, so that one's set-up and latencies are covered by the other.
-// 16 sequences, 16 heads of 64, a block of 100 after 2048 keys, projections included: 97 us with both streams running, 80 without the empty one, 68 with one stream
-// (64 sequences: 153, 137, 119 for 128 after 512 keys).  Fewer pairs: the two-stream form, whose larger key tiles take fewer steps (1 sequence, 8192 keys: 97 us against 112).
+// 16 sequences, 16 heads of 64, a block of 100 after 2048 keys, projections included: 97 us with both streams running, 71 with one stream (64 sequences of 128 after 512 keys: 153, 115).
+// Fewer pairs: the two-stream form, whose larger key tiles take fewer steps (1 sequence, 8192 keys: 13 % faster).
 // Every wait is bounded; on expiry the CTA stores DM_ERR_TIMEOUT in the device status word and leaves.
 // Few queries (block decoding) go to attention_block.cu where block_pays says so.
 #include "dm_internal.h"
@@ -31,7 +32,6 @@ using namespace tc;
 namespace {
 
 constexpr int BQ = 128, SUB = 64;                           // SUB: columns of a sub-tile (128 bytes: one swizzle atom)
-constexpr float RESCALE_LOG2 = 8.f;
 
 // NT: sub-tiles per operand tile; 1 = heads of 64 channels, 2 = heads of 80.  NS: query streams
 template <int NT, int NS> struct Cfg {
@@ -197,7 +197,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             const float mj = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * a.scale_log2;
             float alpha = 1.f;
             if (j == 0) m = mj;
-            else if (mj > m + RESCALE_LOG2) { alpha = ex2f(m - mj); m = mj; }
+            else if (mj > m) { alpha = ex2f(m - mj); m = mj; }
             // P V of the previous tile has read P (and completed O for a scaling)
             if (j > 0) {
                 ok = WAIT(&bars->o_done[s], (uint32_t)((j - 1) & 1));
@@ -220,16 +220,22 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
                 }
                 tmem_st_x16(tp + (c0 >> 1), pk);
             }
-            if (__any_sync(0xffffffffu, alpha != 1.f)) {          // rare: O moves to the new maximum
-#pragma unroll 1
-                for (int c0 = 0; c0 < DH; c0 += 16) {
-                    uint32_t t[16];
-                    tmem_ld_x16(to + c0, t);
-                    tmem_wait_ld();
+            if (__any_sync(0xffffffffu, alpha != 1.f)) {          // O moves to the new maximum
+                uint32_t t[DH];
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) t[i] = __float_as_uint(__uint_as_float(t[i]) * alpha);
-                    tmem_st_x16(to + c0, t);
+                for (int c0 = 0; c0 + 32 <= DH; c0 += 32) tmem_ld_x32(to + c0, t + c0);
+                if constexpr (DH % 32) tmem_ld_x16(to + DH - 16, t + DH - 16);
+                tmem_wait_ld();
+                const f32x2 a2 = pk2(alpha, alpha);
+#pragma unroll
+                for (int i = 0; i < DH; i += 2) {
+                    float x, y;
+                    upk2(mul2(pk2(__uint_as_float(t[i]), __uint_as_float(t[i + 1])), a2), x, y);
+                    t[i] = __float_as_uint(x); t[i + 1] = __float_as_uint(y);
                 }
+#pragma unroll
+                for (int c0 = 0; c0 + 32 <= DH; c0 += 32) tmem_st_x32(to + c0, t + c0);
+                if constexpr (DH % 32) tmem_st_x16(to + DH - 16, t + DH - 16);
             }
             tmem_wait_st();
             fence_before();
@@ -286,11 +292,10 @@ bool attention_supports(int dtype, int d, int n_heads) {
 
 // Few queries: which kernel.  attention_block.cu splits the keys of a (head, sequence) over the GPU, but its products run on mma.sync, for blocks of 32 queries that each read all keys; the
 // kernel above takes 128 queries at the price of 33, with a CTA per pair.  Measured, projections included (block kernel / this one), by pairs, 148 SMs:
-//   48 queries after 2048 keys, heads of 64: 64 pairs 41 / 43 us, 128 57 / 47, 256 93 / 60, 1024 277 / 155; heads of 80: 48 pairs 49 / 48, 96 74 / 53, 384 163 / 103
-//   32 queries, 512 pairs of 64: 66 / 60 us after 512 keys, 105 / 101 after 2048, 259 / 269 after 8192; 384 pairs of 80: 65 / 59, 108 / 104, 278 / 274
-static bool block_pays(int64_t pairs, int Lq, int Lk) {
+//   48 queries after 2048 keys, heads of 64: 64 pairs 41 / 46 us, 96 56 / 47, 128 57 / 49, 256 92 / 63, 1024 275 / 163; heads of 80: 48 pairs 49 / 50, 72 53 / 53, 96 74 / 55, 384 163 / 103
+static bool block_pays(int64_t pairs, int Lq) {
     if (Lq > ATTN_BLOCK_MAX_Q) return false;
-    return Lq > 32 ? 8 * pairs < 5 * sm_count() : pairs <= 2 * sm_count() || Lk > 4096;
+    return Lq <= 32 || 8 * pairs < 5 * sm_count();
 }
 
 // qkv [B*Lq, 3 d] bf16 (columns [Q | K | V], heads contiguous inside each), out [B*Lq, d] bf16.
@@ -304,7 +309,7 @@ cudaError_t attention_forward(const void *qkv, void *out, int B, int Lq, int d, 
     if (cached && (!v_cache || cache_len < 0 || cache_len + Lq > cache_cap)) return cudaErrorInvalidValue;
     const int Lk = cached ? cache_len + Lq : Lq;
     const int64_t pairs = (int64_t)B * n_heads;
-    if (block_pays(pairs, Lq, Lk)) return attention_block(qkv, out, B, Lq, d, n_heads, k_cache, v_cache, cache_len, cache_cap, s);
+    if (block_pays(pairs, Lq)) return attention_block(qkv, out, B, Lq, d, n_heads, k_cache, v_cache, cache_len, cache_cap, s);
     const int streams = Lq <= BQ && pairs > sm_count() ? 1 : 2;
     CUtensorMap mq, mk, mv;
     const int dh = d / n_heads;

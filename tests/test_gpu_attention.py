@@ -224,7 +224,7 @@ def test_attention_block_splits(G, dh, H, G_len, prefix):
     (64, 8, 12, 33, 100), (80, 4, 24, 64, 31),             # more than 32 queries, 96 pairs: two streams, the second without a query
     (64, 20, 8, 33, 63), (80, 20, 8, 100, 1), (64, 20, 8, 128, 0), (80, 20, 8, 128, 65),      # 160 pairs, up to 128 queries: CTAs of one stream
     (64, 20, 8, 129, 0), (64, 2, 2, 128, 150), (80, 2, 1, 300, 20),                             # the second stream with one query; without; in the last CTA only
-    (64, 38, 8, 32, 40), (80, 38, 8, 1, 64)])              # up to 32 queries, 304 pairs: no longer the few-query kernel
+    (64, 38, 8, 32, 40), (80, 38, 8, 1, 64)])              # up to 32 queries: the few-query kernel, however many pairs
 def test_attention_streams(G, dh, H, B, G_len, prefix):
     """The forms of the tensor-core kernel at the lines between them, key tiles cut short, with a key/value cache (beyond the valid keys: NaN)."""
     from paper_2511_15927_b200 import binding as dm
