@@ -1,5 +1,5 @@
 """GPU parity of the dense projection (dm_linear) against the oracle's in_proj / out_proj rows: sizes that
-span several 128 x 256 tiles with ragged tails in every dimension, the row-scale and addend epilogue, and
+span several tiles of every kernel with ragged tails in every dimension, the row-scale and addend epilogue, and
 in-place accumulation into an fp32 output."""
 import numpy as np
 import pytest
