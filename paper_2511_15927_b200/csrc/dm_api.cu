@@ -195,7 +195,7 @@ static int run_mixer(const dm_mixer_cfg *c, const Dims &m, const dm_dir_weights 
     sa.B = m.B; sa.L = m.L; sa.d_inner = m.d_inner; sa.H = m.H; sa.P = m.P; sa.N = m.N; sa.k = m.k;
     sa.d_in_proj = m.ldz; sa.conv_ch = m.conv_ch;          // the kernels use it as the row pitch only
     sa.dtype = c->dtype; sa.flags = c->flags; sa.dir_mask = c->dir_mask; sa.chunk = c->chunk;
-    sa.zx = zx; sa.g = g; sa.ssq = norm_on ? ssq : nullptr;
+    sa.zx = zx; sa.g = g;
     for (int dir = 0; dir < 2; ++dir) {
         sa.dir[dir].conv_w = w[dir].conv_w; sa.dir[dir].conv_b = w[dir].conv_b; sa.dir[dir].norm_w = w[dir].norm_w;
         sa.dir[dir].dt_bias = w[dir].dt_bias; sa.dir[dir].A_log = w[dir].A_log; sa.dir[dir].D = w[dir].D;
@@ -208,6 +208,12 @@ static int run_mixer(const dm_mixer_cfg *c, const Dims &m, const dm_dir_weights 
     sa.z_gated = 1;
     const bool ssd = scan_ssd_supports(sa);
     sa.z_gated = ssd ? 1 : 0;
+    // The scan of a narrow state can leave its sums of squares per 32 channels, more of them than the ssq region holds when heads are wider.  They then lie in ytmp's place, which is written, if at
+    // all, after they have become rstd.
+    sa.ssq_room = m.d_inner / 32 * 2 <= m.d ? m.d_inner / 32 : m.H;
+    const int parts = ssd ? scan_ssq_parts(sa) : m.H;
+    if (parts > m.H) ssq = ytmp;
+    sa.ssq = norm_on ? ssq : nullptr;
 
     {
         GemmArgs ga[2];
@@ -253,7 +259,7 @@ static int run_mixer(const dm_mixer_cfg *c, const Dims &m, const dm_dir_weights 
             a.A = g + (size_t)dir * m.T * m.d_inner * m.es; a.lda = m.d_inner;
             a.B = w[dir].w_out; a.ldb = m.d_inner;
             a.in_dtype = c->dtype; a.M = (int)m.T; a.N = m.d; a.K = m.d_inner;
-            if (norm_on) { a.rs_ssq = ssq + (size_t)dir * m.T * m.H; a.rs_n = m.H; a.rs_inv = 1.f / (float)m.d_inner; a.rs_eps = c->norm_eps; }
+            if (norm_on) { a.rs_ssq = ssq + (size_t)dir * m.T * parts; a.rs_n = parts; a.rs_inv = 1.f / (float)m.d_inner; a.rs_eps = c->norm_eps; }
             a.col_scale = out.col_scale; a.cs_rows = out.cs_rows; a.ld_cs = out.ld_cs;        // the gate distributes over the sum of the directions
             a.addend = out.addend; a.ld_add = out.ld_add;
             a.C = out.y; a.ldc = m.d; a.c_dtype = out.y_dtype;
@@ -272,7 +278,7 @@ static int run_mixer(const dm_mixer_cfg *c, const Dims &m, const dm_dir_weights 
         }
     }
     if (norm_on) {
-        e = rstd_from_ssq(ssq, rstd, (int)(2 * m.T), m.H, m.d_inner, c->norm_eps, s);
+        e = rstd_from_ssq(ssq, rstd, (int)(2 * m.T), parts, m.d_inner, c->norm_eps, s);
         if (e != cudaSuccess) return cuda_fail(e, "rstd");
     }
     if (tied && c->dir_mask == DM_DIR_BOTH) {

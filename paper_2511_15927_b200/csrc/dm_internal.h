@@ -140,7 +140,8 @@ struct ScanArgs {
     int zx_tied;             // both directions read zx[0] (shared in_proj, DM_FLAG_TIED_PROJ)
     int z_gated;             // the z columns of zx already hold SiLU(z) (applied by the in_proj epilogue); the tensor-core scan requires it
     void *g;                 // [2][B*L][d_inner]   dtype: gated output (times norm_w when the norm is on)
-    float *ssq;              // [2][B*L][H] per-head sum of squares of the gated output (norm on), or NULL
+    float *ssq;              // [2][B*L][H] per-head sum of squares of the gated output (norm on), or [2][B*L][scan_ssq_parts] of smaller pieces, or NULL
+    int ssq_room;            // pieces per row that fit at ssq
     ScanDir dir[2];
     const float *ssm_in;     // [B,H,P,N] or NULL   (left-to-right direction only)
     const void *conv_in;     // [B,k-1,conv_ch] or NULL
@@ -153,6 +154,8 @@ bool scan_ssd_supports(const ScanArgs &a);
 bool scan_ssd_chunk_ok(int dtype, int d_state, int chunk);
 void scan_ssd_selftest_withhold(int on);
 bool scan_selftest_withheld();
+// Sums of squares per row that scan_ssd writes: one per head, or (with that room) one per 32 channels
+int scan_ssq_parts(const ScanArgs &a);
 size_t scan_ssd_workspace_bytes(const ScanArgs &a);
 cudaError_t scan_ssd(const ScanArgs &a, void *ws, cudaStream_t s);
 

@@ -1,0 +1,529 @@
+// Fused conv + scan + gate for sequences of d_state 16: the identities of scan_ssd.cu over sub-chunks of 32 tokens, with every product on mma.sync tiles and every intermediate in registers.
+// At d_state 16 the tcgen05 kernel's chunk of 128 tokens does eight times the state work the model has and a mask of 128 x 128 per 64 channels; at 32 tokens the mask is a fourth of that per
+// channel, the state of a head of 64 is 32 registers per lane, and one warp can carry a tile of 32 tokens x 64 (or 32) channels from its raw rows to its gated output, meeting other warps only
+// where it takes the state over.
+// A CTA is one chain (batch row, direction, head or half a head): tile warps, of which warp w of n takes the tiles w, w + n, ... in the direction's time order, and a state warp.  A tile:
+//     loads    x rows with their conv history, [B' | C'] rows and decays by TMA into the warp's own buffers, the next tile's as soon as this one's have been read; z a step later
+//     conv     lane = 4 channels x 8 or 16 rows, results as bf16 over the raw rows, rows in time order
+//     St       the tile's own contribution to the state, x'^T (w o B'), left in shared memory for the state warp
+//     S, W     C' B'^T; its accumulators, masked and weighted, are the B operand of the next product as they stand
+//     chain    waits for the state before the tile: the state warp keeps the state in registers and, tile by tile, leaves its bf16 copy and takes h <- 2^Lambda_last h + St
+//     y, gate  y^T = 2^Lambda_i (h_in C'^T) + x'^T W^T, 16 channels at a time; z enters in the accumulators' layout (ldmatrix.trans), g = y SiLU(z), sums of squares, * norm_w; out through
+//              stmatrix.trans and a TMA store
+// Time order is a matter of row addresses (<- reads its rows backwards), so that the mask is the same for both directions.
+// The launch before (narrow_prep) leaves B' | C' as bf16 rows of 32 columns and the decays relative to each sub-chunk.
+// Bound by the shared-memory pipe (60 % of its wavefronts on average, 70 % on an SM with two chains) and by latencies at 20 warps an SM: 1500 instructions per warp and tile of 64 channels, an issue
+// slot used half of the time.  Scan alone, 32 heads of 64: 4 x 4096 tokens 190 us on the tcgen05 kernel, 113 here (2.9 TB/s of the rows' traffic where a copy reaches 6.5); 1 x 32768 650 -> 300, 8 x 512
+// 70 -> 38 behind the prep launch; a layer of 4 x 4096 475 -> 402 us.  With the state handed from tile warp to tile warp a step of the chain took 800 to 1800 clocks and 1 x 32768 436 us; through mbarriers 515.
+#include "ssd_common.cuh"
+
+namespace dm {
+namespace {
+
+using namespace ssd;
+
+constexpr int NS = 16;                       // d_state
+constexpr int XR = QB + 3;                   // raw rows of a tile with the conv's history
+constexpr int PER_SM = 4;                    // CTAs per SM at most
+
+// Tiles of MT x 16 channels: rows of 64 or 128 bytes with the swizzle of that width (tiles aligned to eight rows)
+template <int MT> struct Tile {
+    static constexpr int CW = 16 * MT, RB = 2 * CW;
+    static constexpr int WARPS = 20;                             // (16 of 128 registers: level; 24 of 80 for half heads: 8 % slower on one long sequence) resident on an SM, by registers: in CTAs of WARPS / 1 .. 4, one of them the state warp
+    static constexpr int QR = CW / 4, RG = 32 / QR, RPG = QB / RG;      // conv: lanes to a row (4 channels each), groups of rows, rows of a group
+    // a warp's buffers
+    static constexpr uint32_t X = 0, LAM = XR * RB, E = LAM + 256, Z = (E + 256 + 8 * RB - 1) / (8 * RB) * (8 * RB), BC = Z + QB * RB, SLOT = BC + QB * 64;
+    static constexpr uint32_t TX_X = XR * RB + QB * 64 + 256, TX_Z = QB * RB;
+    static constexpr uint32_t ST = X;                            // over x' once that is in registers: St, then the state's copy, 512 bytes (a 16-byte piece of each lane) at a time
+    static_assert(LAM % 16 == 0 && BC % 512 == 0 && SLOT % (8 * RB) == 0, "slot layout");
+    // 16-byte piece p of row r lies at piece p ^ swz(r)
+    static __host__ __device__ constexpr uint32_t swz(uint32_t r) { return RB == 64 ? (r >> 1) & 3 : r & 7; }
+};
+template <int MT> struct Shared {
+    float conv[5][16 * MT];                  // taps by steps back in time, then the bias; all halved (SiLU(v) = v/2 + v/2 tanh(v/2))
+    float norm_w[16 * MT];
+    uint64_t x[Tile<MT>::WARPS], z[Tile<MT>::WARPS];
+    int ready[Tile<MT>::WARPS];              // by tile warp: 1 + the last tile whose St it left
+    int done;                                // tiles whose incoming state is there
+    int abort;
+};
+template <int MT> constexpr size_t smem_bytes(int nw) { return 1024 + (size_t)(nw - 1) * Tile<MT>::SLOT + sizeof(Shared<MT>); }
+
+__device__ __forceinline__ void prefetch_tile(const CUtensorMap *map, int x, int y, int z) {
+    asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];" ::"l"(map), "r"(x), "r"(y), "r"(z) : "memory");
+}
+__device__ __forceinline__ float2 lds2(uint32_t addr) {
+    float2 v;
+    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(addr));
+    return v;
+}
+__device__ __forceinline__ float lds1(uint32_t addr) {
+    float v;
+    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr));
+    return v;
+}
+__device__ __forceinline__ float4 lds4(uint32_t addr) {
+    float4 v;
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr));
+    return v;
+}
+__device__ __forceinline__ void sts1(uint32_t addr, float v) { asm volatile("st.shared.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory"); }
+
+// Non-volatile, so that the compiler may mix products with what surrounds them
+__device__ __forceinline__ void mma(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ void raise_flag(uint32_t addr, int v) { asm volatile("st.release.cta.shared::cta.s32 [%0], %1;" ::"r"(addr), "r"(v) : "memory"); }
+// Bounded wait until a counter in shared memory has reached `target` (same abort protocol as mbar_wait).  A plain load is answered in a third of the time an mbarrier's probe takes, and these waits
+// are the chain's serial part.
+__device__ __forceinline__ bool flag_reached(uint32_t addr, int target, volatile int *abort_flag, int *status) {
+    auto seen = [&] {
+        int v;
+        asm volatile("ld.acquire.cta.shared::cta.s32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+        return v >= target;
+    };
+    if (seen()) return true;
+    const uint64_t t0 = globaltimer_ns();
+    for (;;) {
+#pragma unroll 1
+        for (int i = 0; i < 256; ++i)
+            if (seen()) return true;
+        if (*abort_flag) return false;
+        if (globaltimer_ns() - t0 > WAIT_LIMIT_NS) {
+            *abort_flag = 1;
+            atomicExch(status, (int)DM_ERR_TIMEOUT);
+            return false;
+        }
+    }
+}
+
+// The state warp: 16 x 16 tiles [channels][states] in the accumulators' layout
+template <int MT>
+__device__ __forceinline__ void state_role(const SsdArgs &a, const uint8_t *slots, Shared<MT> *sh, int nt, int nsub, const float *h_in, float *h_out, int *status) {
+    using T = Tile<MT>;
+    const int lane = threadIdx.x & 31, gr = lane >> 2, qc = lane & 3;
+    volatile int *abort_flag = &sh->abort;
+    const uint32_t sb = smem_u32(slots), ready = smem_u32(sh->ready), done = smem_u32(&sh->done);
+    float h[MT][2][4];
+#pragma unroll
+    for (int m = 0; m < MT; ++m)
+#pragma unroll
+        for (int n = 0; n < 2; ++n)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) h[m][n][e] = h_in ? h_in[(16 * m + gr + (e >> 1) * 8) * NS + 8 * n + 2 * qc + (e & 1)] : 0.f;
+    int w = 0;
+    for (int k = 0; k < nsub; ++k) {
+        const uint32_t slot = sb + w * T::SLOT;
+        if (!__all_sync(0xffffffffu, flag_reached(ready + 4 * w, k + 1, abort_flag, status))) return;
+        float4 st[MT][2];
+#pragma unroll
+        for (int m = 0; m < MT; ++m)
+#pragma unroll
+            for (int n = 0; n < 2; ++n) st[m][n] = lds4(slot + T::ST + lane * 16 + (2 * m + n) * 512);
+        const float dec = lds1(slot + T::E + (QB - 1) * 4);
+#pragma unroll
+        for (int m = 0; m < MT; ++m)
+            asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(slot + T::ST + lane * 16 + m * 512), "r"(pack_bf16(h[m][0][0], h[m][0][1])), "r"(pack_bf16(h[m][0][2], h[m][0][3])),
+                         "r"(pack_bf16(h[m][1][0], h[m][1][1])), "r"(pack_bf16(h[m][1][2], h[m][1][3])) : "memory");
+        __syncwarp();
+        if (lane == 0) raise_flag(done, k + 1);
+        const f32x2 dec2 = pk2(dec, dec);
+#pragma unroll
+        for (int m = 0; m < MT; ++m)
+#pragma unroll
+            for (int n = 0; n < 2; ++n) {
+                upk2(fma2(dec2, pk2(h[m][n][0], h[m][n][1]), pk2(st[m][n].x, st[m][n].y)), h[m][n][0], h[m][n][1]);
+                upk2(fma2(dec2, pk2(h[m][n][2], h[m][n][3]), pk2(st[m][n].z, st[m][n].w)), h[m][n][2], h[m][n][3]);
+            }
+        if (++w == nt) w = 0;
+    }
+    if (h_out) {
+#pragma unroll
+        for (int m = 0; m < MT; ++m)
+#pragma unroll
+            for (int n = 0; n < 2; ++n)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) h_out[(16 * m + gr + (e >> 1) * 8) * NS + 8 * n + 2 * qc + (e & 1)] = h[m][n][e];
+    }
+}
+
+template <int MT, bool REV>
+__device__ __forceinline__ void chain(const CUtensorMap &map_x, const CUtensorMap &map_z, const CUtensorMap &map_bc, const CUtensorMap &map_g, const SsdArgs &a,
+                                      const float *__restrict__ dl, uint8_t *slots, Shared<MT> *sh, int grp, int b, int *status) {
+    using T = Tile<MT>;
+    constexpr int CW = T::CW, RB = T::RB;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, gr = lane >> 2, qc = lane & 3, nt = (blockDim.x >> 5) - 1;      // nt: tile warps
+    const int L = a.L, nsub = (L + QB - 1) / QB, seq = (REV ? a.B : 0) + b, zseq = a.zx_tied ? b : seq, ch0 = grp * CW, h = ch0 / a.Pr, G = a.d_inner / CW;
+    volatile int *abort_flag = &sh->abort;
+    uint8_t *const slot = slots + warp * T::SLOT;
+    const uint32_t sb = smem_u32(slot), conv_w = smem_u32(&sh->conv[0][0]), stp = sb + T::ST + lane * 16;
+    uint64_t *const bx = &sh->x[warp], *const bz = &sh->z[warp];
+    const float *dl_head = dl + ((int64_t)seq * a.H + h) * 2 * a.Lp;
+    const float Dh = (a.flags & DM_FLAG_D_SKIP) ? a.dir[REV ? 1 : 0].D[h] : 0.f;
+    if (warp == nt) {
+        const int64_t state0 = (((int64_t)b * a.H + h) * a.Pr + ch0 % a.Pr) * NS;
+        state_role<MT>(a, slots, sh, nt, nsub, !REV && a.ssm_in ? a.ssm_in + state0 : nullptr, !REV && a.ssm_out ? a.ssm_out + state0 : nullptr, status);
+        return;
+    }
+
+    auto WAIT = [&](uint64_t *bar, uint32_t parity) { return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, status)); };
+    auto first_row = [&](int k) { return (REV ? nsub - 1 - k : k) * QB; };         // of the k-th tile in time
+    auto load_x = [&](int k) {
+        const int r0 = first_row(k);
+        mbar_expect_tx(bx, T::TX_X);
+        tma_load_3d(slot + T::X, &map_x, a.d_inner + ch0, REV ? r0 : r0 - 3, zseq, bx);
+        tma_load_3d(slot + T::BC, &map_bc, 0, r0, seq, bx);
+        bulk_load(slot + T::LAM, dl_head + (int64_t)(r0 / QB) * 2 * QB, 2 * QB * 4, bx);
+    };
+    auto load_z = [&](int k) {
+        mbar_expect_tx(bz, T::TX_Z);
+        tma_load_3d(slot + T::Z, &map_z, ch0, first_row(k), zseq, bz);
+    };
+
+    const int cg = lane / T::QR, cq = lane % T::QR;                               // conv: rows RPG cg + .., channels 4 cq ..
+    auto conv_at = [&](uint32_t row) { return (uint32_t)(((cq >> 1) ^ T::swz(row)) << 4) + (cq & 1) * 8 + row * RB; };       // (row: without the group's, which leave the swizzle alone)
+    uint32_t xo, zo, bco, bno;
+    {
+        const int ri = (lane & 7) + ((lane >> 3) & 1) * 8, rj = (lane & 7) + (lane >> 4) * 8, ra = REV ? QB - 1 - ri : ri, rb = REV ? QB - 1 - rj : rj, lo = (lane >> 3) & 1;
+        xo = sb + T::X + rj * RB + ((lo ^ T::swz(rj)) << 4);                      // x'^T (rows in time order): pieces p lo | hi, then rows j lo | hi
+        zo = sb + T::Z + rb * RB + ((lo ^ T::swz(rb)) << 4);                      // z^T: pieces p lo | hi, then two i tiles
+        bco = sb + T::BC + ra * 64 + (((lane >> 4) ^ ((ra >> 1) & 3)) << 4);      // rows lo | hi, then pieces: B'^T of St; ^ 32: C'
+        bno = sb + T::BC + rb * 64 + ((lo ^ ((rb >> 1) & 3)) << 4);               // pieces lo | hi, then rows: B' of S
+    }
+    constexpr uint32_t BC16 = REV ? (uint32_t)(-16 * 64) : 16 * 64, Z16 = REV ? (uint32_t)(-16 * RB) : 16 * RB;      // 16 rows later in time
+
+    if (lane == 0 && warp < nsub) load_x(warp);
+    int it = 0;
+    for (int k = warp; k < nsub; k += nt, ++it) {
+        const int r0 = first_row(k);
+        if (!WAIT(bx, it & 1)) break;
+        // ---- conv: a group's rows in time order, history first
+        if (!REV && k == 0 && a.conv_in) {                                        // rows before the sequence: the carried conv state (the load left zeros)
+            for (int u = lane; u < 3 * CW / 2; u += 32) {
+                const int r = u / (CW / 2), c = u % (CW / 2), m = a.k - 1 + r - 3;
+                if (m >= 0)
+                    *reinterpret_cast<uint32_t *>(slot + T::X + r * RB + (((c >> 2) ^ T::swz(r)) << 4) + (c & 3) * 4) =
+                        *reinterpret_cast<const uint32_t *>(a.conv_in + ((int64_t)b * (a.k - 1) + m) * a.conv_ch + ch0 + 2 * c);
+            }
+            __syncwarp();
+        }
+        uint2 raw[T::RPG + 3];
+#pragma unroll
+        for (int u = 0; u < T::RPG + 3; ++u) {
+            const uint32_t ad = sb + T::X + conv_at(REV ? QB + 2 - u : u) + (REV ? -cg : cg) * (T::RPG * RB);
+            asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(raw[u].x), "=r"(raw[u].y) : "r"(ad));
+        }
+        const float lam_t = lds1(sb + T::LAM + lane * 4), lamp_t = lds1(sb + T::LAM + QB * 4 + lane * 4);
+        const float lam_last = lds1(sb + T::LAM + (QB - 1) * 4);
+        __syncwarp();                                                             // the rows are in registers: x' goes over them
+        if (lane == 0) {
+            bulk_wait_read0();                                                    // the last tile's output has left the z buffer
+            load_z(k);
+            if (k + nt < nsub) prefetch_tile(&map_x, a.d_inner + ch0, first_row(k + nt), zseq);
+        }
+        sts1(sb + T::E + lane * 4, ex2f(lam_t));
+        sts1(sb + T::E + QB * 4 + lane * 4, ex2f(lam_last - lamp_t));             // w_j
+        {
+            f32x2 wt[5][2];
+#pragma unroll
+            for (int m = 0; m < 5; ++m) {
+                const float4 v = lds4(conv_w + m * CW * 4 + cq * 16);
+                wt[m][0] = pk2(v.x, v.y); wt[m][1] = pk2(v.z, v.w);
+            }
+            f32x2 w0[2], w1[2], w2[2];                                            // the three rows before
+            w2[0] = bf2_to_f2(raw[0].x); w2[1] = bf2_to_f2(raw[0].y);
+            w1[0] = bf2_to_f2(raw[1].x); w1[1] = bf2_to_f2(raw[1].y);
+            w0[0] = bf2_to_f2(raw[2].x); w0[1] = bf2_to_f2(raw[2].y);
+#pragma unroll
+            for (int t = 0; t < T::RPG; ++t) {
+                const f32x2 cur[2] = {bf2_to_f2(raw[t + 3].x), bf2_to_f2(raw[t + 3].y)};
+                uint32_t o[2];
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    f32x2 hv = fma2(wt[3][e], w2[e], wt[4][e]);
+                    hv = fma2(wt[2][e], w1[e], hv); hv = fma2(wt[1][e], w0[e], hv); hv = fma2(wt[0][e], cur[e], hv);
+                    float ha, hb;
+                    upk2(hv, ha, hb);
+                    o[e] = f2_to_bf2(fma2(hv, pk2(tanh_fast(ha), tanh_fast(hb)), hv));
+                    w2[e] = w1[e]; w1[e] = w0[e]; w0[e] = cur[e];
+                }
+                asm volatile("st.shared.v2.u32 [%0], {%1, %2};" ::"r"(sb + T::X + conv_at(t) + cg * (T::RPG * RB)), "r"(o[0]), "r"(o[1]) : "memory");
+            }
+        }
+        __syncwarp();
+        // ---- St = x'^T (w o B')
+        uint32_t xa[MT][2][4];
+        {
+            float st[MT][2][4];
+            uint32_t wb[2][4];                                                    // [16 rows j][(j lo, n lo), (j hi, n lo), (j lo, n hi), (j hi, n hi)]
+#pragma unroll
+            for (int kt = 0; kt < 2; ++kt) {
+                ldmatrix_x4_t(wb[kt][0], wb[kt][1], wb[kt][2], wb[kt][3], bco + kt * BC16);
+                const float2 wl = lds2(sb + T::E + QB * 4 + (16 * kt + 2 * qc) * 4), wh = lds2(sb + T::E + QB * 4 + (16 * kt + 8 + 2 * qc) * 4);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) wb[kt][e] = f2_to_bf2(mul2(bf2_to_f2(wb[kt][e]), (e & 1) ? pk2(wh.x, wh.y) : pk2(wl.x, wl.y)));
+            }
+#pragma unroll
+            for (int m = 0; m < MT; ++m) {
+#pragma unroll
+                for (int kt = 0; kt < 2; ++kt) ldmatrix_x4_t(xa[m][kt][0], xa[m][kt][1], xa[m][kt][2], xa[m][kt][3], (xo ^ (32 * m)) + kt * 16 * RB);
+#pragma unroll
+                for (int n = 0; n < 2; ++n) {
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) st[m][n][e] = 0.f;
+#pragma unroll
+                    for (int kt = 0; kt < 2; ++kt) mma(st[m][n], xa[m][kt], wb[kt][2 * n], wb[kt][2 * n + 1]);
+                }
+            }
+            __syncwarp();                                                         // x' is in registers: St goes over it
+#pragma unroll
+            for (int m = 0; m < MT; ++m)
+#pragma unroll
+                for (int n = 0; n < 2; ++n)
+                    asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(stp + (2 * m + n) * 512), "f"(st[m][n][0]), "f"(st[m][n][1]), "f"(st[m][n][2]), "f"(st[m][n][3]) : "memory");
+            __syncwarp();
+            if (lane == 0) raise_flag(smem_u32(&sh->ready[warp]), k + 1);
+        }
+        // ---- S, W: C' tiles of 16 rows (the same registers are A operand here and B operand of Yb)
+        uint32_t cf[2][4], wf[4][4];                                              // W: (8 rows i, 8 columns j) as the B operand of y^T = x'^T W^T
+        f32x2 ei[4];
+        {
+            uint32_t bf[2][4];
+            ldmatrix_x4(cf[0][0], cf[0][1], cf[0][2], cf[0][3], bco ^ 32);
+            ldmatrix_x4(cf[1][0], cf[1][1], cf[1][2], cf[1][3], (bco ^ 32) + BC16);
+            ldmatrix_x4(bf[0][0], bf[0][1], bf[0][2], bf[0][3], bno);
+            ldmatrix_x4(bf[1][0], bf[1][1], bf[1][2], bf[1][3], bno + BC16);
+            float2 lp[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) lp[j] = lds2(sb + T::LAM + QB * 4 + (8 * j + 2 * qc) * 4);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) { const float2 v = lds2(sb + T::E + (8 * i + 2 * qc) * 4); ei[i] = pk2(v.x, v.y); }
+#pragma unroll
+            for (int mt = 0; mt < 2; ++mt) {
+                float s[4][4];
+#pragma unroll
+                for (int j = 0; j < 2 * mt + 2; ++j) {
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) s[j][e] = 0.f;
+                    mma(s[j], cf[mt], bf[j >> 1][(j & 1) * 2], bf[j >> 1][(j & 1) * 2 + 1]);
+                }
+#pragma unroll
+                for (int hf = 0; hf < 2; ++hf) {
+                    const int i = 2 * mt + hf;
+                    const float li = lds1(sb + T::LAM + (8 * i + gr) * 4);
+#pragma unroll
+                    for (int j = 0; j <= i; ++j) {
+                        float e0 = li - lp[j].x, e1 = li - lp[j].y;
+                        if (j == i) { e0 = 2 * qc <= gr ? e0 : -INFINITY; e1 = 2 * qc + 1 <= gr ? e1 : -INFINITY; }      // 2^-inf = 0 after i
+                        float v0 = s[j][2 * hf] * ex2f(e0), v1 = s[j][2 * hf + 1] * ex2f(e1);
+                        if (j == i) { v0 += 2 * qc == gr ? Dh : 0.f; v1 += 2 * qc + 1 == gr ? Dh : 0.f; }
+                        wf[i][j] = pack_bf16(v0, v1);
+                    }
+                }
+            }
+        }
+        // ---- the state before the tile: A operand of Yb
+        if (!__all_sync(0xffffffffu, flag_reached(smem_u32(&sh->done), k + 1, abort_flag, status))) break;
+        uint32_t hb[MT][4];
+#pragma unroll
+        for (int m = 0; m < MT; ++m)
+            asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(hb[m][0]), "=r"(hb[m][1]), "=r"(hb[m][2]), "=r"(hb[m][3]) : "r"(stp + m * 512));
+        fence_proxy_async();
+        __syncwarp();                                                             // all but z has been read: the next tile's may come
+        if (lane == 0 && k + nt < nsub) {
+            load_x(k + nt);
+            prefetch_tile(&map_z, ch0, first_row(k + nt), zseq);
+        }
+        // ---- y and the gate, 16 channels at a time
+        if (!WAIT(bz, it & 1)) break;
+        f32x2 sq[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) sq[i] = pk2(0.f, 0.f);
+#pragma unroll
+        for (int m = 0; m < MT; ++m) {
+            float y[4][4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) y[i][e] = 0.f;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) mma(y[i], hb[m], cf[i >> 1][i & 1], cf[i >> 1][2 + (i & 1)]);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                upk2(mul2(ei[i], pk2(y[i][0], y[i][1])), y[i][0], y[i][1]);
+                upk2(mul2(ei[i], pk2(y[i][2], y[i][3])), y[i][2], y[i][3]);
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i) mma(y[i], xa[m][0], wf[i][0], i > 0 ? wf[i][1] : 0u);
+#pragma unroll
+            for (int i = 2; i < 4; ++i) mma(y[i], xa[m][1], wf[i][2], i > 2 ? wf[i][3] : 0u);
+            const float nl = sh->norm_w[16 * m + gr], nh = sh->norm_w[16 * m + 8 + gr];
+            const f32x2 nl2 = pk2(nl, nl), nh2 = pk2(nh, nh);
+#pragma unroll
+            for (int ip = 0; ip < 2; ++ip) {
+                const uint32_t ad = (zo ^ (32 * m)) + ip * Z16;
+                uint32_t z[4];                                                    // (i tile 2 ip, p lo | hi), (i tile 2 ip + 1, p lo | hi)
+                ldmatrix_x4_t(z[0], z[1], z[2], z[3], ad);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const int i = 2 * ip + (e >> 1);
+                    const f32x2 g = mul2(pk2(y[i][(e & 1) * 2], y[i][(e & 1) * 2 + 1]), bf2_to_f2(z[e]));
+                    sq[i] = fma2(g, g, sq[i]);
+                    z[e] = f2_to_bf2(mul2(g, (e & 1) ? nh2 : nl2));
+                }
+                stmatrix_x4_t(ad, z[0], z[1], z[2], z[3]);
+            }
+        }
+        fence_proxy_async();
+        __syncwarp();
+        if (lane == 0) {
+            tma_store_3d(&map_g, slot + T::Z, ch0, r0, seq);
+            bulk_commit();
+        }
+        if (a.ssq) {
+            // eight sums per lane over the lanes of equal qc: halves exchanged, so that each lane ends with one token's sum
+            float v[4][2], u[2][2], t[2];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) upk2(sq[i], v[i][0], v[i][1]);
+            const bool b4 = lane & 16, b3 = lane & 8, b2 = lane & 4;
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+#pragma unroll
+                for (int e = 0; e < 2; ++e) u[i][e] = (b4 ? v[2 + i][e] : v[i][e]) + __shfl_xor_sync(0xffffffffu, b4 ? v[i][e] : v[2 + i][e], 16);
+#pragma unroll
+            for (int e = 0; e < 2; ++e) t[e] = (b3 ? u[1][e] : u[0][e]) + __shfl_xor_sync(0xffffffffu, b3 ? u[0][e] : u[1][e], 8);
+            const float s = (b2 ? t[1] : t[0]) + __shfl_xor_sync(0xffffffffu, b2 ? t[0] : t[1], 4);
+            const int i = (b4 ? 16 : 0) + (b3 ? 8 : 0) + 2 * qc + (b2 ? 1 : 0), row = r0 + (REV ? QB - 1 - i : i);
+            if (row < L) a.ssq[((int64_t)seq * L + row) * G + grp] = s;
+        }
+    }
+    if (*abort_flag && lane == 0 && warp < nsub) {                                // aborting: bounded wait for the loads still in flight
+        // whichever phase is open: a load that has landed completes it, and a phase without a load runs into the limit
+        mbar_wait_quiet(bx, it & 1, 100000000ull);
+        mbar_wait_quiet(bx, (it & 1) ^ 1, 100000000ull);
+        mbar_wait_quiet(bz, it & 1, 100000000ull);
+    }
+    if (lane == 0) bulk_wait0();
+}
+
+template <int MT>
+__global__ void __launch_bounds__(Tile<MT>::WARPS * 32, 1)
+narrow_scan_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_z, const __grid_constant__ CUtensorMap map_bc,
+                   const __grid_constant__ CUtensorMap map_g, const __grid_constant__ SsdArgs a, const float *__restrict__ dl, int ndir, int dir0, int *status) {
+    using T = Tile<MT>;
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t *slots = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+    const int tid = threadIdx.x, nt = (blockDim.x >> 5) - 1;
+    Shared<MT> *sh = reinterpret_cast<Shared<MT> *>(slots + nt * T::SLOT);
+    const int G = a.d_inner / T::CW, grp = blockIdx.x % G, dir = dir0 + (blockIdx.x / G) % ndir, b = blockIdx.x / (G * ndir);
+    const ScanDir &w = a.dir[dir];
+    if (tid == 0) {
+        for (int i = 0; i < nt; ++i) { mbar_init(&sh->x[i], 1); mbar_init(&sh->z[i], 1); sh->ready[i] = 0; }
+        sh->done = 0;
+        sh->abort = 0;
+        mbar_fence_init();
+    }
+    for (int i = tid; i < T::CW; i += blockDim.x) {
+        const int c = grp * T::CW + i;
+        const __nv_bfloat16 *cw = static_cast<const __nv_bfloat16 *>(w.conv_w) + (int64_t)c * a.k;
+        for (int m = 0; m < 4; ++m) sh->conv[m][i] = m < a.k ? 0.5f * __bfloat162float(cw[a.k - 1 - m]) : 0.f;
+        sh->conv[4][i] = (a.flags & DM_FLAG_CONV_BIAS) && w.conv_b ? 0.5f * __bfloat162float(static_cast<const __nv_bfloat16 *>(w.conv_b)[c]) : 0.f;
+        sh->norm_w[i] = (a.flags & DM_FLAG_GATED_RMSNORM) && w.norm_w ? __bfloat162float(static_cast<const __nv_bfloat16 *>(w.norm_w)[c]) : 1.f;
+    }
+    __syncthreads();
+    pdl_wait();
+    pdl_trigger();
+    if (dir == 1) chain<MT, true>(map_x, map_z, map_bc, map_g, a, dl, slots, sh, grp, b, status);
+    else chain<MT, false>(map_x, map_z, map_bc, map_g, a, dl, slots, sh, grp, b, status);
+}
+
+// B' and C' (conv + SiLU) as bf16 rows [B' 16 | C' 16], and the decays of every sub-chunk.  A CTA takes the 128 rows of a chunk (a thread: a channel pair over four rows) or the decays of 64 heads
+// over them.
+__global__ void __launch_bounds__(PREP_THREADS)
+narrow_prep_kernel(const __grid_constant__ SsdArgs a, __nv_bfloat16 *__restrict__ bc, float *__restrict__ dl, int dir0) {
+    __shared__ __align__(16) float sm[64 * Q];
+    pdl_wait();
+    pdl_trigger();
+    const int per = 1 + (a.H + 63) / 64, c = blockIdx.x / per, part = blockIdx.x - c * per, b = blockIdx.y;
+    const int dir = dir0 + blockIdx.z, r0 = (dir == 1 ? a.nch - 1 - c : c) * Q;
+    if (part > 0) { prep_decay<true>(a, dl, dir, b, r0, (part - 1) * 64, sm); return; }
+    constexpr int RUN = Q * NS / PREP_THREADS;                       // rows of a thread
+    const bool rev = dir == 1;
+    const int tid = threadIdx.x, pi = tid & (NS - 1), L = a.L, k = a.k;
+    const int cc = a.d_inner + 2 * pi;                               // conv channel of the pair's first member (B, then C)
+    const int64_t seq = (int64_t)dir * a.B + b;
+    const ScanDir &w = a.dir[dir];
+    const uint32_t *col = reinterpret_cast<const uint32_t *>(a.zx + ((int64_t)(a.zx_tied ? 0 : dir) * a.B + b) * L * a.d_in_proj + a.d_inner + cc);
+    const int64_t ld32 = a.d_in_proj / 2;
+    const int lo = r0 + tid / NS * RUN, first = rev ? lo + RUN - 1 : lo, step = rev ? -1 : 1;
+    const uint32_t *cin = (!rev && a.conv_in) ? reinterpret_cast<const uint32_t *>(a.conv_in + (int64_t)b * (k - 1) * a.conv_ch + cc) : nullptr;
+    uint32_t raw[RUN + 3];
+#pragma unroll
+    for (int i = 0; i < RUN + 3; ++i) {
+        const int t = first + (i - 3) * step;
+        raw[i] = (t >= 0 && t < L) ? __ldg(col + (int64_t)t * ld32) : 0u;
+        if (cin && t < 0 && k - 1 + t >= 0) raw[i] = __ldg(cin + (int64_t)(k - 1 + t) * (a.conv_ch / 2));
+    }
+    float wl[2][4], bias[2] = {0.f, 0.f};
+    const __nv_bfloat16 *cw = static_cast<const __nv_bfloat16 *>(w.conv_w) + (int64_t)cc * k;
+#pragma unroll
+    for (int e = 0; e < 2; ++e)
+#pragma unroll
+        for (int m = 0; m < 4; ++m) wl[e][m] = m < k ? __bfloat162float(cw[e * k + k - 1 - m]) : 0.f;
+    if ((a.flags & DM_FLAG_CONV_BIAS) && w.conv_b) {
+        bias[0] = __bfloat162float(static_cast<const __nv_bfloat16 *>(w.conv_b)[cc]);
+        bias[1] = __bfloat162float(static_cast<const __nv_bfloat16 *>(w.conv_b)[cc + 1]);
+    }
+    uint32_t *dst = reinterpret_cast<uint32_t *>(bc) + seq * L * NS + pi;
+#pragma unroll
+    for (int i = 0; i < RUN; ++i) {
+        const int t = first + i * step;
+        const uint32_t win[4] = {raw[i + 3], raw[i + 2], raw[i + 1], raw[i]};
+        const uint32_t pk = prep_conv_pair(wl, bias, win);
+        if (t < L) dst[(int64_t)t * NS] = pk;
+    }
+}
+
+template <int MT>
+cudaError_t launch(const SsdArgs &a, __nv_bfloat16 *bc, float *dl, int ndir, int dir0, cudaStream_t s) {
+    using T = Tile<MT>;
+    const int nsub = (a.L + QB - 1) / QB;
+    CUtensorMap mx, mz, mb, mg;
+    auto map = [&](CUtensorMap *m, const void *p, int64_t ld, int cols, int rows) {
+        const uint64_t dims[3] = {(uint64_t)ld, (uint64_t)a.L, (uint64_t)2 * a.B}, str[2] = {(uint64_t)ld, (uint64_t)a.L * ld};
+        const uint32_t box[3] = {(uint32_t)cols, (uint32_t)rows, 1};
+        return make_map_bf16(m, p, 3, dims, str, box, cols == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B);
+    };
+    if (!map(&mx, a.zx, a.d_in_proj, T::CW, XR) || !map(&mz, a.zx, a.d_in_proj, T::CW, QB) || !map(&mb, bc, 2 * NS, 2 * NS, QB) || !map(&mg, a.g, a.d_inner, T::CW, QB))
+        return cudaErrorInvalidValue;
+    int *status = device_status_ptr();
+    if (!status) return cudaErrorUnknown;
+    const dim3 pgrid(a.nch * (1 + (a.H + 63) / 64), a.B, ndir);
+    cudaError_t e = launch_chain(narrow_prep_kernel, pgrid, PREP_THREADS, 0, s, 0, a, bc, dl, dir0);
+    if (e != cudaSuccess) return e;
+    // as many warps to a chain as leave all chains resident, up to PER_SM of them to an SM.  Chains that share an SM are launched without overlap behind a prep grid that fills the GPU (chain_spread): 4 x 4096
+    // tokens of 32 heads 402 -> 399 us a layer; behind smaller grids the overlap is worth 3 us (8 x 512: 124 / 128).
+    const int64_t chains = (int64_t)(a.d_inner / T::CW) * ndir * a.B;
+    const int sms = sm_count();
+    const int per_sm = chains > (int64_t)PER_SM * sms ? PER_SM : (int)((chains + sms - 1) / sms);
+    int nw = T::WARPS / per_sm;
+    if (nw > nsub + 1) nw = nsub + 1;
+    e = cudaFuncSetAttribute(narrow_scan_kernel<MT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes<MT>(T::WARPS));
+    if (e != cudaSuccess) return e;
+    if (per_sm > 1) chain_spread((int64_t)pgrid.x * pgrid.y * pgrid.z, chains, sms);      // several CTAs to an SM, but not packed
+    return launch_chain(narrow_scan_kernel<MT>, (unsigned)chains, 32 * nw, smem_bytes<MT>(nw), s, 0, mx, mz, mb, mg, a, dl, ndir, dir0, status);
+}
+
+}  // namespace
+
+bool scan_narrow_shape(int headdim, int d_state) { return d_state == NS && headdim % 32 == 0; }
+// Few chains: heads of 64 are split, so that twice as many SMs have one.  Everywhere else the whole head is the better tile, since mask, decays, B' and C' serve twice the channels (32 heads, half heads / whole:
+// 2 x 4096 218 / 211 us a layer, 4 x 4096 412 / 399).
+int scan_narrow_width(int headdim, int64_t heads) { return headdim == 64 && 2 * heads > sm_count() ? 64 : 32; }
+
+cudaError_t scan_narrow(const ssd::SsdArgs &a, __nv_bfloat16 *bc, float *dl, int ndir, int dir0, int width, cudaStream_t s) {
+    return width == 64 ? launch<4>(a, bc, dl, ndir, dir0, s) : launch<2>(a, bc, dl, ndir, dir0, s);
+}
+
+}  // namespace dm

@@ -43,7 +43,6 @@ namespace {
 
 using namespace ssd;
 
-constexpr int Q = 128;            // tokens per chunk
 constexpr int P = 64;             // headdim
 constexpr int HALO = 8;           // conv look-back rows kept with the x tile (8 keeps the tile 1024-byte aligned)
 constexpr int XROWS = Q + HALO;
@@ -87,29 +86,6 @@ struct Misc {
 static_assert(sizeof(Misc) <= 7168, "Misc must fit its slot");
 static_assert(offsetof(Misc, norm_w) % 16 == 0 && offsetof(Misc, wbuf) % 16 == 0 && offsetof(Misc, cbuf) % 16 == 0, "float4 access");
 
-// One warp, one head, one 128-token chunk: d[e] = Delta of the token 4 lane + e in the direction's time order.  Writes Lambda (inclusive cumulative
-// Delta A in that order, log2 units) of physical chunk row r to dl[r] and Lambda' = Lambda - log2 Delta to dl[Lp + r].
-__device__ __forceinline__ void prep_lambda_head(const float (&d)[4], float A_log, bool rev, int lane, float *dl, int Lp) {
-    const float Ah = -expf(A_log) * 1.4426950408889634f;
-    float cum[4];
-    cum[0] = d[0] * Ah; cum[1] = fmaf(d[1], Ah, cum[0]); cum[2] = fmaf(d[2], Ah, cum[1]); cum[3] = fmaf(d[3], Ah, cum[2]);
-    float run = cum[3];
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-        const float up = __shfl_up_sync(0xffffffffu, run, off);
-        if (lane >= off) run += up;
-    }
-    const float base = run - cum[3];                             // sum over the lanes before this one
-    float lam[4], lamp[4];
-#pragma unroll
-    for (int e = 0; e < 4; ++e) { lam[e] = base + cum[e]; lamp[e] = lam[e] - __log2f(d[e]); }    // Delta = 0 (padding): Lambda' = +inf
-    const int rlo = rev ? Q - 4 - 4 * lane : 4 * lane;           // lowest physical row of this lane's four
-    const float4 v0 = rev ? make_float4(lam[3], lam[2], lam[1], lam[0]) : make_float4(lam[0], lam[1], lam[2], lam[3]);
-    const float4 v1 = rev ? make_float4(lamp[3], lamp[2], lamp[1], lamp[0]) : make_float4(lamp[0], lamp[1], lamp[2], lamp[3]);
-    *reinterpret_cast<float4 *>(dl + rlo) = v0;
-    *reinterpret_cast<float4 *>(dl + Lp + rlo) = v1;
-}
-
 // --------------------------------------------------------------------------------------------------
 // Launch 1: B', C' (bf16) and Lambda, Lambda' (fp32, log2 units).  CTAs of two kinds per physical chunk of one (direction, batch row): 64 of its rows
 // of B' and C' (a thread filters one channel pair over 16 rows), or the decays of 64 heads over all 128 rows (a thread takes the 16 heads
@@ -118,7 +94,7 @@ __device__ __forceinline__ void prep_lambda_head(const float (&d)[4], float A_lo
 // tokens of 64 heads took 35 us (20 now), 1 x 1024 of 120 heads 23 us (8 now).
 // --------------------------------------------------------------------------------------------------
 constexpr int PREP_PARTS = 4;               // sub-chunks of the short-block kernel per chunk
-constexpr int PREP_THREADS = 512, PREP_RUN = 16, PREP_ROWS = PREP_THREADS / N * PREP_RUN, PREP_BC = Q / PREP_ROWS;      // rows per thread, per B', C' unit; units per chunk
+constexpr int PREP_RUN = 16, PREP_ROWS = PREP_THREADS / N * PREP_RUN, PREP_BC = Q / PREP_ROWS;      // rows per thread, per B', C' unit; units per chunk
 constexpr int BCT_LD = N / 2 + 4;           // row pitch (32-bit words) of the B' / C' tile S is computed from: 16-byte rows, conflict-free ldmatrix
 static_assert(QB == Q / PREP_PARTS && PREP_ROWS == 2 * QB, "a B', C' unit covers two sub-chunks");
 
@@ -201,40 +177,6 @@ __device__ __forceinline__ void prep_bc(const SsdArgs &a, __nv_bfloat16 *__restr
         }
     }
 }
-// Delta and the cumulative log-decays of heads [h0, h0 + 64) over the chunk that starts at row r0; dsm: [64][Q] floats
-__device__ __forceinline__ void prep_decay(const SsdArgs &a, float *__restrict__ dA, int dir, int b, int r0, int h0, float *dsm) {
-    const bool rev = dir == 1;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const ScanDir &w = a.dir[dir];
-    const int64_t seq = (int64_t)dir * a.B + b;
-    {
-        const int row = tid & (Q - 1), hg = tid / Q * 16, t = r0 + row, hb = h0 + hg;
-        // the dt columns start on a 16-byte boundary (all widths are multiples of 8), and the rows are padded to one
-        const __nv_bfloat16 *src = a.zx + (((int64_t)(a.zx_tied ? 0 : dir) * a.B + b) * a.L + t) * a.d_in_proj + a.d_inner + a.conv_ch + hb;
-        uint4 v[2] = {make_uint4(0u, 0u, 0u, 0u), make_uint4(0u, 0u, 0u, 0u)};
-#pragma unroll
-        for (int i = 0; i < 2; ++i) if (t < a.L && hb + 8 * i < a.H) v[i] = __ldg(reinterpret_cast<const uint4 *>(src) + i);
-        float bias[16];
-#pragma unroll
-        for (int j = 0; j < 16; ++j) bias[j] = hb + j < a.H ? __ldg(w.dt_bias + hb + j) : 0.f;
-#pragma unroll
-        for (int j = 0; j < 16; ++j) {
-            const uint32_t word = reinterpret_cast<const uint32_t *>(v)[j >> 1];
-            const float dt = (j & 1) ? bf16_hi(word) : bf16_lo(word);
-            dsm[(hg + j) * Q + row] = t < a.L ? prep_delta(dt, bias[j]) : 0.f;
-        }
-    }
-    __syncthreads();
-#pragma unroll 2
-    for (int hh = warp; hh < 64; hh += PREP_THREADS / 32) {
-        const int h = h0 + hh;
-        if (h >= a.H) break;
-        const float4 q = *reinterpret_cast<const float4 *>(dsm + hh * Q + (rev ? Q - 4 - 4 * lane : 4 * lane));
-        const float d[4] = {rev ? q.w : q.x, rev ? q.z : q.y, rev ? q.y : q.z, rev ? q.x : q.w};
-        prep_lambda_head(d, __ldg(w.A_log + h), rev, lane, dA + ((seq * a.H + h) * 2) * a.Lp + r0, a.Lp);
-    }
-}
-
 // grid.x: for every chunk that the direction visits first (in time order), PREP_BC units of B', C' and one of decays per 64 heads
 template <bool WITH_S>
 __global__ void __launch_bounds__(PREP_THREADS)
@@ -246,7 +188,7 @@ ssd_prep_kernel(const __grid_constant__ SsdArgs a, __nv_bfloat16 *__restrict__ B
     const int per = PREP_BC + (a.H + 63) / 64, c = blockIdx.x / per, part = blockIdx.x - c * per;
     const int dir = dir0 + blockIdx.z, pc = dir == 1 ? a.nch - 1 - c : c;
     if (part < PREP_BC) prep_bc<WITH_S>(a, Bp, Cp, Sb, dir, blockIdx.y, pc * Q + part * PREP_ROWS, sm);
-    else prep_decay(a, dA, dir, blockIdx.y, pc * Q, (part - PREP_BC) * 64, reinterpret_cast<float *>(sm));
+    else prep_decay<false>(a, dA, dir, blockIdx.y, pc * Q, (part - PREP_BC) * 64, reinterpret_cast<float *>(sm));
 }
 
 // --------------------------------------------------------------------------------------------------
@@ -377,7 +319,7 @@ __device__ __noinline__ void prep_role(const SsdArgs &a, const PrepJob &pj, int 
                 float d[4];
 #pragma unroll
                 for (int e = 0; e < 4; ++e) d[e] = dsm[(rev ? Q - 1 - 4 * lane - e : 4 * lane + e) * 65 + hh];
-                prep_lambda_head(d, w.A_log[h], rev, lane, pj.dA + ((seq * a.H + h) * 2) * a.Lp + r0, a.Lp);
+                prep_lambda_head<false>(d, w.A_log[h], rev, lane, pj.dA + ((seq * a.H + h) * 2) * a.Lp + r0, a.Lp);
             }
         }
         // ---- publish the item
@@ -1236,6 +1178,13 @@ constexpr int BLOCK_MAX_L = 2 * QB;       // sequences up to this length take th
 
 bool block_mode(const ScanArgs &a) { return a.chunk == QB || (a.chunk == 0 && a.L <= BLOCK_MAX_L); }
 
+// d_state 16, beyond the short blocks
+bool narrow_mode(const ScanArgs &a) { return a.chunk == 0 && !block_mode(a) && scan_narrow_shape(a.P, a.N); }
+int narrow_width(const ScanArgs &a) {
+    const int w = scan_narrow_width(a.P, (int64_t)a.H * a.B * (a.dir_mask == DM_DIR_BOTH ? 2 : 1));
+    return a.ssq_room >= a.d_inner / w ? w : a.P;
+}
+
 struct Scratch {
     size_t bp, cp, da, sb, sy, total;
     int nch, Lp;
@@ -1282,6 +1231,8 @@ bool scan_ssd_supports(const ScanArgs &a) {
     return encode_fn() != nullptr;
 }
 
+int scan_ssq_parts(const ScanArgs &a) { return scan_ssd_supports(a) && narrow_mode(a) ? a.d_inner / narrow_width(a) : a.H; }
+
 size_t scan_ssd_workspace_bytes(const ScanArgs &a) {
     if (!shape_ok(a)) return 0;
     return scratch_layout(a).total;
@@ -1304,6 +1255,7 @@ cudaError_t scan_ssd(const ScanArgs &a, void *ws, cudaStream_t s) {
     float *Sb = blk ? reinterpret_cast<float *>(base + l.sb) : nullptr;
 
     if (blk && scan_step_supports(k)) return scan_step(k, a.P, ndir, dir0, s);
+    if (narrow_mode(a)) return scan_narrow(k, Bp, dA, ndir, dir0, narrow_width(a), s);
 
     // One long sequence leaves SMs without a scan CTA: they take the prep work inside the scan launch (see prep_role), except for
     // the first PRE_CHUNKS chunks of every sequence and direction, which a small prep launch of their own has ready by the time the

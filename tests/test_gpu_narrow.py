@@ -1,0 +1,72 @@
+"""The scan of narrow states (bf16, d_state 16, more than 64 tokens) against the CPU oracle: lengths around its sub-chunks of 32 tokens and around one round of a chain's warps, both head
+widths, odd head counts, carried state in and out, flags, single directions; and its error beside that of the 128-token kernel on the same inputs."""
+import numpy as np
+import pytest
+
+from oracle import bimamba_oracle as O
+from paper_2511_15927_b200 import inputs as I
+
+pytestmark = pytest.mark.gpu
+BF16_REL, BF16_ABS = 1e-2, 5e-2
+
+
+@pytest.fixture(scope="module")
+def G():
+    from paper_2511_15927_b200 import build
+    build.build()
+    import tests.gpu_util as g
+    return g
+
+
+def _check(G, got, want):
+    assert np.all(np.isfinite(got))
+    assert G.rel_l2(got, want) <= BF16_REL, G.rel_l2(got, want)
+    assert G.max_abs(got, want) <= BF16_ABS, G.max_abs(got, want)
+
+
+# (batch, heads, headdim, length, conv width, flags, directions).  Chains of half heads with 20 warps where heads are few (640 tokens a round), of whole heads with 16 warps (512 tokens) from 75
+# heads of all sequences and directions, with 8, 5 and 4 warps from 149, 297 and 445; (40, 16): more chains than are resident
+@pytest.mark.parametrize("B,H,P,L,k,flags,dirs", [
+    (1, 2, 64, 65, 4, 7, 3), (2, 8, 64, 96, 4, 7, 3), (2, 8, 32, 97, 4, 7, 3), (1, 8, 64, 128, 4, 7, 3), (3, 8, 32, 129, 3, 7, 3), (1, 16, 32, 159, 2, 6, 3),
+    (2, 8, 64, 161, 4, 5, 1), (2, 8, 64, 255, 4, 3, 2), (1, 8, 64, 640, 4, 7, 3), (1, 8, 64, 641, 4, 7, 3), (2, 24, 64, 513, 4, 7, 3), (4, 24, 64, 225, 4, 7, 3), (10, 16, 64, 161, 3, 7, 3),
+    (40, 16, 64, 130, 4, 7, 3), (1, 4, 64, 1301, 4, 0, 3), (2, 72, 64, 100, 4, 7, 3)])
+def test_forward_and_state(G, B, H, P, L, k, flags, dirs):
+    shape = I.MixerShape(B, L, P * H // 2, 2, 16, k, H)
+    wf, wr = I.make_mixer_weights(shape, 80 + L, I.BF16, perturb=True)
+    x = I.make_activations(shape, 80 + L, I.BF16)
+    kw = G.oracle_kwargs(shape, flags)
+    want = O.bimamba_forward(x, wf, wr, dir_mask=dirs, **kw)
+    got = G.run_forward(shape, I.BF16, wf, wr, x, flags=flags, dir_mask=dirs)
+    _check(G, got, want)
+    np.testing.assert_array_equal(got, G.run_forward(shape, I.BF16, wf, wr, x, flags=flags, dir_mask=dirs))          # run to run
+    if not dirs & 1:
+        return
+    ssm_in, conv_in = I.make_states(shape, 80 + L, I.BF16)
+    y_o, s_o, c_o = O.bimamba_block_step(x, wf, wr, ssm_state_in=ssm_in, conv_state_in=conv_in, dir_mask=dirs, **kw)
+    y_g, s_g, c_g = G.run_block_step(shape, I.BF16, wf, wr, x, ssm_in, conv_in, flags=flags, dir_mask=dirs)
+    _check(G, y_g, y_o)
+    _check(G, s_g, s_o)
+    _check(G, c_g, c_o)
+
+
+@pytest.mark.parametrize("P,L", [(64, 500), (32, 333)])
+def test_error_is_that_of_the_128_token_kernel(G, P, L):
+    """Both kernels round x', W, the weighted operand of the state update and the state's copy to bf16 and sum in fp32: their errors are of one size.  A tenth more is allowed for the shorter chunk,
+    which passes more of the history through the state's copy and less through W."""
+    shape = I.MixerShape(2, L, P * 8 // 2, 2, 16, 4, 8)
+    wf, wr = I.make_mixer_weights(shape, 9, I.BF16, perturb=True)
+    x = I.make_activations(shape, 9, I.BF16)
+    want = O.bimamba_forward(x, wf, wr, **G.oracle_kwargs(shape))
+    e = [G.rel_l2(G.run_forward(shape, I.BF16, wf, wr, x, chunk=c), want) for c in (0, 128)]
+    assert e[0] <= 1.1 * e[1], e
+
+
+def test_causality(G):
+    shape = I.MixerShape(2, 300, 256, 2, 16, 4, 8)
+    wf, wr = I.make_mixer_weights(shape, 4, I.BF16, perturb=True)
+    x = I.make_activations(shape, 4, I.BF16)
+    x2 = x.copy(); x2[0, 150] += 1.0
+    for dirs in (1, 2):
+        d = G.run_forward(shape, I.BF16, wf, wr, x2, dir_mask=dirs) - G.run_forward(shape, I.BF16, wf, wr, x, dir_mask=dirs)
+        before, after = (d[0, :150], d[0, 150:]) if dirs == 1 else (d[0, 151:], d[0, :151])
+        assert np.all(before == 0) and np.any(after != 0) and np.all(d[1] == 0)
