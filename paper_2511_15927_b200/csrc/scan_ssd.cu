@@ -340,6 +340,60 @@ __device__ __noinline__ void prep_role(const SsdArgs &a, const PrepJob &pj, int 
 // the B', C' tiles and S; each has its own Lambda, Lambda' (two per stage), its own mask W (mask group g builds head g's W, the second
 // one in the TMEM columns the other modes leave unused) and its own 32-wide Ya = W x' product; Yb, St, the state (two 32-column halves)
 // and the tiles are those of a 64-channel head, with the decay factors taken per column half.
+// The mask works on tiles of 8 x 8 in the accumulators' layout of mma.sync: a lane has two neighbouring columns of four rows (8 a + lane / 4 of its warp's 32), so that a column's factor serves four
+// entries and the tiles of the diagonal block that lie off its diagonal need no comparison, or no work at all.
+// W of 16 columns before the diagonal block: two products per entry, column factors in cf (shared memory), row factors in ri2.
+__device__ __forceinline__ void mask_before(uint32_t s_addr, uint32_t w_addr, const float *cf, const f32x2 (&ri2)[4], int qc) {
+    uint32_t r[2][8];
+    tmem_ld_tile16(s_addr, r[0]);
+    tmem_ld_tile16(s_addr + (16u << 16), r[1]);
+    const float2 c0 = *reinterpret_cast<const float2 *>(cf + 2 * qc), c1 = *reinterpret_cast<const float2 *>(cf + 8 + 2 * qc);
+    const f32x2 cf2[2] = {pk2(c0.x, c0.y), pk2(c1.x, c1.y)};
+    tmem_wait_ld();
+#pragma unroll
+    for (int hh = 0; hh < 2; ++hh) {
+        uint32_t out[4];
+#pragma unroll
+        for (int b = 0; b < 2; ++b)
+#pragma unroll
+            for (int a = 0; a < 2; ++a)
+                out[2 * b + a] = f2_to_bf2(mul2(mul2(pk2(__uint_as_float(r[hh][4 * b + 2 * a]), __uint_as_float(r[hh][4 * b + 2 * a + 1])), cf2[b]), ri2[2 * hh + a]));
+        tmem_st_tile16_h(w_addr + hh * (16u << 16), out);
+    }
+}
+// W of columns 16 HF .. of the diagonal block (s_addr, w_addr: the block's first column): one exponential per entry, none after i in time; rows without entries keep the zeros they were given once.
+template <bool REV, int HF>
+__device__ __forceinline__ void mask_diagonal(uint32_t s_addr, uint32_t w_addr, const float *lamp, const float (&li)[4], int gr, int qc, float Dh) {
+    constexpr bool USED[2] = {!(HF == 1 && !REV), !(HF == 0 && REV)};       // rows 0-15, rows 16-31
+    uint32_t r[2][8];
+#pragma unroll
+    for (int hh = 0; hh < 2; ++hh) if (USED[hh]) tmem_ld_tile16(s_addr + 16 * HF + hh * (16u << 16), r[hh]);
+    float2 lp[2];
+#pragma unroll
+    for (int b = 0; b < 2; ++b) lp[b] = *reinterpret_cast<const float2 *>(lamp + 16 * HF + 8 * b + 2 * qc);
+    tmem_wait_ld();
+#pragma unroll
+    for (int hh = 0; hh < 2; ++hh) {
+        if (!USED[hh]) continue;
+        uint32_t out[4];
+#pragma unroll
+        for (int b = 0; b < 2; ++b)
+#pragma unroll
+            for (int a = 0; a < 2; ++a) {
+                const int ta = 2 * hh + a, tb = 2 * HF + b, rel = REV ? tb - ta : ta - tb;      // > 0: all of the tile's entries count, < 0: none
+                if (rel < 0) { out[2 * b + a] = 0u; continue; }
+                float e0 = li[ta] - lp[b].x, e1 = li[ta] - lp[b].y;
+                if (rel == 0) {
+                    e0 = (REV ? 2 * qc >= gr : 2 * qc <= gr) ? e0 : -INFINITY;                  // 2^-inf = 0
+                    e1 = (REV ? 2 * qc + 1 >= gr : 2 * qc + 1 <= gr) ? e1 : -INFINITY;
+                }
+                const float s0 = __uint_as_float(r[hh][4 * b + 2 * a]), s1 = __uint_as_float(r[hh][4 * b + 2 * a + 1]);
+                out[2 * b + a] = rel == 0 ? pack_bf16(fmaf(s0, ex2f(e0), 2 * qc == gr ? Dh : 0.f), fmaf(s1, ex2f(e1), 2 * qc + 1 == gr ? Dh : 0.f)) : pack_bf16(s0 * ex2f(e0), s1 * ex2f(e1));
+            }
+        tmem_st_tile16_h(w_addr + 8 * HF + hh * (16u << 16), out);
+    }
+}
+
 template <int HM>
 __global__ void __launch_bounds__(NTHREADS, 1)
 ssd_scan_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_z,
@@ -348,7 +402,7 @@ ssd_scan_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
     extern __shared__ uint8_t smem_raw[];
     // 1024-byte aligned base, derived by offsetting the __shared__ array so that accesses stay shared-space loads and stores
     uint8_t *smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
-    constexpr bool HALFP = HM == 1, PAIR = HM == 2;
+    constexpr bool HALFP = HM == 1, PAIR = HM == 2, ALLPOLL = !PAIR;
     constexpr int NH = PAIR ? 2 : 1;                               // heads per CTA
     constexpr uint32_t DL_STAGE = NH * DL_HEAD;                    // bytes of one (Lambda, Lambda') stage
     Misc *misc = reinterpret_cast<Misc *>(smem + OFF_DL + NDL * DL_STAGE);
@@ -530,7 +584,7 @@ ssd_scan_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
                     if (leader) umma_ss<1>(tmem + TM_S, dC + o, dBk + o, I128);
                 }
                 if (leader) umma_commit(&misc->s_full);
-                if constexpr (HALFP) { if (c > 0 && !issue_ya(c - 1)) break; }
+                if constexpr (HALFP || PAIR) { if (c > 0 && !issue_ya(c - 1)) break; }
                 // Yb = C' h_in  (A = C' K-major, B = bf16 state [n][p] MN-major) into the buffer the epilogue of chunk c-2 has drained;
                 // its completion releases C' (S was issued before it) and the state copy
                 const uint32_t tyb = tmem + (par ? TM_YB1 : TM_YB0);
@@ -540,7 +594,7 @@ ssd_scan_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
 #pragma unroll
                 for (int kk = 1; kk < 8; ++kk) if (leader) umma_ss<1>(tyb, dC + (kk >> 2) * (T16 >> 4) + 2 * (kk & 3), dH + kk * 128, I64);
                 if (leader) umma_commit(&misc->empty_c);             // also releases the bf16 state copy
-                if constexpr (!HALFP) { if (c > 0 && !issue_ya(c - 1)) break; }
+                if constexpr (!HALFP && !PAIR) { if (c > 0 && !issue_ya(c - 1)) break; }
                 // h += B'^T (w o x')  (A = B' [j][n] MN-major, B = w o x' [j][p] MN-major), onto the state the conv groups have scaled
                 if (!WAIT2(&misc->xs_full, par, &misc->hs_ready, par)) break;
                 fence_after();
@@ -552,7 +606,7 @@ ssd_scan_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
                 if (c == nch - 1) ok = issue_ya(c);
             }
         };
-        if constexpr (HALFP) mma_role(elect_one());
+        if constexpr (HALFP || PAIR) mma_role(elect_one());
         else if (lane == 0) mma_role(true);
     } else if (warp < 4 + 4 * NWG) {
         // ============================================================ state update; conv + SiLU of the x tile; w o x'
@@ -635,7 +689,7 @@ ssd_scan_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
         for (int c = 0; c < nch; ++c) {
             const int sx = c % NX, sd = c % NDL;
             const uint32_t par = c & 1;
-            if (ok) ok = WAIT3(&misc->full_x[sx], (c / NX) & 1, &misc->full_dl[sd], (c / NDL) & 1, &misc->st_full, par ^ 1);
+            if (ok && (ALLPOLL || warp == 4)) ok = WAIT3(&misc->full_x[sx], (c / NX) & 1, &misc->full_dl[sd], (c / NDL) & 1, &misc->st_full, par ^ 1);
             if (!named_all(1, ROLE, ok)) { ok = false; break; }
             // (Lambda, Lambda') of the head whose state columns this thread hands over (two heads per CTA: the column half sh)
             const float *lam = reinterpret_cast<const float *>(smem + OFF_DL + sd * DL_STAGE + (PAIR ? sh : 0) * DL_HEAD), *lamp = lam + Q;
@@ -720,12 +774,19 @@ ssd_scan_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
         // The NWG groups share every row: group g takes the 16-column groups gi = g, g + NWG, ... of the mask and the
         // state columns [g, g+1) * P / NWG, so the triangular mask is split evenly between them.
         const int mg = (warp - 4 - 4 * NWG) >> 2;       // group index
-        const int row = (tid - (4 + 4 * NWG) * 32) & (WG - 1);      // token row i (mask) / state row n (state)
+        const int gr = lane >> 2, qc = lane & 3;        // rows 32 q + 8 a + gr, columns 2 qc and 2 qc + 1 of every eight
         const int q = warp & 3;
         // two heads per CTA: group mg builds the whole mask of head h + mg (its own Lambda, D and W columns) instead of half of one mask
         const float Dh = (a.flags & DM_FLAG_D_SKIP) ? w.D[h + (PAIR ? mg : 0)] : 0.f;
         const uint32_t tm_w = (PAIR && mg) ? TM_W1 : TM_W;
         float *cbuf = misc->cbuf[mg][q];
+        {                                                // what lies after i in time is zero in every chunk
+            uint32_t zero[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) zero[i] = 0u;
+            for (int gi = PAIR ? 0 : mg; gi < 8; gi += PAIR ? 1 : NWG) tmem_st_x8(tlane + tm_w + gi * 8, zero);
+            tmem_wait_st();
+        }
         bool ok = true;
         for (int c = 0; c < nch; ++c) {
             const int sd = c % NDL;
@@ -734,67 +795,35 @@ ssd_scan_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
             if (ok) ok = WAIT(&misc->full_dl[sd], (c / NDL) & 1);
             if (!named_all(3 + mg, WG, ok)) { ok = false; break; }
             const float *lam = reinterpret_cast<const float *>(smem + OFF_DL + sd * DL_STAGE + (PAIR ? mg : 0) * DL_HEAD), *lamp = lam + Q;
-            const float li = lam[row];
+            float li[4];
+#pragma unroll
+            for (int a4 = 0; a4 < 4; ++a4) li[a4] = lam[32 * q + 8 * a4 + gr];
             // ---- W_ij = S_ij 2^(Lambda_i - Lambda'_j) for j not after i in time, + D on the diagonal; 0 elsewhere.
             // Blocks of 32 x 32: the block on the diagonal takes one exponential per entry; a block before it (in
             // time) uses 2^(Lambda_i - Lambda_ref) * 2^(Lambda_ref - Lambda'_j) with Lambda_ref the last row before this
             // warp's rows -- both exponents are non-positive -- so it costs one exponential per row and per column.
             const int n_off = rev ? 3 - q : q;
-            float ri = 1.f;
+            f32x2 ri2[4] = {};
             if (n_off > 0) {
                 const float ref = lam[rev ? 32 * (q + 1) : 32 * q - 1];
-                ri = ex2f(li - ref);
+#pragma unroll
+                for (int a4 = 0; a4 < 4; ++a4) { const float v = ex2f(li[a4] - ref); ri2[a4] = pk2(v, v); }
                 for (int i = 0; i < n_off; ++i) {
                     const int j = (rev ? 32 * (q + 1) : 0) + 32 * i + lane;
                     cbuf[j] = ex2f(ref - lamp[j]);
                 }
                 __syncwarp();
             }
-            const f32x2 ri2 = pk2(ri, ri);
-            // validity of the diagonal block's entries as integers: entry jj (0..31) of the block counts iff key(jj) >= 0,
-            // and carries the D skip iff key(jj) == 0
-            const int ksign = rev ? 1 : -1, kbase = rev ? -(row & 31) : (row & 31);
             if (!WAIT2(&misc->s_full, par, &misc->y_full, par ^ 1)) { ok = false; continue; }
             fence_after();
+            {                                            // this group's share of the groups of 16 columns
+                const uint32_t s_q = tlane + TM_S + 32 * q, w_q = tlane + tm_w + 16 * q;
+                const float *lp_q = lamp + 32 * q;
+                if (PAIR || mg == 0) { if (rev) mask_diagonal<true, 0>(s_q, w_q, lp_q, li, gr, qc, Dh); else mask_diagonal<false, 0>(s_q, w_q, lp_q, li, gr, qc, Dh); }
+                if (PAIR || mg == 1) { if (rev) mask_diagonal<true, 1>(s_q, w_q, lp_q, li, gr, qc, Dh); else mask_diagonal<false, 1>(s_q, w_q, lp_q, li, gr, qc, Dh); }
 #pragma unroll 1
-            for (int gi = PAIR ? 0 : mg; gi < 8; gi += PAIR ? 1 : NWG) {        // this group's share of the 8 groups of 16 columns
-                const int jb = gi >> 1, j0 = gi * 16;
-                uint32_t out[8];
-                if (rev ? jb > q : jb < q) {
-                    uint32_t r[16];
-                    tmem_ld_x16(tlane + TM_S + j0, r);
-                    tmem_wait_ld();
-                    const float4 *cp = reinterpret_cast<const float4 *>(cbuf + j0);
-#pragma unroll
-                    for (int v4 = 0; v4 < 4; ++v4) {
-                        const float4 cv = cp[v4];
-                        out[2 * v4] = f2_to_bf2(mul2(mul2(pk2(__uint_as_float(r[4 * v4]), __uint_as_float(r[4 * v4 + 1])), pk2(cv.x, cv.y)), ri2));
-                        out[2 * v4 + 1] = f2_to_bf2(mul2(mul2(pk2(__uint_as_float(r[4 * v4 + 2]), __uint_as_float(r[4 * v4 + 3])), pk2(cv.z, cv.w)), ri2));
-                    }
-                } else if (jb == q) {
-                    uint32_t r[16];
-                    tmem_ld_x16(tlane + TM_S + j0, r);
-                    tmem_wait_ld();
-                    const float4 *lp4 = reinterpret_cast<const float4 *>(lamp + j0);
-#pragma unroll
-                    for (int v4 = 0; v4 < 4; ++v4) {
-                        const float4 lp = lp4[v4];
-                        const float lpv[4] = {lp.x, lp.y, lp.z, lp.w};
-                        float v[4];
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            const int key = ksign * ((j0 & 31) + 4 * v4 + e) + kbase;
-                            const float m = ex2f(key >= 0 ? li - lpv[e] : -INFINITY);      // 2^-inf = 0: no branch around the exponential
-                            v[e] = fmaf(__uint_as_float(r[4 * v4 + e]), m, key == 0 ? Dh : 0.f);
-                        }
-                        out[2 * v4] = pack_bf16(v[0], v[1]);
-                        out[2 * v4 + 1] = pack_bf16(v[2], v[3]);
-                    }
-                } else {
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) out[i] = 0u;
-                }
-                tmem_st_x8(tlane + tm_w + gi * 8, out);
+                for (int gi = (rev ? 2 * (q + 1) : 0) + (PAIR ? 0 : mg); gi < (rev ? 8 : 2 * q); gi += PAIR ? 1 : NWG)
+                    mask_before(tlane + TM_S + 16 * gi, tlane + tm_w + 8 * gi, cbuf + 16 * gi, ri2, qc);
             }
             fence_before();
             mbar_arrive(&misc->s_empty);                 // every read of S has completed (wait::ld above)
@@ -812,7 +841,7 @@ ssd_scan_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
         for (int c = 0; c < nch; ++c) {
             const int sz = c % NZ, sd = c % NDL, pc = rev ? nch - 1 - c : c;
             const uint32_t par = c & 1;
-            if (ok) ok = WAIT3(&misc->full_z[sz], (c / NZ) & 1, &misc->full_dl[sd], (c / NDL) & 1, &misc->y_full, par);
+            if (ok && (ALLPOLL || warp == 4 + 8 * NWG)) ok = WAIT3(&misc->full_z[sz], (c / NZ) & 1, &misc->full_dl[sd], (c / NDL) & 1, &misc->y_full, par);
             if (!named_all(2, ROLE, ok)) { ok = false; break; }
             fence_after();
             const float *lam = reinterpret_cast<const float *>(smem + OFF_DL + sd * DL_STAGE + (PAIR ? eg : 0) * DL_HEAD);      // two heads per CTA: group eg = head h + eg
