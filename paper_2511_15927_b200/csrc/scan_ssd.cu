@@ -341,7 +341,9 @@ __device__ __noinline__ void prep_role(const SsdArgs &a, const PrepJob &pj, int 
 // one in the TMEM columns the other modes leave unused) and its own 32-wide Ya = W x' product; Yb, St, the state (two 32-column halves)
 // and the tiles are those of a 64-channel head, with the decay factors taken per column half.
 // The mask works on tiles of 8 x 8 in the accumulators' layout of mma.sync: a lane has two neighbouring columns of four rows (8 a + lane / 4 of its warp's 32), so that a column's factor serves four
-// entries and the tiles of the diagonal block that lie off its diagonal need no comparison, or no work at all.
+// entries and the tiles of the diagonal block that lie off its diagonal need no comparison, or no work at all.  With a lane per row (32x32b loads) 16 columns took four 16-byte broadcasts from shared memory, which
+// this SM answers in 250 clocks at that load, and the diagonal block 32 compared exponentials per lane instead of 20, 8 of them compared: 213 -> 200 us for 8 x 1024 tokens of 120 heads of 32, 355 -> 340 us for
+// 8 x 2048 of 64 heads of 64.
 // W of 16 columns before the diagonal block: two products per entry, column factors in cf (shared memory), row factors in ri2.
 __device__ __forceinline__ void mask_before(uint32_t s_addr, uint32_t w_addr, const float *cf, const f32x2 (&ri2)[4], int qc) {
     uint32_t r[2][8];
@@ -402,7 +404,8 @@ ssd_scan_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
     extern __shared__ uint8_t smem_raw[];
     // 1024-byte aligned base, derived by offsetting the __shared__ array so that accesses stay shared-space loads and stores
     uint8_t *smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
-    constexpr bool HALFP = HM == 1, PAIR = HM == 2, ALLPOLL = !PAIR;
+    constexpr bool HALFP = HM == 1, PAIR = HM == 2;
+    constexpr bool ALL_POLL = !PAIR;                               // conv and epilogue groups: every warp asks the barriers, or one warp does and the others sleep at the group barrier (216 -> 213 us with two heads per CTA, 1 % slower with one)
     constexpr int NH = PAIR ? 2 : 1;                               // heads per CTA
     constexpr uint32_t DL_STAGE = NH * DL_HEAD;                    // bytes of one (Lambda, Lambda') stage
     Misc *misc = reinterpret_cast<Misc *>(smem + OFF_DL + NDL * DL_STAGE);
@@ -529,11 +532,12 @@ ssd_scan_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
         // Order per iteration: S(c), Yb(c), Ya(c-1), St(c).  S(c) goes out as soon as the mask of chunk c-1 has read
         // S(c-1); Yb(c) follows at once (its accumulator is double-buffered, so it does not wait for the epilogue of
         // chunk c-1), which frees the single C' buffer early enough for the next chunk's load.
-        // Half-width heads: the whole warp walks the loop and waits, one elected lane issues the products and their
+        // 32-wide heads: the whole warp walks the loop and waits, one elected lane issues the products and their
         // commits (the operand descriptors then live in uniform registers and a product takes a third of the time to
-        // issue), and Ya(c-1) goes out before Yb(c) so that the mask of chunk c starts earlier.  With full-width heads
-        // the conv groups are the longer chain and both changes only take issue slots from them at the wrong time
-        // (measured 5 % slower), so there one lane runs the loop and Ya(c-1) follows Yb(c).
+        // issue), and Ya(c-1) goes out before Yb(c), so that the mask of chunk c starts earlier: the masks, two whole ones
+        // where a CTA carries two heads, are the longest chain there (120 heads, 8 x 1024 tokens: 242 -> 216 us).  With
+        // 64-wide heads the conv groups are, and both changes only take issue slots from them at the wrong time
+        // (340 -> 359 us for 8 x 2048 tokens of 64 heads, either change alone 348 and 356), so there one lane runs the loop and Ya(c-1) follows Yb(c).
         auto mma_role = [&](const bool leader) {
             // low halves of the operand descriptors; a K step of 16 advances a K-major operand by 32 bytes inside its
             // 64-wide tile (+2) or to the next tile (+T16/16), an MN-major operand by 16 rows (+2048/16)
@@ -689,7 +693,7 @@ ssd_scan_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
         for (int c = 0; c < nch; ++c) {
             const int sx = c % NX, sd = c % NDL;
             const uint32_t par = c & 1;
-            if (ok && (ALLPOLL || warp == 4)) ok = WAIT3(&misc->full_x[sx], (c / NX) & 1, &misc->full_dl[sd], (c / NDL) & 1, &misc->st_full, par ^ 1);
+            if (ok && (ALL_POLL || warp == 4)) ok = WAIT3(&misc->full_x[sx], (c / NX) & 1, &misc->full_dl[sd], (c / NDL) & 1, &misc->st_full, par ^ 1);
             if (!named_all(1, ROLE, ok)) { ok = false; break; }
             // (Lambda, Lambda') of the head whose state columns this thread hands over (two heads per CTA: the column half sh)
             const float *lam = reinterpret_cast<const float *>(smem + OFF_DL + sd * DL_STAGE + (PAIR ? sh : 0) * DL_HEAD), *lamp = lam + Q;
@@ -841,7 +845,7 @@ ssd_scan_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
         for (int c = 0; c < nch; ++c) {
             const int sz = c % NZ, sd = c % NDL, pc = rev ? nch - 1 - c : c;
             const uint32_t par = c & 1;
-            if (ok && (ALLPOLL || warp == 4 + 8 * NWG)) ok = WAIT3(&misc->full_z[sz], (c / NZ) & 1, &misc->full_dl[sd], (c / NDL) & 1, &misc->y_full, par);
+            if (ok && (ALL_POLL || warp == 4 + 8 * NWG)) ok = WAIT3(&misc->full_z[sz], (c / NZ) & 1, &misc->full_dl[sd], (c / NDL) & 1, &misc->y_full, par);
             if (!named_all(2, ROLE, ok)) { ok = false; break; }
             fence_after();
             const float *lam = reinterpret_cast<const float *>(smem + OFF_DL + sd * DL_STAGE + (PAIR ? eg : 0) * DL_HEAD);      // two heads per CTA: group eg = head h + eg
