@@ -67,7 +67,8 @@ typedef struct {
     int32_t dir_mask;   /* DM_DIR_BOTH; one direction alone is meant for invariant tests */
     int32_t chunk;      /* tokens per scan chunk; 0 = library default.  Results do not depend on it
                            beyond rounding order.  bf16 with d_state <= 128 runs the chunked form of the
-                           recurrence and takes 0, 128 (tensor-core kernel; the default above 64 tokens)
+                           recurrence and takes 0, 128 (tensor-core kernel; the default above 64 tokens,
+                           except for d_state 16, whose default has a kernel of its own with tiles of 32)
                            or 32 (CUDA-core kernel; the default up to 64 tokens, i.e. for the blocks of
                            block-autoregressive decoding) -- other values: DM_ERR_UNSUPPORTED.  fp32, and
                            d_state 256, run the sequential form, where any chunk > 0 only sizes the
@@ -361,7 +362,7 @@ int dm_bimamba_forward_static(const dm_mixer_cfg *cfg, const dm_dir_weights w[2]
 int dm_selftest_wait_timeout(uint32_t limit_us, uint64_t *out, void *cuda_stream);
 
 /* Self-test switch for the same failure path inside the tensor-core scan (no counterpart in the paper).  While on, a mixer call
- * whose scan can do its prep work inside the scan launch (fewer scan CTAs than SMs, more than eight chunks; outside the test one
+ * whose scan can do its prep work inside the scan launch (the tensor-core kernel, fewer scan CTAs than SMs, more than eight chunks; outside the test one
  * sequence of 32 chunks or more does) launches the scan without the CTAs of that role: the flags its load warps wait for from the ninth chunk on are never raised,
  * the waits run out after their regular limit (2 s), and every role of every CTA has to leave through the abort path -- loads in
  * flight waited for, TMEM freed.  A call on the sequential scan (fp32, or d_state 256) of more than two chunks leaves out the
