@@ -208,7 +208,7 @@ static int run_mixer(const dm_mixer_cfg *c, const Dims &m, const dm_dir_weights 
     sa.z_gated = 1;
     const bool ssd = scan_ssd_supports(sa);
     sa.z_gated = ssd ? 1 : 0;
-    // The scan of a narrow state can leave its sums of squares per 32 channels, more of them than the ssq region holds when heads are wider.  They then lie in ytmp's place, which is written, if at
+    // The scan of a narrow state leaves its sums of squares per 32 channels, more of them than the ssq region holds when heads are wider.  They then lie in ytmp's place, which is written, if at
     // all, after they have become rstd.
     sa.ssq_room = m.d_inner / 32 * 2 <= m.d ? m.d_inner / 32 : m.H;
     const int parts = ssd ? scan_ssq_parts(sa) : m.H;

@@ -154,7 +154,7 @@ bool scan_ssd_supports(const ScanArgs &a);
 bool scan_ssd_chunk_ok(int dtype, int d_state, int chunk);
 void scan_ssd_selftest_withhold(int on);
 bool scan_selftest_withheld();
-// Sums of squares per row that scan_ssd writes: one per head, or (with that room) one per 32 channels
+// Sums of squares per row that scan_ssd writes: one per head, or (narrow state, with that room) one per 32 channels, whatever the batch
 int scan_ssq_parts(const ScanArgs &a);
 size_t scan_ssd_workspace_bytes(const ScanArgs &a);
 cudaError_t scan_ssd(const ScanArgs &a, void *ws, cudaStream_t s);

@@ -98,6 +98,21 @@ __device__ __forceinline__ bool flag_reached(uint32_t addr, int target, volatile
     }
 }
 
+// Eight sums per lane (of tokens 8 i + 2 qc + e) over the lanes of equal qc: halves exchanged, so that each lane ends with one token's sum
+__device__ __forceinline__ float token_sum(const f32x2 (&sq)[4], int lane) {
+    float v[4][2], u[2][2], t[2];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) upk2(sq[i], v[i][0], v[i][1]);
+    const bool b4 = lane & 16, b3 = lane & 8, b2 = lane & 4;
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int e = 0; e < 2; ++e) u[i][e] = (b4 ? v[2 + i][e] : v[i][e]) + __shfl_xor_sync(0xffffffffu, b4 ? v[i][e] : v[2 + i][e], 16);
+#pragma unroll
+    for (int e = 0; e < 2; ++e) t[e] = (b3 ? u[1][e] : u[0][e]) + __shfl_xor_sync(0xffffffffu, b3 ? u[0][e] : u[1][e], 8);
+    return (b2 ? t[1] : t[0]) + __shfl_xor_sync(0xffffffffu, b2 ? t[0] : t[1], 4);
+}
+
 // The state warp: 16 x 16 tiles [channels][states] in the accumulators' layout
 template <int MT>
 __device__ __forceinline__ void state_role(const SsdArgs &a, const uint8_t *slots, Shared<MT> *sh, int nt, int nsub, const float *h_in, float *h_out, int *status) {
@@ -154,7 +169,7 @@ __device__ __forceinline__ void chain(const CUtensorMap &map_x, const CUtensorMa
     using T = Tile<MT>;
     constexpr int CW = T::CW, RB = T::RB;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, gr = lane >> 2, qc = lane & 3, nt = (blockDim.x >> 5) - 1;      // nt: tile warps
-    const int L = a.L, nsub = (L + QB - 1) / QB, seq = (REV ? a.B : 0) + b, zseq = a.zx_tied ? b : seq, ch0 = grp * CW, h = ch0 / a.Pr, G = a.d_inner / CW;
+    const int L = a.L, nsub = (L + QB - 1) / QB, seq = (REV ? a.B : 0) + b, zseq = a.zx_tied ? b : seq, ch0 = grp * CW, h = ch0 / a.Pr;
     volatile int *abort_flag = &sh->abort;
     uint8_t *const slot = slots + warp * T::SLOT;
     const uint32_t sb = smem_u32(slot), conv_w = smem_u32(&sh->conv[0][0]), stp = sb + T::ST + lane * 16;
@@ -338,10 +353,13 @@ __device__ __forceinline__ void chain(const CUtensorMap &map_x, const CUtensorMa
         // ---- y and the gate, 16 channels at a time
         if (!WAIT(bz, it & 1)) break;
         f32x2 sq[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) sq[i] = pk2(0.f, 0.f);
+        float part[MT / 2];                                                       // this lane's token: sums of squares of 32 channels each
 #pragma unroll
         for (int m = 0; m < MT; ++m) {
+            if (m % 2 == 0) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) sq[i] = pk2(0.f, 0.f);
+            }
             float y[4][4];
 #pragma unroll
             for (int i = 0; i < 4; ++i)
@@ -374,6 +392,7 @@ __device__ __forceinline__ void chain(const CUtensorMap &map_x, const CUtensorMa
                 }
                 stmatrix_x4_t(ad, z[0], z[1], z[2], z[3]);
             }
+            if (m % 2 && m < MT - 1 && a.ssq) part[m / 2] = token_sum(sq, lane);
         }
         fence_proxy_async();
         __syncwarp();
@@ -382,20 +401,14 @@ __device__ __forceinline__ void chain(const CUtensorMap &map_x, const CUtensorMa
             bulk_commit();
         }
         if (a.ssq) {
-            // eight sums per lane over the lanes of equal qc: halves exchanged, so that each lane ends with one token's sum
-            float v[4][2], u[2][2], t[2];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) upk2(sq[i], v[i][0], v[i][1]);
-            const bool b4 = lane & 16, b3 = lane & 8, b2 = lane & 4;
-#pragma unroll
-            for (int i = 0; i < 2; ++i)
-#pragma unroll
-                for (int e = 0; e < 2; ++e) u[i][e] = (b4 ? v[2 + i][e] : v[i][e]) + __shfl_xor_sync(0xffffffffu, b4 ? v[i][e] : v[2 + i][e], 16);
-#pragma unroll
-            for (int e = 0; e < 2; ++e) t[e] = (b3 ? u[1][e] : u[0][e]) + __shfl_xor_sync(0xffffffffu, b3 ? u[0][e] : u[1][e], 8);
-            const float s = (b2 ? t[1] : t[0]) + __shfl_xor_sync(0xffffffffu, b2 ? t[0] : t[1], 4);
-            const int i = (b4 ? 16 : 0) + (b3 ? 8 : 0) + 2 * qc + (b2 ? 1 : 0), row = r0 + (REV ? QB - 1 - i : i);
-            if (row < L) a.ssq[((int64_t)seq * L + row) * G + grp] = s;
+            part[MT / 2 - 1] = token_sum(sq, lane);
+            const int i = ((lane >> 3) << 3) + 2 * qc + ((lane >> 2) & 1), row = r0 + (REV ? QB - 1 - i : i);      // token_sum's
+            float *dst = a.ssq + ((int64_t)seq * L + row) * a.ssq_parts;
+            if (row < L) {
+                if constexpr (MT == 2) dst[grp] = part[0];
+                else if (a.ssq_parts > a.H) *reinterpret_cast<float2 *>(dst + 2 * grp) = make_float2(part[0], part[1]);
+                else dst[grp] = part[0] + part[1];
+            }
         }
     }
     if (*abort_flag && lane == 0 && warp < nsub) {                                // aborting: bounded wait for the loads still in flight

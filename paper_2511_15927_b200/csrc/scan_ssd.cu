@@ -1213,10 +1213,9 @@ bool block_mode(const ScanArgs &a) { return a.chunk == QB || (a.chunk == 0 && a.
 
 // d_state 16, beyond the short blocks
 bool narrow_mode(const ScanArgs &a) { return a.chunk == 0 && !block_mode(a) && scan_narrow_shape(a.P, a.N); }
-int narrow_width(const ScanArgs &a) {
-    const int w = scan_narrow_width(a.P, (int64_t)a.H * a.B * (a.dir_mask == DM_DIR_BOTH ? 2 : 1));
-    return a.ssq_room >= a.d_inner / w ? w : a.P;
-}
+// Halves of a head each leave a sum of squares; whole heads leave two as well, wherever halves could have been the choice
+bool narrow_halves(const ScanArgs &a) { return a.ssq_room >= a.d_inner / 32; }
+int narrow_width(const ScanArgs &a) { return narrow_halves(a) ? scan_narrow_width(a.P, (int64_t)a.H * a.B * (a.dir_mask == DM_DIR_BOTH ? 2 : 1)) : a.P; }
 
 struct Scratch {
     size_t bp, cp, da, sb, sy, total;
@@ -1264,7 +1263,7 @@ bool scan_ssd_supports(const ScanArgs &a) {
     return encode_fn() != nullptr;
 }
 
-int scan_ssq_parts(const ScanArgs &a) { return scan_ssd_supports(a) && narrow_mode(a) ? a.d_inner / narrow_width(a) : a.H; }
+int scan_ssq_parts(const ScanArgs &a) { return scan_ssd_supports(a) && narrow_mode(a) && narrow_halves(a) ? a.d_inner / 32 : a.H; }
 
 size_t scan_ssd_workspace_bytes(const ScanArgs &a) {
     if (!shape_ok(a)) return 0;
@@ -1280,7 +1279,7 @@ cudaError_t scan_ssd(const ScanArgs &a, void *ws, cudaStream_t s) {
     SsdArgs k{};
     k.B = a.B; k.L = a.L; k.H = a.H; k.d_inner = a.d_inner; k.d_in_proj = a.d_in_proj; k.conv_ch = a.conv_ch; k.k = a.k;
     k.flags = a.flags; k.nch = l.nch; k.Lp = l.Lp; k.Nr = a.N; k.Pr = a.P; k.zx_tied = a.zx_tied; k.g = static_cast<__nv_bfloat16 *>(a.g);
-    k.zx = static_cast<const __nv_bfloat16 *>(a.zx); k.ssq = a.ssq; k.dA = dA;
+    k.zx = static_cast<const __nv_bfloat16 *>(a.zx); k.ssq = a.ssq; k.ssq_parts = scan_ssq_parts(a); k.dA = dA;
     k.ssm_in = a.ssm_in; k.ssm_out = a.ssm_out; k.conv_in = static_cast<const __nv_bfloat16 *>(a.conv_in);
     k.dir[0] = a.dir[0]; k.dir[1] = a.dir[1];
     const int ndir = a.dir_mask == DM_DIR_BOTH ? 2 : 1, dir0 = a.dir_mask == DM_DIR_REV ? 1 : 0;

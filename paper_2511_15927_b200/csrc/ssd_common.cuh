@@ -22,7 +22,8 @@ struct SsdArgs {
     int zx_tied;                 // both directions read the in_proj output of direction 0 (shared projections)
     __nv_bfloat16 *g;            // [2][B*L][d_inner] gated output (written with plain stores when Pr < P, else through map_g)
     const __nv_bfloat16 *zx;
-    float *ssq;
+    float *ssq;                  // [2][B*L][ssq_parts] sums of squares of the gated output, or NULL
+    int ssq_parts;               // H, or (narrow-state kernel) one per 32 channels
     const float *dA;             // [2][B][H][2][Lp]: Lambda, Lambda' (log2 units)
     const float *ssm_in; float *ssm_out;
     const __nv_bfloat16 *conv_in;  // [B][k-1][conv_ch] pre-conv rows before the first token (left-to-right layer), or NULL
@@ -134,7 +135,8 @@ __device__ __forceinline__ uint4 ld8_bf16(const __nv_bfloat16 *p) {
 bool scan_step_supports(const ssd::SsdArgs &a);
 cudaError_t scan_step(const ssd::SsdArgs &a, int headdim, int ndir, int dir0, cudaStream_t s);
 // Sequences of more than two sub-chunks with d_state 16, in chains of `width` channels (scan_narrow_width; heads: of all sequences and directions): see scan_narrow.cu.
-// bc: [2][B][L][32] bf16, dl: [2][B][H][Lp / 32][2][32] fp32 of scratch; a.ssq: [2][B][L][d_inner / width].
+// bc: [2][B][L][32] bf16, dl: [2][B][H][Lp / 32][2][32] fp32 of scratch.  The sums of squares do not depend on the width, so that a row's result does not depend on how many others share the
+// call: a.ssq_parts is d_inner / 32, or H where heads are as wide as the chains.
 bool scan_narrow_shape(int headdim, int d_state);
 int scan_narrow_width(int headdim, int64_t heads);
 cudaError_t scan_narrow(const ssd::SsdArgs &a, __nv_bfloat16 *bc, float *dl, int ndir, int dir0, int width, cudaStream_t s);

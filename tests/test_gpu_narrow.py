@@ -70,3 +70,25 @@ def test_causality(G):
         d = G.run_forward(shape, I.BF16, wf, wr, x2, dir_mask=dirs) - G.run_forward(shape, I.BF16, wf, wr, x, dir_mask=dirs)
         before, after = (d[0, :150], d[0, 150:]) if dirs == 1 else (d[0, 151:], d[0, :151])
         assert np.all(before == 0) and np.any(after != 0) and np.all(d[1] == 0)
+
+
+def test_a_row_does_not_depend_on_the_rows_beside_it(G):
+    """Few heads are split into halves, many are not: the sums of squares, and with them every bit of a row, are the same either way.  20 rows of 4 heads are 160 chains, 3 rows 24 (d_model 128: the
+    products' tiles are the same for both); the host-buffer call cuts its batch into pieces of 3 rows."""
+    shape = I.MixerShape(20, 2100, 128, 2, 16, 4, 4)
+    wf, wr = I.make_mixer_weights(shape, 6, I.BF16, perturb=True)
+    x = I.make_activations(shape, 6, I.BF16)
+    whole = G.run_forward(shape, I.BF16, wf, wr, x)
+    few = I.MixerShape(3, 2100, 128, 2, 16, 4, 4)
+    np.testing.assert_array_equal(G.run_forward(few, I.BF16, wf, wr, np.ascontiguousarray(x[7:10])), whole[7:10])
+    np.testing.assert_array_equal(G.run_forward_host(shape, I.BF16, wf, wr, x), whole)
+
+
+@pytest.mark.parametrize("B", [2, 3])
+def test_no_room_for_sums_of_half_heads(G, B):
+    """expand 32: the sums of squares of 32 channels each have no place in the workspace, so heads of 64 stay whole at any batch (64 and 96 chains) and leave one sum each."""
+    shape = I.MixerShape(B, 200, 32, 32, 16, 4, 16)
+    assert shape.headdim == 64
+    wf, wr = I.make_mixer_weights(shape, 7, I.BF16, perturb=True)
+    x = I.make_activations(shape, 7, I.BF16)
+    _check(G, G.run_forward(shape, I.BF16, wf, wr, x), O.bimamba_forward(x, wf, wr, **G.oracle_kwargs(shape)))
