@@ -8,7 +8,7 @@
 //     St       the tile's own contribution to the state, x'^T (w o B'), left in shared memory for the state warp
 //     S, W     C' B'^T; its accumulators, masked and weighted, are the B operand of the next product as they stand
 //     chain    waits for the state before the tile: the state warp keeps the state in registers and, tile by tile, leaves its bf16 copy and takes h <- 2^Lambda_last h + St
-//     y, gate  y^T = 2^Lambda_i (h_in C'^T) + x'^T W^T, 16 channels at a time; z enters in the accumulators' layout (ldmatrix.trans), g = y SiLU(z), sums of squares, * norm_w; out through
+//     y, gate  y^T = 2^Lambda_i (h_in C'^T) + D x'^T + x'^T W^T, 16 channels at a time; z enters in the accumulators' layout (ldmatrix.trans), g = y SiLU(z), sums of squares, * norm_w; out through
 //              stmatrix.trans and a TMA store
 // Time order is a matter of row addresses (<- reads its rows backwards), so that the mask is the same for both directions.
 // The launch before (narrow_prep) leaves B' | C' as bf16 rows of 32 columns and the decays relative to each sub-chunk.
@@ -74,6 +74,13 @@ __device__ __forceinline__ void mma(float (&d)[4], const uint32_t (&a)[4], uint3
     asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
         : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
+// v = hi + lo to 16 bits.  Where v is infinite its rest is NaN: the minimum makes it a number that leaves the infinity alone
+__device__ __forceinline__ void split_bf16(f32x2 v, uint32_t &hi, uint32_t &lo) {
+    hi = f2_to_bf2(v);
+    const uint32_t r = f2_to_bf2(fma2(pk2(-1.f, -1.f), bf2_to_f2(hi), v));
+    const __nv_bfloat162 c = __hmin2(*reinterpret_cast<const __nv_bfloat162 *>(&r), __float2bfloat162_rn(0x1p100f));
+    lo = *reinterpret_cast<const uint32_t *>(&c);
+}
 __device__ __forceinline__ void raise_flag(uint32_t addr, int v) { asm volatile("st.release.cta.shared::cta.s32 [%0], %1;" ::"r"(addr), "r"(v) : "memory"); }
 // Bounded wait until a counter in shared memory has reached `target` (same abort protocol as mbar_wait).  A plain load is answered in a third of the time an mbarrier's probe takes, and these waits
 // are the chain's serial part.
@@ -113,9 +120,9 @@ __device__ __forceinline__ float token_sum(const f32x2 (&sq)[4], int lane) {
     return (b2 ? t[1] : t[0]) + __shfl_xor_sync(0xffffffffu, b2 ? t[0] : t[1], 4);
 }
 
-// The state warp: 16 x 16 tiles [channels][states] in the accumulators' layout
-template <int MT>
-__device__ __forceinline__ void state_role(const SsdArgs &a, const uint8_t *slots, Shared<MT> *sh, int nt, int nsub, const float *h_in, float *h_out, int *status) {
+// The state warp: 16 x 16 tiles [channels][states] in the accumulators' layout.  PARTS: bf16 numbers to an entry of the state's copy
+template <int MT, int PARTS>
+__device__ __forceinline__ void state_role(const uint8_t *slots, Shared<MT> *sh, int nt, int nsub, const float *h_in, float *h_out, int *status) {
     using T = Tile<MT>;
     const int lane = threadIdx.x & 31, gr = lane >> 2, qc = lane & 3;
     volatile int *abort_flag = &sh->abort;
@@ -138,9 +145,18 @@ __device__ __forceinline__ void state_role(const SsdArgs &a, const uint8_t *slot
             for (int n = 0; n < 2; ++n) st[m][n] = lds4(slot + T::ST + lane * 16 + (2 * m + n) * 512);
         const float dec = lds1(slot + T::E + (QB - 1) * 4);
 #pragma unroll
-        for (int m = 0; m < MT; ++m)
-            asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(slot + T::ST + lane * 16 + m * 512), "r"(pack_bf16(h[m][0][0], h[m][0][1])), "r"(pack_bf16(h[m][0][2], h[m][0][3])),
-                         "r"(pack_bf16(h[m][1][0], h[m][1][1])), "r"(pack_bf16(h[m][1][2], h[m][1][3])) : "memory");
+        for (int m = 0; m < MT; ++m) {
+            uint32_t c[2][4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const f32x2 v = pk2(h[m][e >> 1][(e & 1) * 2], h[m][e >> 1][(e & 1) * 2 + 1]);
+                if constexpr (PARTS == 2) split_bf16(v, c[0][e], c[1][e]);
+                else c[0][e] = f2_to_bf2(v);
+            }
+#pragma unroll
+            for (int u = 0; u < PARTS; ++u)
+                asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(slot + T::ST + lane * 16 + (PARTS * m + u) * 512), "r"(c[u][0]), "r"(c[u][1]), "r"(c[u][2]), "r"(c[u][3]) : "memory");
+        }
         __syncwarp();
         if (lane == 0) raise_flag(done, k + 1);
         const f32x2 dec2 = pk2(dec, dec);
@@ -163,11 +179,13 @@ __device__ __forceinline__ void state_role(const SsdArgs &a, const uint8_t *slot
     }
 }
 
-template <int MT, bool REV>
+// The state's copy is bf16, of which the history of every tile is read: without the D skip beside it that made y up to 1 % less accurate than the 128-token kernel's (which takes more of the history
+// through its mask), so that the copy has two parts there (6 to 8 % of a layer's time).  With the skip, D x' is added in fp32 instead of in W, and y is 9 % more accurate than that kernel's.
+template <int MT, bool SKIP, bool REV>
 __device__ __forceinline__ void chain(const CUtensorMap &map_x, const CUtensorMap &map_z, const CUtensorMap &map_bc, const CUtensorMap &map_g, const SsdArgs &a,
                                       const float *__restrict__ dl, uint8_t *slots, Shared<MT> *sh, int grp, int b, int *status) {
     using T = Tile<MT>;
-    constexpr int CW = T::CW, RB = T::RB;
+    constexpr int CW = T::CW, RB = T::RB, PARTS = SKIP ? 1 : 2;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, gr = lane >> 2, qc = lane & 3, nt = (blockDim.x >> 5) - 1;      // nt: tile warps
     const int L = a.L, nsub = (L + QB - 1) / QB, seq = (REV ? a.B : 0) + b, zseq = a.zx_tied ? b : seq, ch0 = grp * CW, h = ch0 / a.Pr;
     volatile int *abort_flag = &sh->abort;
@@ -175,10 +193,11 @@ __device__ __forceinline__ void chain(const CUtensorMap &map_x, const CUtensorMa
     const uint32_t sb = smem_u32(slot), conv_w = smem_u32(&sh->conv[0][0]), stp = sb + T::ST + lane * 16;
     uint64_t *const bx = &sh->x[warp], *const bz = &sh->z[warp];
     const float *dl_head = dl + ((int64_t)seq * a.H + h) * 2 * a.Lp;
-    const float Dh = (a.flags & DM_FLAG_D_SKIP) ? a.dir[REV ? 1 : 0].D[h] : 0.f;
+    const float D1 = SKIP ? a.dir[REV ? 1 : 0].D[h] : 0.f;
+    const f32x2 Dh = pk2(D1, D1);
     if (warp == nt) {
         const int64_t state0 = (((int64_t)b * a.H + h) * a.Pr + ch0 % a.Pr) * NS;
-        state_role<MT>(a, slots, sh, nt, nsub, !REV && a.ssm_in ? a.ssm_in + state0 : nullptr, !REV && a.ssm_out ? a.ssm_out + state0 : nullptr, status);
+        state_role<MT, PARTS>(slots, sh, nt, nsub, !REV && a.ssm_in ? a.ssm_in + state0 : nullptr, !REV && a.ssm_out ? a.ssm_out + state0 : nullptr, status);
         return;
     }
 
@@ -270,33 +289,33 @@ __device__ __forceinline__ void chain(const CUtensorMap &map_x, const CUtensorMa
         // ---- St = x'^T (w o B')
         uint32_t xa[MT][2][4];
         {
-            float st[MT][2][4];
-            uint32_t wb[2][4];                                                    // [16 rows j][(j lo, n lo), (j hi, n lo), (j lo, n hi), (j hi, n hi)]
+            // B' comes rounded to bf16, and rounding w o B' once more made the state 11 % less accurate than the 128-token kernel's (which rounds w o x' once): w o B' is the sum of two bf16 numbers
+            // (1 to 2 % of a layer's time)
+            uint32_t wb[2][4], wc[2][4];                                          // [16 rows j][(j lo, n lo), (j hi, n lo), (j lo, n hi), (j hi, n hi)]
 #pragma unroll
             for (int kt = 0; kt < 2; ++kt) {
                 ldmatrix_x4_t(wb[kt][0], wb[kt][1], wb[kt][2], wb[kt][3], bco + kt * BC16);
                 const float2 wl = lds2(sb + T::E + QB * 4 + (16 * kt + 2 * qc) * 4), wh = lds2(sb + T::E + QB * 4 + (16 * kt + 8 + 2 * qc) * 4);
 #pragma unroll
-                for (int e = 0; e < 4; ++e) wb[kt][e] = f2_to_bf2(mul2(bf2_to_f2(wb[kt][e]), (e & 1) ? pk2(wh.x, wh.y) : pk2(wl.x, wl.y)));
+                for (int e = 0; e < 4; ++e) split_bf16(mul2(bf2_to_f2(wb[kt][e]), (e & 1) ? pk2(wh.x, wh.y) : pk2(wl.x, wl.y)), wb[kt][e], wc[kt][e]);
             }
 #pragma unroll
             for (int m = 0; m < MT; ++m) {
 #pragma unroll
                 for (int kt = 0; kt < 2; ++kt) ldmatrix_x4_t(xa[m][kt][0], xa[m][kt][1], xa[m][kt][2], xa[m][kt][3], (xo ^ (32 * m)) + kt * 16 * RB);
-#pragma unroll
-                for (int n = 0; n < 2; ++n) {
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) st[m][n][e] = 0.f;
-#pragma unroll
-                    for (int kt = 0; kt < 2; ++kt) mma(st[m][n], xa[m][kt], wb[kt][2 * n], wb[kt][2 * n + 1]);
-                }
             }
             __syncwarp();                                                         // x' is in registers: St goes over it
 #pragma unroll
             for (int m = 0; m < MT; ++m)
 #pragma unroll
-                for (int n = 0; n < 2; ++n)
-                    asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(stp + (2 * m + n) * 512), "f"(st[m][n][0]), "f"(st[m][n][1]), "f"(st[m][n][2]), "f"(st[m][n][3]) : "memory");
+                for (int n = 0; n < 2; ++n) {
+                    float st[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+                    for (int kt = 0; kt < 2; ++kt) mma(st, xa[m][kt], wc[kt][2 * n], wc[kt][2 * n + 1]);
+#pragma unroll
+                    for (int kt = 0; kt < 2; ++kt) mma(st, xa[m][kt], wb[kt][2 * n], wb[kt][2 * n + 1]);
+                    asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(stp + (2 * m + n) * 512), "f"(st[0]), "f"(st[1]), "f"(st[2]), "f"(st[3]) : "memory");
+                }
             __syncwarp();
             if (lane == 0) raise_flag(smem_u32(&sh->ready[warp]), k + 1);
         }
@@ -332,7 +351,6 @@ __device__ __forceinline__ void chain(const CUtensorMap &map_x, const CUtensorMa
                         float e0 = li - lp[j].x, e1 = li - lp[j].y;
                         if (j == i) { e0 = 2 * qc <= gr ? e0 : -INFINITY; e1 = 2 * qc + 1 <= gr ? e1 : -INFINITY; }      // 2^-inf = 0 after i
                         float v0 = s[j][2 * hf] * ex2f(e0), v1 = s[j][2 * hf + 1] * ex2f(e1);
-                        if (j == i) { v0 += 2 * qc == gr ? Dh : 0.f; v1 += 2 * qc + 1 == gr ? Dh : 0.f; }
                         wf[i][j] = pack_bf16(v0, v1);
                     }
                 }
@@ -340,10 +358,12 @@ __device__ __forceinline__ void chain(const CUtensorMap &map_x, const CUtensorMa
         }
         // ---- the state before the tile: A operand of Yb
         if (!__all_sync(0xffffffffu, flag_reached(smem_u32(&sh->done), k + 1, abort_flag, status))) break;
-        uint32_t hb[MT][4];
+        uint32_t hb[MT][PARTS][4];
 #pragma unroll
         for (int m = 0; m < MT; ++m)
-            asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(hb[m][0]), "=r"(hb[m][1]), "=r"(hb[m][2]), "=r"(hb[m][3]) : "r"(stp + m * 512));
+#pragma unroll
+            for (int u = 0; u < PARTS; ++u)
+                asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(hb[m][u][0]), "=r"(hb[m][u][1]), "=r"(hb[m][u][2]), "=r"(hb[m][u][3]) : "r"(stp + (PARTS * m + u) * 512));
         fence_proxy_async();
         __syncwarp();                                                             // all but z has been read: the next tile's may come
         if (lane == 0 && k + nt < nsub) {
@@ -366,11 +386,16 @@ __device__ __forceinline__ void chain(const CUtensorMap &map_x, const CUtensorMa
 #pragma unroll
                 for (int e = 0; e < 4; ++e) y[i][e] = 0.f;
 #pragma unroll
-            for (int i = 0; i < 4; ++i) mma(y[i], hb[m], cf[i >> 1][i & 1], cf[i >> 1][2 + (i & 1)]);
+            for (int u = PARTS - 1; u >= 0; --u)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) mma(y[i], hb[m][u], cf[i >> 1][i & 1], cf[i >> 1][2 + (i & 1)]);
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                upk2(mul2(ei[i], pk2(y[i][0], y[i][1])), y[i][0], y[i][1]);
-                upk2(mul2(ei[i], pk2(y[i][2], y[i][3])), y[i][2], y[i][3]);
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {                                     // (the A operand's words are laid out as the accumulators)
+                    const f32x2 v = pk2(y[i][2 * e], y[i][2 * e + 1]);
+                    upk2(SKIP ? fma2(ei[i], v, mul2(Dh, bf2_to_f2(xa[m][i >> 1][(i & 1) * 2 + e]))) : mul2(ei[i], v), y[i][2 * e], y[i][2 * e + 1]);
+                }
             }
 #pragma unroll
             for (int i = 0; i < 4; ++i) mma(y[i], xa[m][0], wf[i][0], i > 0 ? wf[i][1] : 0u);
@@ -420,7 +445,7 @@ __device__ __forceinline__ void chain(const CUtensorMap &map_x, const CUtensorMa
     if (lane == 0) bulk_wait0();
 }
 
-template <int MT>
+template <int MT, bool SKIP>
 __global__ void __launch_bounds__(Tile<MT>::WARPS * 32, 1)
 narrow_scan_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_z, const __grid_constant__ CUtensorMap map_bc,
                    const __grid_constant__ CUtensorMap map_g, const __grid_constant__ SsdArgs a, const float *__restrict__ dl, int ndir, int dir0, int *status) {
@@ -447,8 +472,8 @@ narrow_scan_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
     __syncthreads();
     pdl_wait();
     pdl_trigger();
-    if (dir == 1) chain<MT, true>(map_x, map_z, map_bc, map_g, a, dl, slots, sh, grp, b, status);
-    else chain<MT, false>(map_x, map_z, map_bc, map_g, a, dl, slots, sh, grp, b, status);
+    if (dir == 1) chain<MT, SKIP, true>(map_x, map_z, map_bc, map_g, a, dl, slots, sh, grp, b, status);
+    else chain<MT, SKIP, false>(map_x, map_z, map_bc, map_g, a, dl, slots, sh, grp, b, status);
 }
 
 // B' and C' (conv + SiLU) as bf16 rows [B' 16 | C' 16], and the decays of every sub-chunk.  A CTA takes the 128 rows of a chunk (a thread: a channel pair over four rows) or the decays of 64 heads
@@ -522,10 +547,11 @@ cudaError_t launch(const SsdArgs &a, __nv_bfloat16 *bc, float *dl, int ndir, int
     const int per_sm = chains > (int64_t)PER_SM * sms ? PER_SM : (int)((chains + sms - 1) / sms);
     int nw = T::WARPS / per_sm;
     if (nw > nsub + 1) nw = nsub + 1;
-    e = cudaFuncSetAttribute(narrow_scan_kernel<MT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes<MT>(T::WARPS));
+    auto kern = (a.flags & DM_FLAG_D_SKIP) ? narrow_scan_kernel<MT, true> : narrow_scan_kernel<MT, false>;
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes<MT>(T::WARPS));
     if (e != cudaSuccess) return e;
     if (per_sm > 1) chain_spread((int64_t)pgrid.x * pgrid.y * pgrid.z, chains, sms);      // several CTAs to an SM, but not packed
-    return launch_chain(narrow_scan_kernel<MT>, (unsigned)chains, 32 * nw, smem_bytes<MT>(nw), s, 0, mx, mz, mb, mg, a, dl, ndir, dir0, status);
+    return launch_chain(kern, (unsigned)chains, 32 * nw, smem_bytes<MT>(nw), s, 0, mx, mz, mb, mg, a, dl, ndir, dir0, status);
 }
 
 }  // namespace
@@ -533,7 +559,8 @@ cudaError_t launch(const SsdArgs &a, __nv_bfloat16 *bc, float *dl, int ndir, int
 bool scan_narrow_shape(int headdim, int d_state) { return d_state == NS && headdim % 32 == 0; }
 // Few chains: heads of 64 are split, so that twice as many SMs have one.  Everywhere else the whole head is the better tile, since mask, decays, B' and C' serve twice the channels (32 heads, half heads / whole:
 // 2 x 4096 218 / 211 us a layer, 4 x 4096 412 / 399).
-int scan_narrow_width(int headdim, int64_t heads) { return headdim == 64 && 2 * heads > sm_count() ? 64 : 32; }
+// Without the D skip the state's copy has two parts and a whole head's registers spill: halves always (2 x 2048 131 / 134 us, 4 x 4096 436 / 446, 5 x 4096 572 / 604).
+int scan_narrow_width(int headdim, int64_t heads, bool skip) { return headdim == 64 && skip && 2 * heads > sm_count() ? 64 : 32; }
 
 cudaError_t scan_narrow(const ssd::SsdArgs &a, __nv_bfloat16 *bc, float *dl, int ndir, int dir0, int width, cudaStream_t s) {
     return width == 64 ? launch<4>(a, bc, dl, ndir, dir0, s) : launch<2>(a, bc, dl, ndir, dir0, s);

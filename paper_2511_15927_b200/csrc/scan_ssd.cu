@@ -1215,7 +1215,7 @@ bool block_mode(const ScanArgs &a) { return a.chunk == QB || (a.chunk == 0 && a.
 bool narrow_mode(const ScanArgs &a) { return a.chunk == 0 && !block_mode(a) && scan_narrow_shape(a.P, a.N); }
 // Halves of a head each leave a sum of squares; whole heads leave two as well, wherever halves could have been the choice
 bool narrow_halves(const ScanArgs &a) { return a.ssq_room >= a.d_inner / 32; }
-int narrow_width(const ScanArgs &a) { return narrow_halves(a) ? scan_narrow_width(a.P, (int64_t)a.H * a.B * (a.dir_mask == DM_DIR_BOTH ? 2 : 1)) : a.P; }
+int narrow_width(const ScanArgs &a) { return narrow_halves(a) ? scan_narrow_width(a.P, (int64_t)a.H * a.B * (a.dir_mask == DM_DIR_BOTH ? 2 : 1), (a.flags & DM_FLAG_D_SKIP) != 0) : a.P; }
 
 struct Scratch {
     size_t bp, cp, da, sb, sy, total;

@@ -49,16 +49,22 @@ def test_forward_and_state(G, B, H, P, L, k, flags, dirs):
     _check(G, c_g, c_o)
 
 
-@pytest.mark.parametrize("P,L", [(64, 500), (32, 333)])
-def test_error_is_that_of_the_128_token_kernel(G, P, L):
-    """Both kernels round x', W, the weighted operand of the state update and the state's copy to bf16 and sum in fp32: their errors are of one size.  A tenth more is allowed for the shorter chunk,
-    which passes more of the history through the state's copy and less through W."""
-    shape = I.MixerShape(2, L, P * 8 // 2, 2, 16, 4, 8)
-    wf, wr = I.make_mixer_weights(shape, 9, I.BF16, perturb=True)
-    x = I.make_activations(shape, 9, I.BF16)
-    want = O.bimamba_forward(x, wf, wr, **G.oracle_kwargs(shape))
-    e = [G.rel_l2(G.run_forward(shape, I.BF16, wf, wr, x, chunk=c), want) for c in (0, 128)]
-    assert e[0] <= 1.1 * e[1], e
+@pytest.mark.parametrize("d,P,L,flags", [(512, 64, 300, 7), (512, 32, 300, 7), (512, 64, 500, 3), (1024, 64, 1000, 3), (512, 32, 300, 2), (768, 64, 96, 7)])
+def test_error_is_no_larger_than_that_of_the_128_token_kernel(G, d, P, L, flags):
+    """From a carried state, with and without the D skip and the norm, mean of three seeds.  The output: not larger.  The state: both kernels round B' and one factor of each term beside it once (x' here,
+    w x' there) and sum in fp32, so that their errors are two samples of one distribution; 6 % between them (they came out 0.93 to 1.03 apart; rounding w B' a second time gave 1.11 to 1.14)."""
+    e = []
+    for seed in range(3):
+        shape = I.MixerShape(1, L, d, 2, 16, 4, 2 * d // P)
+        wf, wr = I.make_mixer_weights(shape, seed, I.BF16, perturb=True)
+        x = I.make_activations(shape, seed, I.BF16)
+        ssm_in, conv_in = I.make_states(shape, seed, I.BF16)
+        y_o, s_o, _ = O.bimamba_block_step(x, wf, wr, ssm_state_in=ssm_in, conv_state_in=conv_in, **G.oracle_kwargs(shape, flags))
+        for c in (0, 128):
+            y, s, _ = G.run_block_step(shape, I.BF16, wf, wr, x, ssm_in, conv_in, flags=flags, chunk=c)
+            e.append((G.rel_l2(y, y_o), G.rel_l2(s, s_o)))
+    narrow, wide = np.mean(e[0::2], axis=0), np.mean(e[1::2], axis=0)
+    assert narrow[0] <= wide[0] and narrow[1] <= 1.06 * wide[1], (narrow, wide)
 
 
 def test_causality(G):
@@ -84,11 +90,11 @@ def test_a_row_does_not_depend_on_the_rows_beside_it(G):
     np.testing.assert_array_equal(G.run_forward_host(shape, I.BF16, wf, wr, x), whole)
 
 
-@pytest.mark.parametrize("B", [2, 3])
-def test_no_room_for_sums_of_half_heads(G, B):
+@pytest.mark.parametrize("B,flags", [(2, 7), (3, 7), (3, 3)])
+def test_no_room_for_sums_of_half_heads(G, B, flags):
     """expand 32: the sums of squares of 32 channels each have no place in the workspace, so heads of 64 stay whole at any batch (64 and 96 chains) and leave one sum each."""
     shape = I.MixerShape(B, 200, 32, 32, 16, 4, 16)
     assert shape.headdim == 64
     wf, wr = I.make_mixer_weights(shape, 7, I.BF16, perturb=True)
     x = I.make_activations(shape, 7, I.BF16)
-    _check(G, G.run_forward(shape, I.BF16, wf, wr, x), O.bimamba_forward(x, wf, wr, **G.oracle_kwargs(shape)))
+    _check(G, G.run_forward(shape, I.BF16, wf, wr, x, flags=flags), O.bimamba_forward(x, wf, wr, **G.oracle_kwargs(shape, flags)))
