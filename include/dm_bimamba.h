@@ -365,7 +365,9 @@ int dm_selftest_wait_timeout(uint32_t limit_us, uint64_t *out, void *cuda_stream
  * whose scan can do its prep work inside the scan launch (the tensor-core kernel, fewer scan CTAs than SMs, more than eight chunks; outside the test one
  * sequence of 32 chunks or more does) launches the scan without the CTAs of that role: the flags its load warps wait for from the ninth chunk on are never raised,
  * the waits run out after their regular limit (2 s), and every role of every CTA has to leave through the abort path -- loads in
- * flight waited for, TMEM freed.  A call on the sequential scan (fp32, or d_state 256) of more than two chunks leaves out the
+ * flight waited for, TMEM freed.  On the scan of narrow states (bf16, d_state 16, more than 64 tokens, chunk 0) every CTA's
+ * state warp waits for a flag that is never raised at the third tile of 32 tokens, and the tile warps for the states from
+ * there on.  A call on the sequential scan (fp32, or d_state 256) of more than two chunks leaves out the
  * copies of every CTA's third chunk, with the same consequences.  The call itself returns DM_OK; dm_check then reports
  * DM_ERR_TIMEOUT; y is unspecified.  Nothing faults or hangs.  Process-wide; switch it off again. */
 int dm_selftest_withhold_prep(int on);

@@ -15,6 +15,8 @@
 // Bound by the shared-memory pipe (60 % of its wavefronts on average, 70 % on an SM with two chains) and by latencies at 20 warps an SM: 1500 instructions per warp and tile of 64 channels, an issue
 // slot used half of the time.  Scan alone, 32 heads of 64: 4 x 4096 tokens 190 us on the tcgen05 kernel, 113 here (2.9 TB/s of the rows' traffic where a copy reaches 6.5); 1 x 32768 650 -> 300, 8 x 512
 // 70 -> 38 behind the prep launch; a layer of 4 x 4096 475 -> 402 us.  With the state handed from tile warp to tile warp a step of the chain took 800 to 1800 clocks and 1 x 32768 436 us; through mbarriers 515.
+#include <climits>
+
 #include "ssd_common.cuh"
 
 namespace dm {
@@ -120,9 +122,10 @@ __device__ __forceinline__ float token_sum(const f32x2 (&sq)[4], int lane) {
     return (b2 ? t[1] : t[0]) + __shfl_xor_sync(0xffffffffu, b2 ? t[0] : t[1], 4);
 }
 
-// The state warp: 16 x 16 tiles [channels][states] in the accumulators' layout.  PARTS: bf16 numbers to an entry of the state's copy
+// The state warp: 16 x 16 tiles [channels][states] in the accumulators' layout.  PARTS: bf16 numbers to an entry of the state's copy.
+// held: tile at which it waits for a flag that nobody raises (self-test), or -1
 template <int MT, int PARTS>
-__device__ __forceinline__ void state_role(const uint8_t *slots, Shared<MT> *sh, int nt, int nsub, const float *h_in, float *h_out, int *status) {
+__device__ __forceinline__ void state_role(const uint8_t *slots, Shared<MT> *sh, int nt, int nsub, const float *h_in, float *h_out, int held, int *status) {
     using T = Tile<MT>;
     const int lane = threadIdx.x & 31, gr = lane >> 2, qc = lane & 3;
     volatile int *abort_flag = &sh->abort;
@@ -137,7 +140,7 @@ __device__ __forceinline__ void state_role(const uint8_t *slots, Shared<MT> *sh,
     int w = 0;
     for (int k = 0; k < nsub; ++k) {
         const uint32_t slot = sb + w * T::SLOT;
-        if (!__all_sync(0xffffffffu, flag_reached(ready + 4 * w, k + 1, abort_flag, status))) return;
+        if (!__all_sync(0xffffffffu, flag_reached(ready + 4 * w, k == held ? INT_MAX : k + 1, abort_flag, status))) return;
         float4 st[MT][2];
 #pragma unroll
         for (int m = 0; m < MT; ++m)
@@ -183,7 +186,7 @@ __device__ __forceinline__ void state_role(const uint8_t *slots, Shared<MT> *sh,
 // through its mask), so that the copy has two parts there (6 to 8 % of a layer's time).  With the skip, D x' is added in fp32 instead of in W, and y is 9 % more accurate than that kernel's.
 template <int MT, bool SKIP, bool REV>
 __device__ __forceinline__ void chain(const CUtensorMap &map_x, const CUtensorMap &map_z, const CUtensorMap &map_bc, const CUtensorMap &map_g, const SsdArgs &a,
-                                      const float *__restrict__ dl, uint8_t *slots, Shared<MT> *sh, int grp, int b, int *status) {
+                                      const float *__restrict__ dl, uint8_t *slots, Shared<MT> *sh, int grp, int b, int held, int *status) {
     using T = Tile<MT>;
     constexpr int CW = T::CW, RB = T::RB, PARTS = SKIP ? 1 : 2;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, gr = lane >> 2, qc = lane & 3, nt = (blockDim.x >> 5) - 1;      // nt: tile warps
@@ -197,7 +200,7 @@ __device__ __forceinline__ void chain(const CUtensorMap &map_x, const CUtensorMa
     const f32x2 Dh = pk2(D1, D1);
     if (warp == nt) {
         const int64_t state0 = (((int64_t)b * a.H + h) * a.Pr + ch0 % a.Pr) * NS;
-        state_role<MT, PARTS>(slots, sh, nt, nsub, !REV && a.ssm_in ? a.ssm_in + state0 : nullptr, !REV && a.ssm_out ? a.ssm_out + state0 : nullptr, status);
+        state_role<MT, PARTS>(slots, sh, nt, nsub, !REV && a.ssm_in ? a.ssm_in + state0 : nullptr, !REV && a.ssm_out ? a.ssm_out + state0 : nullptr, held, status);
         return;
     }
 
@@ -448,7 +451,7 @@ __device__ __forceinline__ void chain(const CUtensorMap &map_x, const CUtensorMa
 template <int MT, bool SKIP>
 __global__ void __launch_bounds__(Tile<MT>::WARPS * 32, 1)
 narrow_scan_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_z, const __grid_constant__ CUtensorMap map_bc,
-                   const __grid_constant__ CUtensorMap map_g, const __grid_constant__ SsdArgs a, const float *__restrict__ dl, int ndir, int dir0, int *status) {
+                   const __grid_constant__ CUtensorMap map_g, const __grid_constant__ SsdArgs a, const float *__restrict__ dl, int ndir, int dir0, int held, int *status) {
     using T = Tile<MT>;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *slots = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
@@ -472,8 +475,8 @@ narrow_scan_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
     __syncthreads();
     pdl_wait();
     pdl_trigger();
-    if (dir == 1) chain<MT, SKIP, true>(map_x, map_z, map_bc, map_g, a, dl, slots, sh, grp, b, status);
-    else chain<MT, SKIP, false>(map_x, map_z, map_bc, map_g, a, dl, slots, sh, grp, b, status);
+    if (dir == 1) chain<MT, SKIP, true>(map_x, map_z, map_bc, map_g, a, dl, slots, sh, grp, b, held, status);
+    else chain<MT, SKIP, false>(map_x, map_z, map_bc, map_g, a, dl, slots, sh, grp, b, held, status);
 }
 
 // B' and C' (conv + SiLU) as bf16 rows [B' 16 | C' 16], and the decays of every sub-chunk.  A CTA takes the 128 rows of a chunk (a thread: a channel pair over four rows) or the decays of 64 heads
@@ -551,7 +554,7 @@ cudaError_t launch(const SsdArgs &a, __nv_bfloat16 *bc, float *dl, int ndir, int
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes<MT>(T::WARPS));
     if (e != cudaSuccess) return e;
     if (per_sm > 1) chain_spread((int64_t)pgrid.x * pgrid.y * pgrid.z, chains, sms);      // several CTAs to an SM, but not packed
-    return launch_chain(kern, (unsigned)chains, 32 * nw, smem_bytes<MT>(nw), s, 0, mx, mz, mb, mg, a, dl, ndir, dir0, status);
+    return launch_chain(kern, (unsigned)chains, 32 * nw, smem_bytes<MT>(nw), s, 0, mx, mz, mb, mg, a, dl, ndir, dir0, scan_selftest_withheld() ? 2 : -1, status);
 }
 
 }  // namespace

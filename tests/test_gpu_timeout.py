@@ -93,6 +93,34 @@ def test_the_sequential_scan_leaves_when_a_copy_never_comes(G):
         assert G.rel_l2(got, O.bimamba_forward(x, wf, wr, **G.oracle_kwargs(shape))) <= (1e-4 if dtype == I.F32 else 1e-2)
 
 
+@pytest.mark.parametrize("B", [2, 5])
+def test_the_narrow_scan_leaves_when_a_flag_is_never_raised(G, B):
+    """The scan of narrow states, heads in halves (B = 2) and whole (B = 5): the state warp's wait for the third tile is for a flag that nobody raises; it and the tile warps' waits for
+    the states from there on run out (2 s), loads in flight are waited for and every warp leaves.  DM_ERR_TIMEOUT once, and the same call is correct again afterwards."""
+    import time
+    import torch
+    from oracle import bimamba_oracle as O
+    from paper_2511_15927_b200 import binding as dm
+    shape = I.MixerShape(B, 300, 256, 2, 16, 4, 8)
+    wf, wr = I.make_mixer_weights(shape, 6, I.BF16)
+    x = I.make_activations(shape, 6, I.BF16)
+    st = torch.cuda.current_stream().cuda_stream
+    dm.dm_check(st)
+    dm.dm_selftest_withhold_prep(True)
+    try:
+        t0 = time.time()
+        with pytest.raises(dm.DmError) as e:
+            G.run_forward(shape, I.BF16, wf, wr, x)
+        waited = time.time() - t0
+    finally:
+        dm.dm_selftest_withhold_prep(False)
+    assert e.value.status == dm.DM_ERR_TIMEOUT
+    assert 1.5 < waited < 20.0
+    dm.dm_check(st)
+    got = G.run_forward(shape, I.BF16, wf, wr, x)
+    assert G.rel_l2(got, O.bimamba_forward(x, wf, wr, **G.oracle_kwargs(shape))) <= 1e-2
+
+
 def test_selftest_argument_checks(G):
     from paper_2511_15927_b200 import binding as dm
     before = dm.dm_kernel_launch_count()
