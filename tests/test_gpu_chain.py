@@ -94,11 +94,15 @@ CASES = {
     "mixer_long": lambda G: _mixer(G, I.BF16, I.MixerShape(1, 4100, 128, 2, 128, 4, 4)),               # prep partly inside the scan launch
     "mixer_1k_pairs": lambda G: _mixer(G, I.BF16, I.MixerShape(2, 700, 512, 2, 128, 4, 32)),
     "mixer_chunk32": lambda G: _mixer(G, I.BF16, I.MixerShape(1, 2100, 128, 2, 16, 4, 4), chunk=32),
+    "mixer_narrow": lambda G: _mixer(G, I.BF16, I.MixerShape(2, 300, 256, 2, 16, 4, 8), state=True),       # d_state 16: chains of half heads, whole ones, two to an SM
+    "mixer_narrow_whole": lambda G: _mixer(G, I.BF16, I.MixerShape(5, 300, 256, 2, 16, 4, 8), state=True),
+    "mixer_narrow_two": lambda G: _mixer(G, I.BF16, I.MixerShape(10, 300, 256, 2, 16, 4, 8)),
     "mixer_tied": lambda G: _mixer(G, I.BF16, I.MixerShape(2, 200, 256, 2, 64, 4, 8), flags=15),
     "mixer_f32": lambda G: _mixer(G, I.F32, I.MixerShape(2, 300, 128, 2, 16, 4, 8), state=True),
     "block_32": lambda G: _mixer(G, I.BF16, I.MixerShape(4, 32, 512, 2, 128, 4, 16), state=True),
     "block_48": lambda G: _mixer(G, I.BF16, I.MixerShape(4, 48, 256, 2, 128, 4, 16), state=True),
     "stack": lambda G: _stack(G, "plain", I.MixerShape(2, 150, 256, 2, 32, 4, 8)),
+    "stack_narrow": lambda G: _stack(G, "plain", I.MixerShape(2, 150, 256, 2, 16, 4, 8)),
     "stack_few_rows": lambda G: _stack(G, "plain", I.MixerShape(1, 100, 256, 2, 32, 4, 8), V=38016),     # the vocabulary's tiles taken in turn
     "stack_cond": lambda G: _stack(G, "cond", I.MixerShape(2, 150, 256, 2, 32, 4, 8)),
     "hybrid_block": lambda G: _stack(G, "hybrid_block", I.MixerShape(3, 32, 256, 2, 64, 4, 8)),

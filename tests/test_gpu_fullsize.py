@@ -82,7 +82,7 @@ def test_cfg3_32k_prefix_and_suffix_independence(G):
 
 
 def test_cfg2_layer_sampled_row_against_the_oracle(G):
-    """d_state 16 (zero-padded to 128 on the tensor-core scan) at B=4, L=4096, d_model 1024."""
+    """d_state 16 (the scan of narrow states, two chains to an SM) at B=4, L=4096, d_model 1024."""
     shape, dtype = I.CONFIGS["cfg2_layer"]
     wf, wr = I.make_mixer_weights(shape, 0, dtype)
     x = I.make_activations(shape, 0, dtype)

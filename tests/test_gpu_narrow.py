@@ -24,12 +24,16 @@ def _check(G, got, want):
     assert G.max_abs(got, want) <= BF16_ABS, G.max_abs(got, want)
 
 
-# (batch, heads, headdim, length, conv width, flags, directions).  Chains of half heads with 20 warps where heads are few (640 tokens a round), of whole heads with 16 warps (512 tokens) from 75
-# heads of all sequences and directions, with 8, 5 and 4 warps from 149, 297 and 445; (40, 16): more chains than are resident
+# (batch, heads, headdim, length, conv width, flags, directions).  A chain's tile warps take 32 tokens each in turn: 19 warps (608 tokens a round) for up to 148 chains, 9 (288), 5 (160) and 4 (128) from
+# 149, 297 and 445.  Heads of 64 are chains of half a head each for up to 74 heads of all sequences and directions, and without the D skip (flag 4), and one chain elsewhere.  (40, 16): more chains
+# than are resident
 @pytest.mark.parametrize("B,H,P,L,k,flags,dirs", [
     (1, 2, 64, 65, 4, 7, 3), (2, 8, 64, 96, 4, 7, 3), (2, 8, 32, 97, 4, 7, 3), (1, 8, 64, 128, 4, 7, 3), (3, 8, 32, 129, 3, 7, 3), (1, 16, 32, 159, 2, 6, 3),
     (2, 8, 64, 161, 4, 5, 1), (2, 8, 64, 255, 4, 3, 2), (1, 8, 64, 640, 4, 7, 3), (1, 8, 64, 641, 4, 7, 3), (2, 24, 64, 513, 4, 7, 3), (4, 24, 64, 225, 4, 7, 3), (10, 16, 64, 161, 3, 7, 3),
-    (40, 16, 64, 130, 4, 7, 3), (1, 4, 64, 1301, 4, 0, 3), (2, 72, 64, 100, 4, 7, 3)])
+    (40, 16, 64, 130, 4, 7, 3), (1, 4, 64, 1301, 4, 0, 3), (2, 72, 64, 100, 4, 7, 3),
+    (1, 8, 64, 608, 4, 7, 3), (1, 8, 64, 609, 4, 7, 3), (5, 8, 64, 608, 4, 7, 3), (5, 8, 64, 609, 4, 7, 3), (5, 8, 64, 641, 2, 6, 3), (4, 24, 64, 288, 4, 7, 3), (4, 24, 64, 289, 4, 7, 3),
+    (4, 24, 64, 321, 3, 7, 3), (10, 16, 64, 160, 4, 7, 3), (6, 16, 32, 289, 4, 7, 3), (2, 24, 64, 321, 4, 3, 3), (2, 3, 64, 100, 4, 7, 3), (3, 5, 64, 193, 4, 7, 3), (2, 3, 32, 97, 4, 7, 3),
+    (1, 5, 32, 66, 3, 5, 3), (26, 3, 64, 72, 4, 7, 3)])
 def test_forward_and_state(G, B, H, P, L, k, flags, dirs):
     shape = I.MixerShape(B, L, P * H // 2, 2, 16, k, H)
     wf, wr = I.make_mixer_weights(shape, 80 + L, I.BF16, perturb=True)

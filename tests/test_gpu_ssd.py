@@ -91,29 +91,29 @@ def test_state_in_and_out(G):
     assert G.rel_l2(s2_, s_whole) <= 5e-3
 
 
-@pytest.mark.parametrize("N,H", [(16, 8), (32, 8), (64, 8)])
-def test_smaller_d_state_runs_zero_padded(G, N, H):
-    """d_state below 128 takes the same kernel with B', C' and the state zero-padded: parity of the output, and the
-    carried state in the model's own [B, H, P, d_state] layout, in and out."""
+@pytest.mark.parametrize("N,H,chunk", [(16, 8, 0), (16, 8, 128), (32, 8, 0), (64, 8, 0)])
+def test_smaller_d_state_runs_zero_padded(G, N, H, chunk):
+    """d_state below 128 takes the same kernel with B', C' and the state zero-padded (16: with chunk = 128, its default is a
+    kernel of its own): parity of the output, and the carried state in the model's own [B, H, P, d_state] layout, in and out."""
     shape = I.MixerShape(2, 300, 32 * H, 2, N, 4, H)
     assert shape.d_in_proj % 8 == 0                         # 16-byte rows: the tensor-core path takes the shape
     wf, wr = I.make_mixer_weights(shape, 20 + N, I.BF16, perturb=True)
     x = I.make_activations(shape, 20 + N, I.BF16)
     kw = G.oracle_kwargs(shape)
-    _check(G, G.run_forward(shape, I.BF16, wf, wr, x), O.bimamba_forward(x, wf, wr, **kw))
+    _check(G, G.run_forward(shape, I.BF16, wf, wr, x, chunk=chunk), O.bimamba_forward(x, wf, wr, **kw))
     ssm_in, conv_in = I.make_states(shape, 20 + N, I.BF16)
     y_o, s_o, c_o = O.bimamba_block_step(x, wf, wr, ssm_state_in=ssm_in, conv_state_in=conv_in, **kw)
-    y_g, s_g, c_g = G.run_block_step(shape, I.BF16, wf, wr, x, ssm_in, conv_in)
+    y_g, s_g, c_g = G.run_block_step(shape, I.BF16, wf, wr, x, ssm_in, conv_in, chunk=chunk)
     assert s_g.shape == s_o.shape == (2, H, 64, N)
     _check(G, y_g, y_o)
     _check(G, s_g, s_o)
     _check(G, c_g, c_o)
 
 
-@pytest.mark.parametrize("N", [128, 16])
-def test_half_width_heads_run_with_padded_channels(G, N):
-    """headdim 32 (the paper's 1.3B shape: 120 heads of 32, App. A.1) takes the same kernel: a CTA loads 64 channels, of
-    which the second half (the next head's) is padding that never leaves it.  Parity of the output, the last head
+@pytest.mark.parametrize("N,chunk", [(128, 0), (16, 0), (16, 128)])
+def test_half_width_heads_run_with_padded_channels(G, N, chunk):
+    """headdim 32 (the paper's 1.3B shape: 120 heads of 32, App. A.1) takes the same kernel (d_state 16: with chunk = 128): a
+    CTA has two heads, or, where their number is odd, loads 64 channels, of which the second half (the next head's) is padding that never leaves it.  Parity of the output, the last head
     included, and of the carried state in the model's [B, H, 32, d_state] layout."""
     H = 8
     shape = I.MixerShape(2, 300, 128, 2, N, 4, H)           # d_inner 256 = 8 heads of 32
@@ -122,10 +122,10 @@ def test_half_width_heads_run_with_padded_channels(G, N):
     x = I.make_activations(shape, 40 + N, I.BF16)
     kw = G.oracle_kwargs(shape)
     for flags in (7, 6):                                    # with and without the gated norm (its sum of squares covers 32 channels)
-        _check(G, G.run_forward(shape, I.BF16, wf, wr, x, flags=flags), O.bimamba_forward(x, wf, wr, **G.oracle_kwargs(shape, flags)))
+        _check(G, G.run_forward(shape, I.BF16, wf, wr, x, flags=flags, chunk=chunk), O.bimamba_forward(x, wf, wr, **G.oracle_kwargs(shape, flags)))
     ssm_in, conv_in = I.make_states(shape, 40 + N, I.BF16)
     y_o, s_o, c_o = O.bimamba_block_step(x, wf, wr, ssm_state_in=ssm_in, conv_state_in=conv_in, **kw)
-    y_g, s_g, c_g = G.run_block_step(shape, I.BF16, wf, wr, x, ssm_in, conv_in)
+    y_g, s_g, c_g = G.run_block_step(shape, I.BF16, wf, wr, x, ssm_in, conv_in, chunk=chunk)
     assert s_g.shape == s_o.shape == (2, H, 32, N)
     _check(G, y_g, y_o)
     _check(G, s_g, s_o)
