@@ -138,9 +138,10 @@ __device__ __forceinline__ void state_role(const uint8_t *slots, Shared<MT> *sh,
 #pragma unroll
             for (int e = 0; e < 4; ++e) h[m][n][e] = h_in ? h_in[(16 * m + gr + (e >> 1) * 8) * NS + 8 * n + 2 * qc + (e & 1)] : 0.f;
     int w = 0;
-    for (int k = 0; k < nsub; ++k) {
+    const int last = held < 0 ? nsub : min(held, nsub);                          // (asked for in the loop, the chain's serial part, `held` cost 5 % of the scan: 1 x 32768 tokens 375 / 393 us)
+    for (int k = 0; k < last; ++k) {
         const uint32_t slot = sb + w * T::SLOT;
-        if (!__all_sync(0xffffffffu, flag_reached(ready + 4 * w, k == held ? INT_MAX : k + 1, abort_flag, status))) return;
+        if (!__all_sync(0xffffffffu, flag_reached(ready + 4 * w, k + 1, abort_flag, status))) return;
         float4 st[MT][2];
 #pragma unroll
         for (int m = 0; m < MT; ++m)
@@ -172,6 +173,7 @@ __device__ __forceinline__ void state_role(const uint8_t *slots, Shared<MT> *sh,
             }
         if (++w == nt) w = 0;
     }
+    if (last < nsub) { flag_reached(done, INT_MAX, abort_flag, status); return; }
     if (h_out) {
 #pragma unroll
         for (int m = 0; m < MT; ++m)
@@ -183,12 +185,13 @@ __device__ __forceinline__ void state_role(const uint8_t *slots, Shared<MT> *sh,
 }
 
 // The state's copy is bf16, of which the history of every tile is read: without the D skip beside it that made y up to 1 % less accurate than the 128-token kernel's (which takes more of the history
-// through its mask), so that the copy has two parts there (6 to 8 % of a layer's time).  With the skip, D x' is added in fp32 instead of in W, and y is 9 % more accurate than that kernel's.
-template <int MT, bool SKIP, bool REV>
+// through its mask), so that the copy has two parts there (6 to 8 % of a layer's time).  With the skip, D x' is added in fp32 instead of in W, for which the scan takes the same time (5 x 4096 tokens of 32
+// heads: 5 % more), and y is 9 % more accurate than that kernel's.
+template <int MT, int PARTS, bool REV>
 __device__ __forceinline__ void chain(const CUtensorMap &map_x, const CUtensorMap &map_z, const CUtensorMap &map_bc, const CUtensorMap &map_g, const SsdArgs &a,
                                       const float *__restrict__ dl, uint8_t *slots, Shared<MT> *sh, int grp, int b, int held, int *status) {
     using T = Tile<MT>;
-    constexpr int CW = T::CW, RB = T::RB, PARTS = SKIP ? 1 : 2;
+    constexpr int CW = T::CW, RB = T::RB;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, gr = lane >> 2, qc = lane & 3, nt = (blockDim.x >> 5) - 1;      // nt: tile warps
     const int L = a.L, nsub = (L + QB - 1) / QB, seq = (REV ? a.B : 0) + b, zseq = a.zx_tied ? b : seq, ch0 = grp * CW, h = ch0 / a.Pr;
     volatile int *abort_flag = &sh->abort;
@@ -196,7 +199,7 @@ __device__ __forceinline__ void chain(const CUtensorMap &map_x, const CUtensorMa
     const uint32_t sb = smem_u32(slot), conv_w = smem_u32(&sh->conv[0][0]), stp = sb + T::ST + lane * 16;
     uint64_t *const bx = &sh->x[warp], *const bz = &sh->z[warp];
     const float *dl_head = dl + ((int64_t)seq * a.H + h) * 2 * a.Lp;
-    const float D1 = SKIP ? a.dir[REV ? 1 : 0].D[h] : 0.f;
+    const float D1 = (a.flags & DM_FLAG_D_SKIP) ? a.dir[REV ? 1 : 0].D[h] : 0.f;
     const f32x2 Dh = pk2(D1, D1);
     if (warp == nt) {
         const int64_t state0 = (((int64_t)b * a.H + h) * a.Pr + ch0 % a.Pr) * NS;
@@ -394,11 +397,10 @@ __device__ __forceinline__ void chain(const CUtensorMap &map_x, const CUtensorMa
                 for (int i = 0; i < 4; ++i) mma(y[i], hb[m][u], cf[i >> 1][i & 1], cf[i >> 1][2 + (i & 1)]);
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-#pragma unroll
-                for (int e = 0; e < 2; ++e) {                                     // (the A operand's words are laid out as the accumulators)
-                    const f32x2 v = pk2(y[i][2 * e], y[i][2 * e + 1]);
-                    upk2(SKIP ? fma2(ei[i], v, mul2(Dh, bf2_to_f2(xa[m][i >> 1][(i & 1) * 2 + e]))) : mul2(ei[i], v), y[i][2 * e], y[i][2 * e + 1]);
-                }
+                const uint32_t *xi = &xa[m][i >> 1][(i & 1) * 2];                 // (the A operand's words are laid out as the accumulators)
+                const f32x2 lo = pk2(y[i][0], y[i][1]), hi = pk2(y[i][2], y[i][3]);
+                upk2(PARTS == 1 ? fma2(ei[i], lo, mul2(Dh, bf2_to_f2(xi[0]))) : mul2(ei[i], lo), y[i][0], y[i][1]);
+                upk2(PARTS == 1 ? fma2(ei[i], hi, mul2(Dh, bf2_to_f2(xi[1]))) : mul2(ei[i], hi), y[i][2], y[i][3]);
             }
 #pragma unroll
             for (int i = 0; i < 4; ++i) mma(y[i], xa[m][0], wf[i][0], i > 0 ? wf[i][1] : 0u);
@@ -448,7 +450,7 @@ __device__ __forceinline__ void chain(const CUtensorMap &map_x, const CUtensorMa
     if (lane == 0) bulk_wait0();
 }
 
-template <int MT, bool SKIP>
+template <int MT, int PARTS>
 __global__ void __launch_bounds__(Tile<MT>::WARPS * 32, 1)
 narrow_scan_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_z, const __grid_constant__ CUtensorMap map_bc,
                    const __grid_constant__ CUtensorMap map_g, const __grid_constant__ SsdArgs a, const float *__restrict__ dl, int ndir, int dir0, int held, int *status) {
@@ -475,8 +477,8 @@ narrow_scan_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
     __syncthreads();
     pdl_wait();
     pdl_trigger();
-    if (dir == 1) chain<MT, SKIP, true>(map_x, map_z, map_bc, map_g, a, dl, slots, sh, grp, b, held, status);
-    else chain<MT, SKIP, false>(map_x, map_z, map_bc, map_g, a, dl, slots, sh, grp, b, held, status);
+    if (dir == 1) chain<MT, PARTS, true>(map_x, map_z, map_bc, map_g, a, dl, slots, sh, grp, b, held, status);
+    else chain<MT, PARTS, false>(map_x, map_z, map_bc, map_g, a, dl, slots, sh, grp, b, held, status);
 }
 
 // B' and C' (conv + SiLU) as bf16 rows [B' 16 | C' 16], and the decays of every sub-chunk.  A CTA takes the 128 rows of a chunk (a thread: a channel pair over four rows) or the decays of 64 heads
@@ -543,23 +545,24 @@ cudaError_t launch(const SsdArgs &a, __nv_bfloat16 *bc, float *dl, int ndir, int
     const dim3 pgrid(a.nch * (1 + (a.H + 63) / 64), a.B, ndir);
     cudaError_t e = launch_chain(narrow_prep_kernel, pgrid, PREP_THREADS, 0, s, 0, a, bc, dl, dir0);
     if (e != cudaSuccess) return e;
-    // as many warps to a chain as leave all chains resident, up to PER_SM of them to an SM.  Chains that share an SM are launched without overlap behind a prep grid that fills the GPU (chain_spread): 4 x 4096
-    // tokens of 32 heads 402 -> 399 us a layer; behind smaller grids the overlap is worth 3 us (8 x 512: 124 / 128).
+    // as many warps to a chain as leave all chains resident, up to PER_SM of them to an SM.  One to two chains to an SM are launched without overlap behind a prep grid that fills the GPU (chain_spread): 4 x 4096
+    // tokens of 32 heads 402 -> 399 us a layer; behind smaller grids the overlap is worth 3 us (8 x 512: 124 / 128).  With more chains every SM is filled either way: 2 % apart at most, in both directions
+    // (overlap / none: 5 x 4096 603 / 599, 8 x 2048 440 / 433, 4 x 1024 of 120 heads of 32 379 / 383).
     const int64_t chains = (int64_t)(a.d_inner / T::CW) * ndir * a.B;
     const int sms = sm_count();
     const int per_sm = chains > (int64_t)PER_SM * sms ? PER_SM : (int)((chains + sms - 1) / sms);
     int nw = T::WARPS / per_sm;
     if (nw > nsub + 1) nw = nsub + 1;
-    auto kern = (a.flags & DM_FLAG_D_SKIP) ? narrow_scan_kernel<MT, true> : narrow_scan_kernel<MT, false>;
+    auto kern = (a.flags & DM_FLAG_D_SKIP) ? narrow_scan_kernel<MT, 1> : narrow_scan_kernel<MT, 2>;
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes<MT>(T::WARPS));
     if (e != cudaSuccess) return e;
-    if (per_sm > 1) chain_spread((int64_t)pgrid.x * pgrid.y * pgrid.z, chains, sms);      // several CTAs to an SM, but not packed
+    if (per_sm == 2) chain_spread((int64_t)pgrid.x * pgrid.y * pgrid.z, chains, sms);      // several CTAs to an SM, but not packed
     return launch_chain(kern, (unsigned)chains, 32 * nw, smem_bytes<MT>(nw), s, 0, mx, mz, mb, mg, a, dl, ndir, dir0, scan_selftest_withheld() ? 2 : -1, status);
 }
 
 }  // namespace
 
-bool scan_narrow_shape(int headdim, int d_state) { return d_state == NS && headdim % 32 == 0; }
+bool scan_narrow_shape(int d_state) { return d_state == NS; }
 // Few chains: heads of 64 are split, so that twice as many SMs have one.  Everywhere else the whole head is the better tile, since mask, decays, B' and C' serve twice the channels (32 heads, half heads / whole:
 // 2 x 4096 218 / 211 us a layer, 4 x 4096 412 / 399).
 // Without the D skip the state's copy has two parts and a whole head's registers spill: halves always (2 x 2048 131 / 134 us, 4 x 4096 436 / 446, 5 x 4096 572 / 604).

@@ -1212,7 +1212,7 @@ constexpr int BLOCK_MAX_L = 2 * QB;       // sequences up to this length take th
 bool block_mode(const ScanArgs &a) { return a.chunk == QB || (a.chunk == 0 && a.L <= BLOCK_MAX_L); }
 
 // d_state 16, beyond the short blocks
-bool narrow_mode(const ScanArgs &a) { return a.chunk == 0 && !block_mode(a) && scan_narrow_shape(a.P, a.N); }
+bool narrow_mode(const ScanArgs &a) { return a.chunk == 0 && !block_mode(a) && scan_narrow_shape(a.N); }
 // Halves of a head each leave a sum of squares; whole heads leave two as well, wherever halves could have been the choice
 bool narrow_halves(const ScanArgs &a) { return a.ssq_room >= a.d_inner / 32; }
 int narrow_width(const ScanArgs &a) { return narrow_halves(a) ? scan_narrow_width(a.P, (int64_t)a.H * a.B * (a.dir_mask == DM_DIR_BOTH ? 2 : 1), (a.flags & DM_FLAG_D_SKIP) != 0) : a.P; }

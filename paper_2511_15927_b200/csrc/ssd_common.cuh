@@ -137,7 +137,7 @@ cudaError_t scan_step(const ssd::SsdArgs &a, int headdim, int ndir, int dir0, cu
 // Sequences of more than two sub-chunks with d_state 16, in chains of `width` channels (scan_narrow_width; heads: of all sequences and directions): see scan_narrow.cu.
 // bc: [2][B][L][32] bf16, dl: [2][B][H][Lp / 32][2][32] fp32 of scratch.  The sums of squares do not depend on the width, so that a row's result does not depend on how many others share the
 // call: a.ssq_parts is d_inner / 32, or H where heads are as wide as the chains.
-bool scan_narrow_shape(int headdim, int d_state);
+bool scan_narrow_shape(int d_state);
 int scan_narrow_width(int headdim, int64_t heads, bool skip);
 cudaError_t scan_narrow(const ssd::SsdArgs &a, __nv_bfloat16 *bc, float *dl, int ndir, int dir0, int width, cudaStream_t s);
 
