@@ -1,4 +1,4 @@
-// Fused conv + scan + gate for sequences of d_state 16: the identities of scan_ssd.cu over sub-chunks of 32 tokens, with every product on mma.sync tiles and every intermediate in registers.
+// Fused conv + scan + gate for sequences of d_state 16: the identities of scan_ssd.cu over sub-chunks of 32 tokens, with every product on mma.sync tiles and the intermediates in registers (34 words a thread of whole heads spill).
 // At d_state 16 the tcgen05 kernel's chunk of 128 tokens does eight times the state work the model has and a mask of 128 x 128 per 64 channels; at 32 tokens the mask is a fourth of that per
 // channel, the state of a head of 64 is 32 registers per lane, and one warp can carry a tile of 32 tokens x 64 (or 32) channels from its raw rows to its gated output, meeting other warps only
 // where it takes the state over.
@@ -12,9 +12,9 @@
 //              stmatrix.trans and a TMA store
 // Time order is a matter of row addresses (<- reads its rows backwards), so that the mask is the same for both directions.
 // The launch before (narrow_prep) leaves B' | C' as bf16 rows of 32 columns and the decays relative to each sub-chunk.
-// Bound by the shared-memory pipe (60 % of its wavefronts on average, 70 % on an SM with two chains) and by latencies at 20 warps an SM: 1500 instructions per warp and tile of 64 channels, an issue
-// slot used half of the time.  Scan alone, 32 heads of 64: 4 x 4096 tokens 190 us on the tcgen05 kernel, 113 here (2.9 TB/s of the rows' traffic where a copy reaches 6.5); 1 x 32768 650 -> 300, 8 x 512
-// 70 -> 38 behind the prep launch; a layer of 4 x 4096 475 -> 402 us.  With the state handed from tile warp to tile warp a step of the chain took 800 to 1800 clocks and 1 x 32768 436 us; through mbarriers 515.
+// Bound by the shared-memory pipe (54 % of its wavefronts on average, 65 % on an SM with two chains) and by latencies at 20 warps an SM: 1750 instructions per warp and tile of 64 channels, an issue
+// slot used half of the time.  Prep and scan, 32 heads of 64: 4 x 4096 tokens 196 us on the tcgen05 kernel, 142 here (2.9 TB/s of the rows' traffic where a copy reaches 6.5); 1 x 32768 736 -> 345, 8 x 512
+// 81 -> 49, 1 x 4096 99 -> 49.  With the state handed from tile warp to tile warp a step of the chain took 800 to 1800 clocks and the scan of 1 x 32768 436 us, where it took 300; through mbarriers 515.
 #include <climits>
 
 #include "ssd_common.cuh"
@@ -31,7 +31,7 @@ constexpr int PER_SM = 4;                    // CTAs per SM at most
 // Tiles of MT x 16 channels: rows of 64 or 128 bytes with the swizzle of that width (tiles aligned to eight rows)
 template <int MT> struct Tile {
     static constexpr int CW = 16 * MT, RB = 2 * CW;
-    static constexpr int WARPS = 20;                             // (16 of 128 registers: level; 24 of 80 for half heads: 8 % slower on one long sequence) resident on an SM, by registers: in CTAs of WARPS / 1 .. 4, one of them the state warp
+    static constexpr int WARPS = 20;                             // (16 of 128 registers: level, 32 x 128 tokens 6 % slower; 24 of 80 for half heads: 8 % slower on one long sequence) resident on an SM, by registers: in CTAs of WARPS / 1 .. 4, one of them the state warp
     static constexpr int QR = CW / 4, RG = 32 / QR, RPG = QB / RG;      // conv: lanes to a row (4 channels each), groups of rows, rows of a group
     // a warp's buffers
     static constexpr uint32_t X = 0, LAM = XR * RB, E = LAM + 256, Z = (E + 256 + 8 * RB - 1) / (8 * RB) * (8 * RB), BC = Z + QB * RB, SLOT = BC + QB * 64;
@@ -563,8 +563,9 @@ cudaError_t launch(const SsdArgs &a, __nv_bfloat16 *bc, float *dl, int ndir, int
 }  // namespace
 
 bool scan_narrow_shape(int d_state) { return d_state == NS; }
-// Few chains: heads of 64 are split, so that twice as many SMs have one.  Everywhere else the whole head is the better tile, since mask, decays, B' and C' serve twice the channels (32 heads, half heads / whole:
-// 2 x 4096 218 / 211 us a layer, 4 x 4096 412 / 399).
+// Few chains: heads of 64 are split, so that twice as many SMs have one.  Everywhere else the whole head is the better tile, since mask, decays, B' and C' serve twice the channels.  A layer with half heads /
+// whole ones, by heads of all sequences and directions: 64 1 x 1024 tokens 52 / 57 us, 1 x 4096 121 / 138; 72 65 / 69, 158 / 175; 76 1 x 512 54 / 55, 1 x 2048 110 / 106; 80 1 x 4096 208 / 195;
+// 128 2 x 2048 127 / 123; 256 4 x 4096 412 / 399.
 // Without the D skip the state's copy has two parts and a whole head's registers spill: halves always (2 x 2048 131 / 134 us, 4 x 4096 436 / 446, 5 x 4096 572 / 604).
 int scan_narrow_width(int headdim, int64_t heads, bool skip) { return headdim == 64 && skip && 2 * heads > sm_count() ? 64 : 32; }
 
